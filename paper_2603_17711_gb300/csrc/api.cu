@@ -96,6 +96,8 @@ struct ttn_ctx {
   float *mlp_x = nullptr, *mlp_ws = nullptr, *mlp_logits = nullptr;
   double* rs_norm = nullptr;
   uint64_t n_splits = 0;
+  double2* xs_planes = nullptr;  // leg / part planes of the FP64 tensor-core lists (xs_apply.cu)
+  int64_t xs_elems = 0;
   double2* rdm_vec = nullptr;
   double2* rho_dev = nullptr;
   int* flag_dev = nullptr;
@@ -230,7 +232,8 @@ struct Layout {
   int64_t tc_bsplit_floats = 0;  // FP32 mode only
   size_t tc_pool = 0, tc_off = 0;
   std::vector<int64_t> tc_off_host;  // float offset of each matrix in tc_pool, -1 if none
-  size_t svd_small = 0, rsvd = 0, mlp = 0;
+  size_t svd_small = 0, rsvd = 0, mlp = 0, xs = 0;
+  int64_t xs_elems = 0;
   // direct integration (vmf): committed state, per-node saves, 7 stage
   // derivatives (all as flat copies of the node region), edge scratch
   size_t vmf_y = 0, vmf_save = 0, vmf_k = 0, vmf_tmp = 0, vmf_r = 0, vmf_aug = 0, vmf_dmi = 0, vmf_x = 0,
@@ -295,6 +298,9 @@ Layout layout_of(const Plan& p, int prec) {
   L.rsvd = take(3 * p.theta_cap * sizeof(double2));
   L.mlp = take((24 + 13 + mlp_ws_floats(1) + 8) * sizeof(float) + 2 * sizeof(double));
   L.flag = take(sizeof(int) * 4);
+  // one plane per leg always fits; small nodes may cut their terms into more
+  L.xs_elems = std::max<int64_t>(4 * S, std::min<int64_t>(24 * p.P_cap_max, 1 << 20));
+  L.xs = take(L.xs_elems * sizeof(double2));
   if (prec == PREC_F64) {
     L.nodes_elems = acc;
     L.vmf_y = take(acc * sizeof(double2));
@@ -410,7 +416,20 @@ struct Exec {
       });
       return;
     }
-    run(kind, L.flops, [&] { launch_apply(h->prec, h->Tlo, L, e, s); });
+    run(kind, L.flops, [&] {
+      if (h->prec == PREC_F64)
+        apply64(L, e);
+      else
+        launch_apply(h->prec, h->Tlo, L, e, s);
+    });
+  }
+  // an FP64 list: large ones on the tensor cores (exact digit split), the others on the CUDA cores
+  void apply64(const ApList& L, const Epi& e) {
+    if (xs_applicable(L, p.ap_outs.data(), p.ap_terms.data()) &&
+        launch_apply_xs(h->h_bufs.data(), h->h_mats.data(), L, e, p.ap_outs.data(), p.ap_terms.data(), h->xs_planes,
+                        h->xs_elems, h->params.max_split, s))
+      return;
+    launch_apply(PREC_F64, h->T, L, e, s);
   }
   void store(int kind, int list) { apply(kind, list, Epi{EPI_STORE, nullptr, nullptr, nullptr, nullptr, 0.0}); }
 
@@ -455,8 +474,15 @@ struct Exec {
   void absorb(int v, int u) {
     const int li = p.tree.leg_index(v, u);
     const ApList& L = p.ap_lists[p.absorb[v][li]];
+    // the mixed form keeps the CUDA-core order of the sums: its FP32 roundings
+    // turn a last-bit difference here into one of 1e-7 within a few flows, so
+    // its trajectories stay reproducible only if the FP64 bits do
     run(3, L.flops, [&] {
-      launch_apply(PREC_F64, h->T, L, Epi{EPI_STORE, nullptr, nullptr, nullptr, nullptr, 0.0}, s);
+      const Epi store{EPI_STORE, nullptr, nullptr, nullptr, nullptr, 0.0};
+      if (h->prec == PREC_F64)
+        apply64(L, store);
+      else
+        launch_apply(PREC_F64, h->T, L, store, s);
     });
     run(3, 0.0, [&] { launch_copy(h->h_bufs[v], lo_copy(v), h->h_bufs[p.buf.tmp], p.P[v], s); });
   }
@@ -1169,6 +1195,8 @@ ttn_status ttn_set_workspace(ttn_t h, void* dptr, size_t bytes) {
     h->rdm_off = L.rdm_off;
     h->rho_dev = (double2*)(base + L.rho);
     h->flag_dev = (int*)(base + L.flag);
+    h->xs_planes = (double2*)(base + L.xs);
+    h->xs_elems = L.xs_elems;
     h->node_off = L.node_off;
     if (h->prec == PREC_F64) {
       h->vmf_n = L.nodes_elems;
@@ -2027,6 +2055,7 @@ ttn_status ttn_autotune(ttn_t h, int32_t reps) {
       if (!f64[i] && h->prec == PREC_F32 && h->params.tensor_cores &&
           tc_applicable(L, p.ap_outs.data(), p.ap_terms.data()))
         continue;
+      if (h->prec == PREC_F64 && xs_applicable(L, p.ap_outs.data(), p.ap_terms.data())) continue;
       const bool epi = p.ap_outs[L.out_begin].dst < 0;
       const TuneKey key = ap_key(p, L, prec);
       auto seen = done.find(key);

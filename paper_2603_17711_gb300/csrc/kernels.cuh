@@ -125,6 +125,22 @@ struct TcEmbedBatch {
 };
 int64_t tc_pool_floats(int d);
 void launch_tc_embed(void* const* mats32, const TcEmbedJob* jobs, int n, float* pool, cudaStream_t s);
+// FP64 lists on the tensor cores by an exact digit split (xs_apply.cu).
+// xs_applicable: the list qualifies (3 or 4 legs, contracted legs <= 64, all
+// outputs alike, work above kXsMinFlops). bufs / mats: host copies of the FP64
+// address tables (baked into the launch). planes: FP64 scratch of plane_elems
+// complex values (one-output lists: one plane per leg and term part, at most
+// max_split parts a leg). Returns
+// false (nothing launched) when the scratch or the launch's tables are too small.
+// The line: below about 8 MFLOP the CUDA-core launch is not bound by FP64 issue
+// and the second launch (plane sum) is not won back: 32x12x12, 12 terms (8.3
+// MFLOP) 16.6 us on the CUDA cores, 15.6 here; 19x11x11, 8 terms (2.1 MFLOP)
+// 8.7 / 13.3; 20^3, 12 terms (15 MFLOP) 26.7 / 13.5.
+constexpr double kXsMinFlops = 8.0e6;
+bool xs_applicable(const ApList& L, const ApOut* outs_host, const ApTerm* terms_host);
+bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L, const Epi& e,
+                     const ApOut* outs_host, const ApTerm* terms_host, double2* planes, int64_t plane_elems,
+                     int max_split, cudaStream_t s);
 void launch_project(int prec, const DevTables& T, const PjList& L, cudaStream_t s);
 // The same projections for wide bonds in the FP32 form (every output d x d
 // with d >= 32 and a reduction range of >= 1024 positions, all outputs of the

@@ -1,0 +1,620 @@
+// FP64 mode products on the tensor cores by an exact split into 8-bit digits.
+//
+// What bounds the FP64 contractions is the FP64 pipe: an SM sub-partition of
+// GB300 retires one FP64 warp instruction per 64-76 cycles (0.42 FMA/clk),
+// while a warp-level m16n8k16 f16 MMA (2048 multiply-adds, f32 accumulators)
+// takes 8.2 cycles, both measured. Here a real FP64 operand becomes a 62-bit
+// fixed-point integer, scaled by the largest exponent of its row (operator) or
+// fiber (tensor), and the integer eight signed 8-bit digits, held exactly in
+// f16. The product of two digits is below 2^14 and at most 8 * 128 of them
+// enter one f32 accumulator (2d <= 128, digit pairs i + j = g <= 7), so every
+// accumulator is an exact integer below 2^24: the only errors are the two
+// truncations at 2^-62 and the dropped digit pairs i + j > 7, together below
+// 2^-60 of (row maximum x fiber maximum), where a chain of FP64 FMAs loses
+// 2^-53 per addition. 36 digit products replace 64-cycle FMAs by MMAs at
+// 2048 * 592 / (36 * 8.2) = 4.1k multiply-adds per clock against 259 FMAs.
+//
+// One term Y += M x_l X (complex, d = d_l <= 64) is a real GEMM: output index
+// i gives rows i (real part) and i + 8 (imaginary part) of an MMA tile, leg
+// index x the two K columns (Re, Im), a position n of the other legs one N
+// column. A lane loads the complex values of its own fragment slots from
+// global memory (L1 / L2), so there is no shared-memory staging and no barrier
+// in the term loop; the digits live in registers. A warp owns 8 output indices x
+// 16 positions. Columns x of the operator block are first scaled to equal
+// size, the scale moved to the tensor operand: both fixed-point scales then
+// refer to the largest contribution |M[i][x]| |X[x][n]| and an operator whose
+// columns differ by many orders of magnitude loses nothing.
+//
+// A non-finite operand makes its whole row or column of outputs NaN.
+//
+// Measured (graph replay, CUDA-core kernel / this one): 64^3 node, 14 terms
+// 1785 / 273 us (6.9 TFLOP/s of FP64 results against the 1.1 of the FP64 pipe;
+// the tensor pipe is a third busy, the rest is operand latency and digit
+// arithmetic); 20^3, 12 terms 26.7 / 13.5 us; 20x25x25, 12 terms 40.6 / 21.4 us.
+// Relative 2-norm error against 128-bit sums: 1.15e-16 / 2.35e-16 (64^3),
+// 1.14e-16 / 1.70e-16 (20^3), 4.7e-17 / 1.4e-16 for a single product.
+#include <algorithm>
+#include <cstdint>
+
+#include <cuda_fp16.h>
+
+#include "kernels.cuh"
+
+namespace ttn {
+
+namespace {
+
+constexpr int kXsWarps = 8;
+constexpr int kXsThreads = 32 * kXsWarps;
+constexpr int kXsNT = 2;              // n tiles (8 positions) per warp
+constexpr int kXsCols = 8 * kXsNT;    // positions per warp
+constexpr int kXsTermSplit = 2;       // more terms than this on a leg: the warp groups split the terms
+constexpr int kXsMaxD = 64;           // 2 d <= 128: exactness of the f32 accumulators
+constexpr unsigned kFull = 0xffffffffu;
+
+__device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+__device__ __forceinline__ int exp_field(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+__device__ __forceinline__ int exp_c(double2 v) { return max(exp_field(v.x), exp_field(v.y)); }
+
+// v as a fixed-point integer with 62 bits below 2^(top + 1 - 1023), plus the
+// bias that turns its bytes into digits - 128 .. 127 offset by 128. Subnormal v is zero.
+__device__ __forceinline__ uint64_t fixed_biased(double v, int top) {
+  const uint64_t u = (uint64_t)__double_as_longlong(v);
+  const int e = (int)(u >> 52) & 0x7ff;
+  const uint64_t m = e == 0 ? 0ull : ((u & 0xfffffffffffffull) | 0x10000000000000ull) << 9;
+  const int s = min(max(top - e, 0), 63);
+  const uint64_t f = m >> s;
+  const uint64_t sg = (uint64_t)((int64_t)u >> 63);
+  return (f ^ sg) - sg + 0x8080808080808080ull;
+}
+// Digit i (0 = most significant) of the pair (re, im) as f16x2.
+template <int I>
+__device__ __forceinline__ uint32_t digit_pair(uint64_t re, uint64_t im) {
+  constexpr int b = 7 - I;
+  const uint32_t wr = b >= 4 ? (uint32_t)(re >> 32) : (uint32_t)re;
+  const uint32_t wi = b >= 4 ? (uint32_t)(im >> 32) : (uint32_t)im;
+  constexpr uint32_t sel = (uint32_t)(b & 3) | ((uint32_t)(4 + (b & 3)) << 8);  // byte 0: re, byte 2: im
+  uint32_t r = (__byte_perm(wr, wi, sel) & 0x00ff00ffu) | 0x64006400u;          // 1024 + byte
+  const __half2 h = __hsub2(*reinterpret_cast<__half2*>(&r), __half2half2(__ushort_as_half(0x6480)));  // - 1152
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+__device__ __forceinline__ void digits8(double2 v, int top, uint32_t (&d)[8]) {
+  const uint64_t re = fixed_biased(v.x, top), im = fixed_biased(v.y, top);
+  d[0] = digit_pair<0>(re, im);
+  d[1] = digit_pair<1>(re, im);
+  d[2] = digit_pair<2>(re, im);
+  d[3] = digit_pair<3>(re, im);
+  d[4] = digit_pair<4>(re, im);
+  d[5] = digit_pair<5>(re, im);
+  d[6] = digit_pair<6>(re, im);
+  d[7] = digit_pair<7>(re, im);
+}
+
+// sum_g C_g 2^(8 (7 - g)) times 2^ex, rounded to nearest, built from integers
+// (a conversion instruction would occupy the FP64 pipe as long as an FMA).
+__device__ __forceinline__ double join(const float (&c)[8], int ex) {
+  int C[8];
+#pragma unroll
+  for (int g = 0; g < 8; ++g) C[g] = __float2int_rn(c[g]);
+  // value = H 2^32 + l, |H| < 2^45: 96 bits, so no digit product is rounded before the end
+  const int64_t lo = (int64_t)C[4] * (1 << 24) + (int64_t)C[5] * (1 << 16) + (int64_t)C[6] * 256 + C[7];
+  int64_t H = (int64_t)C[0] * (1 << 24) + (int64_t)C[1] * (1 << 16) + (int64_t)C[2] * 256 + C[3] + (lo >> 32);
+  uint32_t l = (uint32_t)lo;
+  const uint64_t sg = (uint64_t)H & 0x8000000000000000ull;
+  if (H < 0) {
+    H = ~H + (l == 0 ? 1 : 0);
+    l = 0u - l;
+  }
+  if (H == 0) {  // leading digits cancelled: take the low word up
+    if (l == 0) return 0.0;
+    H = l;
+    l = 0;
+    ex -= 32;
+  }
+  const int lz = __clzll(H);  // >= 19
+  const uint64_t n = ((uint64_t)H << lz) | (lz >= 32 ? (uint64_t)l << (lz - 32) : (uint64_t)(l >> (32 - lz)));
+  const uint64_t m = (n >> 11) + ((n >> 10) & 1ull);
+  const int E = 1023 + 63 - lz + 32 + ex;
+  if (E <= 0) return 0.0;
+  if (E >= 0x7ff) return __longlong_as_double((long long)(sg | 0x7ff0000000000000ull));
+  return __longlong_as_double((long long)(sg | (((uint64_t)E << 52) + (m - 0x10000000000000ull))));
+}
+
+// One block product: 8 MT output indices (8 per warp of a group of MT warps) x 16
+// positions, K <= 8 MT complex K positions. The tensor operand's digits are
+// made once per group (warp m makes those of K positions 8m .. 8m+7) and
+// shared through shared memory; the operator's are made by the warp that uses
+// them.
+struct XsGroup {
+  int m, MT, bar;   // warp of the group, warps, named barrier
+  int* cx;          // [64] largest exponent of every operator column (group maximum)
+  int* col;         // [16] largest tensor exponent + cx of every position
+  int* craw;        // [16] largest raw tensor exponent (0x7ff: not finite)
+  uint4* bd;        // [MT][8][32] digits: x, y = K halves of positions 0..7, z, w = of positions 8..15
+};
+struct XsSrc {
+  const double2* a;  // operator row of this lane, or null
+  const double2* b[kXsNT];  // tensor fiber of this lane's positions, or null
+};
+__device__ __forceinline__ void gsync(const XsGroup& G) {
+  if (G.MT == 1)
+    __syncwarp();
+  else
+    asm volatile("bar.sync %0, %1;" ::"r"(G.bar), "r"(32 * G.MT) : "memory");
+}
+
+// acc += block product. PROJ: conj(A) instead of A.
+template <bool PROJ, typename KA, typename KB>
+__device__ __forceinline__ void xs_block(const XsGroup& G, const XsSrc& S, int K, KA ka, KB kb,
+                                         double (&acc)[kXsNT][4]) {
+  const int lane = threadIdx.x & 31, kq = lane & 3;
+  const double2 zero = make_double2(0.0, 0.0);
+  const int KS = (K + 7) >> 3;
+  // 1: raw tensor values of this warp's K positions; column exponents of the operator
+  double2 braw[kXsNT][2];
+#pragma unroll
+  for (int hf = 0; hf < 2; ++hf) {
+    const int k = G.m * 8 + 4 * hf + kq;
+#pragma unroll
+    for (int t = 0; t < kXsNT; ++t) braw[t][hf] = (k < K && S.b[t]) ? S.b[t][kb(k)] : zero;
+  }
+  int rraw = 0;
+  uint32_t ep[8];  // operator exponents of both K halves, so the operator is read once more only for its digits
+#pragma unroll
+  for (int ks = 0; ks < 8; ++ks) {
+    ep[ks] = 0;
+    if (ks < KS) {
+      const int k = ks * 8 + kq;
+      const int e0 = (k < K && S.a) ? exp_c(S.a[ka(k)]) : 0;
+      const int e1 = (k + 4 < K && S.a) ? exp_c(S.a[ka(k + 4)]) : 0;
+      ep[ks] = (uint32_t)e0 | ((uint32_t)e1 << 16);
+    }
+  }
+#pragma unroll
+  for (int ks = 0; ks < 8; ++ks)
+    if (ks < KS) {  // both halves' column maxima at once (packed 16-bit maxima)
+      uint32_t cx = ep[ks];
+      cx = __vmaxu2(cx, __shfl_xor_sync(kFull, cx, 4));
+      cx = __vmaxu2(cx, __shfl_xor_sync(kFull, cx, 8));
+      cx = __vmaxu2(cx, __shfl_xor_sync(kFull, cx, 16));
+      if (lane < 8) atomicMax(&G.cx[ks * 8 + lane], lane < 4 ? (int)(cx & 0xffff) : (int)(cx >> 16));
+      rraw = max(rraw, max((int)(ep[ks] & 0xffff), (int)(ep[ks] >> 16)));
+    }
+  gsync(G);
+  // 2: row scale of the scaled operator, position scales
+  int row = -4096;
+#pragma unroll
+  for (int ks = 0; ks < 8; ++ks)
+    if (ks < KS) {
+      const int e0 = ep[ks] & 0xffff, e1 = ep[ks] >> 16;
+      if (e0) row = max(row, e0 - G.cx[ks * 8 + kq]);
+      if (e1) row = max(row, e1 - G.cx[ks * 8 + 4 + kq]);
+    }
+  row = max(row, __shfl_xor_sync(kFull, row, 1));
+  row = max(row, __shfl_xor_sync(kFull, row, 2));
+  rraw = max(rraw, __shfl_xor_sync(kFull, rraw, 1));
+  rraw = max(rraw, __shfl_xor_sync(kFull, rraw, 2));
+  const int cb[2] = {G.cx[G.m * 8 + kq], G.cx[G.m * 8 + 4 + kq]};
+#pragma unroll
+  for (int t = 0; t < kXsNT; ++t) {
+    int c = 0, r = 0;
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+      const int eb = exp_c(braw[t][hf]);
+      if (eb && cb[hf]) c = max(c, eb + cb[hf]);
+      r = max(r, eb);
+    }
+    c = max(c, __shfl_xor_sync(kFull, c, 1));
+    c = max(c, __shfl_xor_sync(kFull, c, 2));
+    r = max(r, __shfl_xor_sync(kFull, r, 1));
+    r = max(r, __shfl_xor_sync(kFull, r, 2));
+    if (kq == 0) {
+      atomicMax(&G.col[8 * t + (lane >> 2)], c);
+      atomicMax(&G.craw[8 * t + (lane >> 2)], r);
+    }
+  }
+  gsync(G);
+  // 3: tensor digits of this warp's K positions
+  {
+    uint32_t d[kXsNT][2][8];
+#pragma unroll
+    for (int t = 0; t < kXsNT; ++t) {
+      const int top = G.col[8 * t + (lane >> 2)];
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf)  // a zero operator column contributes nothing whatever the tensor holds
+        digits8(cb[hf] ? braw[t][hf] : zero, top - cb[hf], d[t][hf]);
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) G.bd[(G.m * 8 + j) * 32 + lane] = make_uint4(d[0][0][j], d[0][1][j], d[1][0][j], d[1][1][j]);
+  }
+  gsync(G);
+  // 4: operator digits and MMAs
+  float c[kXsNT][8][4];
+#pragma unroll
+  for (int t = 0; t < kXsNT; ++t)
+#pragma unroll
+    for (int g = 0; g < 8; ++g)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) c[t][g][r] = 0.f;
+  auto ld_a = [&](int k) { return (k < K && S.a) ? S.a[ka(k)] : zero; };
+  double2 nv[2] = {ld_a(kq), ld_a(4 + kq)};
+#pragma unroll 1
+  for (int ks = 0; ks < KS; ++ks) {
+    uint32_t a[8][4];
+    const double2 v[2] = {nv[0], nv[1]};
+    if (ks + 1 < KS) {
+      nv[0] = ld_a(ks * 8 + 8 + kq);
+      nv[1] = ld_a(ks * 8 + 12 + kq);
+    }
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+      uint32_t ad[8];
+      digits8(v[hf], row + G.cx[ks * 8 + 4 * hf + kq], ad);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const uint32_t sw = __byte_perm(ad[i], ad[i], 0x1032);  // (im, re)
+        a[i][2 * hf] = PROJ ? ad[i] : ad[i] ^ 0x80000000u;      // (re, -+im)
+        a[i][2 * hf + 1] = PROJ ? sw ^ 0x00008000u : sw;        // (+-im, re)
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const uint4 b = G.bd[(ks * 8 + j) * 32 + lane];
+#pragma unroll
+      for (int i = 0; i + j < 8; ++i) {
+        mma_f16(c[0][i + j], a[i], b.x, b.y);
+        mma_f16(c[1][i + j], a[i], b.z, b.w);
+      }
+    }
+  }
+  // lane holds rows (lane >> 2) re / im of columns 2 kq, 2 kq + 1
+#pragma unroll
+  for (int t = 0; t < kXsNT; ++t)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int n = 8 * t + 2 * kq + j, ec = G.col[n];
+      const bool bad = rraw == 0x7ff || G.craw[n] == 0x7ff;
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        float cc[8];
+#pragma unroll
+        for (int g = 0; g < 8; ++g) cc[g] = c[t][g][2 * p + j];
+        // both fixed points: value = integer * 2^(scale - 1084); the digit pairs of
+        // group g weigh 2^(8 (14 - g)), 2^56 of it outside join()
+        acc[t][2 * j + p] += bad ? __longlong_as_double(0x7ff8000000000000ll) : join(cc, row + ec - 2 * 1084 + 56);
+      }
+    }
+  gsync(G);  // scales and digits consumed
+  for (int e = G.m * 32 + lane; e < 96; e += 32 * G.MT) G.cx[e] = 0;  // cx, col, craw: contiguous
+  gsync(G);
+}
+
+// Leg geometry: element = outer * (d * inner) + x * inner + in, position n = outer * inner + in.
+struct XsLeg {
+  int d, inner, rest;  // all below 2^30 (xs_applicable)
+};
+__device__ __forceinline__ XsLeg leg_of(const int (&dd)[4], int leg) {
+  XsLeg g;
+  g.d = dd[leg];
+  g.inner = 1;
+  for (int l = 3; l > leg; --l) g.inner *= dd[l];
+  g.rest = dd[0] * dd[1] * dd[2] * dd[3] / g.d;
+  return g;
+}
+
+}  // namespace
+
+// Work of one launch, passed by value: operands and term lists sit in the
+// constant bank, where a table in global memory costs three dependent L2 round
+// trips (about 1.4 us of a launch) before the first operand can be loaded.
+constexpr int kXsMaxTerms = 192, kXsMaxOuts = 96;
+struct XsTerm {
+  const double2* M;
+  const double2* X;
+};
+struct XsWork {
+  int dims[4];      // of every output
+  int leg;          // -1: one output, all legs, planes; -2: every output's terms share one leg; else this leg
+  // -1: CTAs [lt[l], lt[l+1]) of grid.x work on leg l, parts[l] term parts x
+  // tiles; part j writes plane plane[l] + j
+  int lt[5], parts[4], plane[4];
+  double2* planes;
+  double2* dst[kXsMaxOuts];
+  short tb[kXsMaxOuts][5];  // terms of output o on leg l: [tb[o][l], tb[o][l+1])
+  XsTerm term[kXsMaxTerms];
+};
+
+// CTA = (output, leg, tile, part). With MT = ceil(d / 8) row blocks the 8 warps
+// form G = 8 / MT groups; the groups split the terms (split_terms, one 16-position
+// tile per CTA, summed in group order through shared memory) or the positions
+// (one 16-position tile per group, no sum).
+__global__ void __launch_bounds__(kXsThreads, 2) k_xs_apply(const __grid_constant__ XsWork w) {
+  __shared__ __align__(16) uint4 sm_bd[kXsWarps * 8 * 32];  // digits; the groups' sums at the end
+  __shared__ int sm_sc[kXsWarps][96];
+  double2(*red)[kXsCols * 8] = reinterpret_cast<double2(*)[kXsCols * 8]>(sm_bd);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int o = blockIdx.y;
+  int leg = w.leg, bx = blockIdx.x, part = 0, nparts = 1;
+  const bool pl = leg == -1;
+  if (leg == -2) {
+    leg = 0;
+    while (leg < 3 && w.tb[o][leg + 1] == w.tb[o][0]) ++leg;
+  }
+  if (pl) {
+    leg = 0;
+    while (leg < 3 && bx >= w.lt[leg + 1]) ++leg;
+    nparts = w.parts[leg];
+    const int nt = (w.lt[leg + 1] - w.lt[leg]) / nparts;
+    bx -= w.lt[leg];
+    part = bx / nt;
+    bx = bx % nt;
+  }
+  const XsLeg g = leg_of(w.dims, leg);
+  const int MT = (g.d + 7) >> 3, G = kXsWarps / MT;
+  const int t_begin = w.tb[o][leg], nterm = w.tb[o][leg + 1] - t_begin;
+  const bool earlier = !pl && t_begin > w.tb[o][0];  // an earlier leg's launch wrote the destination
+  if (nterm == 0) return;  // uniform over the CTA
+  const bool split_terms = pl || nterm > kXsTermSplit;
+  const int tiles = (g.rest + kXsCols - 1) / kXsCols;
+  if (!split_terms && bx * G >= tiles) return;
+  const int mt = wid % MT, grp = wid / MT;
+  const int tile = split_terms ? bx : bx * G + grp;
+  const bool on = grp < G && tile < tiles;
+  double acc[kXsNT][4];
+#pragma unroll
+  for (int t = 0; t < kXsNT; ++t)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) acc[t][r] = 0.0;
+  const int i = mt * 8 + (lane >> 2);
+  const XsGroup gp{mt, MT, 1 + grp, sm_sc[grp], sm_sc[grp] + 64, sm_sc[grp] + 80, sm_bd + (size_t)grp * MT * 8 * 32};
+  for (int e = threadIdx.x; e < kXsWarps * 96; e += kXsThreads) sm_sc[0][e] = 0;
+  __syncthreads();
+  if (on) {
+    const int n_split = split_terms ? nparts * G : 1, me = split_terms ? part * G + grp : 0;
+    int boff[kXsNT];
+#pragma unroll
+    for (int t = 0; t < kXsNT; ++t) {
+      const int n = tile * kXsCols + 8 * t + (lane >> 2);
+      boff[t] = n < g.rest ? (n / g.inner) * (g.d * g.inner) + n % g.inner : -1;
+    }
+    const int inner = g.inner;
+    for (int q = me; q < nterm; q += n_split) {
+      const XsTerm tm = w.term[t_begin + q];
+      XsSrc S;
+      S.a = i < g.d ? tm.M + (int64_t)i * g.d : nullptr;
+#pragma unroll
+      for (int t = 0; t < kXsNT; ++t) S.b[t] = boff[t] >= 0 ? tm.X + boff[t] : nullptr;
+      xs_block<false>(gp, S, g.d, [](int k) { return k; }, [inner](int k) { return k * inner; }, acc);
+    }
+  }
+  double2* Y = pl ? w.planes + (int64_t)(w.plane[leg] + part) * ((int64_t)g.rest * g.d) : w.dst[o];
+  auto put = [&](int n, int ii, double2 v) {
+    if (n >= g.rest || ii >= g.d) return;
+    const int at = (n / g.inner) * (g.d * g.inner) + n % g.inner + ii * g.inner;
+    if (earlier) {
+      const double2 y = Y[at];
+      v.x += y.x;
+      v.y += y.y;
+    }
+    Y[at] = v;
+  };
+  if (!split_terms || G == 1) {
+    if (on)
+#pragma unroll
+      for (int t = 0; t < kXsNT; ++t)
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+          put(tile * kXsCols + 8 * t + 2 * (lane & 3) + j, i, make_double2(acc[t][2 * j], acc[t][2 * j + 1]));
+    return;
+  }
+  // groups added in order; slot = column * 8 + row of the block
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < kXsNT; ++t)
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      red[wid][(8 * t + 2 * (lane & 3) + j) * 8 + (lane >> 2)] = make_double2(acc[t][2 * j], acc[t][2 * j + 1]);
+  __syncthreads();
+  for (int e = threadIdx.x; e < MT * kXsCols * 8; e += kXsThreads) {
+    // consecutive threads along the faster of (row, position) in the destination
+    int cc, ii;
+    if (g.inner == 1) {
+      ii = e % (MT * 8);
+      cc = e / (MT * 8);
+    } else {
+      cc = e % kXsCols;
+      ii = e / kXsCols;
+    }
+    const int m = ii >> 3, slot = cc * 8 + (ii & 7);
+    double2 v = red[m][slot];
+    for (int q = 1; q < G; ++q) {
+      const double2 w = red[q * MT + m][slot];
+      v.x += w.x;
+      v.y += w.y;
+    }
+    put(tile * kXsCols + cc, ii, v);
+  }
+}
+
+// RK4 stage update of element e with the computed derivative k (kernels.cuh, Epi), FP64.
+__device__ __forceinline__ void rk_update(const Epi& ep, int64_t e, double2 k) {
+  const double2 y = ep.y[e];
+  double2* ys = (double2*)ep.ys;
+  const double h = ep.mode == EPI_RK3 ? ep.h : 0.5 * ep.h;
+  if (ep.mode == EPI_RK4) {
+    const double2 a = ep.acc[e];
+    const double w = ep.h / 6.0;
+    ep.y[e] = make_double2(y.x + w * (a.x + k.x), y.y + w * (a.y + k.y));
+    return;
+  }
+  if (ep.mode == EPI_RK1) {
+    ep.acc[e] = k;
+  } else {
+    const double2 a = ep.acc[e];
+    ep.acc[e] = make_double2(a.x + 2.0 * k.x, a.y + 2.0 * k.y);
+  }
+  ys[e] = make_double2(y.x + h * k.x, y.y + h * k.y);
+}
+
+// Sum of the planes of a one-output list, in order, and its epilogue.
+__global__ void __launch_bounds__(128) k_xs_epilogue(const double2* planes, int n_planes, int64_t P, Epi ep,
+                                                     double2* dst) {
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e >= P) return;
+  double2 k = planes[e];
+  for (int q = 1; q < n_planes; ++q) {
+    const double2 v = planes[(int64_t)q * P + e];
+    k.x += v.x;
+    k.y += v.y;
+  }
+  if (ep.mode == EPI_STORE) {
+    dst[e] = k;
+    return;
+  }
+  rk_update(ep, e, k);
+}
+
+namespace {
+
+int sm_count() {
+  static int n = [] {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1)
+      v = 152;
+    return v;
+  }();
+  return n;
+}
+
+}  // namespace
+
+// Lists that take this path: contracted legs of at most 64, all outputs alike,
+// fewer than 2^31 elements, and enough multiply-adds that the CUDA-core kernel
+// would be bound by FP64 issue instead of by its launch.
+bool xs_applicable(const ApList& L, const ApOut* outs, const ApTerm* terms) {
+  if (L.n_tiles <= 0) return false;
+  const ApOut& f = outs[L.out_begin];
+  const int64_t P = (int64_t)f.d0 * f.d1 * f.d2 * f.d3;
+  if (P >= (int64_t)1 << 30 || L.out_end - L.out_begin > 65535) return false;
+  for (int o = L.out_begin; o < L.out_end; ++o) {
+    const ApOut& u = outs[o];
+    if (u.d0 != f.d0 || u.d1 != f.d1 || u.d2 != f.d2 || u.d3 != f.d3) return false;
+    const int dd[4] = {u.d0, u.d1, u.d2, u.d3};
+    if (u.term_begin == u.term_end) return false;
+    for (int t = u.term_begin; t < u.term_end; ++t) {
+      const ApTerm& tm = terms[t];
+      if (tm.mat < 0 || tm.leg < 0 || tm.leg > 3 || dd[tm.leg] > kXsMaxD) return false;
+    }
+  }
+  return L.flops >= kXsMinFlops;
+}
+
+bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L, const Epi& e, const ApOut* outs,
+                     const ApTerm* terms, double2* planes, int64_t plane_elems, int max_split,
+                     cudaStream_t s) {
+  const int n_outs = L.out_end - L.out_begin;
+  const ApOut& u = outs[L.out_begin];
+  const int dd[4] = {u.d0, u.d1, u.d2, u.d3};
+  const int64_t P = (int64_t)u.d0 * u.d1 * u.d2 * u.d3;
+  int nterm[4] = {0, 0, 0, 0};
+  bool multi_leg = false;
+  for (int o = L.out_begin; o < L.out_end; ++o)
+    for (int t = outs[o].term_begin; t < outs[o].term_end; ++t) {
+      ++nterm[terms[t].leg];
+      multi_leg = multi_leg || terms[t].leg != terms[outs[o].term_begin].leg;
+    }
+  int tiles[4];
+  for (int l = 0; l < 4; ++l) tiles[l] = (int)((P / dd[l] + kXsCols - 1) / kXsCols);
+  XsWork gr{};
+  if (n_outs > kXsMaxOuts || outs[L.out_end - 1].term_end - outs[L.out_begin].term_begin > kXsMaxTerms) return false;
+  int nq = 0;
+  for (int i = 0; i < 4; ++i) gr.dims[i] = dd[i];
+  for (int o = 0; o < n_outs; ++o) {
+    const ApOut& v = outs[L.out_begin + o];
+    gr.dst[o] = v.dst >= 0 ? bufs[v.dst] : nullptr;
+    gr.tb[o][0] = (short)nq;
+    for (int l = 0; l < 4; ++l) {
+      for (int t = v.term_begin; t < v.term_end; ++t)
+        if (terms[t].leg == l) gr.term[nq++] = XsTerm{mats[terms[t].mat], bufs[terms[t].src]};
+      gr.tb[o][l + 1] = (short)nq;
+    }
+  }
+  if (n_outs == 1) {
+    // all legs in one launch, each leg's terms cut into parts while a warp
+    // still has more than one term and the launch stays below four CTAs per SM
+    // (two are resident at a time)
+    int ctas = 0, n_planes = 0, groups[4];
+    for (int l = 0; l < 4; ++l) {
+      groups[l] = kXsWarps / ((dd[l] + 7) / 8);
+      gr.parts[l] = 1;
+      if (nterm[l]) {
+        ctas += tiles[l];
+        ++n_planes;
+      }
+    }
+    if ((int64_t)n_planes * P > plane_elems) return false;
+    for (;;) {
+      int best = -1;
+      double chain = 1.0;
+      for (int l = 0; l < 4; ++l) {
+        const int q = groups[l] * gr.parts[l];
+        const double c = (double)((nterm[l] + q - 1) / q) * ((dd[l] + 7) / 8);
+        if (nterm[l] > q && gr.parts[l] < max_split && c > chain) {
+          chain = c;
+          best = l;
+        }
+      }
+      if (best < 0 || ctas + tiles[best] > 4 * sm_count() || (int64_t)(n_planes + 1) * P > plane_elems) break;
+      ++gr.parts[best];
+      ctas += tiles[best];
+      ++n_planes;
+    }
+    int q = 0;
+    for (int l = 0; l < 4; ++l) {
+      gr.plane[l] = q;
+      gr.lt[l + 1] = gr.lt[l] + (nterm[l] ? tiles[l] * gr.parts[l] : 0);
+      if (nterm[l]) q += gr.parts[l];
+    }
+    gr.leg = -1;
+    gr.planes = planes;
+    k_xs_apply<<<dim3(gr.lt[4], 1), kXsThreads, 0, s>>>(gr);
+    k_xs_epilogue<<<(int)((P + 127) / 128), 128, 0, s>>>(planes, q, P, e, gr.dst[0]);
+    return true;
+  }
+  if (e.mode != EPI_STORE) return false;
+  // several outputs: one launch when no output has terms on two legs, else one
+  // launch per leg, later legs adding to what earlier ones wrote. Outputs of
+  // at most two terms a leg use the groups for positions, so fewer CTAs.
+  int most[4] = {0, 0, 0, 0};
+  for (int o = L.out_begin; o < L.out_end; ++o) {
+    int c[4] = {0, 0, 0, 0};
+    for (int t = outs[o].term_begin; t < outs[o].term_end; ++t) ++c[terms[t].leg];
+    for (int l = 0; l < 4; ++l) most[l] = std::max(most[l], c[l]);
+  }
+  int gx[4], gmax = 0;
+  for (int l = 0; l < 4; ++l) {
+    const int G = kXsWarps / ((dd[l] + 7) / 8);
+    gx[l] = nterm[l] == 0 ? 0 : most[l] > kXsTermSplit ? tiles[l] : (tiles[l] + G - 1) / G;
+    gmax = std::max(gmax, gx[l]);
+  }
+  if (!multi_leg) {
+    gr.leg = -2;
+    k_xs_apply<<<dim3(gmax, n_outs), kXsThreads, 0, s>>>(gr);
+    return true;
+  }
+  for (int l = 0; l < 4; ++l)
+    if (nterm[l]) {
+      gr.leg = l;
+      k_xs_apply<<<dim3(gx[l], n_outs), kXsThreads, 0, s>>>(gr);
+    }
+  return true;
+}
+
+}  // namespace ttn
