@@ -374,6 +374,14 @@ struct Exec {
   cudaStream_t s;
   explicit Exec(ttn_t hh) : h(hh), p(hh->plan), s(hh->stream) {}
 
+  HostTables ht_64() const {
+    return HostTables{(void* const*)h->h_bufs.data(), (void* const*)h->h_mats.data(), p.ap_outs.data(),
+                      p.ap_terms.data(), p.pj_outs.data()};
+  }
+  HostTables ht_lo() const {
+    return HostTables{h->h_bufs_lo.data(), h->h_mats_lo.data(), p.ap_outs.data(), p.ap_terms.data(), p.pj_outs.data()};
+  }
+
   // account one kernel launch of class `kind` and, when profiling, bracket it
   // with CUDA events on the handle's stream
   template <typename F>
@@ -411,7 +419,7 @@ struct Exec {
                              h->tc_pool_on ? h->tc_pool : nullptr, h->tc_pool_on ? h->tc_off_dev : nullptr, s,
                              h->tc_off.data(), ring ? h->tc_bsplit : nullptr, ring ? h->tc_bsplit_floats : 0,
                              &used_ring))
-          launch_apply(h->prec, h->Tlo, L, e, s);
+          launch_apply(h->prec, h->Tlo, ht_lo(), L, e, s);
         if (used_ring) ++h->n_ring;
       });
       return;
@@ -420,7 +428,7 @@ struct Exec {
       if (h->prec == PREC_F64)
         apply64(L, e);
       else
-        launch_apply(h->prec, h->Tlo, L, e, s);
+        launch_apply(h->prec, h->Tlo, ht_lo(), L, e, s);
     });
   }
   // an FP64 list: large ones on the tensor cores (exact digit split), the others on the CUDA cores
@@ -429,7 +437,7 @@ struct Exec {
         launch_apply_xs(h->h_bufs.data(), h->h_mats.data(), L, e, p.ap_outs.data(), p.ap_terms.data(), h->xs_planes,
                         h->xs_elems, h->params.max_split, s))
       return;
-    launch_apply(PREC_F64, h->T, L, e, s);
+    launch_apply(PREC_F64, h->T, ht_64(), L, e, s);
   }
   void store(int kind, int list) { apply(kind, list, Epi{EPI_STORE, nullptr, nullptr, nullptr, nullptr, 0.0}); }
 
@@ -444,7 +452,7 @@ struct Exec {
       const int dq = q.leg == 0 ? q.d0 : q.leg == 1 ? q.d1 : q.d2;
       const int64_t nrest = (int64_t)q.d0 * q.d1 * q.d2 / dq;
       run(1, L.flops, [&] {
-        if (!launch_project_tiled(h->prec, h->Tlo, L, dq, nrest, p.sm_count, s)) launch_project(h->prec, h->Tlo, L, s);
+        if (!launch_project_tiled(h->prec, h->Tlo, L, dq, nrest, p.sm_count, s)) launch_project(h->prec, h->Tlo, ht_lo(), L, s);
       });
       if (h->tc_pool_on) {
         const int d = p.dims[a][p.tree.leg_index(a, b)];  // current rank of the bond
@@ -482,7 +490,7 @@ struct Exec {
       if (h->prec == PREC_F64)
         apply64(L, store);
       else
-        launch_apply(PREC_F64, h->T, L, store, s);
+        launch_apply(PREC_F64, h->T, ht_64(), L, store, s);
     });
     run(3, 0.0, [&] { launch_copy(h->h_bufs[v], lo_copy(v), h->h_bufs[p.buf.tmp], p.P[v], s); });
   }
@@ -1017,6 +1025,7 @@ ttn_status ttn_create(const ttn_tree* tree, const int32_t* leg_dims, const int32
     else
       cudaGetLastError();
   }
+  h->plan.fp64 = precision == TTN_FP64;
   try {
     e = h->plan.build(tree->n_nodes, tree->parent, tree->n_legs, tree->leg_node, leg_dims, ranks);
   } catch (...) {
@@ -2021,6 +2030,7 @@ ttn_status ttn_autotune(ttn_t h, int32_t reps) {
     if (reps < 1 || reps > 100) return h->fail(TTN_EINVAL, "reps must be 1..100");
     Plan& p = h->plan;
     cudaStream_t s = h->stream;
+    Exec ex(h);
     std::vector<char> f64(p.ap_lists.size(), 0);  // absorb lists run in FP64 in both forms
     for (const auto& a : p.absorb)
       for (int id : a)
@@ -2052,6 +2062,7 @@ ttn_status ttn_autotune(ttn_t h, int32_t reps) {
       if (L.n_tiles <= 0) continue;
       const int prec = f64[i] ? PREC_F64 : h->prec;
       const DevTables& T = f64[i] ? h->T : h->Tlo;
+      const HostTables H = f64[i] ? ex.ht_64() : ex.ht_lo();
       if (!f64[i] && h->prec == PREC_F32 && h->params.tensor_cores &&
           tc_applicable(L, p.ap_outs.data(), p.ap_terms.data()))
         continue;
@@ -2076,7 +2087,7 @@ ttn_status ttn_autotune(ttn_t h, int32_t reps) {
           L2.w = w;
           L2.k = k;
           L2.useful = useful;
-          const float t = time_of([&] { launch_apply(prec, T, L2, epi ? rk1 : store, s); });
+          const float t = time_of([&] { launch_apply(prec, T, H, L2, epi ? rk1 : store, s); });
           if (t < 0.97f * tb) {
             tb = t;
             best_w = w;
@@ -2108,7 +2119,7 @@ ttn_status ttn_autotune(ttn_t h, int32_t reps) {
       for (int k = 1; k <= kmax; ++k) {
         PjList L2 = L;
         L2.k = k;
-        const float t = time_of([&] { launch_project(h->prec, h->Tlo, L2, s); });
+        const float t = time_of([&] { launch_project(h->prec, h->Tlo, ex.ht_lo(), L2, s); });
         if (t < 0.97f * tb) {
           tb = t;
           best = k;

@@ -82,7 +82,56 @@ template <> struct Cx<float> {
 // make a small contraction fast; when many lists run at once (batched
 // instances) fewer warps per tile waste less on idle warps and reductions.
 // NW (warps per CTA: 2, 4 or 8) and k are chosen per list (ApList::w, k).
+//
+// A small launch is a latency chain, so the chain is kept short: job tables in
+// the constant bank (three dependent L2 reads saved), the next unit of a warp by
+// addition instead of a modulo per term, real and imaginary sums on two
+// sub-partitions, the stage update's state and accumulator loaded before the
+// sum, its step coefficient divided on the host. Same sums in the same order.
+// Measured in the rank-10 spin-boson train: 8-CTA bond lists 5.0 -> 3.9 us,
+// 1-CTA lists 5.0 -> 3.6 us; rank-20 chain, 160-CTA lists 6.1 -> 4.6 us, 500-CTA
+// (FP64-issue bound) 20 -> 20 us.
 // ---------------------------------------------------------------------------
+
+// Job tables as seen by the kernels: in global memory (any list), or as kernel
+// parameters (lists of at most NT terms and NO outputs, all addresses resolved).
+template <typename V>
+struct ApTermV {
+  const V* M;  // null: identity
+  const V* X;
+  int leg;
+  int diag;  // ApTerm::pad: packed diagonals of a sparse operator, 0: dense
+};
+template <typename V>
+struct ApOutV {
+  int d0, d1, d2, d3, tb, te, tile0;
+  V* dst;
+};
+template <typename V>
+struct ApMem {
+  DevTables T;
+  __device__ __forceinline__ int find(const ApList& L, int tile) const {
+    return list_output(T.outs, L.out_begin, L.out_end, L.tpo, tile);
+  }
+  __device__ __forceinline__ ApOutV<V> out(int o) const {
+    const ApOut u = T.outs[o];
+    return ApOutV<V>{u.d0, u.d1, u.d2, u.d3, u.term_begin, u.term_end, u.tile0, u.dst >= 0 ? (V*)T.bufs[u.dst] : nullptr};
+  }
+  __device__ __forceinline__ ApTermV<V> term(int t) const {
+    const ApTerm a = T.terms[t];
+    return ApTermV<V>{a.mat < 0 ? nullptr : (const V*)T.mats[a.mat], (const V*)T.bufs[a.src], a.leg, a.pad};
+  }
+};
+template <typename V, int NT, int NO>
+struct ApPar {
+  ApOutV<V> outs[NO];
+  ApTermV<V> terms[NT];
+  __device__ __forceinline__ int find(const ApList& L, int tile) const {
+    return list_output(outs, 0, L.out_end - L.out_begin, L.tpo, tile);
+  }
+  __device__ __forceinline__ const ApOutV<V>& out(int o) const { return outs[o]; }
+  __device__ __forceinline__ const ApTermV<V>& term(int t) const { return terms[t]; }
+};
 
 // Leg geometry of one output element (kept in registers: selected by switch,
 // never indexed dynamically).
@@ -91,37 +140,44 @@ struct Geo {
   int i0, i1, i2, i3;
   int64_t s0, s1, s2;  // s3 = 1
 };
-
-template <typename R>
-__device__ __forceinline__ int term_dim(const ApTerm& term, const Geo& g) {
-  switch (term.leg) {
-    case 0: return g.d0;
-    case 1: return g.d1;
-    case 2: return g.d2;
-    default: return g.d3;
-  }
-}
-
-// contribution of positions [x0, x0 + kApChunk) of one term (the whole term if identity)
-template <typename R>
-__device__ __forceinline__ typename Cx<R>::T unit_dot(const ApTerm& term, const DevTables& T, int64_t idx,
-                                                      const Geo& g, int x0) {
-  using C = Cx<R>;
-  using V = typename C::T;
-  const V* __restrict__ src = (const V*)T.bufs[term.src];
-  if (term.mat < 0) return src[idx];
-  const V* __restrict__ M = (const V*)T.mats[term.mat];
-  int dl, il;
-  int64_t stride;
-  switch (term.leg) {
+__device__ __forceinline__ void geo_leg(const Geo& g, int leg, int& dl, int& il, int64_t& stride) {
+  switch (leg) {
     case 0: dl = g.d0; il = g.i0; stride = g.s0; break;
     case 1: dl = g.d1; il = g.i1; stride = g.s1; break;
     case 2: dl = g.d2; il = g.i2; stride = g.s2; break;
     default: dl = g.d3; il = g.i3; stride = 1; break;
   }
-  const V* __restrict__ row = M + (int64_t)il * dl;
-  const V* __restrict__ col = src + (idx - (int64_t)il * stride);
+}
+
+// contribution of positions [x0, x0 + kApChunk) of one term (the whole term if
+// identity or sparse)
+template <typename R>
+__device__ __forceinline__ typename Cx<R>::T unit_dot(const ApTermV<typename Cx<R>::T>& term, int64_t idx, const Geo& g,
+                                                      int x0) {
+  using C = Cx<R>;
+  using V = typename C::T;
+  if (!term.M) return term.X[idx];
+  int dl, il;
+  int64_t stride;
+  geo_leg(g, term.leg, dl, il, stride);
+  const V* __restrict__ row = term.M + (int64_t)il * dl;
+  const V* __restrict__ col = term.X + (idx - (int64_t)il * stride);
   V mv[kApChunk], sv[kApChunk];
+  if (sizeof(R) == 8 && term.diag) {  // at most three diagonals: x = il + offset
+    const int nd = term.diag >> 24;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int x = il + (int)(int8_t)(term.diag >> (8 * k));
+      const bool in = k < nd && x >= 0 && x < dl;
+      mv[k] = in ? row[x] : C::zero();
+      sv[k] = in ? col[(int64_t)x * stride] : C::zero();
+    }
+    V acc = C::zero();
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      if (k < nd) acc = C::fma(mv[k], sv[k], acc);
+    return acc;
+  }
 #pragma unroll
   for (int k = 0; k < kApChunk; ++k) {
     const int x = x0 + k;
@@ -137,25 +193,98 @@ __device__ __forceinline__ typename Cx<R>::T unit_dot(const ApTerm& term, const 
   return acc;
 }
 
+// Sum of n per-warp (or per-CTA) partials of one tile, in order: warp 0 adds the
+// real parts, warp 1 the imaginary parts. An FP64 addition holds an SM
+// sub-partition for 64 cycles whatever the lane count, so the two components
+// on two sub-partitions take half the time of one warp adding complex values,
+// with the same sums; the epilogue follows the same split.
+template <typename R>
+__device__ __forceinline__ R comp_sum(const typename Cx<R>::T (*part)[32], int n) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  R acc = R(0);
+  if (wid < 2) {
+    const R* p = reinterpret_cast<const R*>(part) + 2 * lane + wid;
+    acc = p[0];
+    for (int w = 1; w < n; ++w) acc += p[64 * w];
+  }
+  return acc;
+}
+
 // Sum of one output tile over the units of CTA `rank` of the k sharing it;
-// the CTA's total (fixed order over warps) is returned in warp 0.
-template <typename R, int NW>
-__device__ __forceinline__ typename Cx<R>::T tile_sum(const DevTables& T, const ApList& L, int tile, int rank, int K,
-                                                      typename Cx<R>::T (*part)[32], ApOut& out, int64_t& idx,
-                                                      int64_t& P) {
+// the CTA's total (fixed order over warps) is returned in warps 0 (real part)
+// and 1 (imaginary part).
+template <typename R, int NW, typename TAB>
+__device__ __forceinline__ R tile_sum(const TAB& tab, const ApOutV<typename Cx<R>::T>& out, const Geo& g,
+                                                      int64_t idx, bool in, int rank, int K,
+                                                      typename Cx<R>::T (*part)[32]) {
   using C = Cx<R>;
   using V = typename C::T;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  out = T.outs[list_output(T.outs, L.out_begin, L.out_end, L.tpo, tile)];
+  V acc = C::zero();
+  const int W = K * NW;
+  int off = rank * NW + wid;  // this warp's first unit, relative to the current term's
+  for (int t = out.tb; t < out.te; ++t) {
+    const ApTermV<V> term = tab.term(t);
+    int nch = 1;
+    if (term.M && !(sizeof(R) == 8 && term.diag)) {
+      const int dl = term.leg == 0 ? g.d0 : term.leg == 1 ? g.d1 : term.leg == 2 ? g.d2 : g.d3;
+      nch = (dl + kApChunk - 1) / kApChunk;
+    }
+    int c = off;
+    for (; c < nch; c += W)
+      if (in) acc = C::add(acc, unit_dot<R>(term, idx, g, c * kApChunk));
+    off = c - nch;
+  }
+  part[wid][lane] = acc;
+  __syncthreads();
+  return comp_sum<R>(part, NW);
+}
+
+// Epilogue of one component of one output element (warp `comp` of the CTA
+// owning the tile; at = 2 idx + comp); y0, a0: the state and the stage
+// accumulator, loaded ahead of the sum.
+template <typename R>
+__device__ __forceinline__ void tile_store(R* dst, const Epi& ep, int64_t at, R acc, double y0, double a0) {
+  if (ep.mode == EPI_STORE) {
+    dst[at] = acc;
+    return;
+  }
+  const double k = acc;
+  if (ep.mode == EPI_RK4) {
+    const double yn = y0 + ep.c * (a0 + k);
+    ((double*)ep.y)[at] = yn;
+    if ((void*)ep.y_lo != (void*)ep.y) ((R*)ep.y_lo)[at] = (R)yn;
+    return;
+  }
+  ((double*)ep.acc)[at] = ep.mode == EPI_RK1 ? k : a0 + 2.0 * k;
+  ((R*)ep.ys)[at] = (R)(y0 + ep.c * k);
+}
+
+template <typename R, int NW, typename TAB>
+__global__ void __launch_bounds__(32 * NW, 32 / NW) k_apply(const __grid_constant__ TAB tab, ApList L, Epi ep) {
+  using C = Cx<R>;
+  using V = typename C::T;
+  __shared__ V part[NW][32];
+  __shared__ V slot[kMaxSplit][32];
+  const int K = L.k;
+  const int tile = blockIdx.x / K, rank = blockIdx.x % K;  // rank == block rank in the cluster
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const ApOutV<V> out = tab.out(tab.find(L, tile));
   Geo g;
   g.d0 = out.d0; g.d1 = out.d1; g.d2 = out.d2; g.d3 = out.d3;
   g.s2 = g.d3;
   g.s1 = (int64_t)g.d2 * g.d3;
   g.s0 = g.s1 * g.d1;
-  P = g.s0 * g.d0;
-  idx = (int64_t)(tile - out.tile0) * kApTile + lane;
-  V acc = C::zero();
-  if (idx < P) {
+  const int64_t P = g.s0 * g.d0, idx = (int64_t)(tile - out.tile0) * kApTile + lane;
+  const bool in = idx < P;
+  g.i0 = g.i1 = g.i2 = g.i3 = 0;
+  const int64_t at = 2 * idx + (wid & 1);
+  double y0 = 0.0, a0 = 0.0;
+  if (in) {
+    if (ep.mode != EPI_STORE && wid < 2 && rank == 0) {
+      y0 = ((const double*)ep.y)[at];
+      if (ep.mode != EPI_RK1) a0 = ((const double*)ep.acc)[at];
+    }
     if (P <= 0x7fffffff) {  // every tensor of these trees: 32-bit index arithmetic
       const unsigned x = (unsigned)idx, s1 = (unsigned)g.s1, s2 = (unsigned)g.s2;
       const unsigned q2 = x / s2, q1 = x / s1;
@@ -169,90 +298,22 @@ __device__ __forceinline__ typename Cx<R>::T tile_sum(const DevTables& T, const 
       g.i2 = (int)((idx / g.s2) % g.d2);
       g.i3 = (int)(idx % g.d3);
     }
-    const int W = K * NW, me = rank * NW + wid;
-    int u = 0;  // index of the term's first unit in the tile's unit list
-    for (int t = out.term_begin; t < out.term_end; ++t) {
-      const ApTerm term = T.terms[t];
-      const int nch = term.mat < 0 ? 1 : (term_dim<R>(term, g) + kApChunk - 1) / kApChunk;
-      for (int c = ((me - u) % W + W) % W; c < nch; c += W)
-        acc = C::add(acc, unit_dot<R>(term, T, idx, g, c * kApChunk));
-      u += nch;
-    }
   }
-  part[wid][lane] = acc;
-  __syncthreads();
-  if (wid == 0) {
-    acc = part[0][lane];
-    for (int w = 1; w < NW; ++w) acc = C::add(acc, part[w][lane]);
-  }
-  __syncthreads();  // part may be reused by the caller's next tile
-  return acc;
-}
-
-// Epilogue of one output element (warp 0 of the CTA owning the tile).
-template <typename R>
-__device__ __forceinline__ void tile_store(const DevTables& T, const ApOut& out, const Epi& ep, int64_t idx,
-                                           typename Cx<R>::T acc) {
-  using C = Cx<R>;
-  using V = typename C::T;
-  if (ep.mode == EPI_STORE) {
-    ((V*)T.bufs[out.dst])[idx] = acc;
-    return;
-  }
-  const double2 k = C::wide(acc);
-  double2* __restrict__ y = ep.y;
-  double2* __restrict__ ac = ep.acc;
-  V* __restrict__ ys = (V*)ep.ys;
-  const double h = ep.h;
-  switch (ep.mode) {
-    case EPI_RK1:
-      ac[idx] = k;
-      ys[idx] = C::narrow(cadd(y[idx], cscale(0.5 * h, k)));
-      break;
-    case EPI_RK2:
-      ac[idx] = cadd(ac[idx], cscale(2.0, k));
-      ys[idx] = C::narrow(cadd(y[idx], cscale(0.5 * h, k)));
-      break;
-    case EPI_RK3:
-      ac[idx] = cadd(ac[idx], cscale(2.0, k));
-      ys[idx] = C::narrow(cadd(y[idx], cscale(h, k)));
-      break;
-    default: {
-      const double2 yn = cadd(y[idx], cscale(h / 6.0, cadd(ac[idx], k)));
-      y[idx] = yn;
-      if ((void*)ep.y_lo != (void*)ep.y) ((V*)ep.y_lo)[idx] = C::narrow(yn);
-      break;
-    }
-  }
-}
-
-template <typename R, int NW>
-__global__ void __launch_bounds__(32 * NW, 32 / NW) k_apply(DevTables T, ApList L, Epi ep) {
-  using C = Cx<R>;
-  using V = typename C::T;
-  __shared__ V part[NW][32];
-  __shared__ V slot[kMaxSplit][32];
-  const int K = L.k;
-  const int tile = blockIdx.x / K, rank = blockIdx.x % K;  // rank == block rank in the cluster
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  ApOut out;
-  int64_t idx, P;
-  V acc = tile_sum<R, NW>(T, L, tile, rank, K, part, out, idx, P);
+  R acc = tile_sum<R, NW>(tab, out, g, idx, in, rank, K, part);
   if (K > 1) {
     cg::cluster_group cluster = cg::this_cluster();
-    if (wid == 0 && rank > 0) cluster.map_shared_rank(&slot[0][0], 0)[rank * 32 + lane] = acc;
+    if (wid < 2) reinterpret_cast<R*>(cluster.map_shared_rank(&slot[0][0], 0))[rank * 64 + 2 * lane + wid] = acc;
     cluster.sync();
     if (rank > 0) return;
-    if (wid == 0)
-      for (int r = 1; r < K; ++r) acc = C::add(acc, slot[r][lane]);
+    acc = comp_sum<R>(slot, K);
   }
-  if (wid != 0 || idx >= P) return;
-  tile_store<R>(T, out, ep, idx, acc);
+  if (wid > 1 || !in) return;
+  tile_store<R>(reinterpret_cast<R*>(out.dst), ep, at, acc, y0, a0);
 }
 
 // Launch n_tiles * k CTAs; k > 1 makes every k consecutive CTAs one cluster.
 template <typename Kern, typename... Args>
-static void launch_split(Kern kern, int n_tiles, int k, int warps, cudaStream_t s, Args... args) {
+static void launch_split(Kern kern, int n_tiles, int k, int warps, cudaStream_t s, const Args&... args) {
   if (k <= 1) {
     kern<<<n_tiles, 32 * warps, 0, s>>>(args...);
     return;
@@ -272,21 +333,49 @@ static void launch_split(Kern kern, int n_tiles, int k, int warps, cudaStream_t 
   cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-template <typename R>
-static void launch_apply_w(const DevTables& T, const ApList& L, const Epi& e, cudaStream_t s) {
+template <typename R, typename TAB>
+static void launch_apply_w(const TAB& tab, const ApList& L, const Epi& e, cudaStream_t s) {
   switch (L.w) {
-    case 2: launch_split(k_apply<R, 2>, L.n_tiles, L.k, 2, s, T, L, e); break;
-    case 4: launch_split(k_apply<R, 4>, L.n_tiles, L.k, 4, s, T, L, e); break;
-    default: launch_split(k_apply<R, 8>, L.n_tiles, L.k, 8, s, T, L, e); break;
+    case 2: launch_split(k_apply<R, 2, TAB>, L.n_tiles, L.k, 2, s, tab, L, e); break;
+    case 4: launch_split(k_apply<R, 4, TAB>, L.n_tiles, L.k, 4, s, tab, L, e); break;
+    default: launch_split(k_apply<R, 8, TAB>, L.n_tiles, L.k, 8, s, tab, L, e); break;
   }
 }
 
-void launch_apply(int prec, const DevTables& T, const ApList& L, const Epi& e, cudaStream_t s) {
+template <typename R, int NT, int NO>
+static bool apply_par(const HostTables& H, const ApList& L, const Epi& e, cudaStream_t s) {
+  using V = typename Cx<R>::T;
+  const int t0 = H.outs[L.out_begin].term_begin, t1 = H.outs[L.out_end - 1].term_end;
+  if (L.out_end - L.out_begin > NO || t1 - t0 > NT) return false;
+  ApPar<V, NT, NO> tab{};
+  for (int o = L.out_begin; o < L.out_end; ++o) {
+    const ApOut& u = H.outs[o];
+    tab.outs[o - L.out_begin] = ApOutV<V>{u.d0, u.d1, u.d2, u.d3, u.term_begin - t0, u.term_end - t0, u.tile0,
+                                          u.dst >= 0 ? (V*)H.bufs[u.dst] : nullptr};
+  }
+  for (int t = t0; t < t1; ++t) {
+    const ApTerm& a = H.terms[t];
+    tab.terms[t - t0] = ApTermV<V>{a.mat < 0 ? nullptr : (const V*)H.mats[a.mat], (const V*)H.bufs[a.src], a.leg, a.pad};
+  }
+  launch_apply_w<R>(tab, L, e, s);
+  return true;
+}
+
+// Three parameter sizes (a launch's parameters are copied whole), then the tables in memory.
+template <typename R>
+static void launch_apply_r(const DevTables& T, const HostTables& H, const ApList& L, const Epi& e, cudaStream_t s) {
+  if (apply_par<R, 12, 4>(H, L, e, s)) return;
+  if (apply_par<R, 32, 32>(H, L, e, s)) return;
+  if (apply_par<R, 120, 40>(H, L, e, s)) return;
+  launch_apply_w<R>(ApMem<typename Cx<R>::T>{T}, L, e, s);
+}
+
+void launch_apply(int prec, const DevTables& T, const HostTables& H, const ApList& L, const Epi& e, cudaStream_t s) {
   if (L.n_tiles <= 0) return;
   if (prec == PREC_F32)
-    launch_apply_w<float>(T, L, e, s);
+    launch_apply_r<float>(T, H, L, with_coef(e), s);
   else
-    launch_apply_w<double>(T, L, e, s);
+    launch_apply_r<double>(T, H, L, with_coef(e), s);
 }
 
 // ---------------------------------------------------------------------------
@@ -299,8 +388,31 @@ void launch_apply(int prec, const DevTables& T, const ApList& L, const Epi& e, c
 // ---------------------------------------------------------------------------
 constexpr int kPjWarps = kSplitWarps;
 
-template <typename R>
-__global__ void __launch_bounds__(32 * kPjWarps, 4) k_project(DevTables T, PjList L) {
+template <typename V>
+struct PjOutV {
+  int d0, d1, d2, leg, tile0;
+  const V* u;
+  const V* w;
+  V* dst;
+};
+template <typename V>
+struct PjMem {
+  DevTables T;
+  __device__ __forceinline__ PjOutV<V> out(const PjList& L, int tile) const {
+    const PjOut p = T.pjs[list_output(T.pjs, L.out_begin, L.out_end, L.tpo, tile)];
+    return PjOutV<V>{p.d0, p.d1, p.d2, p.leg, p.tile0, (const V*)T.bufs[p.u_buf], (const V*)T.bufs[p.w_buf], (V*)T.mats[p.dst_mat]};
+  }
+};
+template <typename V, int NO>
+struct PjPar {
+  PjOutV<V> outs[NO];
+  __device__ __forceinline__ PjOutV<V> out(const PjList& L, int tile) const {
+    return outs[list_output(outs, 0, L.out_end - L.out_begin, L.tpo, tile)];
+  }
+};
+
+template <typename R, typename TAB>
+__global__ void __launch_bounds__(32 * kPjWarps, 4) k_project(const __grid_constant__ TAB tab, PjList L) {
   using C = Cx<R>;
   using V = typename C::T;
   __shared__ V part[kPjWarps][32];
@@ -308,7 +420,7 @@ __global__ void __launch_bounds__(32 * kPjWarps, 4) k_project(DevTables T, PjLis
   const int K = L.k;
   const int tile = blockIdx.x / K, rank = blockIdx.x % K;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const PjOut pj = T.pjs[list_output(T.pjs, L.out_begin, L.out_end, L.tpo, tile)];
+  const PjOutV<V> pj = tab.out(L, tile);
   const int dd[3] = {pj.d0, pj.d1, pj.d2};
   const int64_t st[3] = {(int64_t)pj.d1 * pj.d2, pj.d2, 1};
   const int l = pj.leg;
@@ -319,8 +431,8 @@ __global__ void __launch_bounds__(32 * kPjWarps, 4) k_project(DevTables T, PjLis
   V acc = C::zero();
   if (e < d * d) {
     const int xp = e / d, x = e % d;
-    const V* __restrict__ U = (const V*)T.bufs[pj.u_buf] + (int64_t)xp * st[l];
-    const V* __restrict__ Wt = (const V*)T.bufs[pj.w_buf] + (int64_t)x * st[l];
+    const V* __restrict__ U = pj.u + (int64_t)xp * st[l];
+    const V* __restrict__ Wt = pj.w + (int64_t)x * st[l];
     const int W = K * kPjWarps, me = rank * kPjWarps + wid;
     for (int r0 = me; r0 < nrest; r0 += 4 * W) {
       V uv[4], wv[4];
@@ -340,20 +452,16 @@ __global__ void __launch_bounds__(32 * kPjWarps, 4) k_project(DevTables T, PjLis
   }
   part[wid][lane] = acc;
   __syncthreads();
-  if (wid == 0) {
-    acc = part[0][lane];
-    for (int w = 1; w < kPjWarps; ++w) acc = C::add(acc, part[w][lane]);
-  }
+  R sum = comp_sum<R>(part, kPjWarps);
   if (K > 1) {
     cg::cluster_group cluster = cg::this_cluster();
-    if (wid == 0 && rank > 0) cluster.map_shared_rank(&slot[0][0], 0)[rank * 32 + lane] = acc;
+    if (wid < 2) reinterpret_cast<R*>(cluster.map_shared_rank(&slot[0][0], 0))[rank * 64 + 2 * lane + wid] = sum;
     cluster.sync();
     if (rank > 0) return;
-    if (wid == 0)
-      for (int r = 1; r < K; ++r) acc = C::add(acc, slot[r][lane]);
+    sum = comp_sum<R>(slot, K);
   }
-  if (wid != 0 || e >= d * d) return;
-  ((V*)T.mats[pj.dst_mat])[e] = acc;
+  if (wid > 1 || e >= d * d) return;
+  reinterpret_cast<R*>(pj.dst)[2 * e + wid] = sum;
 }
 
 // Projection of wide bonds (d >= 32, reduction range >= 1024): 32 x 32 output
@@ -476,28 +584,62 @@ bool launch_project_tiled(int prec, const DevTables& T, const PjList& L, int d, 
   return cudaLaunchKernelEx(&cfg, k_project_tiled<double>, T, L, ntx, KS) == cudaSuccess;
 }
 
-void launch_project(int prec, const DevTables& T, const PjList& L, cudaStream_t s) {
+template <typename R, int NO>
+static bool project_par(const HostTables& H, const PjList& L, cudaStream_t s) {
+  using V = typename Cx<R>::T;
+  if (L.out_end - L.out_begin > NO) return false;
+  PjPar<V, NO> tab{};
+  for (int o = L.out_begin; o < L.out_end; ++o) {
+    const PjOut& p = H.pjs[o];
+    tab.outs[o - L.out_begin] = PjOutV<V>{p.d0, p.d1, p.d2, p.leg, p.tile0, (const V*)H.bufs[p.u_buf],
+                                          (const V*)H.bufs[p.w_buf], (V*)H.mats[p.dst_mat]};
+  }
+  launch_split(k_project<R, PjPar<V, NO>>, L.n_tiles, L.k, kPjWarps, s, tab, L);
+  return true;
+}
+template <typename R>
+static void launch_project_r(const DevTables& T, const HostTables& H, const PjList& L, cudaStream_t s) {
+  if (project_par<R, 8>(H, L, s) || project_par<R, 48>(H, L, s)) return;
+  launch_split(k_project<R, PjMem<typename Cx<R>::T>>, L.n_tiles, L.k, kPjWarps, s, PjMem<typename Cx<R>::T>{T}, L);
+}
+
+void launch_project(int prec, const DevTables& T, const HostTables& H, const PjList& L, cudaStream_t s) {
   if (L.n_tiles <= 0) return;
   if (prec == PREC_F32)
-    launch_split(k_project<float>, L.n_tiles, L.k, kPjWarps, s, T, L);
+    launch_project_r<float>(T, H, L, s);
   else
-    launch_split(k_project<double>, L.n_tiles, L.k, kPjWarps, s, T, L);
+    launch_project_r<double>(T, H, L, s);
 }
 
 // Clusters of more than 8 CTAs are non-portable: allowed once per process for
 // every contraction and projection kernel, before any launch (and outside any
 // graph capture).
+template <typename K>
+static void allow_wide(K kern) {
+  cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+}
+template <typename R, typename TAB>
+static void allow_wide_apply() {
+  allow_wide(k_apply<R, 8, TAB>);
+  allow_wide(k_apply<R, 4, TAB>);
+  allow_wide(k_apply<R, 2, TAB>);
+}
+template <typename R>
+static void allow_wide_r() {
+  using V = typename Cx<R>::T;
+  allow_wide_apply<R, ApPar<V, 12, 4>>();
+  allow_wide_apply<R, ApPar<V, 32, 32>>();
+  allow_wide_apply<R, ApPar<V, 120, 40>>();
+  allow_wide_apply<R, ApMem<V>>();
+  allow_wide(k_project<R, PjPar<V, 8>>);
+  allow_wide(k_project<R, PjPar<V, 48>>);
+  allow_wide(k_project<R, PjMem<V>>);
+}
 void allow_wide_splits() {
   static std::once_flag once;
   std::call_once(once, [] {
-    cudaFuncSetAttribute(k_apply<double, 8>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaFuncSetAttribute(k_apply<double, 4>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaFuncSetAttribute(k_apply<double, 2>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaFuncSetAttribute(k_apply<float, 8>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaFuncSetAttribute(k_apply<float, 4>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaFuncSetAttribute(k_apply<float, 2>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaFuncSetAttribute(k_project<double>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaFuncSetAttribute(k_project<float>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    allow_wide_r<double>();
+    allow_wide_r<float>();
     cudaGetLastError();
   });
 }

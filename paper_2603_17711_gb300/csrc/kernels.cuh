@@ -24,6 +24,18 @@ struct DevTables {
   const PjOut* pjs;
 };
 
+// Host copies of the same tables. A launch whose list fits takes its outputs,
+// terms and operand addresses as kernel parameters (constant bank): reading
+// them from global memory is a chain of three dependent L2 round trips before
+// the first operand can be loaded, about 1.4 us of a 5 us launch.
+struct HostTables {
+  void* const* bufs;
+  void* const* mats;
+  const ApOut* outs;
+  const ApTerm* terms;
+  const PjOut* pjs;
+};
+
 // q = a / b and r = a - q b for a >= 0, b > 0, in 32-bit arithmetic when both
 // fit: a 64-bit integer division is a long instruction sequence on the GPU,
 // and index decompositions sit in the inner loops of the gather, scatter and
@@ -70,7 +82,12 @@ struct Epi {
   void* ys;      // stage input (contraction type)
   double2* acc;  // FP64 stage accumulator
   double h;
+  double c = 0.0;  // coefficient of k in the update (h/2, h/2, h, h/6), set by the launch: a division per thread costs ~370 cycles
 };
+inline Epi with_coef(Epi e) {
+  e.c = e.mode == EPI_RK3 ? e.h : e.mode == EPI_RK4 ? e.h / 6.0 : 0.5 * e.h;
+  return e;
+}
 
 // One time-dependent open-leg matrix: cur = stat + sum_d g_d * part_d.
 constexpr int kMaxDrives = 8;
@@ -83,7 +100,7 @@ struct DriveArgs {
   double g[kMaxDrives];
 };
 
-void launch_apply(int prec, const DevTables& T, const ApList& L, const Epi& e, cudaStream_t s);
+void launch_apply(int prec, const DevTables& T, const HostTables& H, const ApList& L, const Epi& e, cudaStream_t s);
 // Allows the contraction and projection kernels clusters of up to kMaxSplit
 // (16) CTAs; called once before the first launch.
 void allow_wide_splits();
@@ -141,7 +158,7 @@ bool xs_applicable(const ApList& L, const ApOut* outs_host, const ApTerm* terms_
 bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L, const Epi& e,
                      const ApOut* outs_host, const ApTerm* terms_host, double2* planes, int64_t plane_elems,
                      int max_split, cudaStream_t s);
-void launch_project(int prec, const DevTables& T, const PjList& L, cudaStream_t s);
+void launch_project(int prec, const DevTables& T, const HostTables& H, const PjList& L, cudaStream_t s);
 // The same projections for wide bonds in the FP32 form (every output d x d
 // with d >= 32 and a reduction range of >= 1024 positions, all outputs of the
 // list alike):

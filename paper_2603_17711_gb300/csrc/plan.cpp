@@ -374,6 +374,34 @@ int Plan::new_mat(int d) {
   return (int)mats.size() - 1;
 }
 
+// Packed diagonals (plan.hpp, mat_diag) of an open-leg operator and its drive
+// parts; 0 (dense) when they fill more than three, or when a dense row is at
+// most three chunks of the apply kernel (d <= 12): there the whole row costs a
+// warp or two more per tile and no time. Above, it does: Table 1 spin-boson
+// (depth 25), leaf-node combine 21.2 -> 10.5 us, pair products 18.3 -> 6.0 us;
+// FMO (depth 20), step 40.4 -> 37.1 ms.
+static int32_t diagonals_of(const LocalMat& lm, int d) {
+  std::vector<int> offs;
+  auto scan = [&](const std::vector<cd>& m) {
+    if (m.empty()) return;
+    for (int i = 0; i < d; ++i)
+      for (int x = 0; x < d; ++x)
+        if (m[(size_t)i * d + x] != cd(0) && std::find(offs.begin(), offs.end(), x - i) == offs.end())
+          offs.push_back(x - i);
+  };
+  scan(lm.stat);
+  for (const auto& dr : lm.drive) scan(dr);
+  if (offs.empty()) offs.push_back(0);
+  if (offs.size() > 3 || d <= 3 * kApChunk) return 0;
+  std::sort(offs.begin(), offs.end());
+  int32_t v = (int32_t)offs.size() << 24;
+  for (size_t k = 0; k < offs.size(); ++k) {
+    if (offs[k] < -127 || offs[k] > 127) return 0;
+    v |= (int32_t)((uint32_t)(uint8_t)(int8_t)offs[k] << (8 * k));
+  }
+  return v;
+}
+
 std::string Plan::build_classes() {
   const int n = tree.n_nodes, nl = tree.n_legs;
   // keys: the factor shared by more two-factor terms (ties: lower leg)
@@ -477,6 +505,9 @@ std::string Plan::build_classes() {
   }
   bond_mat = (int)mats.size();  // alias of the bond buffer (no pool storage)
   mats.push_back(MatSlot{r_cap_max, -1});
+  mat_diag.assign(mats.size(), 0);
+  if (fp64)
+    for (const LocalMat& lm : locals) mat_diag[lm.slot] = diagonals_of(lm, leg_dims[lm.leg]);
   return "";
 }
 
@@ -515,9 +546,10 @@ int Plan::add_list(const std::vector<ApOut>& outs, const std::vector<std::vector
     o.term_begin = (int)ap_terms.size();
     if (o.d3 < 1) o.d3 = 1;
     const int dd[4] = {o.d0, o.d1, o.d2, o.d3};
-    for (const ApTerm& t : tl[i]) {
+    for (ApTerm t : tl[i]) {
+      t.pad = t.mat >= 0 ? mat_diag[t.mat] : 0;
       ap_terms.push_back(t);
-      if (t.mat >= 0) L.flops += 8.0 * o.d0 * o.d1 * o.d2 * o.d3 * dd[t.leg];
+      if (t.mat >= 0) L.flops += 8.0 * o.d0 * o.d1 * o.d2 * o.d3 * (t.pad ? t.pad >> 24 : dd[t.leg]);
     }
     o.term_end = (int)ap_terms.size();
     o.tile0 = tiles;
@@ -536,7 +568,8 @@ int Plan::add_list(const std::vector<ApOut>& outs, const std::vector<std::vector
   for (size_t i = 0; i < outs.size(); ++i) {
     const int dd[4] = {outs[i].d0, outs[i].d1, outs[i].d2, outs[i].d3 < 1 ? 1 : outs[i].d3};
     int u = 0;
-    for (const ApTerm& t : tl[i]) u += t.mat < 0 ? 1 : (dd[t.leg] + kApChunk - 1) / kApChunk;
+    for (const ApTerm& t : tl[i])
+      u += t.mat < 0 || mat_diag[t.mat] ? 1 : (dd[t.leg] + kApChunk - 1) / kApChunk;
     units_max = std::max(units_max, u);
   }
   L.units = units_max;
@@ -609,6 +642,27 @@ void Plan::vl_terms(const std::vector<std::pair<int, int>>& vl, int src, std::ve
       pairs.push_back({xs, l1, ps, l2});
     }
   }
+}
+
+// Partners that share their X factor share its product too:
+// X (P_a x_a U + P_b x_b U) costs one mode product with X instead of two. Done
+// where the P are sparse (mat_diag; FP64 form): their sum is a few FMAs per
+// element. Dense P stay apart: on the tensor cores a list with terms on two legs
+// needs a launch per leg. Leg 0 is kept apart from the others (the down-only list
+// of vmf needs them apart).
+std::vector<Plan::PairGroup> Plan::group_pairs(const std::vector<std::array<int, 4>>& pairs) const {
+  std::vector<PairGroup> out;
+  for (const auto& q : pairs) {
+    PairGroup* g = nullptr;
+    if (mat_diag[q[2]])
+      for (PairGroup& c : out)
+        if (c.xs == q[0] && c.l1 == q[1] && mat_diag[c.p[0].first] && (c.p[0].second == 0) == (q[3] == 0)) g = &c;
+    if (g)
+      g->p.push_back({q[2], q[3]});
+    else
+      out.push_back(PairGroup{q[0], q[1], {{q[2], q[3]}}});
+  }
+  return out;
 }
 
 void Plan::node_terms(int u, int src, int, std::vector<ApTerm>& singles,
@@ -708,26 +762,28 @@ std::string Plan::build_jobs() {
       int src = var == 0 ? u : var == 1 ? buf.ys : buf.ys2;
       node_terms(u, src, 0, singles, pairs);
       ApOut base{dims[u][0], dims[u][1], dims[u][2], 0, 0, -1, 0, 0};
-      if (!pairs.empty()) {
+      const std::vector<PairGroup> gs = group_pairs(pairs);
+      if (!gs.empty()) {
         std::vector<ApOut> outs;
         std::vector<std::vector<ApTerm>> tl;
-        for (size_t g = 0; g < pairs.size(); ++g) {
+        for (size_t g = 0; g < gs.size(); ++g) {
           ApOut o = base;
           o.dst = buf.t0 + (int)g;
           outs.push_back(o);
-          tl.push_back({ApTerm{pairs[g][2], pairs[g][3], src, 0}});
+          tl.push_back({});
+          for (const auto& q : gs[g].p) tl.back().push_back(ApTerm{q.first, q.second, src, 0});
         }
         node_flow[u].first[var] = add_list(outs, tl);
       }
       std::vector<ApTerm> all = singles;
-      for (size_t g = 0; g < pairs.size(); ++g) all.push_back(ApTerm{pairs[g][0], pairs[g][1], buf.t0 + (int)g, 0});
+      for (size_t g = 0; g < gs.size(); ++g) all.push_back(ApTerm{gs[g].xs, gs[g].l1, buf.t0 + (int)g, 0});
       node_flow[u].combine[var] = add_list({base}, {all});
       if (var == 0 && u != 0) {
         std::vector<ApTerm> down;
         for (const ApTerm& t : singles)
           if (t.leg != 0) down.push_back(t);
-        for (size_t g = 0; g < pairs.size(); ++g)
-          if (pairs[g][1] != 0 && pairs[g][3] != 0) down.push_back(ApTerm{pairs[g][0], pairs[g][1], buf.t0 + (int)g, 0});
+        for (size_t g = 0; g < gs.size(); ++g)
+          if (gs[g].l1 != 0 && gs[g].p[0].second != 0) down.push_back(ApTerm{gs[g].xs, gs[g].l1, buf.t0 + (int)g, 0});
         node_down[u] = add_list({base}, {down});
       }
     }
@@ -780,20 +836,21 @@ std::string Plan::build_jobs() {
         int src = var == 0 ? buf.th_y : var == 1 ? buf.th_ys : buf.th_ys2;
         vl_terms(vl, src, singles, pairs);
         ApOut base{td[0], td[1], td[2], 0, 0, -1, 0, td[3]};
-        if (!pairs.empty()) {
+        const std::vector<PairGroup> gs = group_pairs(pairs);
+        if (!gs.empty()) {
           std::vector<ApOut> outs;
           std::vector<std::vector<ApTerm>> tl;
-          for (size_t g = 0; g < pairs.size(); ++g) {
+          for (size_t g = 0; g < gs.size(); ++g) {
             ApOut o = base;
             o.dst = buf.t0 + (int)g;
             outs.push_back(o);
-            tl.push_back({ApTerm{pairs[g][2], pairs[g][3], src, 0}});
+            tl.push_back({});
+            for (const auto& q : gs[g].p) tl.back().push_back(ApTerm{q.first, q.second, src, 0});
           }
           two_site[e].first[var] = add_list(outs, tl);
         }
         std::vector<ApTerm> all = singles;
-        for (size_t g = 0; g < pairs.size(); ++g)
-          all.push_back(ApTerm{pairs[g][0], pairs[g][1], buf.t0 + (int)g, 0});
+        for (size_t g = 0; g < gs.size(); ++g) all.push_back(ApTerm{gs[g].xs, gs[g].l1, buf.t0 + (int)g, 0});
         two_site[e].combine[var] = add_list({base}, {all});
       }
     }

@@ -92,7 +92,7 @@ struct ApTerm {
   int32_t mat;
   int32_t leg;
   int32_t src;  // buffer id
-  int32_t pad;
+  int32_t pad;  // FP64 form: packed diagonals of a sparse operator (Plan::mat_diag), 0 = dense
 };
 // One output tensor of an apply job list.
 struct ApOut {
@@ -191,6 +191,13 @@ struct Plan {
   std::vector<LocalMat> locals;                   // open-leg matrices
   std::vector<MatSlot> mats;                      // all matrix slots in the pool
   int64_t mat_pool = 0;                           // complex elements
+  // per matrix: an open-leg operator whose entries lie on at most three
+  // diagonals (x - i = offset; the ladder and number operators of a Fock leg, a
+  // site projector on a system leg), packed as n << 24 | three signed bytes;
+  // 0 = dense. The contractions of the FP64 form then touch n entries per row
+  // instead of d. The mixed form stays dense: its sums keep their order.
+  std::vector<int32_t> mat_diag;
+  bool fp64 = true;  // precision of the handle's contractions
   int bond_mat = -1;                              // matrix id aliasing the bond buffer
 
   // job lists
@@ -242,6 +249,13 @@ struct Plan {
   int split_factor(int tiles, int useful) const;
   void node_terms(int u, int src, int t_base, std::vector<ApTerm>& singles,
                   std::vector<std::array<int, 4>>& pairs) const;
+  // A pair term of a node: X on one leg, and the partners P on other legs behind
+  // the same X.
+  struct PairGroup {
+    int xs, l1;
+    std::vector<std::pair<int, int>> p;  // (P slot, leg)
+  };
+  std::vector<PairGroup> group_pairs(const std::vector<std::array<int, 4>>& pairs) const;
   // operator terms on an arbitrary list of (node, leg) "virtual legs"
   void vl_terms(const std::vector<std::pair<int, int>>& vl, int src, std::vector<ApTerm>& singles,
                 std::vector<std::array<int, 4>>& pairs) const;

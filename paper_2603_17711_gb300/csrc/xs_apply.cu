@@ -445,12 +445,10 @@ __global__ void __launch_bounds__(kXsThreads, 2) k_xs_apply(const __grid_constan
 // RK4 stage update of element e with the computed derivative k (kernels.cuh, Epi), FP64.
 __device__ __forceinline__ void rk_update(const Epi& ep, int64_t e, double2 k) {
   const double2 y = ep.y[e];
-  double2* ys = (double2*)ep.ys;
-  const double h = ep.mode == EPI_RK3 ? ep.h : 0.5 * ep.h;
+  const double c = ep.c;
   if (ep.mode == EPI_RK4) {
     const double2 a = ep.acc[e];
-    const double w = ep.h / 6.0;
-    ep.y[e] = make_double2(y.x + w * (a.x + k.x), y.y + w * (a.y + k.y));
+    ep.y[e] = make_double2(y.x + c * (a.x + k.x), y.y + c * (a.y + k.y));
     return;
   }
   if (ep.mode == EPI_RK1) {
@@ -459,19 +457,40 @@ __device__ __forceinline__ void rk_update(const Epi& ep, int64_t e, double2 k) {
     const double2 a = ep.acc[e];
     ep.acc[e] = make_double2(a.x + 2.0 * k.x, a.y + 2.0 * k.y);
   }
-  ys[e] = make_double2(y.x + h * k.x, y.y + h * k.y);
+  ((double2*)ep.ys)[e] = make_double2(y.x + c * k.x, y.y + c * k.y);
 }
 
-// Sum of the planes of a one-output list, in order, and its epilogue.
+// Sum of the planes of a one-output list, in order, the list's sparse terms (at
+// most three entries a row: a few FMAs an element, not worth a tensor-core
+// term) and its epilogue.
+constexpr int kXsMaxSparse = 24;
+struct XsSparse {
+  int n;
+  int dims[4];
+  XsTerm term[kXsMaxSparse];
+  int leg[kXsMaxSparse], diag[kXsMaxSparse];
+};
 __global__ void __launch_bounds__(128) k_xs_epilogue(const double2* planes, int n_planes, int64_t P, Epi ep,
-                                                     double2* dst) {
+                                                     double2* dst, const __grid_constant__ XsSparse sp) {
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= P) return;
-  double2 k = planes[e];
+  double2 k = n_planes > 0 ? planes[e] : make_double2(0.0, 0.0);
   for (int q = 1; q < n_planes; ++q) {
     const double2 v = planes[(int64_t)q * P + e];
     k.x += v.x;
     k.y += v.y;
+  }
+  for (int t = 0; t < sp.n; ++t) {
+    int inner = 1;
+    for (int l = 3; l > sp.leg[t]; --l) inner *= sp.dims[l];
+    const int d = sp.dims[sp.leg[t]], i = (int)(e / inner) % d, nd = sp.diag[t] >> 24;
+    for (int q = 0; q < nd; ++q) {
+      const int off = (int)(int8_t)(sp.diag[t] >> (8 * q)), x = i + off;
+      if (x < 0 || x >= d) continue;
+      const double2 m = sp.term[t].M[i * d + x], v = sp.term[t].X[e + (int64_t)off * inner];
+      k.x = fma(m.x, v.x, fma(-m.y, v.y, k.x));
+      k.y = fma(m.x, v.y, fma(m.y, v.x, k.y));
+    }
   }
   if (ep.mode == EPI_STORE) {
     dst[e] = k;
@@ -502,6 +521,7 @@ bool xs_applicable(const ApList& L, const ApOut* outs, const ApTerm* terms) {
   if (L.n_tiles <= 0) return false;
   const ApOut& f = outs[L.out_begin];
   const int64_t P = (int64_t)f.d0 * f.d1 * f.d2 * f.d3;
+  double dense = 0.0;  // sparse operators are cheap on the CUDA cores
   if (P >= (int64_t)1 << 30 || L.out_end - L.out_begin > 65535) return false;
   for (int o = L.out_begin; o < L.out_end; ++o) {
     const ApOut& u = outs[o];
@@ -511,9 +531,10 @@ bool xs_applicable(const ApList& L, const ApOut* outs, const ApTerm* terms) {
     for (int t = u.term_begin; t < u.term_end; ++t) {
       const ApTerm& tm = terms[t];
       if (tm.mat < 0 || tm.leg < 0 || tm.leg > 3 || dd[tm.leg] > kXsMaxD) return false;
+      if (!tm.pad) dense += 8.0 * P * dd[tm.leg];
     }
   }
-  return L.flops >= kXsMinFlops;
+  return dense >= kXsMinFlops;
 }
 
 bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L, const Epi& e, const ApOut* outs,
@@ -533,20 +554,27 @@ bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L
   int tiles[4];
   for (int l = 0; l < 4; ++l) tiles[l] = (int)((P / dd[l] + kXsCols - 1) / kXsCols);
   XsWork gr{};
+  XsSparse sp{};
   if (n_outs > kXsMaxOuts || outs[L.out_end - 1].term_end - outs[L.out_begin].term_begin > kXsMaxTerms) return false;
   int nq = 0;
-  for (int i = 0; i < 4; ++i) gr.dims[i] = dd[i];
+  for (int i = 0; i < 4; ++i) gr.dims[i] = sp.dims[i] = dd[i];
   for (int o = 0; o < n_outs; ++o) {
     const ApOut& v = outs[L.out_begin + o];
     gr.dst[o] = v.dst >= 0 ? bufs[v.dst] : nullptr;
     gr.tb[o][0] = (short)nq;
     for (int l = 0; l < 4; ++l) {
       for (int t = v.term_begin; t < v.term_end; ++t)
-        if (terms[t].leg == l) gr.term[nq++] = XsTerm{mats[terms[t].mat], bufs[terms[t].src]};
+        if (terms[t].leg == l && n_outs == 1 && terms[t].pad && sp.n < kXsMaxSparse) {
+          sp.leg[sp.n] = l;
+          sp.diag[sp.n] = terms[t].pad;
+          sp.term[sp.n++] = XsTerm{mats[terms[t].mat], bufs[terms[t].src]};
+        } else if (terms[t].leg == l)
+          gr.term[nq++] = XsTerm{mats[terms[t].mat], bufs[terms[t].src]};
       gr.tb[o][l + 1] = (short)nq;
     }
   }
   if (n_outs == 1) {
+    for (int l = 0; l < 4; ++l) nterm[l] = gr.tb[0][l + 1] - gr.tb[0][l];
     // all legs in one launch, each leg's terms cut into parts while a warp
     // still has more than one term and the launch stays below four CTAs per SM
     // (two are resident at a time)
@@ -585,7 +613,7 @@ bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L
     gr.leg = -1;
     gr.planes = planes;
     k_xs_apply<<<dim3(gr.lt[4], 1), kXsThreads, 0, s>>>(gr);
-    k_xs_epilogue<<<(int)((P + 127) / 128), 128, 0, s>>>(planes, q, P, e, gr.dst[0]);
+    k_xs_epilogue<<<(int)((P + 127) / 128), 128, 0, s>>>(planes, q, P, with_coef(e), gr.dst[0], sp);
     return true;
   }
   if (e.mode != EPI_STORE) return false;
