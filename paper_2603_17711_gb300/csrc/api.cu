@@ -287,7 +287,7 @@ Layout layout_of(const Plan& p, int prec) {
   }
   L.rdm_elems = ra;
   L.rdm = take(ra * sizeof(double2));
-  L.rho = take((size_t)p.leg_dims[0] * p.leg_dims[0] * sizeof(double2));
+  L.rho = take(((size_t)p.leg_dims[0] * p.leg_dims[0] + 1) * sizeof(double2));  // rho, then the error flag
   L.bufs_tab = take(p.buf.n_bufs * sizeof(double2*));
   L.mats_tab = take(p.mats.size() * sizeof(double2*));
   L.terms = take(p.ap_terms.size() * sizeof(ApTerm));
@@ -869,17 +869,31 @@ struct Exec {
     for (int c : p.tree.postorder)
       if (c != 0) env(c, p.tree.parent[c]);
   }
-  void rdm(double2* out) {
+  // rho into out, one launch per tree level; flag_out (nullable): the error flag as a number
+  void rdm(double2* out, double2* flag_out = nullptr) {
+    const int n = p.tree.n_nodes;
+    std::vector<int> level(n, 0);
+    int top = 0;
     for (int u : p.tree.postorder) {
-      const auto& d = p.dims[u];
-      const double2* w[3] = {nullptr, nullptr, nullptr};
-      for (int li = (u == 0 ? 2 : 1); li < 3; ++li) {
-        const Leg& L = p.tree.legs[u][li];
-        if (L.kind == 'n') w[li] = h->rdm_vec + h->rdm_off[L.v];
+      for (int c : p.tree.children[u]) level[u] = std::max(level[u], level[c] + 1);
+      top = std::max(top, level[u]);
+    }
+    std::vector<RdmJob> jobs;
+    for (int l = 0; l <= top; ++l) {
+      jobs.clear();
+      for (int u = 0; u < n; ++u) {
+        if (level[u] != l) continue;
+        const auto& d = p.dims[u];
+        const double2* w[3] = {nullptr, nullptr, nullptr};
+        for (int li = (u == 0 ? 2 : 1); li < 3; ++li) {
+          const Leg& L = p.tree.legs[u][li];
+          if (L.kind == 'n') w[li] = h->rdm_vec + h->rdm_off[L.v];
+        }
+        jobs.push_back(RdmJob{h->h_bufs[u], w[1], w[2], u == 0 ? out : h->rdm_vec + h->rdm_off[u], d[1], d[2],
+                              u == 0 ? d[0] * d[1] : d[0], u == 0 ? 1 : 0, 0});
       }
       run(3, 0.0, [&] {
-        launch_rdm_node(h->h_bufs[u], d[0], d[1], d[2], u == 0, w[1], w[2],
-                        u == 0 ? out : h->rdm_vec + h->rdm_off[u], s);
+        launch_rdm_level(jobs.data(), (int)jobs.size(), h->flag_dev, l == top ? flag_out : nullptr, s);
       });
     }
   }
@@ -1575,15 +1589,18 @@ ttn_status ttn_step(ttn_t h, double dt, int32_t scheme, int32_t n_steps) {
   return st;
 }
 
-static ttn_status check_flag(ttn_t h) {
-  int flag = 0;
-  CUDA_TRY(h, cudaMemcpyAsync(&flag, h->flag_dev, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-  CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+static ttn_status flag_status(ttn_t h, int flag) {
   if (flag & 2) return h->fail(TTN_ETIMEOUT, "a cluster or grid exchange of the QR kernels gave up");
   if (flag & 8) return h->fail(TTN_ETIMEOUT, "a tensor-core MMA wait gave up after 1 s");
   if (flag & 16) return h->fail(TTN_ETIMEOUT, "a grid barrier of the Jacobi SVD gave up after wait_s");
   if (flag) return h->fail(TTN_ENUMERIC, "non-finite amplitude in the root tensor");
   return TTN_OK;
+}
+static ttn_status check_flag(ttn_t h) {
+  int flag = 0;
+  CUDA_TRY(h, cudaMemcpyAsync(&flag, h->flag_dev, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+  return flag_status(h, flag);
 }
 
 ttn_status ttn_rdm_device(ttn_t h, void* rho_dev) {
@@ -1602,12 +1619,14 @@ ttn_status ttn_rdm(ttn_t h, double* rho_out) {
     if (!h->ws_bound) return h->fail(TTN_ESTATE, "bind the workspace first");
     if (!rho_out) return h->fail(TTN_EINVAL, "null output");
     Exec ex(h);
-    ex.rdm(h->rho_dev);
-    const int M = h->plan.leg_dims[0];
+    const size_t n = (size_t)h->plan.leg_dims[0] * h->plan.leg_dims[0];
+    ex.rdm(h->rho_dev, h->rho_dev + n);
     CUDA_TRY(h, cudaGetLastError());
-    CUDA_TRY(h, cudaMemcpyAsync(rho_out, h->rho_dev, (size_t)M * M * sizeof(double2), cudaMemcpyDeviceToHost,
-                                h->stream));
-    return check_flag(h);
+    std::vector<double2> back(n + 1);  // rho and the error flag in one copy
+    CUDA_TRY(h, cudaMemcpyAsync(back.data(), h->rho_dev, (n + 1) * sizeof(double2), cudaMemcpyDeviceToHost, h->stream));
+    CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+    std::memcpy(rho_out, back.data(), n * sizeof(double2));
+    return flag_status(h, (int)back[n].x);
   });
 }
 

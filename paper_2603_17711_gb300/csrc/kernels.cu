@@ -826,47 +826,71 @@ void launch_copy(double2* dst, float2* dst_lo, const double2* src, int64_t n, cu
 // Reduced density matrix (rho_S = <0|Omega>): contraction of one node with
 // the vectors of its two child legs (the n = 0 unit vector on open legs).
 // ---------------------------------------------------------------------------
-// One CTA per output; warp w takes the rows b = w, w + 8, ... of the output's
-// slice (for the root: one row, the output itself), the lanes split the row
-// over c and a fixed butterfly adds them, and the warps' sums are added in warp
-// order, so the result is reproducible.
-__global__ void __launch_bounds__(256) k_rdm_node(const double2* U, int d0, int d1, int d2, int root,
-                                                  const double2* w1, const double2* w2, double2* out) {
-  // root: out[i*d1 + j] = sum_c U[i, j, c] w2[c]; else out[a] = sum_{b,c} U[a,b,c] w1[b] w2[c]
-  __shared__ double2 part[8];
-  const int e = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nrow = root ? 1 : (w1 ? d1 : 1);
-  const double2* blk = U + (int64_t)e * (root ? d2 : (int64_t)d1 * d2);
+// All nodes of one tree level in one launch, one CTA per output. Lanes own the
+// positions c of the last leg, warp w the rows b = w, w + 8, ...: a lane adds
+// w1[b] U[a, b, c] over its rows, multiplies by w2[c] once, and only that is
+// summed over lanes (fixed butterfly) and warps (in order), so an element costs
+// four FP64 operations; a butterfly per row, as one launch per node had it, costs
+// ten more per row. 21-node chain at rank 20: 21 launches of 4.2 us -> 7 of about 3 us.
+struct RdmLevel {
+  int n;
+  RdmJob job[kRdmLevelMax];
+};
+__global__ void __launch_bounds__(256) k_rdm_level(const __grid_constant__ RdmLevel lv, const int* flag,
+                                                   double2* flag_out) {
+  __shared__ double part[8][2];
+  int q = 0;
+  while (q + 1 < lv.n && (int)blockIdx.x >= lv.job[q + 1].cta0) ++q;
+  const RdmJob jb = lv.job[q];
+  const int e = blockIdx.x - jb.cta0, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // root: e = i*d1 + j, out[e] = sum_c U[i, j, c] w2[c]; else out[a] = sum_{b,c} U[a, b, c] w1[b] w2[c]
+  const int nb = jb.w1 ? jb.d1 : 1, nc = jb.w2 ? jb.d2 : 1;
+  const double2* blk = jb.U + (int64_t)e * (jb.root ? jb.d2 : (int64_t)jb.d1 * jb.d2);
   double2 acc = make_double2(0.0, 0.0);
-  for (int b = warp; b < nrow; b += 8) {
-    const double2* row = blk + (int64_t)b * d2;
-    double2 inner = make_double2(0.0, 0.0);
-    if (w2) {
-      for (int c = lane; c < d2; c += 32) inner = cfma(row[c], w2[c], inner);
-      for (int o = 16; o > 0; o >>= 1) {
-        inner.x += __shfl_xor_sync(0xffffffffu, inner.x, o);
-        inner.y += __shfl_xor_sync(0xffffffffu, inner.y, o);
+  if (jb.w2) {
+    for (int c = lane; c < nc; c += 32) {
+      double2 t = make_double2(0.0, 0.0);
+      if (jb.w1) {
+        for (int b = warp; b < nb; b += 8) t = cfma(jb.w1[b], blk[(int64_t)b * jb.d2 + c], t);
+      } else if (warp == 0) {
+        t = blk[c];
       }
-    } else {
-      inner = row[0];
+      acc = cfma(t, jb.w2[c], acc);
     }
-    acc = (!root && w1) ? cfma(w1[b], inner, acc) : inner;
+  } else if (jb.w1) {  // the n = 0 position of the last leg: threads over the rows
+    for (int b = threadIdx.x; b < nb; b += 256) acc = cfma(jb.w1[b], blk[(int64_t)b * jb.d2], acc);
+  } else if (threadIdx.x == 0) {
+    acc = blk[0];
   }
-  if (lane == 0) part[warp] = acc;
+  for (int o = 16; o > 0; o >>= 1) {
+    acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+    acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+  }
+  if (lane == 0) {
+    part[warp][0] = acc.x;
+    part[warp][1] = acc.y;
+  }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double2 t = part[0];
-    for (int w = 1; w < 8 && w < nrow; ++w) {
-      t.x += part[w].x;
-      t.y += part[w].y;
-    }
-    out[e] = t;
+  if (threadIdx.x < 2) {
+    double t = part[0][threadIdx.x];
+    for (int w = 1; w < 8; ++w) t += part[w][threadIdx.x];
+    reinterpret_cast<double*>(jb.out)[2 * e + threadIdx.x] = t;
   }
+  // the error flag beside rho, so that one copy brings both to the host
+  if (flag_out && blockIdx.x == 0 && threadIdx.x == 0) flag_out->x = (double)*flag;
 }
-void launch_rdm_node(const double2* U, int d0, int d1, int d2, bool root, const double2* w1,
-                     const double2* w2, double2* out, cudaStream_t s) {
-  const int nout = root ? d0 * d1 : d0;
-  if (nout > 0) k_rdm_node<<<nout, 256, 0, s>>>(U, d0, d1, d2, root ? 1 : 0, w1, w2, out);
+void launch_rdm_level(RdmJob* jobs, int n, const int* flag, double2* flag_out, cudaStream_t s) {
+  for (int i0 = 0; i0 < n; i0 += kRdmLevelMax) {
+    RdmLevel lv{};
+    int ctas = 0;
+    for (int i = i0; i < n && lv.n < kRdmLevelMax; ++i) {
+      RdmJob j = jobs[i];
+      j.cta0 = ctas;
+      ctas += j.n_out;
+      lv.job[lv.n++] = j;
+    }
+    if (ctas > 0) k_rdm_level<<<ctas, 256, 0, s>>>(lv, flag, flag_out);
+  }
 }
 
 __global__ void k_drive(double2* const* mats, float2* const* mats32, const DriveMat* list, int n, DriveArgs g) {

@@ -218,10 +218,20 @@ bool launch_qr_blocked(double2* U, int d0, int d1, int d2, int leg, double tol, 
                        cudaStream_t s, uint64_t grid_wait_ns = 2000000000ull);
 // dst = src (FP64); dst_lo (nullable) = FP32 copy.
 void launch_copy(double2* dst, float2* dst_lo, const double2* src, int64_t n, cudaStream_t s);
-// rho / vector contraction for one node: out[a] (non-root) or out[i*d1+j] (root)
-// = sum U[...] w1[.] w2[.] (w = nullptr means the n = 0 unit vector).
-void launch_rdm_node(const double2* U, int d0, int d1, int d2, bool root, const double2* w1,
-                     const double2* w2, double2* out, cudaStream_t s);
+// rho / vector contraction of nodes that do not depend on one another (one tree
+// level): out[a] (non-root, n_out = d0) or out[i*d1+j] (root, n_out = d0*d1) =
+// sum U[...] w1[.] w2[.] (w = nullptr means the n = 0 unit vector). flag_out
+// (nullable): receives *flag as a real number.
+struct RdmJob {
+  const double2* U;
+  const double2* w1;
+  const double2* w2;
+  double2* out;
+  int d1, d2, n_out, root;
+  int cta0;  // set by the launch
+};
+constexpr int kRdmLevelMax = 32;
+void launch_rdm_level(RdmJob* jobs, int n, const int* flag, double2* flag_out, cudaStream_t s);
 // cur = stat + sum_d g_d part_d in the FP64 table; mats32 (nullable) receives
 // the FP32 copy of cur (same matrix id in the FP32 table).
 void launch_drive(double2* const* mats_dev, float2* const* mats32, const DriveMat* list, int n,

@@ -113,8 +113,9 @@ extern "C" ttn_status ttn_rdm_noalloc(const ttn_tree* tree, const int32_t* leg_d
       const Leg& L = p.tree.legs[u][li];
       if (L.kind == 'n') w[li] = scratch + off[L.v];
     }
-    launch_rdm_node((const double2*)node_dev[u], d[0], d[1], d[2], u == 0, w[1], w[2],
-                    u == 0 ? (double2*)rho_dev : scratch + off[u], s);
+    RdmJob job{(const double2*)node_dev[u], w[1], w[2], u == 0 ? (double2*)rho_dev : scratch + off[u], d[1], d[2],
+               u == 0 ? d[0] * d[1] : d[0], u == 0 ? 1 : 0, 0};
+    launch_rdm_level(&job, 1, nullptr, nullptr, s);
   }
   ce = cudaGetLastError();
   if (ce != cudaSuccess) {
