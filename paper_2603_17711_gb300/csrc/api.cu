@@ -70,6 +70,7 @@ struct ttn_ctx {
   double* svd_sigma = nullptr;
   int* svd_perm = nullptr;
   int* svd_info = nullptr;
+  double* svd_cand = nullptr;  // pivot candidates of the two-site QR
   unsigned* svd_sync = nullptr;  // barrier counters of the grid Jacobi SVD
   // direct integration (vmf), FP64 form only
   double2 *vmf_y = nullptr, *vmf_save = nullptr, *vmf_tmp = nullptr, *vmf_r = nullptr, *vmf_aug = nullptr,
@@ -232,7 +233,7 @@ struct Layout {
   int64_t tc_bsplit_floats = 0;  // FP32 mode only
   size_t tc_pool = 0, tc_off = 0;
   std::vector<int64_t> tc_off_host;  // float offset of each matrix in tc_pool, -1 if none
-  size_t svd_small = 0, rsvd = 0, mlp = 0, xs = 0;
+  size_t svd_cand = 0, svd_small = 0, rsvd = 0, mlp = 0, xs = 0;
   int64_t xs_elems = 0;
   // direct integration (vmf): committed state, per-node saves, 7 stage
   // derivatives (all as flat copies of the node region), edge scratch
@@ -295,6 +296,7 @@ Layout layout_of(const Plan& p, int prec) {
   L.pjs = take(p.pj_outs.size() * sizeof(PjOut));
   L.drives = take(p.locals.size() * sizeof(DriveMat));
   L.svd_small = take(p.theta_cap * sizeof(double) + (p.theta_cap + 4 + kSvdSyncInts) * sizeof(int));
+  L.svd_cand = take(kPivScratch * sizeof(double));
   L.rsvd = take(3 * p.theta_cap * sizeof(double2));
   L.mlp = take((24 + 13 + mlp_ws_floats(1) + 8) * sizeof(float) + 2 * sizeof(double));
   L.flag = take(sizeof(int) * 4);
@@ -590,9 +592,21 @@ struct Exec {
   uint64_t wait_ns() const { return (uint64_t)(h->params.wait_s * 1e9); }
   // launch the Jacobi SVD (one CTA or the whole GPU) and read back sigma; false
   // (with fail_st set) when it did not converge or a grid wait gave up
-  bool jacobi(const double2* theta, int m, int n, std::vector<double>& sig) {
+  // pivoted (nullable in): ask for the pivoted-QR route of a two-site matrix with
+  // the isometry on the first / second side; out: whether it was taken
+  bool jacobi(const double2* theta, int m, int n, std::vector<double>& sig, bool iso_first = false,
+              bool* pivoted = nullptr) {
     const int nc = std::min(m, n);
     run(2, 0.0, [&] {
+      if (pivoted) {
+        *pivoted = launch_pivot_svd(theta, m, n, iso_first, h->svd_A, h->svd_V, h->svd_sigma, h->svd_cand, h->svd_info,
+                                    h->svd_sync, h->flag_dev, wait_ns(), s);
+        if (*pivoted) return;
+        if (const cudaError_t e = cudaGetLastError(); e != cudaSuccess) {
+          note(e);
+          return;
+        }
+      }
       if (!launch_jacobi_svd_grid(theta, m, n, h->svd_A, h->svd_V, h->svd_sigma, h->svd_info, h->svd_sync,
                                   h->flag_dev, wait_ns(), s))
         {
@@ -727,7 +741,8 @@ struct Exec {
       }
     }
     if (!accepted) {
-      if (!jacobi(h->h_bufs[tl], m, n, sig)) return;
+      bool pivoted = false;
+      if (!jacobi(h->h_bufs[tl], m, n, sig, iso_first, &pivoted)) return;
       // truncation (host): r0 = #{sigma > ps2_atol}, r = min(cap, max(1, ceil(ratio r0)))
       perm.resize(nc);
       for (int i = 0; i < nc; ++i) perm[i] = i;
@@ -745,8 +760,12 @@ struct Exec {
       h->log_labels.push_back(std::max(-4, std::min(8, r - r_cur)) + 4);
       note(cudaMemcpy(h->svd_perm, perm.data(), r * sizeof(int), cudaMemcpyHostToDevice));
       run(3, 0.0, [&] {
-        launch_svd_vecs(h->svd_A, h->svd_V, h->svd_sigma, m, n, h->svd_perm, r, g, iso_first, h->svd_Z,
-                        h->svd_Zg, h->svd_C, s);
+        if (pivoted)
+          launch_pivot_vecs(h->h_bufs[tl], m, n, iso_first, h->svd_A, h->svd_sigma, h->svd_perm, r, g, h->svd_Z,
+                            h->svd_Zg, h->svd_C, s);
+        else
+          launch_svd_vecs(h->svd_A, h->svd_V, h->svd_sigma, m, n, h->svd_perm, r, g, iso_first, h->svd_Z, h->svd_Zg,
+                          h->svd_C, s);
       });
     }
     ++h->n_splits;
@@ -1193,6 +1212,7 @@ ttn_status ttn_set_workspace(ttn_t h, void* dptr, size_t bytes) {
     h->svd_perm = (int*)(h->svd_sigma + p.theta_cap);
     h->svd_info = h->svd_perm + p.theta_cap;
     h->svd_sync = (unsigned*)(h->svd_info + 4);
+    h->svd_cand = (double*)(base + L.svd_cand);
     h->rs_omega = (double2*)(base + L.rsvd);
     h->rs_Y = h->rs_omega + p.theta_cap;
     h->rs_B = h->rs_Y + p.theta_cap;

@@ -314,9 +314,24 @@ __device__ __forceinline__ double warp_sum4(double v0, double v1, double v2, dou
 // of *flag. Same outputs as launch_jacobi_svd.
 constexpr int kJacOneCtaMaxCols = 16;
 constexpr int kJacClusterMax = 16;
-constexpr int kSvdSyncInts = 128;
+constexpr int kSvdSyncInts = 128 + 2048;  // barrier and sweep counters, column round counters
 bool launch_jacobi_svd_grid(const double2* theta, int m, int n, double2* A, double2* V, double* sigma, int* info,
                             unsigned* sync, int* flag, uint64_t wait_ns, cudaStream_t s);
+// The split of a two-site matrix theta (m x n, row-major) with more columns on
+// its smaller side than a cluster's Jacobi takes: pivoted QR, then Jacobi on R^H
+// (svd.cu). X (ni x k, column-major; ni rows of the isometry side, k = min(m, n))
+// receives W Sigma, sigma the norms (unsorted, zero beyond the columns found),
+// info[0] the sweeps, info[2] the columns found. Bg: m*n scratch; cand:
+// kPivScratch doubles; info: 4 ints. False (nothing launched, or a launch
+// failed: cudaGetLastError) when the sizes do not fit.
+constexpr int kPivMaxGrid = 256;
+constexpr int kPivScratch = 2 * kPivMaxGrid + kPivMaxGrid + kPivMaxGrid;  // norms, partial sums, indices
+bool launch_pivot_svd(const double2* theta, int m, int n, bool iso_first, double2* X, double2* Bg, double* sigma,
+                      double* cand, int* info, unsigned* sync, int* flag, uint64_t wait_ns, cudaStream_t s);
+// Isometry Z (ni x r, row-major; columns beyond g zero), its copy Zg, and the
+// centre factor Cm = theta contracted with conj(Z), in the layouts of launch_svd_vecs.
+void launch_pivot_vecs(const double2* theta, int m, int n, bool iso_first, const double2* X, const double* sigma,
+                       const int* perm, int r, int g, double2* Z, double2* Zg, double2* Cm, cudaStream_t s);
 void launch_svd_vecs(const double2* A, const double2* V, const double* sigma, int m, int n, const int* perm, int r,
                      int g, bool iso_first, double2* Z, double2* Zg, double2* Cm, cudaStream_t s);
 void launch_restore_cols(double2* Z, const double2* Zg, int rows, int r, int g, cudaStream_t s);

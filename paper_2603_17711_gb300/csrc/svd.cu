@@ -52,7 +52,14 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
+// Jacobi: four warps, one per SM sub-partition. Eight would share the FP64 pipes
+// two by two and double the time of the lane sums.
+constexpr int kJThreads = 128;
+constexpr int kJWarps = kJThreads / 32;
 constexpr int kBarLanes = 8;
+constexpr int kVerOff = 128;  // first column counter in the sync words
+constexpr int kSvdMaxVer = kSvdSyncInts - kVerOff;
+static_assert(kBarLanes + kJacMaxSweeps <= kVerOff, "sweep counters fit before the column counters");
 
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
   return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -69,6 +76,9 @@ __device__ __forceinline__ uint64_t now_ns() {
 }
 __device__ __forceinline__ void red_release_add(unsigned* p, unsigned v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_release(unsigned* p, unsigned v) {
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
   unsigned v;
@@ -89,10 +99,11 @@ __device__ bool grid_sync(unsigned* lanes, unsigned target, uint64_t wait_ns, in
     if (lane == 0) red_release_add(lanes + blockIdx.x % kBarLanes, 1u);
     const uint64_t t0 = now_ns();
     int ok = 1;
-    for (;;) {
+    for (unsigned it = 0;; ++it) {
       unsigned v = lane < kBarLanes ? ld_acquire(lanes + lane) : 0u;
       for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
       if (__shfl_sync(0xffffffffu, v, 0) >= target) break;
+      if ((it & 15u) != 0) continue;  // the clock is read every 16th poll
       if (__shfl_sync(0xffffffffu, (int)(now_ns() - t0 >= wait_ns), 0)) {  // wait_ns = 0: one poll
         if (lane == 0) atomicOr(flag, 16);
         ok = 0;
@@ -103,6 +114,45 @@ __device__ bool grid_sync(unsigned* lanes, unsigned target, uint64_t wait_ns, in
   }
   __syncthreads();
   return s_ok != 0;
+}
+
+// jacobi_rotation by a whole warp. An FP64 instruction takes 64 cycles for one
+// lane or 32, so what one lane did one after another is laid across lanes: the
+// test |c|^2 > tol^2 a b beside |c|^2, and the two reciprocal square roots of
+// the first stage (of |c|^2 and of d^2 + 4 |c|^2, whose product with its
+// argument is the square root) as one. 3.0k -> 1.5k cycles of a round's ~10k.
+// Results in par (cs, sn, e); *go = 0 (pair left alone), 1 (a small rotation) or
+// 2. Small: the columns' cosine was at most kBigCos and the angle at most
+// kBigSin. A sweep of small rotations only is the last one: what it leaves
+// of the cosines is their product, below 1e-17, so no sweep is spent on
+// finding nothing to rotate.
+constexpr double kBigCos = 1e-10, kBigSin = 1e-8;
+__device__ __forceinline__ void rotate_warp(double a, double b, double cr, double ci, double tol, double tiny2,
+                                            double* par, int* go) {
+  const int lane = threadIdx.x & 31;
+  // lane 0: |c|^2, lane 1: tol^2 a b, lane 2: kBigCos^2 a b
+  const double t = lane == 1 ? tol * tol : lane == 2 ? kBigCos * kBigCos : cr, u0 = lane == 0 ? cr : a * b;
+  double q = t * u0;
+  if (lane == 0) q = fma(ci, ci, q);
+  const double c2 = __shfl_sync(0xffffffffu, q, 0), lim = __shfl_sync(0xffffffffu, q, 1);
+  const double big = __shfl_sync(0xffffffffu, q, 2);
+  if (!(c2 > lim) || c2 == 0.0 || !(fmin(a, b) > tiny2)) {
+    if (lane == 0) *go = 0;
+    return;
+  }
+  const double d = b - a, c4 = 4.0 * c2;
+  const double arg = lane == 1 ? c2 : fma(d, d, c4);
+  const double y = rsqrt(arg);
+  const double ic = __shfl_sync(0xffffffffu, y, 1);   // 1 / |c|
+  const double sr = __shfl_sync(0xffffffffu, arg * y, 0);  // sqrt(d^2 + 4 |c|^2)
+  const double uu = fabs(d) + sr;
+  const double w = rsqrt(fma(uu, uu, c4));
+  // lane 0: cs = u w, lane 1: 2 |c| = 2 |c|^2 / |c|, lanes 2, 3: e = conj(c) / |c|
+  const double l = lane == 0 ? uu : lane == 1 ? 2.0 * c2 : lane == 2 ? cr : -ci;
+  double r = l * (lane == 0 ? w : ic);
+  if (lane == 1) r = d >= 0.0 ? r * w : -(r * w);
+  if (lane < 4) par[lane] = r;
+  if (lane == 1) *go = c2 > big || fabs(r) > kBigSin ? 2 : 1;
 }
 
 // Circle-method pair p of round rd among N (even) columns.
@@ -156,21 +206,35 @@ __device__ __forceinline__ bool phase_sync(unsigned* lanes, unsigned target, uin
   }
 }
 
-// sync: [0, 8) barrier lanes, [8, 8 + max_sweeps) rotations per sweep; zeroed
-// before the launch. kCluster: the CTAs form one thread-block cluster.
+// sync: [0, 8) barrier lanes, [8, 8 + max_sweeps) rotations per sweep, then the columns' rounds; zeroed
+// before the launch. kCluster: the CTAs form one thread-block cluster. V may be
+// null (no right vectors). nc_dev (nullable): the column count, at most nc,
+// found on the device; columns beyond it are zero.
+//
+// Between the rounds of the grid form a CTA waits for its two columns only:
+// ver[j] counts the rounds column j has been through, written with release by
+// the CTA that finished it and polled with acquire by the one that takes it
+// next. A round's hand-over is then one flag to one reader instead of a
+// barrier over all CTAs; one grid barrier a sweep remains, for its rotation count.
+// (sync + kVerOff: up to kSvdMaxVer columns; wider matrices keep the barrier.)
+// The two-site split of the rank-16 driven system (256 x 100 and 256 x 64), per
+// step of 14 splits: 148 ms with accumulated right vectors and one barrier a
+// round; 45 ms with R^H in place of the matrix, 41 with column hand-over and
+// the early last sweep, 40 with four warps a CTA.
 template <bool kCluster>
-__global__ void __launch_bounds__(kThreads) k_jacobi_grid(double2* __restrict__ A, double2* __restrict__ V, int nr,
-                                                          int nc, double* __restrict__ sigma, int* __restrict__ info,
+__global__ void __launch_bounds__(kJThreads) k_jacobi_grid(double2* __restrict__ A, double2* __restrict__ V, int nr,
+                                                          int nc_in, const int* nc_dev, double* __restrict__ sigma, int* __restrict__ info,
                                                           unsigned* sync, int* flag, double tol, int max_sweeps,
                                                           int tr, uint64_t wait_ns) {
-  static_assert(kWarps * 4 == 32, "warp 0 adds four sums of each warp, one per lane");
-  __shared__ double s_red[kWarps][4];
+  static_assert(kJWarps * 4 <= 32 && (kJWarps & (kJWarps - 1)) == 0, "warp 0 adds four sums of each warp, one per lane");
+  __shared__ double s_red[kJWarps][4];
   __shared__ double s_par[4];
   __shared__ int s_go;
   __shared__ unsigned s_total;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int G = gridDim.x;
-  const int N = nc + (nc & 1), npairs = N / 2;
+  const int nc = nc_dev ? max(0, min(*nc_dev, nc_in)) : nc_in;
+  const int N = max(2, nc + (nc & 1)), npairs = N / 2;
   unsigned nbar = 0;
   bool ok = true;
   // ||A||_F^2: column norms of columns jc = blockIdx.x (mod G) into sigma[]
@@ -178,13 +242,13 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_grid(double2* __restrict__ 
   for (int jc = blockIdx.x; jc < nc; jc += G) {
     const double2* x = A + (int64_t)jc * nr;
     double f = 0.0;
-    for (int r = tid; r < nr; r += kThreads) f = fma(x[r].x, x[r].x, fma(x[r].y, x[r].y, f));
+    for (int r = tid; r < nr; r += kJThreads) f = fma(x[r].x, x[r].x, fma(x[r].y, x[r].y, f));
     f = wsum(f);
     if (lane == 0) s_red[wid][0] = f;
     __syncthreads();
     if (tid == 0) {
       double t = 0.0;
-      for (int w = 0; w < kWarps; ++w) t += s_red[w][0];
+      for (int w = 0; w < kJWarps; ++w) t += s_red[w][0];
       sigma[jc] = t;
     }
     __syncthreads();
@@ -195,18 +259,47 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_grid(double2* __restrict__ 
   double fro2 = 0.0;
   for (int jc = 0; jc < nc; ++jc) fro2 += sigma[jc];
   const double tiny2 = jacobi_negligible(nr, fro2);
+  unsigned* ver = sync + kVerOff;
+  const bool p2p = !kCluster && nc <= kSvdMaxVer;
+  __shared__ int s_alive;
   int sweep = 0;
+  unsigned round = 0;  // rounds done, over all sweeps
   for (; sweep < max_sweeps; ++sweep) {
     unsigned rot = 0;
     for (int rd = 0; rd < N - 1 && ok; ++rd) {
       for (int p = blockIdx.x; p < npairs; p += G) {
         int i, j;
         round_pair(N, rd, p, i, j);
-        if (j >= nc) continue;  // the dummy column of an odd count
+        if (p2p) {
+          if (tid < 32) {
+            const int cj = tid == 0 ? i : j;
+            bool alive = true;
+            if (tid < 2 && cj < nc && ld_acquire(ver + cj) != round) {
+              const uint64_t t0 = now_ns();
+              for (unsigned it = 1; ld_acquire(ver + cj) != round; ++it)
+                if ((it & 15u) == 0 && now_ns() - t0 >= wait_ns) {
+                  atomicOr(flag, 16);
+                  alive = false;
+                  break;
+                }
+            }
+            alive = __all_sync(0xffffffffu, alive);
+            if (tid == 0) s_alive = alive ? 1 : 0;
+          }
+          __syncthreads();
+          if (!s_alive) {
+            ok = false;
+            break;
+          }
+        }
+        if (j >= nc) {  // the dummy column of an odd count
+          if (p2p && tid == 0) st_release(ver + i, round + 1);
+          continue;
+        }
         double2* x = A + (int64_t)i * nr;
         double2* y = A + (int64_t)j * nr;
         double a = 0.0, b = 0.0, cr = 0.0, ci = 0.0;
-        for (int r = tid; r < nr; r += kThreads) {
+        for (int r = tid; r < nr; r += kJThreads) {
           const double2 xv = x[r], yv = y[r];
           a = fma(xv.x, xv.x, fma(xv.y, xv.y, a));
           b = fma(yv.x, yv.x, fma(yv.y, yv.y, b));
@@ -216,42 +309,47 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_grid(double2* __restrict__ 
         const double sum = warp_sum4(a, b, cr, ci);
         if ((lane & 7) == 0) s_red[wid][lane >> 3] = sum;
         __syncthreads();
-        if (wid == 0) {  // the rotation, once per pair: warp 0 adds the warps' sums, lane 0 rotates
+        if (wid == 0) {  // the rotation, once per pair: warp 0 adds the warps' sums and rotates
           // lane l holds quantity l & 3 of warp l >> 2; a fixed butterfly over the warp bits
-          double v = s_red[lane >> 2][lane & 3];
-          for (int o = 4; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          double v = s_red[(lane >> 2) % kJWarps][lane & 3];
+          for (int o = 4; o < 4 * kJWarps; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
           const double ga = __shfl_sync(0xffffffffu, v, 0), gb = __shfl_sync(0xffffffffu, v, 1);
           const double gr = __shfl_sync(0xffffffffu, v, 2), gi = __shfl_sync(0xffffffffu, v, 3);
-          if (lane == 0) {
-            double cs, sn;
-            double2 e;
-            s_go = jacobi_rotation(ga, gb, gr, gi, tol, tiny2, cs, sn, e) ? 1 : 0;
-            s_par[0] = cs;
-            s_par[1] = sn;
-            s_par[2] = e.x;
-            s_par[3] = e.y;
-          }
+          rotate_warp(ga, gb, gr, gi, tol, tiny2, s_par, &s_go);
         }
         __syncthreads();  // s_red and s_par are rewritten only after the next pair's sums
-        if (!s_go) continue;
+        const int go = s_go;
+        if (go == 0) {
+          if (p2p && tid < 2) st_release(ver + (tid == 0 ? i : j), round + 1);
+          continue;
+        }
         const double cs = s_par[0], sn = s_par[1];
         const double2 e = make_double2(s_par[2], s_par[3]);
-        for (int r = tid; r < nr; r += kThreads) {
+        for (int r = tid; r < nr; r += kJThreads) {
           const double2 xv = x[r], yv = cmul(e, y[r]);
           x[r] = make_double2(cs * xv.x - sn * yv.x, cs * xv.y - sn * yv.y);
           y[r] = make_double2(sn * xv.x + cs * yv.x, sn * xv.y + cs * yv.y);
         }
-        double2* vx = V + (int64_t)i * nc;
-        double2* vy = V + (int64_t)j * nc;
-        for (int r = tid; r < nc; r += kThreads) {
-          const double2 xv = vx[r], yv = cmul(e, vy[r]);
-          vx[r] = make_double2(cs * xv.x - sn * yv.x, cs * xv.y - sn * yv.y);
-          vy[r] = make_double2(sn * xv.x + cs * yv.x, sn * xv.y + cs * yv.y);
+        if (V) {
+          double2* vx = V + (int64_t)i * nc;
+          double2* vy = V + (int64_t)j * nc;
+          for (int r = tid; r < nc; r += kJThreads) {
+            const double2 xv = vx[r], yv = cmul(e, vy[r]);
+            vx[r] = make_double2(cs * xv.x - sn * yv.x, cs * xv.y - sn * yv.y);
+            vy[r] = make_double2(sn * xv.x + cs * yv.x, sn * xv.y + cs * yv.y);
+          }
         }
-        ++rot;
+        rot += go == 2;
+        if (p2p) {
+          __syncthreads();  // the pair's columns are written
+          if (tid < 2) st_release(ver + (tid == 0 ? i : j), round + 1);
+        }
       }
-      // the sweep's rotation count is published before its last barrier
+      ++round;
+      if (!ok) break;
+      // the sweep's count of rotations that ask for another sweep is published before its last barrier
       if (rd == N - 2 && tid == 0 && rot > 0) atomicAdd(sync + kBarLanes + sweep, rot);
+      if (p2p && rd < N - 2) continue;
       ++nbar;
       ok = phase_sync<kCluster>(sync, nbar * (unsigned)G, wait_ns, flag);
     }
@@ -265,22 +363,232 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_grid(double2* __restrict__ 
   for (int jc = blockIdx.x; jc < nc; jc += G) {
     const double2* x = A + (int64_t)jc * nr;
     double a = 0.0;
-    for (int r = tid; r < nr; r += kThreads) a = fma(x[r].x, x[r].x, fma(x[r].y, x[r].y, a));
+    for (int r = tid; r < nr; r += kJThreads) a = fma(x[r].x, x[r].x, fma(x[r].y, x[r].y, a));
     a = wsum(a);
     if (lane == 0) s_red[wid][0] = a;
     __syncthreads();
     if (tid == 0) {
       double t = 0.0;
-      for (int w = 0; w < kWarps; ++w) t += s_red[w][0];
+      for (int w = 0; w < kJWarps; ++w) t += s_red[w][0];
       sigma[jc] = sqrt(t);
     }
     __syncthreads();
   }
-  if (blockIdx.x == 0 && tid == 0) {
-    info[0] = sweep;
-    info[1] = tr;
+  if (blockIdx.x == 0) {
+    for (int jc = nc + tid; jc < nc_in; jc += kJThreads) sigma[jc] = 0.0;
+    if (tid == 0) {
+      info[0] = sweep;
+      info[1] = tr;
+    }
   }
 }
+
+// Column-pivoted Householder QR of B (nb x ni, nb = the rows of theta that are
+// not the isometry's, ni = the isometry's): B P = Q R, of which only
+// X = R^H (ni x k, column-major, rows in the original order) is kept. One-sided
+// Jacobi on X turns it into W Sigma with W the isometry's singular vectors. R^H
+// is nearly diagonal where the singular values fall fast, so the sweeps drop
+// from 17-20 to 9-11 on the two-site matrices of a run (rank-16 driven
+// system, 256 x 100), and no rotation has to be accumulated.
+//
+// The columns are dealt to the CTAs and live in shared memory. A step is one
+// grid barrier: every CTA publishes its largest remaining column and the norm,
+// then all pick the same pivot (ties: lower index), read that column from L2
+// and apply its reflector to their own columns. A step is a latency chain
+// (barrier, candidates, pivot column, scalars, dot, update) of about 5 us
+// whatever the size. *keff: the number of steps; it stops early when every
+// remaining column is rounding noise of the matrix (jacobi_negligible).
+constexpr int kPivMaxCols = 8;  // columns per CTA
+constexpr int kPivSmem = 200 * 1024;
+__global__ void __launch_bounds__(kThreads) k_pivot_qr(const double2* __restrict__ theta, int m, int n, int iso_first,
+                                                       double2* __restrict__ Bg, double2* __restrict__ X, double* cand,
+                                                       int* cand_i, double* fpart, int* keff, unsigned* sync, int* flag,
+                                                       uint64_t wait_ns) {
+  extern __shared__ double2 sm[];
+  __shared__ double s_nrm[kPivMaxCols], s_part[kWarps][3], s_sc[8];
+  __shared__ int s_done[kPivMaxCols], s_piv;
+  __shared__ long long s_best;
+  const int nb = iso_first ? n : m, ni = iso_first ? m : n;
+  const int k = min(nb, ni), G = gridDim.x;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  double2* v = sm;         // [nb] reflector
+  double2* col = sm + nb;  // [ncl][nb]
+  const int ncl = blockIdx.x < ni ? (ni - 1 - blockIdx.x) / G + 1 : 0;
+  // warps of a column: all eight for one column, down to one for eight
+  const int gs = ncl <= 1 ? 8 : ncl <= 2 ? 4 : ncl <= 4 ? 2 : 1;
+  const int my = wid / gs, gw = wid % gs;  // this warp's column and place in its group
+  const bool on = my < ncl;
+  double2* a = col + (size_t)my * nb;
+  auto group_sum = [&](double x, double y, double z, double& ox, double& oy, double& oz) {
+    // sums over the warps of a column, in order; block-uniform barriers
+    for (int o = 16; o > 0; o >>= 1) {
+      x += __shfl_xor_sync(0xffffffffu, x, o);
+      y += __shfl_xor_sync(0xffffffffu, y, o);
+      z += __shfl_xor_sync(0xffffffffu, z, o);
+    }
+    __syncthreads();
+    if (lane == 0) {
+      s_part[wid][0] = x;
+      s_part[wid][1] = y;
+      s_part[wid][2] = z;
+    }
+    __syncthreads();
+    const int w0 = (wid / gs) * gs;
+    ox = s_part[w0][0];
+    oy = s_part[w0][1];
+    oz = s_part[w0][2];
+    for (int w = w0 + 1; w < w0 + gs; ++w) {
+      ox += s_part[w][0];
+      oy += s_part[w][1];
+      oz += s_part[w][2];
+    }
+  };
+  double nrm = 0.0, u1, u2;
+  {
+    double f = 0.0;
+    if (on) {
+      const int i = blockIdx.x + my * G;
+      for (int r = gw * 32 + lane; r < nb; r += gs * 32) {
+        const double2 t = iso_first ? cconj(theta[(int64_t)i * n + r]) : theta[(int64_t)r * n + i];
+        a[r] = t;
+        f = fma(t.x, t.x, fma(t.y, t.y, f));
+      }
+    }
+    group_sum(f, 0.0, 0.0, nrm, u1, u2);
+    if (on && gw == 0 && lane == 0) {
+      s_nrm[my] = nrm;
+      s_done[my] = 0;
+    }
+  }
+  __syncthreads();
+  if (tid == 0) {
+    double f = 0.0;
+    for (int l = 0; l < ncl; ++l) f += s_nrm[l];
+    fpart[blockIdx.x] = f;
+  }
+  unsigned nbar = 0;
+  double tiny2 = 0.0;
+  int c = 0;
+  for (; c < k; ++c) {
+    // candidate: the largest remaining column of this CTA
+    if (tid == 0) {
+      int best = -1;
+      for (int l = 0; l < ncl; ++l)
+        if (!s_done[l] && (best < 0 || s_nrm[l] > s_nrm[best])) best = l;
+      s_piv = best;
+      const int slot = (c & 1) * G + blockIdx.x;
+      cand[slot] = best < 0 ? -1.0 : s_nrm[best];
+      cand_i[slot] = best < 0 ? 0x7fffffff : (int)blockIdx.x + best * G;
+    }
+    __syncthreads();
+    if (s_piv >= 0) {
+      const double2* src = col + (size_t)s_piv * nb;
+      double2* dst = Bg + (int64_t)(blockIdx.x + s_piv * G) * nb;
+      for (int r = c + tid; r < nb; r += kThreads) dst[r] = src[r];
+    }
+    ++nbar;
+    if (!grid_sync(sync, nbar * (unsigned)G, wait_ns, flag)) return;
+    if (c == 0) {
+      double f = 0.0;
+      for (int q = 0; q < G; ++q) f += __ldcg(fpart + q);
+      tiny2 = jacobi_negligible(max(nb, ni), f);
+      if (!isfinite(f)) {  // nothing to factor: report it, no columns (uniform over the grid)
+        if (blockIdx.x == 0 && tid == 0) atomicOr(flag, 1);
+        break;
+      }
+    }
+    if (wid == 0) {  // pivot: largest norm (positive doubles order like their bits), then lowest index
+      long long bv = -1;
+      int bi = 0x7fffffff;
+      for (int q = lane; q < G; q += 32) {
+        const double cv = __ldcg(cand + (c & 1) * G + q);
+        const long long kb = cv < 0.0 ? -1 : __double_as_longlong(cv);
+        const int ki = __ldcg(cand_i + (c & 1) * G + q);
+        if (kb > bv || (kb == bv && ki < bi)) {
+          bv = kb;
+          bi = ki;
+        }
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        const long long ov = __shfl_xor_sync(0xffffffffu, bv, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (ov > bv || (ov == bv && oi < bi)) {
+          bv = ov;
+          bi = oi;
+        }
+      }
+      if (lane == 0) {
+        s_best = bv;
+        s_piv = bi;
+      }
+    }
+    __syncthreads();
+    const double n2 = s_best < 0 ? 0.0 : __longlong_as_double(s_best);
+    if (!(n2 > tiny2)) break;  // uniform over the grid: every CTA sees the same candidates
+    const int pi = s_piv;
+    const double2* xp = Bg + (int64_t)pi * nb;
+    if (wid == 0) {
+      const double2 x0 = __ldcg(xp + c);
+      // lane 0: alpha = |x|, lane 1: |x_0|
+      const double rt = sqrt(lane == 1 ? fma(x0.x, x0.x, x0.y * x0.y) : n2);
+      const double alpha = __shfl_sync(0xffffffffu, rt, 0), ax0 = __shfl_sync(0xffffffffu, rt, 1);
+      const double rc = 1.0 / (lane == 1 ? alpha * (alpha + ax0) : ax0);
+      const double inv = __shfl_sync(0xffffffffu, rc, 0), beta = __shfl_sync(0xffffffffu, rc, 1);
+      const double2 phi = ax0 > 0.0 ? make_double2(x0.x * inv, x0.y * inv) : make_double2(1.0, 0.0);
+      if (lane == 0) {
+        s_sc[0] = fma(phi.x, alpha, x0.x);  // v_0
+        s_sc[1] = fma(phi.y, alpha, x0.y);
+        s_sc[2] = beta;
+        s_sc[3] = -phi.x * alpha;  // R_cc
+        s_sc[4] = -phi.y * alpha;
+      }
+    }
+    for (int r = c + tid; r < nb; r += kThreads) v[r] = __ldcg(xp + r);
+    __syncthreads();
+    if (tid == 0) v[c] = make_double2(s_sc[0], s_sc[1]);
+    const bool mine = on && (int)blockIdx.x + my * G == pi;
+    const bool act = on && !s_done[my] && !mine;
+    __syncthreads();
+    double wr = 0.0, wi = 0.0;
+    if (act)
+      for (int r = c + gw * 32 + lane; r < nb; r += gs * 32) {
+        const double2 x = v[r], y = a[r];
+        wr = fma(x.x, y.x, fma(x.y, y.y, wr));
+        wi = fma(x.x, y.y, fma(-x.y, y.x, wi));
+      }
+    double sr, si, sn;
+    group_sum(wr, wi, 0.0, sr, si, sn);
+    const double beta = s_sc[2];
+    sr *= beta;
+    si *= beta;
+    double f = 0.0;
+    if (act)
+      for (int r = c + gw * 32 + lane; r < nb; r += gs * 32) {
+        const double2 x = v[r];
+        double2 y = a[r];
+        y.x = fma(-x.x, sr, fma(x.y, si, y.x));
+        y.y = fma(-x.x, si, fma(-x.y, sr, y.y));
+        a[r] = y;
+        if (r > c) f = fma(y.x, y.x, fma(y.y, y.y, f));
+      }
+    group_sum(f, 0.0, 0.0, nrm, u1, u2);
+    if (on && gw == 0 && lane == 0) {
+      const int i = blockIdx.x + my * G;
+      double2 t = make_double2(0.0, 0.0);  // a column finished earlier has no entry in this row of R
+      if (mine)
+        t = make_double2(s_sc[3], -s_sc[4]);
+      else if (act)
+        t = cconj(a[c]);
+      X[(int64_t)c * ni + i] = t;
+      if (mine) s_done[my] = 1;
+      if (act) s_nrm[my] = nrm;
+    }
+    __syncthreads();
+  }
+  if (blockIdx.x == 0 && tid == 0) *keff = c;
+}
+
+size_t pivot_smem(int nb, int ni, int G) { return sizeof(double2) * (size_t)nb * (1 + (ni + G - 1) / G); }
 
 struct GridInfo {
   int sms = 0, coop = 0, occ = 0;
@@ -294,8 +602,9 @@ GridInfo grid_info() {
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&gi.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       gi.sms = 1;
     if (cudaDeviceGetAttribute(&gi.coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess) gi.coop = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&gi.occ, k_jacobi_grid<false>, kThreads, 0) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&gi.occ, k_jacobi_grid<false>, kJThreads, 0) != cudaSuccess)
       gi.occ = 0;
+    cudaFuncSetAttribute(k_pivot_qr, cudaFuncAttributeMaxDynamicSharedMemorySize, kPivSmem);
     gi.cluster16 = cudaFuncSetAttribute(k_jacobi_grid<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
                    cudaSuccess;
   });
@@ -325,7 +634,7 @@ bool launch_jacobi_svd_grid(const double2* theta, int m, int n, double2* A, doub
   const int tr = n > m ? 1 : 0;
   const double tol = jacobi_tol(m, n);
   cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.blockDim = dim3(kJThreads, 1, 1);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   cfg.attrs = at;
@@ -336,15 +645,102 @@ bool launch_jacobi_svd_grid(const double2* theta, int m, int n, double2* A, doub
     at[0].val.clusterDim.x = npairs;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
-    return cudaLaunchKernelEx(&cfg, k_jacobi_grid<true>, A, V, nr, nc, sigma, info, sync, flag, tol, kJacMaxSweeps, tr,
+    return cudaLaunchKernelEx(&cfg, k_jacobi_grid<true>, A, V, nr, nc, (const int*)nullptr, sigma, info, sync, flag, tol, kJacMaxSweeps, tr,
                               wait_ns) == cudaSuccess;
   }
   const int G = std::max(1, std::min(npairs, gi.sms * std::min(gi.occ, 2)));
   cfg.gridDim = dim3(G, 1, 1);
   at[0].id = cudaLaunchAttributeCooperative;
   at[0].val.cooperative = 1;
-  return cudaLaunchKernelEx(&cfg, k_jacobi_grid<false>, A, V, nr, nc, sigma, info, sync, flag, tol, kJacMaxSweeps, tr,
+  return cudaLaunchKernelEx(&cfg, k_jacobi_grid<false>, A, V, nr, nc, (const int*)nullptr, sigma, info, sync, flag, tol, kJacMaxSweeps, tr,
                             wait_ns) == cudaSuccess;
+}
+
+bool launch_pivot_svd(const double2* theta, int m, int n, bool iso_first, double2* X, double2* Bg, double* sigma,
+                      double* cand, int* info, unsigned* sync, int* flag, uint64_t wait_ns, cudaStream_t s) {
+  const int nb = iso_first ? n : m, ni = iso_first ? m : n, k = std::min(m, n);
+  const GridInfo gi = grid_info();
+  // the pivoted QR pays its ~5 us a column where the sweeps it saves are those
+  // of the grid Jacobi (more columns than a cluster holds)
+  if (k <= 2 * kJacClusterMax || !gi.coop || gi.occ < 1 || gi.sms < 2) return false;
+  const int G = std::min({ni, gi.sms, kPivMaxGrid});
+  if ((ni + G - 1) / G > kPivMaxCols || pivot_smem(nb, ni, G) > (size_t)kPivSmem) return false;
+  // the column count stays zero if the factorisation gives up
+  if (cudaMemsetAsync(sync, 0, kSvdSyncInts * sizeof(unsigned), s) != cudaSuccess ||
+      cudaMemsetAsync(info + 2, 0, sizeof(int), s) != cudaSuccess)
+    return false;
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cfg.gridDim = dim3(G, 1, 1);
+  cfg.dynamicSmemBytes = pivot_smem(nb, ni, G);
+  double* fpart = cand + 2 * kPivMaxGrid;
+  int* cand_i = (int*)(fpart + kPivMaxGrid);
+  if (cudaLaunchKernelEx(&cfg, k_pivot_qr, theta, m, n, iso_first ? 1 : 0, Bg, X, cand, cand_i, fpart, info + 2, sync,
+                         flag, wait_ns) != cudaSuccess)
+    return false;
+  if (cudaMemsetAsync(sync, 0, kSvdSyncInts * sizeof(unsigned), s) != cudaSuccess) return false;
+  cfg.dynamicSmemBytes = 0;
+  cfg.blockDim = dim3(kJThreads, 1, 1);
+  cfg.gridDim = dim3(std::max(1, std::min((k + 1) / 2, gi.sms * std::min(gi.occ, 2))), 1, 1);
+  return cudaLaunchKernelEx(&cfg, k_jacobi_grid<false>, X, (double2*)nullptr, ni, k, (const int*)(info + 2), sigma,
+                            info, sync, flag, jacobi_tol(m, n), kJacMaxSweeps, iso_first ? 0 : 1,
+                            wait_ns) == cudaSuccess;
+}
+
+// Isometry columns a < g from W Sigma (X, ni x k column-major), Z = W or its
+// conjugate (second side), zero beyond g; Zg the same; centre = theta
+// contracted with conj(Z), one warp per entry.
+__global__ void k_pivot_iso(const double2* __restrict__ X, const double* __restrict__ sigma, const int* __restrict__ perm,
+                            int ni, int r, int g, int iso_first, double2* Z, double2* Zg) {
+  const int64_t nz = (int64_t)ni * r;
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nz; q += (int64_t)gridDim.x * blockDim.x) {
+    const int a = (int)(q % r), row = (int)(q / r);
+    double2 v = make_double2(0.0, 0.0);
+    if (a < g) {
+      const int j = perm[a];
+      const double2 x = X[(int64_t)j * ni + row];
+      v = make_double2(x.x / sigma[j], (iso_first ? x.y : -x.y) / sigma[j]);
+    }
+    Z[q] = v;
+    Zg[q] = v;
+  }
+}
+__global__ void __launch_bounds__(256) k_pivot_centre(const double2* __restrict__ theta, int m, int n,
+                                                      const double2* __restrict__ Z, int r, int iso_first,
+                                                      double2* __restrict__ Cm) {
+  const int lane = threadIdx.x & 31;
+  const int ni = iso_first ? m : n, no = iso_first ? n : m;
+  const int64_t tot = (int64_t)no * r;
+  for (int64_t w = blockIdx.x * (int64_t)(blockDim.x / 32) + (threadIdx.x >> 5); w < tot;
+       w += (int64_t)gridDim.x * (blockDim.x / 32)) {
+    // iso_first: Cm[a][col] (r x n); second: Cm[row][a] (m x r)
+    const int a = iso_first ? (int)(w / no) : (int)(w % r), o = iso_first ? (int)(w % no) : (int)(w / r);
+    double2 acc = make_double2(0.0, 0.0);
+    for (int i = lane; i < ni; i += 32) {
+      const double2 z = Z[(int64_t)i * r + a], t = iso_first ? theta[(int64_t)i * n + o] : theta[(int64_t)o * n + i];
+      acc.x = fma(z.x, t.x, fma(z.y, t.y, acc.x));
+      acc.y = fma(z.x, t.y, fma(-z.y, t.x, acc.y));
+    }
+    for (int q = 16; q > 0; q >>= 1) {
+      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, q);
+      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, q);
+    }
+    if (lane == 0) Cm[w] = acc;
+  }
+}
+void launch_pivot_vecs(const double2* theta, int m, int n, bool iso_first, const double2* X, const double* sigma,
+                       const int* perm, int r, int g, double2* Z, double2* Zg, double2* Cm, cudaStream_t s) {
+  const int ni = iso_first ? m : n, no = iso_first ? n : m;
+  k_pivot_iso<<<(int)std::min<int64_t>(((int64_t)ni * r + 255) / 256, 1024), 256, 0, s>>>(X, sigma, perm, ni, r, g,
+                                                                                          iso_first ? 1 : 0, Z, Zg);
+  k_pivot_centre<<<(int)std::min<int64_t>(((int64_t)no * r + 7) / 8, 4096), 256, 0, s>>>(theta, m, n, Z, r,
+                                                                                         iso_first ? 1 : 0, Cm);
 }
 
 namespace {
