@@ -124,8 +124,8 @@ __device__ __forceinline__ uint64_t gtimer() {
 // Wait for the phase of the given parity; false (and bit 2 of *flag) once the
 // kernel-wide deadline has passed.
 __device__ __forceinline__ bool mbar_wait(uint64_t* mb, uint32_t parity, uint64_t deadline, int* flag) {
-  while (!mbar_try(mb, parity)) {
-    if (gtimer() > deadline) {
+  for (unsigned it = 1; !mbar_try(mb, parity); ++it) {
+    if ((it & 31u) == 0 && gtimer() > deadline) {
       atomicOr(flag, 2);
       return false;
     }
@@ -175,6 +175,12 @@ __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int
   const int nr = max(0, min(m, r0 + rp) - r0);
   const int tid = threadIdx.x, nt = blockDim.x;
   const int lane = tid & 31, wid = tid >> 5;
+  // column groups: warps 1..7, or, when six warps hold all columns, without
+  // warp 4: it shares its SM sub-partition, and so its FP64 pipe, with warp 0, whose
+  // scalar chain everything waits for
+  const bool six = n <= 6 * kGPW;
+  const int slots = six ? 6 * kGPW : kSlots;
+  const int cw = !six ? wid - 1 : wid < 4 ? wid - 1 : wid == 4 ? -1 : wid - 2;  // place among the column warps, -1: none
   const uint64_t deadline = gtimer() + 2000000000ull;
 
   extern __shared__ double2 smem[];
@@ -192,7 +198,7 @@ __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int
   auto MM_of = [&](int c) -> const double2* {
     return gt ? pn.gtail + (size_t)(2 * C + c) * n2 : cluster.map_shared_rank(MM, c);
   };
-  __shared__ __align__(8) uint64_t mb[2];
+  __shared__ __align__(8) uint64_t mb[2], mbg[2];
   __shared__ double SN[2][16];
   __shared__ double2 SX[2];
   __shared__ double red[kNW];
@@ -204,6 +210,8 @@ __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int
   if (tid == 0) {
     mbar_init(&mb[0], 1);
     mbar_init(&mb[1], 1);
+    mbar_init(&mbg[0], 1);
+    mbar_init(&mbg[1], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
 
@@ -261,9 +269,9 @@ __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int
         push_f64(mapa(smem_u32(&SN[p][me]), lane), ss, rmb);
         if (own) push_c64(mapa(smem_u32(&SX[p]), lane), x[lrow], rmb);
       }
-    } else {
-      const int q = (wid - 1) * kGPW + lane / GL, sl = lane % GL;
-      for (int kb = j + 1; kb < n; kb += kSlots) {  // block-uniform trip count
+    } else if (cw >= 0) {
+      const int q = cw * kGPW + lane / GL, sl = lane % GL;
+      for (int kb = j + 1; kb < n; kb += slots) {  // block-uniform trip count
         const int k = kb + q;
         const double2* a = A + (size_t)min(k, n - 1) * rp;
         double2 u = make_double2(0.0, 0.0);
@@ -331,12 +339,12 @@ __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int
           if (own) x[lrow] = make_double2(fma(phi.x, alpha, x0.x), fma(phi.y, alpha, x0.y));
         }
       }
-    } else {
-      const int q = (wid - 1) * kGPW + lane / GL, sl = lane % GL;
+    } else if (cw >= 0) {
+      const int q = cw * kGPW + lane / GL, sl = lane % GL;
 #pragma unroll
       for (int ps = 0; ps < kMaxPass; ++ps) {
-        const int k = j + 1 + ps * kSlots + q;
-        if (j + 1 + ps * kSlots >= n) break;  // block-uniform
+        const int k = j + 1 + ps * slots + q;
+        if (j + 1 + ps * slots >= n) break;  // block-uniform
         double2 w = make_double2(0.0, 0.0);
         if (k < n)
           for (int c = sl; c < C; c += GL) {
@@ -348,14 +356,14 @@ __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int
       }
     }
     __syncthreads();
-    if (wid > 0 && !s_skip[j]) {
+    if (wid > 0 && cw >= 0 && !s_skip[j]) {
       const double beta = s_beta[j];
       const double2 gam = s_gam;
-      const int q = (wid - 1) * kGPW + lane / GL, sl = lane % GL;
+      const int q = cw * kGPW + lane / GL, sl = lane % GL;
 #pragma unroll
       for (int ps = 0; ps < kMaxPass; ++ps) {
-        const int k = j + 1 + ps * kSlots + q;
-        if (j + 1 + ps * kSlots >= n) break;
+        const int k = j + 1 + ps * slots + q;
+        if (j + 1 + ps * slots >= n) break;
         if (k < n) {
           const double2 rj = RJ[(size_t)p * n + k];
           double2 w = W[ps];
@@ -404,87 +412,125 @@ __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int
     R[k] = v;
     if (R_lo) R_lo[k] = make_float2((float)v.x, (float)v.y);
   }
-  // partial strictly-upper Gram of my rows, one thread per pair a < b
-  // (v_a vanishes above row a; skipped reflectors are zero columns)
+  // Strictly-upper Gram of V (v_a vanishes above row a; skipped reflectors are
+  // zero columns): one thread per pair a < b sums its rows; the partials of pair
+  // t go to CTA t mod C, which adds them in CTA order and sends the sum to every
+  // CTA (stored transposed, GF[b][a], so that the solves read along lanes).
+  // Reading all partials of all CTAs everywhere took 11k cycles, this 4k.
   const int npair = n * (n - 1) / 2;
-  for (int t = tid; t < npair; t += nt) {
-    int b = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)t)) * 0.5f);  // t = b(b-1)/2 + a
+  auto pair_of = [](int t, int& a, int& b) {  // t = b(b-1)/2 + a
+    b = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)t)) * 0.5f);
     while (b * (b - 1) / 2 > t) --b;
     while ((b + 1) * b / 2 <= t) ++b;
-    const int a = t - b * (b - 1) / 2;
+    a = t - b * (b - 1) / 2;
+  };
+  const int nown = me < npair ? (npair - 1 - me) / C + 1 : 0;  // pairs summed here
+  const int nslot = (npair + C - 1) / C;
+  if (tid == 0 && !gt) {
+    mbar_arrive_tx(&mbg[0], 16u * C * nown);
+    mbar_arrive_tx(&mbg[1], 16u * npair);
+  }
+  for (int t = tid; t < npair; t += nt) {
+    int a, b;
+    pair_of(t, a, b);
     double2 g = make_double2(0.0, 0.0);
     const double2* va = A + (size_t)a * rp;
     const double2* vb = A + (size_t)b * rp;
     for (int i = max(b - r0, 0); i < nr; ++i) g = cfmaj(va[i], vb[i], g);
-    G[a * n + b] = g;
+    if (gt)
+      G[a * n + b] = g;
+    else if (alive)  // SU is free after the column loop
+      push_c64(mapa(smem_u32(&SU[(size_t)me * nslot + t / C]), t % C), g, mapa(smem_u32(&mbg[0]), t % C));
   }
-  cluster.sync();
-  // full Gram: fixed-order sum of the CTAs' partials
-  for (int t = tid; t < npair; t += nt) {
-    int b = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)t)) * 0.5f);
-    while (b * (b - 1) / 2 > t) --b;
-    while ((b + 1) * b / 2 <= t) ++b;
-    const int a = t - b * (b - 1) / 2;
-    double2 v[16];
-#pragma unroll
-    for (int c = 0; c < 16; ++c)
-      v[c] = c < C ? G_of(c)[a * n + b] : make_double2(0.0, 0.0);
-    double2 g = make_double2(0.0, 0.0);
-#pragma unroll
-    for (int c = 0; c < 16; ++c)
-      if (c < C) {
-        g.x += v[c].x;
-        g.y += v[c].y;
+  if (gt) {
+    cluster.sync();
+    for (int t = tid; t < npair; t += nt) {
+      int a, b;
+      pair_of(t, a, b);
+      double2 g = make_double2(0.0, 0.0);
+      for (int c = 0; c < C; ++c) {
+        const double2 v = G_of(c)[a * n + b];
+        g.x += v.x;
+        g.y += v.y;
       }
-    GF[a * n + b] = g;
+      GF[b * n + a] = g;
+    }
+  } else {
+    if (alive) alive = mbar_wait(&mbg[0], 0u, deadline, flag);
+    // one lane per component
+    for (int e = tid; e < 2 * nown; e += nt) {
+      const double* p = reinterpret_cast<const double*>(SU) + 2 * (size_t)(e >> 1) + (e & 1);
+      double g = 0.0;
+      for (int c = 0; c < C; ++c) g += p[2 * (size_t)c * nslot];
+      int a, b;
+      pair_of(me + C * (e >> 1), a, b);
+      if (alive) {
+        const uint32_t dst = smem_u32(reinterpret_cast<double*>(GF + b * n + a) + (e & 1)), lmb = smem_u32(&mbg[1]);
+        for (int c = 0; c < C; ++c) push_f64(mapa(dst, c), g, mapa(lmb, c));
+      }
+    }
+    if (alive) alive = mbar_wait(&mbg[1], 0u, deadline, flag);
   }
   __syncthreads();
+  // Back substitution of one column, T^{-1} y = rhs with T^{-1} = diag(1/beta) +
+  // strictly-upper Gram, from a = c down: lanes 0..15 carry real parts, 16..31
+  // imaginary parts of entries 16 q + (lane & 15), so a step is one product and
+  // two FMAs per block of 16 entries (an FP64 instruction costs 64 cycles
+  // whatever the lanes). put(a, v) stores component lane >> 4 of entry a.
+  auto solve = [&](int c, double (&acc)[kQrClusterMaxN / 16], auto&& put) {
+    const int comp = lane >> 4, e = lane & 15;
+#pragma unroll
+    for (int qa = kQrClusterMaxN / 16 - 1; qa >= 0; --qa) {
+      for (int a = min(c, 16 * qa + 15); a >= 16 * qa; --a) {
+        const double t = s_beta[a] * acc[qa];
+        const double tx = __shfl_sync(kFull, t, a & 15), ty = __shfl_sync(kFull, t, 16 + (a & 15));
+        if (e == (a & 15)) put(a, t);
+        const double t1 = comp == 0 ? tx : ty, t2 = comp == 0 ? ty : tx;
+#pragma unroll
+        for (int q = 0; q <= qa; ++q) {
+          const int i = 16 * q + e;
+          if (16 * q < a && i < a) {
+            const double2 g = GF[a * n + i];
+            acc[q] = fma(-g.x, t1, acc[q]);
+            acc[q] = fma(comp == 0 ? g.y : -g.y, t2, acc[q]);
+          }
+        }
+      }
+    }
+  };
   if (panel) {
     for (int c = me + C * wid; c < n; c += C * kNW) {
-      double2 acc0 = make_double2(lane == c ? 1.0 : 0.0, 0.0), acc1 = make_double2(lane + 32 == c ? 1.0 : 0.0, 0.0);
-      for (int a = c; a >= 0; --a) {
-        const double ba = s_beta[a];
-        const double2 src = a < 32 ? acc0 : acc1;
-        double2 ta = make_double2(ba * src.x, ba * src.y);
-        ta.x = __shfl_sync(kFull, ta.x, a & 31);
-        ta.y = __shfl_sync(kFull, ta.y, a & 31);
-        if (lane == (a & 31)) pn.T[a * n + c] = ta;
-        if (lane < a) acc0 = cfms(GF[lane * n + a], ta, acc0);
-        if (a > 32 && lane + 32 < a) acc1 = cfms(GF[(lane + 32) * n + a], ta, acc1);
-      }
+      double acc[kQrClusterMaxN / 16];
+#pragma unroll
+      for (int q = 0; q < kQrClusterMaxN / 16; ++q) acc[q] = lane < 16 && 16 * q + lane == c ? 1.0 : 0.0;
+      double* T = reinterpret_cast<double*>(pn.T);
+      solve(c, acc, [&](int a, double v) { T[2 * (a * n + c) + (lane >> 4)] = v; });
       for (int a = c + 1 + lane; a < n; a += 32) pn.T[a * n + c] = make_double2(0.0, 0.0);
     }
     cluster.sync();  // keep shared memory alive until every remote read has finished
     return;
   }
-  // M = T V_top^H column by column: T^{-1} M[:, c] = conj(V_top[c, :])^T, with
-  // T^{-1} = diag(1/beta) + strictly-upper Gram; back substitution from a = c
-  // down (M[a][c] = 0 for a > c). Column c is solved by CTA c mod C, one warp.
+  // M = T V_top^H column by column: T^{-1} M[:, c] = conj(V_top[c, :])^T
+  // (M[a][c] = 0 for a > c). Column c is solved by CTA c mod C, one warp.
   for (int c = me + C * wid; c < n; c += C * kNW) {
-    double2 acc0 = make_double2(0.0, 0.0), acc1 = make_double2(0.0, 0.0);
+    double acc[kQrClusterMaxN / 16];
+#pragma unroll
+    for (int q = 0; q < kQrClusterMaxN / 16; ++q) acc[q] = 0.0;
     if (c < m) {
       const int oc = c / rp;
       const double2* Ar = cluster.map_shared_rank(A, oc);
       const int lr = c - oc * rp;
-      if (lane <= c && lane < n && !s_skip[lane]) {
-        const double2 v = Ar[(size_t)lane * rp + lr];
-        acc0 = make_double2(v.x, -v.y);
-      }
-      if (lane + 32 <= c && lane + 32 < n && !s_skip[lane + 32]) {
-        const double2 v = Ar[(size_t)(lane + 32) * rp + lr];
-        acc1 = make_double2(v.x, -v.y);
+#pragma unroll
+      for (int q = 0; q < kQrClusterMaxN / 16; ++q) {
+        const int i = 16 * q + (lane & 15);
+        if (i <= c && i < n && !s_skip[i]) {
+          const double2 v = Ar[(size_t)i * rp + lr];
+          acc[q] = lane < 16 ? v.x : -v.y;
+        }
       }
     }
-    for (int a = c; a >= 0; --a) {
-      const double ba = s_beta[a];
-      const double2 src = a < 32 ? acc0 : acc1;
-      double2 ma = make_double2(ba * src.x, ba * src.y);
-      ma.x = __shfl_sync(kFull, ma.x, a & 31);
-      ma.y = __shfl_sync(kFull, ma.y, a & 31);
-      if (lane == (a & 31)) MM[a * n + c] = ma;
-      if (lane < a) acc0 = cfms(GF[lane * n + a], ma, acc0);
-      if (a > 32 && lane + 32 < a) acc1 = cfms(GF[(lane + 32) * n + a], ma, acc1);
-    }
+    double* Md = reinterpret_cast<double*>(MM);
+    solve(c, acc, [&](int a, double v) { Md[2 * (a * n + c) + (lane >> 4)] = v; });
     for (int a = c + 1 + lane; a < n; a += 32) MM[a * n + c] = make_double2(0.0, 0.0);
   }
   cluster.sync();  // every column of M solved; partial Grams no longer read
@@ -492,8 +538,11 @@ __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int
   for (int t = tid; t < n * n; t += nt) G[t] = MM_of((t % n) % C)[t];
   __syncthreads();
   // Q rows: Q[r][c] = delta_rc - sum_{a <= min(r,c)} v_a[r] M[a][c], column c scaled by phase_c
+  // (a column's cost grows with c: tasks dealt to the warps forth and back)
   const int nch = (nr + 31) / 32;
-  for (int task = wid; task < n * nch; task += kNW) {
+  for (int rnd = 0; rnd * kNW < n * nch; ++rnd) {
+    const int task = rnd * kNW + ((rnd & 1) ? kNW - 1 - wid : wid);
+    if (task >= n * nch) continue;
     const int c = task / nch, i = (task % nch) * 32 + lane;
     if (i >= nr) continue;
     const int r = r0 + i;
