@@ -72,14 +72,24 @@ __device__ __forceinline__ double wsum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
   return v;
 }
-// sum over aligned groups of G lanes; every lane of a group gets the same bits
+// Sum over aligned groups of G lanes: lanes of the group's lower half get the
+// real part, the upper half the imaginary part (the first exchange gives each
+// half one component, so a level costs one FP64 addition, 64 cycles, not two;
+// the sums are those of the plain butterfly).
 template <int G>
-__device__ __forceinline__ double2 gsum2(double2 v) {
-  for (int o = G / 2; o > 0; o >>= 1) {
-    v.x += __shfl_xor_sync(kFull, v.x, o);
-    v.y += __shfl_xor_sync(kFull, v.y, o);
-  }
-  return v;
+__device__ __forceinline__ double gsum_split(double2 v) {
+  const bool up = (threadIdx.x & (G / 2)) != 0;
+  double k = up ? v.y : v.x;
+  k += __shfl_xor_sync(kFull, up ? v.x : v.y, G / 2);
+  for (int o = G / 4; o > 0; o >>= 1) k += __shfl_xor_sync(kFull, k, o);
+  return k;
+}
+// (real, imaginary) in every lane from the split form
+template <int G>
+__device__ __forceinline__ double2 join_split(double k) {
+  const bool up = (threadIdx.x & (G / 2)) != 0;
+  const double o = __shfl_xor_sync(kFull, k, G / 2);
+  return up ? make_double2(o, k) : make_double2(k, o);
 }
 // block sum in a fixed order; every thread gets the result
 __device__ double bsum(double v, double* red) {
@@ -277,7 +287,7 @@ __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int
         double2 u = make_double2(0.0, 0.0);
         if (k < n)
           for (int i = i0 + sl; i < nr; i += GL) u = cfmaj(x[i], a[i], u);
-        u = gsum2<GL>(u);
+        u = join_split<GL>(gsum_split<GL>(u));
         if (alive && k < n) {
           const uint32_t su = smem_u32(&SU[((size_t)p * 16 + me) * n + k]);
           const uint32_t rj = smem_u32(&RJ[(size_t)p * n + k]);
@@ -307,9 +317,11 @@ __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int
     const int lrow = j - r0;
     if (alive) alive = mbar_wait(&mb[p], ph[p], deadline, flag);
     ph[p] ^= 1u;
-    double2 W[kMaxPass];
+    double W[kMaxPass];  // split form
     if (wid == 0) {
-      double a2 = lane < C ? SN[p][lane] : 0.0;  // C <= 16: lanes 0..15 carry the sum
+      // C <= 16: a half-warp carries the sum, both halves alike (a zero in any lane
+      // would send the whole warp through the square root's slow path)
+      double a2 = (lane & 15) < C ? SN[p][lane & 15] : 0.0;
       for (int o = 8; o > 0; o >>= 1) a2 += __shfl_xor_sync(kFull, a2, o);
       const double2 x0 = j < m ? SX[p] : make_double2(0.0, 0.0);
       // lane 0: alpha = sqrt(sum), lane 1: |x_0| (one sqrt for both)
@@ -325,18 +337,22 @@ __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int
           s_phase[j] = make_double2(1.0, 0.0);
         }
       } else {
-        // lane 0: 1/|x_0|, lane 1: beta (one division for both)
-        const double rc = 1.0 / (lane == 1 ? alpha * (alpha + ax0) : ax0);
+        // even lanes: 1/|x_0|, odd lanes: beta (one division for both)
+        const double rc = 1.0 / ((lane & 1) ? alpha * (alpha + ax0) : ax0);
         const double inv = __shfl_sync(kFull, rc, 0);
-        const double beta = __shfl_sync(kFull, rc, 1);
-        const double2 phi = ax0 > 0.0 ? make_double2(x0.x * inv, x0.y * inv) : make_double2(1.0, 0.0);
-        if (lane == 0) {
-          s_skip[j] = 0;
-          s_beta[j] = beta;
-          s_alpha[j] = alpha;
-          s_phase[j] = make_double2(-phi.x, -phi.y);
-          s_gam = make_double2(alpha * phi.x, -alpha * phi.y);
-          if (own) x[lrow] = make_double2(fma(phi.x, alpha, x0.x), fma(phi.y, alpha, x0.y));
+        // lane 0 the real, lane 1 the imaginary part of phi, alpha conj(phi) and v_0
+        const double xc = (lane & 1) ? x0.y : x0.x;
+        const double phi = ax0 > 0.0 ? xc * inv : ((lane & 1) ? 0.0 : 1.0);
+        const double ap = alpha * phi;
+        if (lane < 2) {
+          if (lane == 1) s_beta[j] = rc;
+          if (lane == 0) {
+            s_skip[j] = 0;
+            s_alpha[j] = alpha;
+          }
+          reinterpret_cast<double*>(&s_phase[j])[lane] = -phi;
+          reinterpret_cast<double*>(&s_gam)[lane] = lane == 0 ? ap : -ap;
+          if (own) reinterpret_cast<double*>(&x[lrow])[lane] = fma(phi, alpha, xc);
         }
       }
     } else if (cw >= 0) {
@@ -352,7 +368,7 @@ __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int
             w.x += t.x;
             w.y += t.y;
           }
-        W[ps] = gsum2<GL>(w);
+        W[ps] = gsum_split<GL>(w);
       }
     }
     __syncthreads();
@@ -364,12 +380,12 @@ __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int
       for (int ps = 0; ps < kMaxPass; ++ps) {
         const int k = j + 1 + ps * slots + q;
         if (j + 1 + ps * slots >= n) break;
+        const double2 rj = RJ[(size_t)p * n + min(k, n - 1)];
+        // w += gam rj, one component a lane: (gam.x rj.x - gam.y rj.y, gam.x rj.y + gam.y rj.x)
+        const bool up = (lane & (GL / 2)) != 0;
+        const double w = fma(gam.x, up ? rj.y : rj.x, fma(up ? gam.y : -gam.y, up ? rj.x : rj.y, W[ps]));
+        const double2 bw = join_split<GL>(beta * w);
         if (k < n) {
-          const double2 rj = RJ[(size_t)p * n + k];
-          double2 w = W[ps];
-          w.x = fma(gam.x, rj.x, fma(-gam.y, rj.y, w.x));
-          w.y = fma(gam.x, rj.y, fma(gam.y, rj.x, w.y));
-          const double2 bw = make_double2(beta * w.x, beta * w.y);
           double2* a = A + (size_t)k * rp;
           for (int i = i0 + sl; i < nr; i += GL) a[i] = cfms(x[i], bw, a[i]);
         }
@@ -479,21 +495,33 @@ __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int
   // whatever the lanes). put(a, v) stores component lane >> 4 of entry a.
   auto solve = [&](int c, double (&acc)[kQrClusterMaxN / 16], auto&& put) {
     const int comp = lane >> 4, e = lane & 15;
+    double beta = s_beta[c];
 #pragma unroll
     for (int qa = kQrClusterMaxN / 16 - 1; qa >= 0; --qa) {
-      for (int a = min(c, 16 * qa + 15); a >= 16 * qa; --a) {
-        const double t = s_beta[a] * acc[qa];
+      if (c < 16 * qa) continue;
+      double2 g[kQrClusterMaxN / 16];  // row a of the transposed Gram, read a step ahead
+      const int a0 = min(c, 16 * qa + 15);
+#pragma unroll
+      for (int q = 0; q <= qa; ++q) g[q] = 16 * q + e < a0 ? GF[a0 * n + 16 * q + e] : make_double2(0.0, 0.0);
+      for (int a = a0; a >= 16 * qa; --a) {
+        const double t = beta * acc[qa];
+        double2 gn[kQrClusterMaxN / 16];
+        if (a > 0) {
+          beta = s_beta[a - 1];
+#pragma unroll
+          for (int q = 0; q <= qa; ++q)
+            gn[q] = 16 * q + e < a - 1 ? GF[(a - 1) * n + 16 * q + e] : make_double2(0.0, 0.0);
+        }
         const double tx = __shfl_sync(kFull, t, a & 15), ty = __shfl_sync(kFull, t, 16 + (a & 15));
         if (e == (a & 15)) put(a, t);
         const double t1 = comp == 0 ? tx : ty, t2 = comp == 0 ? ty : tx;
 #pragma unroll
         for (int q = 0; q <= qa; ++q) {
-          const int i = 16 * q + e;
-          if (16 * q < a && i < a) {
-            const double2 g = GF[a * n + i];
-            acc[q] = fma(-g.x, t1, acc[q]);
-            acc[q] = fma(comp == 0 ? g.y : -g.y, t2, acc[q]);
+          if (16 * q < a && 16 * q + e < a) {
+            acc[q] = fma(-g[q].x, t1, acc[q]);
+            acc[q] = fma(comp == 0 ? g[q].y : -g[q].y, t2, acc[q]);
           }
+          if (a > 0) g[q] = gn[q];
         }
       }
     }
