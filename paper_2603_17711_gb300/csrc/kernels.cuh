@@ -194,7 +194,8 @@ bool launch_qr_cluster(double2* U, int d0, int d1, int d2, int leg, double tol, 
 // back in place, beta/alpha/phase/skip of those columns at index c0.., and the
 // panel's WY factor T (nb x nb, row-major) with H_c0..H_{c0+nb-1} = I - V T V^H.
 struct QrPanel {
-  double2* gtail;  // full mode: global scratch (3*C*n*n) for the Gram / M buffers, or null
+  double2* gtail;  // full mode: global scratch ((C + 2)*n*n) for the Gram / M buffers, or null
+  bool m_apart;    // full mode: M has shared memory of its own beside the Gram
   double2* A;
   int m, n, c0, nb;
   const double* thr;

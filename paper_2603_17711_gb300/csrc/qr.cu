@@ -160,9 +160,10 @@ __device__ __forceinline__ void push_c64(uint32_t raddr, double2 v, uint32_t rmb
 //   A   [n][rp]     my row block, column-major (v_j overwrites rows >= j of column j)
 //   SU  [2][16][n]  per-parity dot partials u_k pushed by each CTA
 //   RJ  [2][n]      per-parity row j of the trailing columns (from the owner of row j)
-//   G   [n][n]      partial strictly-upper Gram of my rows, later the gathered M
-//   GF  [n][n]      full strictly-upper Gram
-//   MM  [n][n]      the columns of M solved by this CTA
+//   GF  [n][n]      strictly-upper Gram of V, transposed
+//   M   [n][n]      M; its own region where that fits, else GF's (one more
+//                   cluster barrier). When not even GF fits, both are single
+//                   copies in global memory behind the CTAs' partial Grams.
 template <int GL>
 __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int d1, int d2, int leg,
                                                          double tol, double2* R, int* flag, float2* U_lo,
@@ -197,17 +198,10 @@ __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int
   double2* A = smem;
   double2* SU = A + (size_t)n * rp;
   double2* RJ = SU + 32 * (size_t)n;
-  // Gram / M buffers: shared memory, or (large n) per-CTA regions of pn.gtail
   const bool gt = !panel && pn.gtail != nullptr;
   const size_t n2 = (size_t)n * n;
-  double2* G = gt ? pn.gtail + (size_t)me * n2 : RJ + 2 * (size_t)n;
-  double2* GF = gt ? pn.gtail + (size_t)(C + me) * n2 : G + n2;
-  double2* MM = gt ? pn.gtail + (size_t)(2 * C + me) * n2 : GF + n2;
-  // the partial Gram / M of CTA c, as seen from this CTA
-  auto G_of = [&](int c) -> const double2* { return gt ? pn.gtail + (size_t)c * n2 : cluster.map_shared_rank(G, c); };
-  auto MM_of = [&](int c) -> const double2* {
-    return gt ? pn.gtail + (size_t)(2 * C + c) * n2 : cluster.map_shared_rank(MM, c);
-  };
+  double2* GF = gt ? pn.gtail : RJ + 2 * (size_t)n;
+  double2* M = gt ? pn.gtail + n2 : pn.m_apart ? GF + n2 : GF;
   __shared__ __align__(8) uint64_t mb[2], mbg[2];
   __shared__ double SN[2][16];
   __shared__ double2 SX[2];
@@ -454,23 +448,24 @@ __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int
     const double2* vb = A + (size_t)b * rp;
     for (int i = max(b - r0, 0); i < nr; ++i) g = cfmaj(va[i], vb[i], g);
     if (gt)
-      G[a * n + b] = g;
+      pn.gtail[(size_t)(2 + me) * n2 + a * n + b] = g;
     else if (alive)  // SU is free after the column loop
       push_c64(mapa(smem_u32(&SU[(size_t)me * nslot + t / C]), t % C), g, mapa(smem_u32(&mbg[0]), t % C));
   }
   if (gt) {
     cluster.sync();
-    for (int t = tid; t < npair; t += nt) {
+    for (int e = tid; e < nown; e += nt) {
       int a, b;
-      pair_of(t, a, b);
+      pair_of(me + C * e, a, b);
       double2 g = make_double2(0.0, 0.0);
       for (int c = 0; c < C; ++c) {
-        const double2 v = G_of(c)[a * n + b];
+        const double2 v = pn.gtail[(size_t)(2 + c) * n2 + a * n + b];
         g.x += v.x;
         g.y += v.y;
       }
       GF[b * n + a] = g;
     }
+    cluster.sync();
   } else {
     if (alive) alive = mbar_wait(&mbg[0], 0u, deadline, flag);
     // one lane per component
@@ -557,61 +552,61 @@ __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int
         }
       }
     }
-    double* Md = reinterpret_cast<double*>(MM);
-    solve(c, acc, [&](int a, double v) { Md[2 * (a * n + c) + (lane >> 4)] = v; });
-    for (int a = c + 1 + lane; a < n; a += 32) MM[a * n + c] = make_double2(0.0, 0.0);
+    // the column waits in SU (free since the Gram sums) until every CTA may receive it
+    double2* buf = SU + ((size_t)(c / (C * kNW)) * kNW + wid) * n;
+    solve(c, acc, [&](int a, double v) { reinterpret_cast<double*>(buf)[2 * a + (lane >> 4)] = v; });
   }
-  cluster.sync();  // every column of M solved; partial Grams no longer read
-  // gather M into G (column c from CTA c mod C)
-  for (int t = tid; t < n * n; t += nt) G[t] = MM_of((t % n) % C)[t];
-  __syncthreads();
+  if (!gt && !pn.m_apart) cluster.sync();  // M takes GF's place: every solve is done
+  for (int c = me + C * wid; c < n; c += C * kNW) {
+    __syncwarp();
+    const double2* buf = SU + ((size_t)(c / (C * kNW)) * kNW + wid) * n;
+    const int copies = gt ? 1 : C;
+    for (int k = lane; k < (c + 1) * copies; k += 32) {
+      const int a = k % (c + 1), to = k / (c + 1);
+      double2* dst = gt ? M : cluster.map_shared_rank(M, to);
+      dst[a * n + c] = buf[a];
+    }
+  }
+  cluster.sync();  // M complete in every CTA; nobody reads another's rows any more
   // Q rows: Q[r][c] = delta_rc - sum_{a <= min(r,c)} v_a[r] M[a][c], column c scaled by phase_c
-  // (a column's cost grows with c: tasks dealt to the warps forth and back)
-  const int nch = (nr + 31) / 32;
-  for (int rnd = 0; rnd * kNW < n * nch; ++rnd) {
-    const int task = rnd * kNW + ((rnd & 1) ? kNW - 1 - wid : wid);
-    if (task >= n * nch) continue;
-    const int c = task / nch, i = (task % nch) * 32 + lane;
-    if (i >= nr) continue;
+  // Entries (c, row) are laid along the lanes column after column, so that few
+  // rows per CTA still fill the warps; a task is 32 entries and costs as many
+  // steps as its last column needs, so tasks go to the warps forth and back.
+  const int ntask = (n * nr + 31) / 32;
+  for (int rnd = 0; rnd * kNW < ntask; ++rnd) {
+    const int task = rnd * kNW + ((rnd & 1) ? kNW - 1 - wid : wid), e = task * 32 + lane;
+    if (task >= ntask || e >= n * nr) continue;
+    const int c = e / nr, i = e % nr;
     const int r = r0 + i;
     double2 q = make_double2(r == c ? 1.0 : 0.0, 0.0);
     const int amax = min(c, r);
-    for (int a = 0; a <= amax; ++a) q = cfms(A[(size_t)a * rp + i], G[a * n + c], q);
+    for (int a = 0; a <= amax; ++a) q = cfms(A[(size_t)a * rp + i], M[a * n + c], q);
     const double2 p = s_phase[c];
     const double2 qp = make_double2(q.x * p.x - q.y * p.y, q.x * p.y + q.y * p.x);
     const int64_t at = c * st[leg] + (int64_t)(r / dd[lb]) * st[la] + (int64_t)(r % dd[lb]) * st[lb];
     U[at] = qp;
     if (U_lo) U_lo[at] = make_float2((float)qp.x, (float)qp.y);
   }
-  cluster.sync();  // keep shared memory alive until every remote read has finished
 }
 
 constexpr size_t kQrSmemCap = 200 * 1024;
 
-size_t qr_cluster_smem(int m, int n, int C, bool gtail) {
+// nn: n x n buffers in shared memory (2: GF and M, 1: shared, 0: global memory)
+size_t qr_cluster_smem(int m, int n, int C, int nn) {
   const int rp = (m + C - 1) / C;
-  return sizeof(double2) * ((size_t)n * rp + 34 * (size_t)n + (gtail ? 0 : 3 * (size_t)n * n));
+  return sizeof(double2) * ((size_t)n * rp + 34 * (size_t)n + (size_t)nn * n * n);
 }
-size_t qr_cluster_smem(int m, int n, int C) { return qr_cluster_smem(m, n, C, false); }
 
-// Cluster size for an m x n QR (0: does not fit); *gtail set when the Gram / M
-// buffers have to live in global memory.
-int qr_cluster_size(int m, int n, bool* gtail) {
-  *gtail = false;
+// Cluster size for an m x n QR (0: does not fit); *nn as above.
+int qr_cluster_size(int m, int n, int* nn) {
+  *nn = 0;
   if (n > kQrClusterMaxN) return 0;
   int C = (m + 7) / 8;  // about 8 rows per CTA: the factorisation is FP64-issue bound
   C = C < 1 ? 1 : (C > 16 ? 16 : C);
-  if (qr_cluster_smem(m, n, C, false) <= kQrSmemCap) return C;
-  if (qr_cluster_smem(m, n, C, true) <= kQrSmemCap) {
-    *gtail = true;
-    return C;
-  }
+  if (n > 4 * kNW * C) return 0;  // solved columns wait in four rounds of warps
+  for (*nn = 2; *nn >= 0; --*nn)
+    if (qr_cluster_smem(m, n, C, *nn) <= kQrSmemCap) return C;
   return 0;
-}
-int qr_cluster_size(int m, int n) {
-  bool gt;
-  const int C = qr_cluster_size(m, n, &gt);
-  return gt ? 0 : C;
 }
 
 template <int G>
@@ -626,7 +621,7 @@ static bool launch_cluster(double2* U, int d0, int d1, int d2, int leg, double t
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(C, 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = qr_cluster_smem(m, n, C, !pn.A && pn.gtail);
+  cfg.dynamicSmemBytes = qr_cluster_smem(m, n, C, pn.A ? 1 : pn.gtail ? 0 : pn.m_apart ? 2 : 1);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -643,12 +638,13 @@ bool launch_qr_cluster(double2* U, int d0, int d1, int d2, int leg, double tol, 
   const int dd[3] = {d0, d1, d2};
   const int n = dd[leg];
   const int m = (int)((int64_t)d0 * d1 * d2 / n);
-  bool gt = false;
-  const int C = qr_cluster_size(m, n, &gt);
+  int nn = 0;
+  const int C = qr_cluster_size(m, n, &nn);
   if (C == 0) return false;
   QrPanel pn = {};
-  if (gt) {
-    if (!scratch || scratch_elems < 3 * (int64_t)C * n * n) return false;
+  pn.m_apart = nn == 2;
+  if (nn == 0) {
+    if (!scratch || scratch_elems < (C + 2) * (int64_t)n * n) return false;
     pn.gtail = scratch;
   }
   return launch_cluster<8>(U, d0, d1, d2, leg, tol, R, flag, U_lo, R_lo, pn, m, n, C, s);
@@ -657,7 +653,7 @@ bool launch_qr_cluster(double2* U, int d0, int d1, int d2, int leg, double tol, 
 int qr_panel_cluster(int m_act, int nb) {
   int C = (m_act + 7) / 8;
   C = C < 1 ? 1 : (C > 16 ? 16 : C);
-  return qr_cluster_smem(m_act, nb, C) > kQrSmemCap ? 0 : C;
+  return qr_cluster_smem(m_act, nb, C, 1) > kQrSmemCap ? 0 : C;
 }
 
 bool launch_qr_panel(const QrPanel& pn, cudaStream_t s) {
