@@ -454,6 +454,9 @@ struct Exec {
       const int dq = q.leg == 0 ? q.d0 : q.leg == 1 ? q.d1 : q.d2;
       const int64_t nrest = (int64_t)q.d0 * q.d1 * q.d2 / dq;
       run(1, L.flops, [&] {
+        if (h->prec == PREC_F64 && launch_project_xs(h->h_bufs.data(), h->h_mats.data(), L, p.pj_outs.data(),
+                                                     h->params.max_split, s))
+          return;
         if (!launch_project_tiled(h->prec, h->Tlo, L, dq, nrest, p.sm_count, s)) launch_project(h->prec, h->Tlo, ht_lo(), L, s);
       });
       if (h->tc_pool_on) {

@@ -158,6 +158,14 @@ bool xs_applicable(const ApList& L, const ApOut* outs_host, const ApTerm* terms_
 bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L, const Epi& e,
                      const ApOut* outs_host, const ApTerm* terms_host, double2* planes, int64_t plane_elems,
                      int max_split, cudaStream_t s);
+// FP64 projections on the same path; false (nothing launched) below
+// kXsMinPjFlops or when the list does not qualify (all outputs alike, 8 <= bond
+// <= 64, at most 96 outputs).
+// Measured: 64-wide bond, 4096 positions, 5 classes 447 us (FP64 pipe) -> 172;
+// 56 classes' worth of the rank-64 chain's step 30.2 -> 9.9 ms.
+constexpr double kXsMinPjFlops = 8.0e6;
+bool launch_project_xs(double2* const* bufs, double2* const* mats, const PjList& L, const PjOut* pjs_host,
+                       int max_split, cudaStream_t s);
 void launch_project(int prec, const DevTables& T, const HostTables& H, const PjList& L, cudaStream_t s);
 // The same projections for wide bonds in the FP32 form (every output d x d
 // with d >= 32 and a reduction range of >= 1024 positions, all outputs of the

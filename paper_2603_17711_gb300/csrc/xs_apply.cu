@@ -36,9 +36,12 @@
 #include <algorithm>
 #include <cstdint>
 
+#include <cooperative_groups.h>
 #include <cuda_fp16.h>
 
 #include "kernels.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace ttn {
 
@@ -499,6 +502,98 @@ __global__ void __launch_bounds__(128) k_xs_epilogue(const double2* planes, int 
   rk_update(ep, e, k);
 }
 
+// ---------------------------------------------------------------------------
+// Environment projections E[x', x] = sum_r conj(U[x', r]) W[x, r] of wide bonds
+// by the same split: output rows x' in blocks of 8 (one per warp of a group),
+// columns x in tiles of 16, the reduction range in chunks of 8 MT positions, one
+// exact block product per chunk with its own scales, added in FP64. The chunks of
+// a tile are dealt to the groups of KS CTAs (one cluster), whose sums CTA 0 adds
+// in order through distributed shared memory.
+// ---------------------------------------------------------------------------
+constexpr int kXsMaxPj = 96;
+struct XsPj {
+  int dims[3], leg, KS;
+  const double2* u;
+  const double2* w[kXsMaxPj];
+  double2* dst[kXsMaxPj];
+};
+__global__ void __launch_bounds__(kXsThreads, 2) k_xs_project(const __grid_constant__ XsPj w) {
+  __shared__ __align__(16) uint4 sm_bd[kXsWarps * 8 * 32];
+  __shared__ int sm_sc[kXsWarps][96];
+  __shared__ double2 tot[kXsWarps * kXsCols * 8];  // this CTA's 8 MT x 16 tile
+  double2(*red)[kXsCols * 8] = reinterpret_cast<double2(*)[kXsCols * 8]>(sm_bd);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int dd[4] = {w.dims[0], w.dims[1], w.dims[2], 1};
+  const XsLeg g = leg_of(dd, w.leg);
+  const int MT = (g.d + 7) >> 3, G = kXsWarps / MT;
+  const int mt = wid % MT, grp = wid / MT;
+  const int rank = blockIdx.x % w.KS, tile = blockIdx.x / w.KS, o = blockIdx.y;
+  const XsGroup gp{mt, MT, 1 + grp, sm_sc[grp], sm_sc[grp] + 64, sm_sc[grp] + 80, sm_bd + (size_t)grp * MT * 8 * 32};
+  for (int e = threadIdx.x; e < kXsWarps * 96; e += kXsThreads) sm_sc[0][e] = 0;
+  __syncthreads();
+  double acc[kXsNT][4];
+#pragma unroll
+  for (int t = 0; t < kXsNT; ++t)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) acc[t][r] = 0.0;
+  const int chunk = 8 * MT, nch = (g.rest + chunk - 1) / chunk;
+  if (grp < G) {
+    const int i = mt * 8 + (lane >> 2), inner = g.inner, span = g.d * g.inner;
+    XsSrc S;
+    S.a = i < g.d ? w.u + (int64_t)i * inner : nullptr;
+#pragma unroll
+    for (int t = 0; t < kXsNT; ++t) {
+      const int x = tile * kXsCols + 8 * t + (lane >> 2);
+      S.b[t] = x < g.d ? w.w[o] + (int64_t)x * inner : nullptr;
+    }
+    for (int c = rank * G + grp; c < nch; c += w.KS * G) {
+      const int r0 = c * chunk, K = min(chunk, g.rest - r0);
+      auto at = [=](int k) { return (r0 + k) / inner * span + (r0 + k) % inner; };
+      xs_block<true>(gp, S, K, at, at, acc);
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < kXsNT; ++t)
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      red[wid][(8 * t + 2 * (lane & 3) + j) * 8 + (lane >> 2)] = make_double2(acc[t][2 * j], acc[t][2 * j + 1]);
+  __syncthreads();
+  const int ne = MT * kXsCols * 8;
+  for (int e = threadIdx.x; e < ne; e += kXsThreads) {
+    const int m = e / (kXsCols * 8), slot = e % (kXsCols * 8);
+    double2 v = red[m][slot];
+    for (int q = 1; q < G; ++q) {
+      const double2 x = red[q * MT + m][slot];
+      v.x += x.x;
+      v.y += x.y;
+    }
+    tot[e] = v;
+  }
+  if (w.KS > 1) {
+    cg::cluster_group cluster = cg::this_cluster();
+    cluster.sync();
+    // every CTA adds its share of the tile's entries over the CTAs, in order
+    for (int e = rank * kXsThreads + threadIdx.x; e < ne; e += w.KS * kXsThreads) {
+      double2 v = *cluster.map_shared_rank(&tot[e], 0);
+      for (int q = 1; q < w.KS; ++q) {
+        const double2 x = *cluster.map_shared_rank(&tot[e], q);
+        v.x += x.x;
+        v.y += x.y;
+      }
+      const int ii = (e / (kXsCols * 8)) * 8 + (e & 7), x = tile * kXsCols + (e % (kXsCols * 8)) / 8;
+      if (ii < g.d && x < g.d) w.dst[o][(int64_t)ii * g.d + x] = v;
+    }
+    cluster.sync();  // shared memory stays until every CTA has read it
+    return;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < ne; e += kXsThreads) {
+    const int ii = (e / (kXsCols * 8)) * 8 + (e & 7), x = tile * kXsCols + (e % (kXsCols * 8)) / 8;
+    if (ii < g.d && x < g.d) w.dst[o][(int64_t)ii * g.d + x] = tot[e];
+  }
+}
+
 namespace {
 
 int sm_count() {
@@ -643,6 +738,43 @@ bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L
       k_xs_apply<<<dim3(gx[l], n_outs), kXsThreads, 0, s>>>(gr);
     }
   return true;
+}
+
+bool launch_project_xs(double2* const* bufs, double2* const* mats, const PjList& L, const PjOut* pjs, int max_split,
+                       cudaStream_t s) {
+  const int n = L.out_end - L.out_begin;
+  if (n < 1 || n > kXsMaxPj || L.flops < kXsMinPjFlops) return false;
+  const PjOut& f = pjs[L.out_begin];
+  const int dd[3] = {f.d0, f.d1, f.d2}, d = dd[f.leg];
+  const int64_t P = (int64_t)f.d0 * f.d1 * f.d2;
+  if (d > kXsMaxD || d < 8 || P >= (int64_t)1 << 30) return false;
+  XsPj w{};
+  for (int i = 0; i < 3; ++i) w.dims[i] = dd[i];
+  w.leg = f.leg;
+  w.u = bufs[f.u_buf];
+  for (int o = 0; o < n; ++o) {
+    const PjOut& q = pjs[L.out_begin + o];
+    if (q.d0 != f.d0 || q.d1 != f.d1 || q.d2 != f.d2 || q.leg != f.leg || q.u_buf != f.u_buf) return false;
+    w.w[o] = bufs[q.w_buf];
+    w.dst[o] = mats[q.dst_mat];
+  }
+  // split the range while the launch is below two CTAs per SM and a group keeps a chunk
+  const int MT = (d + 7) / 8, G = kXsWarps / MT, tiles = (d + kXsCols - 1) / kXsCols;
+  const int nch = (int)((P / d + 8 * MT - 1) / (8 * MT));
+  w.KS = 1;
+  while (w.KS < std::min(8, max_split) && w.KS * G < nch && (int64_t)tiles * n * w.KS < 2 * sm_count()) ++w.KS;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(tiles * w.KS), (unsigned)n, 1);
+  cfg.blockDim = dim3(kXsThreads, 1, 1);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)w.KS;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_xs_project, w) == cudaSuccess;
 }
 
 }  // namespace ttn
