@@ -99,6 +99,18 @@ __device__ __forceinline__ double wsum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
+// Sum of complex values over aligned groups of G lanes: the group's lower half
+// gets the real part, the upper half the imaginary part. The first exchange
+// leaves each half one component, so a level costs one FP64 addition (64 cycles)
+// instead of two, with the sums of the plain butterfly.
+template <int G>
+__device__ __forceinline__ double gsum_split(double2 v) {
+  const bool up = (threadIdx.x & (G / 2)) != 0;
+  double k = up ? v.y : v.x;
+  k += __shfl_xor_sync(0xffffffffu, up ? v.x : v.y, G / 2);
+  for (int o = G / 4; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+  return k;
+}
 __device__ __forceinline__ bool aborted(const double* sc) { return !isfinite(sc[0]); }
 
 // Acm[c*m + r] = U[row r, column c of the matricisation toward `leg`];
@@ -274,10 +286,11 @@ __device__ bool grid_arrive_wait(unsigned* bar, unsigned target, bool wait, uint
     if (lane == 0) red_release_add(bar + blockIdx.x % kBarLanes, 1u);
     int ok = 1;
     if (wait) {
-      for (;;) {
+      for (unsigned it = 0;; ++it) {
         unsigned v = lane < kBarLanes ? ld_acquire(bar + lane) : 0u;
         for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (__shfl_sync(0xffffffffu, v, 0) >= target) break;
+        if ((it & 15u) != 0) continue;  // the clock is read every 16th poll
         if (__shfl_sync(0xffffffffu, (int)(gtimer() > deadline), 0)) {  // warp-uniform decision
           if (lane == 0) atomicOr(flag, 2);
           ok = 0;
@@ -294,8 +307,9 @@ __device__ bool grid_arrive_wait(unsigned* bar, unsigned target, bool wait, uint
 // Panel factorisation over the whole GPU (cooperative launch, G <= SMs CTAs):
 // the rows [c0, m) of the nb panel columns are split over the CTAs (rp <=
 // kPgRows each, kept in shared memory) and column j costs one grid barrier.
-// Before it every CTA writes its record rec[j][cta] = (|x_j|^2 over its rows,
-// u_k = x_j^H a_k for k > j) and the owner of row j writes own[j] = (x_0,
+// Before it every CTA writes its record rec[j][.][cta] = (|x_j|^2 over its rows,
+// u_k = x_j^H a_k for k > j; CTAs contiguous, so that the 16 threads adding an
+// entry read whole lines) and the owner of row j writes own[j] = (x_0,
 // a_k[j]); after it every CTA adds the G records in the same fixed order, so
 // all CTAs hold bitwise the same alpha, phi, beta and w_k = sum u_k + alpha
 // conj(phi) a_k[j], and updates its own rows. Convention, skipping rule and
@@ -315,8 +329,9 @@ __global__ void __launch_bounds__(256) k_qb_panel_grid(double2* A, int64_t m, in
   __shared__ double2 red[kNB];         // this column's summed record: [0].x = |x|^2, [t] = sum u_{j+t}
   __shared__ double2 s_own[kNB];       // [0] = x_0, [t] = a_{j+t}[j]
   __shared__ double s_beta[kNB], s_alpha[kNB];
-  __shared__ double2 s_phase[kNB], s_gam;
+  __shared__ double2 s_phase[kNB], s_bw[kNB];  // s_bw: beta w_{j+t} of this column
   __shared__ int s_skip[kNB];
+  static_assert(kNB <= 16, "two lanes of one warp per trailing column");
   __shared__ double2 s_gf[kNpair];
   if (aborted(sc)) return;  // uniform over the grid
   const double thr = sc[0];
@@ -345,9 +360,9 @@ __global__ void __launch_bounds__(256) k_qb_panel_grid(double2* A, int64_t m, in
         const int k = j + task;
         for (int i = i0 + lane; i < nr; i += 32) u = cfmaj(X[j][i], X[k][i], u);
       }
-      u.x = wsum(u.x);
-      u.y = wsum(u.y);
-      if (lane == 0) rec[((int64_t)j * kBlkCap + me) * kNB + task] = u;
+      const double t = gsum_split<32>(u);
+      if ((lane & 15) == 0)
+        reinterpret_cast<double*>(&rec[((int64_t)j * kNB + task) * kBlkCap + me])[lane >> 4] = t;
     }
     if (ownr)
       for (int k = j + tid; k < nb; k += blockDim.x) own[j * kNB + k] = X[k][lrow];
@@ -362,22 +377,20 @@ __global__ void __launch_bounds__(256) k_qb_panel_grid(double2* A, int64_t m, in
 #pragma unroll
         for (int q = 0; q < kBlkCap / 16; ++q) {
           const int c = sub + 16 * q;
-          a[q] = c < G ? __ldcg(&rec[((int64_t)j * kBlkCap + c) * kNB + task]) : make_double2(0.0, 0.0);
+          a[q] = c < G ? __ldcg(&rec[((int64_t)j * kNB + task) * kBlkCap + c]) : make_double2(0.0, 0.0);
         }
 #pragma unroll
         for (int h = kBlkCap / 32; h > 0; h >>= 1)  // pairwise, fixed order
 #pragma unroll
-          for (int q = 0; q < h; ++q) {
-            a[q].x += a[q + h].x;
-            a[q].y += a[q + h].y;
-          }
+          for (int q = 0; q < h; ++q)
+            if (16 * (q + h) < G) {  // beyond the grid there are only zeros
+              a[q].x += a[q + h].x;
+              a[q].y += a[q + h].y;
+            }
         v = a[0];
       }
-      for (int o = 8; o > 0; o >>= 1) {  // within each group of 16 lanes
-        v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
-        v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
-      }
-      if (sub == 0 && task < nb - j) red[task] = v;
+      const double t = gsum_split<16>(v);  // within each group of 16 lanes
+      if ((sub & 7) == 0 && task < nb - j) reinterpret_cast<double*>(&red[task])[sub >> 3] = t;
       if (tid < nb - j) s_own[tid] = ow;
     }
     __syncthreads();
@@ -395,17 +408,30 @@ __global__ void __launch_bounds__(256) k_qb_panel_grid(double2* A, int64_t m, in
           s_phase[j] = make_double2(1.0, 0.0);
         }
       } else {
-        const double rc = 1.0 / (lane == 1 ? al * (al + ax0) : ax0);
-        const double inv = __shfl_sync(0xffffffffu, rc, 0);
-        const double be = __shfl_sync(0xffffffffu, rc, 1);
-        const double2 phi = ax0 > 0.0 ? make_double2(x0.x * inv, x0.y * inv) : make_double2(1.0, 0.0);
-        if (lane == 0) {
-          s_skip[j] = 0;
-          s_beta[j] = be;
-          s_alpha[j] = al;
-          s_phase[j] = make_double2(-phi.x, -phi.y);
-          s_gam = make_double2(al * phi.x, -al * phi.y);
-          if (ownr) X[j][lrow] = make_double2(fma(phi.x, al, x0.x), fma(phi.y, al, x0.y));
+        const double rc = 1.0 / ((lane & 1) ? al * (al + ax0) : ax0);
+        const double inv = __shfl_sync(0xffffffffu, rc, 0), be = __shfl_sync(0xffffffffu, rc, 1);
+        // even lanes the real, odd lanes the imaginary part of phi and alpha conj(phi)
+        const int comp = lane & 1;
+        const double xc = comp ? x0.y : x0.x;
+        const double phi = ax0 > 0.0 ? xc * inv : (comp ? 0.0 : 1.0);
+        const double ap = comp ? -(al * phi) : al * phi;
+        const double gx = __shfl_sync(0xffffffffu, ap, 0), gy = __shfl_sync(0xffffffffu, ap, 1);
+        if (lane < 2) {
+          if (lane == 0) {
+            s_skip[j] = 0;
+            s_beta[j] = be;
+            s_alpha[j] = al;
+          }
+          reinterpret_cast<double*>(&s_phase[j])[lane] = -phi;
+          if (ownr) reinterpret_cast<double*>(&X[j][lrow])[lane] = fma(phi, al, xc);
+        }
+        // beta w_k of the trailing columns once, a component a lane (it was
+        // computed again for every updated entry)
+        const int k = lane >> 1;
+        if (k >= 1 && k < nb - j) {
+          const double2 rj = s_own[k], w = red[k];
+          const double wc = fma(gx, comp ? rj.y : rj.x, fma(comp ? gy : -gy, comp ? rj.x : rj.y, comp ? w.y : w.x));
+          reinterpret_cast<double*>(&s_bw[k])[comp] = be * wc;
         }
       }
     }
@@ -413,17 +439,10 @@ __global__ void __launch_bounds__(256) k_qb_panel_grid(double2* A, int64_t m, in
     if (s_skip[j]) {
       for (int i = i0 + tid; i < nr; i += blockDim.x) X[j][i] = make_double2(0.0, 0.0);
     } else {
-      const double be = s_beta[j];
-      const double2 gam = s_gam;
       const int nk = nb - j - 1, len = nr - i0;
       for (int t = tid; len > 0 && t < nk * len; t += blockDim.x) {
         const int k = j + 1 + t / len, i = i0 + t % len;
-        const double2 rj = s_own[k - j];
-        double2 w = red[k - j];
-        w.x = fma(gam.x, rj.x, fma(-gam.y, rj.y, w.x));
-        w.y = fma(gam.x, rj.y, fma(gam.y, rj.x, w.y));
-        const double2 bw = make_double2(be * w.x, be * w.y);
-        X[k][i] = cfms(X[j][i], bw, X[k][i]);
+        X[k][i] = cfms(X[j][i], s_bw[k - j], X[k][i]);
       }
     }
     __syncthreads();
