@@ -154,16 +154,21 @@ void launch_tc_embed(void* const* mats32, const TcEmbedJob* jobs, int n, float* 
 // MFLOP) 16.6 us on the CUDA cores, 15.6 here; 19x11x11, 8 terms (2.1 MFLOP)
 // 8.7 / 13.3; 20^3, 12 terms (15 MFLOP) 26.7 / 13.5.
 constexpr double kXsMinFlops = 8.0e6;
-bool xs_applicable(const ApList& L, const ApOut* outs_host, const ApTerm* terms_host);
+// Instances advanced together (max_split 1) share the FP64 pipes, so the work a
+// list takes off them counts beside its own latency. Batched step of 8 / 16 / 64
+// spin-boson instances: 6.4 / 16.1 / 41.8 ms at 8 MFLOP, 6.5 / 15.9 / 40.9 at 5,
+// 6.9 / 16.6 / 39.5 at 2, 7.4 / 16.9 / 39.4 at 1.
+constexpr double kXsMinFlopsShared = 5.0e6;
+inline double xs_min_flops(int max_split) { return max_split == 1 ? kXsMinFlopsShared : kXsMinFlops; }
+bool xs_applicable(const ApList& L, const ApOut* outs_host, const ApTerm* terms_host, int max_split);
 bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L, const Epi& e,
                      const ApOut* outs_host, const ApTerm* terms_host, double2* planes, int64_t plane_elems,
                      int max_split, cudaStream_t s);
 // FP64 projections on the same path; false (nothing launched) below
-// kXsMinPjFlops or when the list does not qualify (all outputs alike, 8 <= bond
+// xs_min_flops or when the list does not qualify (all outputs alike, 8 <= bond
 // <= 64, at most 96 outputs).
 // Measured: 64-wide bond, 4096 positions, 5 classes 447 us (FP64 pipe) -> 172;
 // 56 classes' worth of the rank-64 chain's step 30.2 -> 9.9 ms.
-constexpr double kXsMinPjFlops = 8.0e6;
 bool launch_project_xs(double2* const* bufs, double2* const* mats, const PjList& L, const PjOut* pjs_host,
                        int max_split, cudaStream_t s);
 void launch_project(int prec, const DevTables& T, const HostTables& H, const PjList& L, cudaStream_t s);

@@ -28,9 +28,11 @@
 // A non-finite operand makes its whole row or column of outputs NaN.
 //
 // Measured (graph replay, CUDA-core kernel / this one): 64^3 node, 14 terms
-// 1785 / 273 us (6.9 TFLOP/s of FP64 results against the 1.1 of the FP64 pipe;
-// the tensor pipe is a third busy, the rest is operand latency and digit
-// arithmetic); 20^3, 12 terms 26.7 / 13.5 us; 20x25x25, 12 terms 40.6 / 21.4 us.
+// 1797 / 249 us (7.6 TFLOP/s of FP64 results against the 1.1 of the FP64 pipe;
+// the tensor pipe is half busy, the rest is operand latency and digit
+// arithmetic); 20^3, 12 terms 26.7 / 13.8 us; 20x25x25, 12 terms 40.6 / 20.8 us.
+// Two scale sets in turn leave three group barriers a product instead of four,
+// and one conversion and one FMA join a digit sum (273 us without both).
 // Relative 2-norm error against 128-bit sums: 1.15e-16 / 2.35e-16 (64^3),
 // 1.14e-16 / 1.70e-16 (20^3), 4.7e-17 / 1.4e-16 for a single product.
 #include <algorithm>
@@ -66,15 +68,23 @@ __device__ __forceinline__ int exp_field(double v) { return (__double2hiint(v) >
 __device__ __forceinline__ int exp_c(double2 v) { return max(exp_field(v.x), exp_field(v.y)); }
 
 // v as a fixed-point integer with 62 bits below 2^(top + 1 - 1023), plus the
-// bias that turns its bytes into digits - 128 .. 127 offset by 128. Subnormal v is zero.
+// bias that turns its bytes into digits - 128 .. 127 offset by 128. Subnormal v
+// is zero; so is everything where top is out of range (kXsNoScale): a shift by
+// 64 or more (or a negative count, taken as unsigned) gives zero.
+constexpr int kXsNoScale = 8192;
 __device__ __forceinline__ uint64_t fixed_biased(double v, int top) {
-  const uint64_t u = (uint64_t)__double_as_longlong(v);
-  const int e = (int)(u >> 52) & 0x7ff;
-  const uint64_t m = e == 0 ? 0ull : ((u & 0xfffffffffffffull) | 0x10000000000000ull) << 9;
-  const int s = min(max(top - e, 0), 63);
-  const uint64_t f = m >> s;
-  const uint64_t sg = (uint64_t)((int64_t)u >> 63);
-  return (f ^ sg) - sg + 0x8080808080808080ull;
+  const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+  const uint32_t e = (hi >> 20) & 0x7ffu, mh = (hi & 0xfffffu) | 0x100000u;
+  const uint32_t s = e == 0 ? 64u : (uint32_t)(top - (int)e);
+  uint64_t f;
+  asm("{\n .reg .b64 m;\n mov.b64 m, {%2, %1};\n shl.b64 m, m, 9;\n shr.u64 %0, m, %3;\n}" : "=l"(f) : "r"(mh), "r"(lo), "r"(s));
+  const uint32_t sg = (uint32_t)((int)hi >> 31);
+  uint32_t tl, th;
+  asm("{\n .reg .b32 a, b, n;\n mov.b64 {a, b}, %2;\n xor.b32 a, a, %3;\n xor.b32 b, b, %3;\n and.b32 n, %3, 1;\n"
+      " add.u32 n, n, 0x80808080;\n add.cc.u32 %0, a, n;\n addc.u32 %1, b, 0x80808080;\n}"
+      : "=r"(tl), "=r"(th)
+      : "l"(f), "r"(sg));
+  return ((uint64_t)th << 32) | tl;
 }
 // Digit i (0 = most significant) of the pair (re, im) as f16x2.
 template <int I>
@@ -99,34 +109,25 @@ __device__ __forceinline__ void digits8(double2 v, int top, uint32_t (&d)[8]) {
   d[7] = digit_pair<7>(re, im);
 }
 
-// sum_g C_g 2^(8 (7 - g)) times 2^ex, rounded to nearest, built from integers
-// (a conversion instruction would occupy the FP64 pipe as long as an FMA).
-__device__ __forceinline__ double join(const float (&c)[8], int ex) {
+// acc += sum_g C_g 2^(8 (7 - g)) 2^ex. The sum is a 76-bit integer H 2^32 + l;
+// its top 63 bits (all of it unless |H| is near its bound) go through one
+// conversion and one FMA on the FP64 pipe, which the digit arithmetic leaves idle:
+// building the double from integers took 60 instructions instead of 30.
+__device__ __forceinline__ double join(const float (&c)[8], int ex, double acc) {
   int C[8];
 #pragma unroll
   for (int g = 0; g < 8; ++g) C[g] = __float2int_rn(c[g]);
-  // value = H 2^32 + l, |H| < 2^45: 96 bits, so no digit product is rounded before the end
   const int64_t lo = (int64_t)C[4] * (1 << 24) + (int64_t)C[5] * (1 << 16) + (int64_t)C[6] * 256 + C[7];
-  int64_t H = (int64_t)C[0] * (1 << 24) + (int64_t)C[1] * (1 << 16) + (int64_t)C[2] * 256 + C[3] + (lo >> 32);
-  uint32_t l = (uint32_t)lo;
-  const uint64_t sg = (uint64_t)H & 0x8000000000000000ull;
-  if (H < 0) {
-    H = ~H + (l == 0 ? 1 : 0);
-    l = 0u - l;
-  }
-  if (H == 0) {  // leading digits cancelled: take the low word up
-    if (l == 0) return 0.0;
-    H = l;
-    l = 0;
-    ex -= 32;
-  }
-  const int lz = __clzll(H);  // >= 19
-  const uint64_t n = ((uint64_t)H << lz) | (lz >= 32 ? (uint64_t)l << (lz - 32) : (uint64_t)(l >> (32 - lz)));
-  const uint64_t m = (n >> 11) + ((n >> 10) & 1ull);
-  const int E = 1023 + 63 - lz + 32 + ex;
-  if (E <= 0) return 0.0;
-  if (E >= 0x7ff) return __longlong_as_double((long long)(sg | 0x7ff0000000000000ull));
-  return __longlong_as_double((long long)(sg | (((uint64_t)E << 52) + (m - 0x10000000000000ull))));
+  const int64_t H = (int64_t)C[0] * (1 << 24) + (int64_t)C[1] * (1 << 16) + (int64_t)C[2] * 256 + C[3] + (lo >> 32);
+  const uint32_t l = (uint32_t)lo, hh = (uint32_t)(H >> 32), hl = (uint32_t)H;
+  // shift the 96-bit value right by sh (0 .. 14) until 64 bits hold it with its sign
+  const int top = 32 - __clz((int)hh ^ ((int)hh >> 31));
+  const int sh = top > 0 ? top + 1 : (int)((hl ^ hh) >> 31);
+  const uint32_t vl = __funnelshift_r(l, hl, sh), vh = __funnelshift_r(hl, hh, sh);
+  const double d = (double)(int64_t)(((uint64_t)vh << 32) | vl);
+  const int E = 1023 + ex + sh;
+  if (E > 0 && E < 0x7ff) return fma(d, __hiloint2double(E << 20, 0), acc);
+  return acc + scalbn(d, ex + sh);  // the scale itself is out of range
 }
 
 // One block product: 8 MT output indices (8 per warp of a group of MT warps) x 16
@@ -136,9 +137,10 @@ __device__ __forceinline__ double join(const float (&c)[8], int ex) {
 // them.
 struct XsGroup {
   int m, MT, bar;   // warp of the group, warps, named barrier
-  int* cx;          // [64] largest exponent of every operator column (group maximum)
-  int* col;         // [16] largest tensor exponent + cx of every position
-  int* craw;        // [16] largest raw tensor exponent (0x7ff: not finite)
+  int* sc;          // [2][96] scales, two sets used in turn (one is cleared while the other is in use):
+                    //   [64] largest exponent of every operator column (group maximum)
+                    //   [16] largest tensor exponent + that of every position
+                    //   [16] largest raw tensor exponent (0x7ff: not finite)
   uint4* bd;        // [MT][8][32] digits: x, y = K halves of positions 0..7, z, w = of positions 8..15
 };
 struct XsSrc {
@@ -154,8 +156,11 @@ __device__ __forceinline__ void gsync(const XsGroup& G) {
 
 // acc += block product. PROJ: conj(A) instead of A.
 template <bool PROJ, typename KA, typename KB>
-__device__ __forceinline__ void xs_block(const XsGroup& G, const XsSrc& S, int K, KA ka, KB kb,
+__device__ __forceinline__ void xs_block(const XsGroup& G, int turn, const XsSrc& S, int K, KA ka, KB kb,
                                          double (&acc)[kXsNT][4]) {
+  int* const scx = G.sc + 96 * (turn & 1);
+  int* const scol = scx + 64;
+  int* const scraw = scx + 80;
   const int lane = threadIdx.x & 31, kq = lane & 3;
   const double2 zero = make_double2(0.0, 0.0);
   const int KS = (K + 7) >> 3;
@@ -186,24 +191,25 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, const XsSrc& S, int K
       cx = __vmaxu2(cx, __shfl_xor_sync(kFull, cx, 4));
       cx = __vmaxu2(cx, __shfl_xor_sync(kFull, cx, 8));
       cx = __vmaxu2(cx, __shfl_xor_sync(kFull, cx, 16));
-      if (lane < 8) atomicMax(&G.cx[ks * 8 + lane], lane < 4 ? (int)(cx & 0xffff) : (int)(cx >> 16));
+      if (lane < 8) atomicMax(&scx[ks * 8 + lane], lane < 4 ? (int)(cx & 0xffff) : (int)(cx >> 16));
       rraw = max(rraw, max((int)(ep[ks] & 0xffff), (int)(ep[ks] >> 16)));
     }
-  gsync(G);
+  gsync(G);  // also: every warp is done with the previous product's scales and digits
+  for (int e = G.m * 32 + lane; e < 96; e += 32 * G.MT) G.sc[96 * ((turn & 1) ^ 1) + e] = 0;
   // 2: row scale of the scaled operator, position scales
   int row = -4096;
 #pragma unroll
   for (int ks = 0; ks < 8; ++ks)
     if (ks < KS) {
       const int e0 = ep[ks] & 0xffff, e1 = ep[ks] >> 16;
-      if (e0) row = max(row, e0 - G.cx[ks * 8 + kq]);
-      if (e1) row = max(row, e1 - G.cx[ks * 8 + 4 + kq]);
+      if (e0) row = max(row, e0 - scx[ks * 8 + kq]);
+      if (e1) row = max(row, e1 - scx[ks * 8 + 4 + kq]);
     }
   row = max(row, __shfl_xor_sync(kFull, row, 1));
   row = max(row, __shfl_xor_sync(kFull, row, 2));
   rraw = max(rraw, __shfl_xor_sync(kFull, rraw, 1));
   rraw = max(rraw, __shfl_xor_sync(kFull, rraw, 2));
-  const int cb[2] = {G.cx[G.m * 8 + kq], G.cx[G.m * 8 + 4 + kq]};
+  const int cb[2] = {scx[G.m * 8 + kq], scx[G.m * 8 + 4 + kq]};
 #pragma unroll
   for (int t = 0; t < kXsNT; ++t) {
     int c = 0, r = 0;
@@ -218,8 +224,8 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, const XsSrc& S, int K
     r = max(r, __shfl_xor_sync(kFull, r, 1));
     r = max(r, __shfl_xor_sync(kFull, r, 2));
     if (kq == 0) {
-      atomicMax(&G.col[8 * t + (lane >> 2)], c);
-      atomicMax(&G.craw[8 * t + (lane >> 2)], r);
+      atomicMax(&scol[8 * t + (lane >> 2)], c);
+      atomicMax(&scraw[8 * t + (lane >> 2)], r);
     }
   }
   gsync(G);
@@ -228,7 +234,7 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, const XsSrc& S, int K
     uint32_t d[kXsNT][2][8];
 #pragma unroll
     for (int t = 0; t < kXsNT; ++t) {
-      const int top = G.col[8 * t + (lane >> 2)];
+      const int cs = scol[8 * t + (lane >> 2)], top = cs ? cs : kXsNoScale;
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf)  // a zero operator column contributes nothing whatever the tensor holds
         digits8(cb[hf] ? braw[t][hf] : zero, top - cb[hf], d[t][hf]);
@@ -258,7 +264,7 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, const XsSrc& S, int K
 #pragma unroll
     for (int hf = 0; hf < 2; ++hf) {
       uint32_t ad[8];
-      digits8(v[hf], row + G.cx[ks * 8 + 4 * hf + kq], ad);
+      digits8(v[hf], row + scx[ks * 8 + 4 * hf + kq], ad);
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const uint32_t sw = __byte_perm(ad[i], ad[i], 0x1032);  // (im, re)
@@ -281,8 +287,8 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, const XsSrc& S, int K
   for (int t = 0; t < kXsNT; ++t)
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      const int n = 8 * t + 2 * kq + j, ec = G.col[n];
-      const bool bad = rraw == 0x7ff || G.craw[n] == 0x7ff;
+      const int n = 8 * t + 2 * kq + j, ec = scol[n];
+      const bool bad = rraw == 0x7ff || scraw[n] == 0x7ff;
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
         float cc[8];
@@ -290,12 +296,10 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, const XsSrc& S, int K
         for (int g = 0; g < 8; ++g) cc[g] = c[t][g][2 * p + j];
         // both fixed points: value = integer * 2^(scale - 1084); the digit pairs of
         // group g weigh 2^(8 (14 - g)), 2^56 of it outside join()
-        acc[t][2 * j + p] += bad ? __longlong_as_double(0x7ff8000000000000ll) : join(cc, row + ec - 2 * 1084 + 56);
+        acc[t][2 * j + p] = bad ? __longlong_as_double(0x7ff8000000000000ll)
+                                : join(cc, row + ec - 2 * 1084 + 56, acc[t][2 * j + p]);
       }
     }
-  gsync(G);  // scales and digits consumed
-  for (int e = G.m * 32 + lane; e < 96; e += 32 * G.MT) G.cx[e] = 0;  // cx, col, craw: contiguous
-  gsync(G);
 }
 
 // Leg geometry: element = outer * (d * inner) + x * inner + in, position n = outer * inner + in.
@@ -339,7 +343,7 @@ struct XsWork {
 // (one 16-position tile per group, no sum).
 __global__ void __launch_bounds__(kXsThreads, 2) k_xs_apply(const __grid_constant__ XsWork w) {
   __shared__ __align__(16) uint4 sm_bd[kXsWarps * 8 * 32];  // digits; the groups' sums at the end
-  __shared__ int sm_sc[kXsWarps][96];
+  __shared__ int sm_sc[kXsWarps][2 * 96];
   double2(*red)[kXsCols * 8] = reinterpret_cast<double2(*)[kXsCols * 8]>(sm_bd);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int o = blockIdx.y;
@@ -375,8 +379,8 @@ __global__ void __launch_bounds__(kXsThreads, 2) k_xs_apply(const __grid_constan
 #pragma unroll
     for (int r = 0; r < 4; ++r) acc[t][r] = 0.0;
   const int i = mt * 8 + (lane >> 2);
-  const XsGroup gp{mt, MT, 1 + grp, sm_sc[grp], sm_sc[grp] + 64, sm_sc[grp] + 80, sm_bd + (size_t)grp * MT * 8 * 32};
-  for (int e = threadIdx.x; e < kXsWarps * 96; e += kXsThreads) sm_sc[0][e] = 0;
+  const XsGroup gp{mt, MT, 1 + grp, sm_sc[grp], sm_bd + (size_t)grp * MT * 8 * 32};
+  for (int e = threadIdx.x; e < kXsWarps * 2 * 96; e += kXsThreads) sm_sc[0][e] = 0;
   __syncthreads();
   if (on) {
     const int n_split = split_terms ? nparts * G : 1, me = split_terms ? part * G + grp : 0;
@@ -387,13 +391,17 @@ __global__ void __launch_bounds__(kXsThreads, 2) k_xs_apply(const __grid_constan
       boff[t] = n < g.rest ? (n / g.inner) * (g.d * g.inner) + n % g.inner : -1;
     }
     const int inner = g.inner;
-    for (int q = me; q < nterm; q += n_split) {
-      const XsTerm tm = w.term[t_begin + q];
+    auto src = [&](int q) {
       XsSrc S;
+      const XsTerm tm = w.term[t_begin + q];
       S.a = i < g.d ? tm.M + (int64_t)i * g.d : nullptr;
 #pragma unroll
       for (int t = 0; t < kXsNT; ++t) S.b[t] = boff[t] >= 0 ? tm.X + boff[t] : nullptr;
-      xs_block<false>(gp, S, g.d, [](int k) { return k; }, [inner](int k) { return k * inner; }, acc);
+      return S;
+    };
+    int turn = 0;
+    for (int q = me; q < nterm; q += n_split, ++turn) {
+      xs_block<false>(gp, turn, src(q), g.d, [](int k) { return k; }, [inner](int k) { return k * inner; }, acc);
     }
   }
   double2* Y = pl ? w.planes + (int64_t)(w.plane[leg] + part) * ((int64_t)g.rest * g.d) : w.dst[o];
@@ -519,7 +527,7 @@ struct XsPj {
 };
 __global__ void __launch_bounds__(kXsThreads, 2) k_xs_project(const __grid_constant__ XsPj w) {
   __shared__ __align__(16) uint4 sm_bd[kXsWarps * 8 * 32];
-  __shared__ int sm_sc[kXsWarps][96];
+  __shared__ int sm_sc[kXsWarps][2 * 96];
   __shared__ double2 tot[kXsWarps * kXsCols * 8];  // this CTA's 8 MT x 16 tile
   double2(*red)[kXsCols * 8] = reinterpret_cast<double2(*)[kXsCols * 8]>(sm_bd);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -528,8 +536,8 @@ __global__ void __launch_bounds__(kXsThreads, 2) k_xs_project(const __grid_const
   const int MT = (g.d + 7) >> 3, G = kXsWarps / MT;
   const int mt = wid % MT, grp = wid / MT;
   const int rank = blockIdx.x % w.KS, tile = blockIdx.x / w.KS, o = blockIdx.y;
-  const XsGroup gp{mt, MT, 1 + grp, sm_sc[grp], sm_sc[grp] + 64, sm_sc[grp] + 80, sm_bd + (size_t)grp * MT * 8 * 32};
-  for (int e = threadIdx.x; e < kXsWarps * 96; e += kXsThreads) sm_sc[0][e] = 0;
+  const XsGroup gp{mt, MT, 1 + grp, sm_sc[grp], sm_bd + (size_t)grp * MT * 8 * 32};
+  for (int e = threadIdx.x; e < kXsWarps * 2 * 96; e += kXsThreads) sm_sc[0][e] = 0;
   __syncthreads();
   double acc[kXsNT][4];
 #pragma unroll
@@ -546,10 +554,11 @@ __global__ void __launch_bounds__(kXsThreads, 2) k_xs_project(const __grid_const
       const int x = tile * kXsCols + 8 * t + (lane >> 2);
       S.b[t] = x < g.d ? w.w[o] + (int64_t)x * inner : nullptr;
     }
-    for (int c = rank * G + grp; c < nch; c += w.KS * G) {
+    int turn = 0;
+    for (int c = rank * G + grp; c < nch; c += w.KS * G, ++turn) {
       const int r0 = c * chunk, K = min(chunk, g.rest - r0);
       auto at = [=](int k) { return (r0 + k) / inner * span + (r0 + k) % inner; };
-      xs_block<true>(gp, S, K, at, at, acc);
+      xs_block<true>(gp, turn, S, K, at, at, acc);
     }
   }
   __syncthreads();
@@ -612,7 +621,7 @@ int sm_count() {
 // Lists that take this path: contracted legs of at most 64, all outputs alike,
 // fewer than 2^31 elements, and enough multiply-adds that the CUDA-core kernel
 // would be bound by FP64 issue instead of by its launch.
-bool xs_applicable(const ApList& L, const ApOut* outs, const ApTerm* terms) {
+bool xs_applicable(const ApList& L, const ApOut* outs, const ApTerm* terms, int max_split) {
   if (L.n_tiles <= 0) return false;
   const ApOut& f = outs[L.out_begin];
   const int64_t P = (int64_t)f.d0 * f.d1 * f.d2 * f.d3;
@@ -629,7 +638,7 @@ bool xs_applicable(const ApList& L, const ApOut* outs, const ApTerm* terms) {
       if (!tm.pad) dense += 8.0 * P * dd[tm.leg];
     }
   }
-  return dense >= kXsMinFlops;
+  return dense >= xs_min_flops(max_split);
 }
 
 bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L, const Epi& e, const ApOut* outs,
@@ -743,7 +752,7 @@ bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L
 bool launch_project_xs(double2* const* bufs, double2* const* mats, const PjList& L, const PjOut* pjs, int max_split,
                        cudaStream_t s) {
   const int n = L.out_end - L.out_begin;
-  if (n < 1 || n > kXsMaxPj || L.flops < kXsMinPjFlops) return false;
+  if (n < 1 || n > kXsMaxPj || L.flops < xs_min_flops(max_split)) return false;
   const PjOut& f = pjs[L.out_begin];
   const int dd[3] = {f.d0, f.d1, f.d2}, d = dd[f.leg];
   const int64_t P = (int64_t)f.d0 * f.d1 * f.d2;
