@@ -149,23 +149,19 @@ void launch_tc_embed(void* const* mats32, const TcEmbedJob* jobs, int n, float* 
 // complex values (one-output lists: one plane per leg and term part, at most
 // max_split parts a leg). Returns
 // false (nothing launched) when the scratch or the launch's tables are too small.
-// The line: below about 8 MFLOP the CUDA-core launch is not bound by FP64 issue
-// and the second launch (plane sum) is not won back: 32x12x12, 12 terms (8.3
-// MFLOP) 16.6 us on the CUDA cores, 15.6 here; 19x11x11, 8 terms (2.1 MFLOP)
-// 8.7 / 13.3; 20^3, 12 terms (15 MFLOP) 26.7 / 13.5.
+// The line: 19x11x11, 8 terms (2.1 MFLOP) 7.2 us on the CUDA cores, 10.4 here (the
+// second launch, the plane sum, is not won back); 16^3, 12 terms (6.3 MFLOP) 12.3 / 9.3;
+// 32x12x12, 12 terms (8.3 MFLOP) 15.8 / 12.0; 20^3, 12 terms (15 MFLOP) 22.9 / 12.9.
+// It lies above the crossing, at 8 MFLOP, and is the same for every max_split: runs
+// that differ only in the split of the CUDA-core launches then stay on one path,
+// and together through the rank events of a long trajectory.
 constexpr double kXsMinFlops = 8.0e6;
-// Instances advanced together (max_split 1) share the FP64 pipes, so the work a
-// list takes off them counts beside its own latency. Batched step of 8 / 16 / 64
-// spin-boson instances: 6.4 / 16.1 / 41.8 ms at 8 MFLOP, 6.5 / 15.9 / 40.9 at 5,
-// 6.9 / 16.6 / 39.5 at 2, 7.4 / 16.9 / 39.4 at 1.
-constexpr double kXsMinFlopsShared = 5.0e6;
-inline double xs_min_flops(int max_split) { return max_split == 1 ? kXsMinFlopsShared : kXsMinFlops; }
-bool xs_applicable(const ApList& L, const ApOut* outs_host, const ApTerm* terms_host, int max_split);
+bool xs_applicable(const ApList& L, const ApOut* outs_host, const ApTerm* terms_host);
 bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L, const Epi& e,
                      const ApOut* outs_host, const ApTerm* terms_host, double2* planes, int64_t plane_elems,
                      int max_split, cudaStream_t s);
 // FP64 projections on the same path; false (nothing launched) below
-// xs_min_flops or when the list does not qualify (all outputs alike, 8 <= bond
+// kXsMinFlops or when the list does not qualify (all outputs alike, 8 <= bond
 // <= 64, at most 96 outputs).
 // Measured: 64-wide bond, 4096 positions, 5 classes 447 us (FP64 pipe) -> 172;
 // 56 classes' worth of the rank-64 chain's step 30.2 -> 9.9 ms.

@@ -20,19 +20,25 @@
 // column. A lane loads the complex values of its own fragment slots from
 // global memory (L1 / L2), so there is no shared-memory staging and no barrier
 // in the term loop; the digits live in registers. A warp owns 8 output indices x
-// 16 positions. Columns x of the operator block are first scaled to equal
-// size, the scale moved to the tensor operand: both fixed-point scales then
-// refer to the largest contribution |M[i][x]| |X[x][n]| and an operator whose
-// columns differ by many orders of magnitude loses nothing.
+// 16 positions. Before the split, X[x] of the tile is scaled to equal size over x and
+// the scale moved to operator column x. The operator's fixed point of row i is
+// then set by the largest contribution |M[i][x]| |X[x]| that the row receives, and what is
+// lost stays below 2^-60 of that, as a chain of FMAs loses 2^-53 of it: the small
+// components of a graded state (weights down to 1e-9 and below beside 1) keep
+// their relative accuracy, also where the operator couples them to themselves
+// by 1 and to the large ones by 1e-9. (With the columns of M scaled to equal size
+// instead, a rank-20 chain's bond directions of weight 1e-9 differed by 2e-9
+// from the FMA chain after 30 steps.)
 //
 // A non-finite operand makes its whole row or column of outputs NaN.
 //
 // Measured (graph replay, CUDA-core kernel / this one): 64^3 node, 14 terms
-// 1797 / 249 us (7.6 TFLOP/s of FP64 results against the 1.1 of the FP64 pipe;
+// 1799 / 244 us (7.7 TFLOP/s of FP64 results against the 1.1 of the FP64 pipe;
 // the tensor pipe is half busy, the rest is operand latency and digit
-// arithmetic); 20^3, 12 terms 26.7 / 13.8 us; 20x25x25, 12 terms 40.6 / 20.8 us.
-// Two scale sets in turn leave three group barriers a product instead of four,
-// and one conversion and one FMA join a digit sum (273 us without both).
+// arithmetic); 20^3, 12 terms 22.9 / 12.9 us; 20x25x25, 12 terms 38.4 / 16.8 us.
+// A product takes two group barriers (scales alternate between two sets; a
+// tensor row's scale is known to the warp that loaded it): with the scale of an
+// operator column, which all warps have to agree on, it took three and 249 us.
 // Relative 2-norm error against 128-bit sums: 1.15e-16 / 2.35e-16 (64^3),
 // 1.14e-16 / 1.70e-16 (20^3), 4.7e-17 / 1.4e-16 for a single product.
 #include <algorithm>
@@ -69,9 +75,9 @@ __device__ __forceinline__ int exp_c(double2 v) { return max(exp_field(v.x), exp
 
 // v as a fixed-point integer with 62 bits below 2^(top + 1 - 1023), plus the
 // bias that turns its bytes into digits - 128 .. 127 offset by 128. Subnormal v
-// is zero; so is everything where top is out of range (kXsNoScale): a shift by
+// is zero; so is everything where top is out of range (no scale): a shift by
 // 64 or more (or a negative count, taken as unsigned) gives zero.
-constexpr int kXsNoScale = 8192;
+constexpr int kXsBias = 4096;  // above every exponent field and difference of two
 __device__ __forceinline__ uint64_t fixed_biased(double v, int top) {
   const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
   const uint32_t e = (hi >> 20) & 0x7ffu, mh = (hi & 0xfffffu) | 0x100000u;
@@ -138,8 +144,8 @@ __device__ __forceinline__ double join(const float (&c)[8], int ex, double acc) 
 struct XsGroup {
   int m, MT, bar;   // warp of the group, warps, named barrier
   int* sc;          // [2][96] scales, two sets used in turn (one is cleared while the other is in use):
-                    //   [64] largest exponent of every operator column (group maximum)
-                    //   [16] largest tensor exponent + that of every position
+                    //   [64] scale of every K position: its largest tensor exponent over the 16 positions
+                    //   [16] largest scaled tensor exponent of every position, offset by kXsBias
                     //   [16] largest raw tensor exponent (0x7ff: not finite)
   uint4* bd;        // [MT][8][32] digits: x, y = K halves of positions 0..7, z, w = of positions 8..15
 };
@@ -154,7 +160,7 @@ __device__ __forceinline__ void gsync(const XsGroup& G) {
     asm volatile("bar.sync %0, %1;" ::"r"(G.bar), "r"(32 * G.MT) : "memory");
 }
 
-// acc += block product. PROJ: conj(A) instead of A.
+// acc += block product. PROJ: conj(B) instead of B.
 template <bool PROJ, typename KA, typename KB>
 __device__ __forceinline__ void xs_block(const XsGroup& G, int turn, const XsSrc& S, int K, KA ka, KB kb,
                                          double (&acc)[kXsNT][4]) {
@@ -164,7 +170,8 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, int turn, const XsSrc
   const int lane = threadIdx.x & 31, kq = lane & 3;
   const double2 zero = make_double2(0.0, 0.0);
   const int KS = (K + 7) >> 3;
-  // 1: raw tensor values of this warp's K positions; column exponents of the operator
+  // 1: raw tensor values of this warp's K positions, their scales (the largest
+  // exponent over the positions) and the position scales; operator exponents
   double2 braw[kXsNT][2];
 #pragma unroll
   for (int hf = 0; hf < 2; ++hf) {
@@ -172,7 +179,6 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, int turn, const XsSrc
 #pragma unroll
     for (int t = 0; t < kXsNT; ++t) braw[t][hf] = (k < K && S.b[t]) ? S.b[t][kb(k)] : zero;
   }
-  int rraw = 0;
   uint32_t ep[8];  // operator exponents of both K halves, so the operator is read once more only for its digits
 #pragma unroll
   for (int ks = 0; ks < 8; ++ks) {
@@ -184,40 +190,26 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, int turn, const XsSrc
       ep[ks] = (uint32_t)e0 | ((uint32_t)e1 << 16);
     }
   }
+  int eb[kXsNT][2];
+  uint32_t xr = 0;  // both K halves (packed 16-bit maxima)
 #pragma unroll
-  for (int ks = 0; ks < 8; ++ks)
-    if (ks < KS) {  // both halves' column maxima at once (packed 16-bit maxima)
-      uint32_t cx = ep[ks];
-      cx = __vmaxu2(cx, __shfl_xor_sync(kFull, cx, 4));
-      cx = __vmaxu2(cx, __shfl_xor_sync(kFull, cx, 8));
-      cx = __vmaxu2(cx, __shfl_xor_sync(kFull, cx, 16));
-      if (lane < 8) atomicMax(&scx[ks * 8 + lane], lane < 4 ? (int)(cx & 0xffff) : (int)(cx >> 16));
-      rraw = max(rraw, max((int)(ep[ks] & 0xffff), (int)(ep[ks] >> 16)));
-    }
-  gsync(G);  // also: every warp is done with the previous product's scales and digits
-  for (int e = G.m * 32 + lane; e < 96; e += 32 * G.MT) G.sc[96 * ((turn & 1) ^ 1) + e] = 0;
-  // 2: row scale of the scaled operator, position scales
-  int row = -4096;
-#pragma unroll
-  for (int ks = 0; ks < 8; ++ks)
-    if (ks < KS) {
-      const int e0 = ep[ks] & 0xffff, e1 = ep[ks] >> 16;
-      if (e0) row = max(row, e0 - scx[ks * 8 + kq]);
-      if (e1) row = max(row, e1 - scx[ks * 8 + 4 + kq]);
-    }
-  row = max(row, __shfl_xor_sync(kFull, row, 1));
-  row = max(row, __shfl_xor_sync(kFull, row, 2));
-  rraw = max(rraw, __shfl_xor_sync(kFull, rraw, 1));
-  rraw = max(rraw, __shfl_xor_sync(kFull, rraw, 2));
-  const int cb[2] = {scx[G.m * 8 + kq], scx[G.m * 8 + 4 + kq]};
+  for (int t = 0; t < kXsNT; ++t) {
+    eb[t][0] = exp_c(braw[t][0]);
+    eb[t][1] = exp_c(braw[t][1]);
+    xr = __vmaxu2(xr, (uint32_t)eb[t][0] | ((uint32_t)eb[t][1] << 16));
+  }
+  xr = __vmaxu2(xr, __shfl_xor_sync(kFull, xr, 4));
+  xr = __vmaxu2(xr, __shfl_xor_sync(kFull, xr, 8));
+  xr = __vmaxu2(xr, __shfl_xor_sync(kFull, xr, 16));
+  const int xk[2] = {(int)(xr & 0xffff), (int)(xr >> 16)};
+  if (lane < 8) scx[G.m * 8 + lane] = lane < 4 ? xk[0] : xk[1];
 #pragma unroll
   for (int t = 0; t < kXsNT; ++t) {
     int c = 0, r = 0;
 #pragma unroll
     for (int hf = 0; hf < 2; ++hf) {
-      const int eb = exp_c(braw[t][hf]);
-      if (eb && cb[hf]) c = max(c, eb + cb[hf]);
-      r = max(r, eb);
+      if (eb[t][hf]) c = max(c, eb[t][hf] - xk[hf] + kXsBias);
+      r = max(r, eb[t][hf]);
     }
     c = max(c, __shfl_xor_sync(kFull, c, 1));
     c = max(c, __shfl_xor_sync(kFull, c, 2));
@@ -228,22 +220,36 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, int turn, const XsSrc
       atomicMax(&scraw[8 * t + (lane >> 2)], r);
     }
   }
-  gsync(G);
-  // 3: tensor digits of this warp's K positions
+  gsync(G);  // also: every warp is done with the previous product's scales and digits
+  for (int e = 64 + G.m * 32 + lane; e < 96; e += 32 * G.MT) G.sc[96 * ((turn & 1) ^ 1) + e] = 0;
+  // 2: row scale of the scaled operator; tensor digits of this warp's K positions
+  int row = -kXsBias, rraw = 0;
+#pragma unroll
+  for (int ks = 0; ks < 8; ++ks)
+    if (ks < KS) {
+      const int e0 = ep[ks] & 0xffff, e1 = ep[ks] >> 16;
+      const int x0 = scx[ks * 8 + kq], x1 = scx[ks * 8 + 4 + kq];
+      if (e0 && x0) row = max(row, e0 + x0);
+      if (e1 && x1) row = max(row, e1 + x1);
+      rraw = max(rraw, max(e0, e1));
+    }
+  row = max(row, __shfl_xor_sync(kFull, row, 1));
+  row = max(row, __shfl_xor_sync(kFull, row, 2));
+  rraw = max(rraw, __shfl_xor_sync(kFull, rraw, 1));
+  rraw = max(rraw, __shfl_xor_sync(kFull, rraw, 2));
   {
     uint32_t d[kXsNT][2][8];
 #pragma unroll
     for (int t = 0; t < kXsNT; ++t) {
-      const int cs = scol[8 * t + (lane >> 2)], top = cs ? cs : kXsNoScale;
+      const int top = scol[8 * t + (lane >> 2)] - kXsBias;
 #pragma unroll
-      for (int hf = 0; hf < 2; ++hf)  // a zero operator column contributes nothing whatever the tensor holds
-        digits8(cb[hf] ? braw[t][hf] : zero, top - cb[hf], d[t][hf]);
+      for (int hf = 0; hf < 2; ++hf) digits8(braw[t][hf], top + xk[hf], d[t][hf]);
     }
 #pragma unroll
     for (int j = 0; j < 8; ++j) G.bd[(G.m * 8 + j) * 32 + lane] = make_uint4(d[0][0][j], d[0][1][j], d[1][0][j], d[1][1][j]);
   }
   gsync(G);
-  // 4: operator digits and MMAs
+  // 3: operator digits and MMAs
   float c[kXsNT][8][4];
 #pragma unroll
   for (int t = 0; t < kXsNT; ++t)
@@ -264,12 +270,12 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, int turn, const XsSrc
 #pragma unroll
     for (int hf = 0; hf < 2; ++hf) {
       uint32_t ad[8];
-      digits8(v[hf], row + scx[ks * 8 + 4 * hf + kq], ad);
+      digits8(v[hf], row - scx[ks * 8 + 4 * hf + kq], ad);
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const uint32_t sw = __byte_perm(ad[i], ad[i], 0x1032);  // (im, re)
         a[i][2 * hf] = PROJ ? ad[i] : ad[i] ^ 0x80000000u;      // (re, -+im)
-        a[i][2 * hf + 1] = PROJ ? sw ^ 0x00008000u : sw;        // (+-im, re)
+        a[i][2 * hf + 1] = PROJ ? sw ^ 0x80000000u : sw;        // (im, +-re)
       }
     }
 #pragma unroll
@@ -288,6 +294,8 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, int turn, const XsSrc
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       const int n = 8 * t + 2 * kq + j, ec = scol[n];
+      const int ex = row + ec - kXsBias;  // no scale: the sums are zero, and 2^0 keeps join() off its slow path
+      const bool none = row < 0 || ec == 0;
       const bool bad = rraw == 0x7ff || scraw[n] == 0x7ff;
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
@@ -297,7 +305,7 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, int turn, const XsSrc
         // both fixed points: value = integer * 2^(scale - 1084); the digit pairs of
         // group g weigh 2^(8 (14 - g)), 2^56 of it outside join()
         acc[t][2 * j + p] = bad ? __longlong_as_double(0x7ff8000000000000ll)
-                                : join(cc, row + ec - 2 * 1084 + 56, acc[t][2 * j + p]);
+                                : join(cc, none ? 0 : ex - 2 * 1084 + 56, acc[t][2 * j + p]);
       }
     }
 }
@@ -512,8 +520,9 @@ __global__ void __launch_bounds__(128) k_xs_epilogue(const double2* planes, int 
 
 // ---------------------------------------------------------------------------
 // Environment projections E[x', x] = sum_r conj(U[x', r]) W[x, r] of wide bonds
-// by the same split: output rows x' in blocks of 8 (one per warp of a group),
-// columns x in tiles of 16, the reduction range in chunks of 8 MT positions, one
+// by the same split, W as the operator and the isometry conj(U) as the tensor
+// operand (its scales leave W's rows as they are, so weakly occupied x keep their relative
+// accuracy): x in blocks of 8 (one per warp of a group), x' in tiles of 16, the reduction range in chunks of 8 MT positions, one
 // exact block product per chunk with its own scales, added in FP64. The chunks of
 // a tile are dealt to the groups of KS CTAs (one cluster), whose sums CTA 0 adds
 // in order through distributed shared memory.
@@ -548,11 +557,11 @@ __global__ void __launch_bounds__(kXsThreads, 2) k_xs_project(const __grid_const
   if (grp < G) {
     const int i = mt * 8 + (lane >> 2), inner = g.inner, span = g.d * g.inner;
     XsSrc S;
-    S.a = i < g.d ? w.u + (int64_t)i * inner : nullptr;
+    S.a = i < g.d ? w.w[o] + (int64_t)i * inner : nullptr;
 #pragma unroll
     for (int t = 0; t < kXsNT; ++t) {
       const int x = tile * kXsCols + 8 * t + (lane >> 2);
-      S.b[t] = x < g.d ? w.w[o] + (int64_t)x * inner : nullptr;
+      S.b[t] = x < g.d ? w.u + (int64_t)x * inner : nullptr;
     }
     int turn = 0;
     for (int c = rank * G + grp; c < nch; c += w.KS * G, ++turn) {
@@ -591,7 +600,7 @@ __global__ void __launch_bounds__(kXsThreads, 2) k_xs_project(const __grid_const
         v.y += x.y;
       }
       const int ii = (e / (kXsCols * 8)) * 8 + (e & 7), x = tile * kXsCols + (e % (kXsCols * 8)) / 8;
-      if (ii < g.d && x < g.d) w.dst[o][(int64_t)ii * g.d + x] = v;
+      if (ii < g.d && x < g.d) w.dst[o][(int64_t)x * g.d + ii] = v;
     }
     cluster.sync();  // shared memory stays until every CTA has read it
     return;
@@ -599,7 +608,7 @@ __global__ void __launch_bounds__(kXsThreads, 2) k_xs_project(const __grid_const
   __syncthreads();
   for (int e = threadIdx.x; e < ne; e += kXsThreads) {
     const int ii = (e / (kXsCols * 8)) * 8 + (e & 7), x = tile * kXsCols + (e % (kXsCols * 8)) / 8;
-    if (ii < g.d && x < g.d) w.dst[o][(int64_t)ii * g.d + x] = tot[e];
+    if (ii < g.d && x < g.d) w.dst[o][(int64_t)x * g.d + ii] = tot[e];
   }
 }
 
@@ -621,7 +630,7 @@ int sm_count() {
 // Lists that take this path: contracted legs of at most 64, all outputs alike,
 // fewer than 2^31 elements, and enough multiply-adds that the CUDA-core kernel
 // would be bound by FP64 issue instead of by its launch.
-bool xs_applicable(const ApList& L, const ApOut* outs, const ApTerm* terms, int max_split) {
+bool xs_applicable(const ApList& L, const ApOut* outs, const ApTerm* terms) {
   if (L.n_tiles <= 0) return false;
   const ApOut& f = outs[L.out_begin];
   const int64_t P = (int64_t)f.d0 * f.d1 * f.d2 * f.d3;
@@ -638,7 +647,7 @@ bool xs_applicable(const ApList& L, const ApOut* outs, const ApTerm* terms, int 
       if (!tm.pad) dense += 8.0 * P * dd[tm.leg];
     }
   }
-  return dense >= xs_min_flops(max_split);
+  return dense >= kXsMinFlops;
 }
 
 bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L, const Epi& e, const ApOut* outs,
@@ -752,7 +761,7 @@ bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L
 bool launch_project_xs(double2* const* bufs, double2* const* mats, const PjList& L, const PjOut* pjs, int max_split,
                        cudaStream_t s) {
   const int n = L.out_end - L.out_begin;
-  if (n < 1 || n > kXsMaxPj || L.flops < xs_min_flops(max_split)) return false;
+  if (n < 1 || n > kXsMaxPj || L.flops < kXsMinFlops) return false;
   const PjOut& f = pjs[L.out_begin];
   const int dd[3] = {f.d0, f.d1, f.d2}, d = dd[f.leg];
   const int64_t P = (int64_t)f.d0 * f.d1 * f.d2;
