@@ -279,6 +279,7 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) k_apply(const __grid_constan
   const bool in = idx < P;
   g.i0 = g.i1 = g.i2 = g.i3 = 0;
   const int64_t at = 2 * idx + (wid & 1);
+  grid_wait();
   double y0 = 0.0, a0 = 0.0;
   if (in) {
     if (ep.mode != EPI_STORE && wid < 2 && rank == 0) {
@@ -300,6 +301,7 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) k_apply(const __grid_constan
     }
   }
   R acc = tile_sum<R, NW>(tab, out, g, idx, in, rank, K, part);
+  grid_release();
   if (K > 1) {
     cg::cluster_group cluster = cg::this_cluster();
     if (wid < 2) reinterpret_cast<R*>(cluster.map_shared_rank(&slot[0][0], 0))[rank * 64 + 2 * lane + wid] = acc;
@@ -314,23 +316,7 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) k_apply(const __grid_constan
 // Launch n_tiles * k CTAs; k > 1 makes every k consecutive CTAs one cluster.
 template <typename Kern, typename... Args>
 static void launch_split(Kern kern, int n_tiles, int k, int warps, cudaStream_t s, const Args&... args) {
-  if (k <= 1) {
-    kern<<<n_tiles, 32 * warps, 0, s>>>(args...);
-    return;
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(n_tiles * k), 1, 1);
-  cfg.blockDim = dim3(32 * warps, 1, 1);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)k;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, kern, args...);
+  launch_dep(kern, dim3((unsigned)(n_tiles * k)), dim3(32 * warps), 0, s, k > 1 ? k : 0, args...);
 }
 
 template <typename R, typename TAB>
@@ -428,6 +414,7 @@ __global__ void __launch_bounds__(32 * kPjWarps, 4) k_project(const __grid_const
   const int e = (tile - pj.tile0) * kPjTile + lane;
   const int la = l == 0 ? 1 : 0, lb = l == 2 ? 1 : 2;  // the two other legs
   const int nrest = dd[la] * dd[lb];
+  grid_wait();
   V acc = C::zero();
   if (e < d * d) {
     const int xp = e / d, x = e % d;
@@ -453,6 +440,7 @@ __global__ void __launch_bounds__(32 * kPjWarps, 4) k_project(const __grid_const
   part[wid][lane] = acc;
   __syncthreads();
   R sum = comp_sum<R>(part, kPjWarps);
+  grid_release();
   if (K > 1) {
     cg::cluster_group cluster = cg::this_cluster();
     if (wid < 2) reinterpret_cast<R*>(cluster.map_shared_rank(&slot[0][0], 0))[rank * 64 + 2 * lane + wid] = sum;
@@ -500,6 +488,7 @@ __global__ void __launch_bounds__(256) k_project_tiled(DevTables T, PjList L, in
   const bool leg_fast = l == 2;  // the leg index is the contiguous one
   const int ty = (tid >> 4) * 2, tx = (tid & 15) * 2;
   V acc[2][2] = {{C::zero(), C::zero()}, {C::zero(), C::zero()}};
+  grid_wait();
   for (int c = c0; c < c1; ++c) {
     const int r0 = c * kPtR;
     if (tid < kPtR) {
@@ -527,6 +516,7 @@ __global__ void __launch_bounds__(256) k_project_tiled(DevTables T, PjList L, in
     }
     __syncthreads();
   }
+  grid_release();
   if (KS > 1) {
     cg::cluster_group cluster = cg::this_cluster();
     if (rank > 0) {
@@ -568,20 +558,10 @@ bool launch_project_tiled(int prec, const DevTables& T, const PjList& L, int d, 
     cudaFuncSetAttribute(k_project_tiled<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
     attr = true;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(items * KS), 1, 1);
-  cfg.blockDim = dim3(256, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr1[1];
-  attr1[0].id = cudaLaunchAttributeClusterDimension;
-  attr1[0].val.clusterDim.x = (unsigned)KS;
-  attr1[0].val.clusterDim.y = 1;
-  attr1[0].val.clusterDim.z = 1;
-  cfg.attrs = attr1;
-  cfg.numAttrs = 1;
-  if (prec == PREC_F32) return cudaLaunchKernelEx(&cfg, k_project_tiled<float>, T, L, ntx, KS) == cudaSuccess;
-  return cudaLaunchKernelEx(&cfg, k_project_tiled<double>, T, L, ntx, KS) == cudaSuccess;
+  const dim3 grid((unsigned)(items * KS));
+  if (prec == PREC_F32)
+    return launch_dep(k_project_tiled<float>, grid, dim3(256), smem, s, KS, T, L, ntx, KS) == cudaSuccess;
+  return launch_dep(k_project_tiled<double>, grid, dim3(256), smem, s, KS, T, L, ntx, KS) == cudaSuccess;
 }
 
 template <typename R, int NO>
@@ -810,6 +790,8 @@ void launch_qr(double2* U, int d0, int d1, int d2, int leg, double tol, double2*
 }
 
 __global__ void k_copy(double2* dst, float2* dst_lo, const double2* src, int64_t n) {
+  grid_wait();
+  grid_release();  // nothing but the copy itself is left
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const double2 v = src[i];
     dst[i] = v;
@@ -819,7 +801,7 @@ __global__ void k_copy(double2* dst, float2* dst_lo, const double2* src, int64_t
 void launch_copy(double2* dst, float2* dst_lo, const double2* src, int64_t n, cudaStream_t s) {
   if (n <= 0) return;
   int blocks = (int)std::min<int64_t>((n + 255) / 256, 1024);
-  k_copy<<<blocks, 256, 0, s>>>(dst, dst_lo, src, n);
+  launch_dep(k_copy, dim3(blocks), dim3(256), 0, s, 0, dst, dst_lo, src, n);
 }
 
 // ---------------------------------------------------------------------------
@@ -843,6 +825,7 @@ __global__ void __launch_bounds__(256) k_rdm_level(const __grid_constant__ RdmLe
   while (q + 1 < lv.n && (int)blockIdx.x >= lv.job[q + 1].cta0) ++q;
   const RdmJob jb = lv.job[q];
   const int e = blockIdx.x - jb.cta0, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  grid_wait();
   // root: e = i*d1 + j, out[e] = sum_c U[i, j, c] w2[c]; else out[a] = sum_{b,c} U[a, b, c] w1[b] w2[c]
   const int nb = jb.w1 ? jb.d1 : 1, nc = jb.w2 ? jb.d2 : 1;
   const double2* blk = jb.U + (int64_t)e * (jb.root ? jb.d2 : (int64_t)jb.d1 * jb.d2);
@@ -866,6 +849,7 @@ __global__ void __launch_bounds__(256) k_rdm_level(const __grid_constant__ RdmLe
     acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
     acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
   }
+  grid_release();
   if (lane == 0) {
     part[warp][0] = acc.x;
     part[warp][1] = acc.y;
@@ -889,7 +873,7 @@ void launch_rdm_level(RdmJob* jobs, int n, const int* flag, double2* flag_out, c
       ctas += j.n_out;
       lv.job[lv.n++] = j;
     }
-    if (ctas > 0) k_rdm_level<<<ctas, 256, 0, s>>>(lv, flag, flag_out);
+    if (ctas > 0) launch_dep(k_rdm_level, dim3(ctas), dim3(256), 0, s, 0, lv, flag, flag_out);
   }
 }
 

@@ -14,6 +14,48 @@ namespace ttn {
 // both modes; PREC_F32 runs the contractions in FP32 on FP32 shadow copies.
 enum Prec : int { PREC_F64 = 0, PREC_F32 = 1 };
 
+// Programmatic dependent launch. The kernels of a step form one chain of short
+// launches. launch_dep lets a launch start its CTAs while the previous kernel of
+// the stream still runs; such a kernel calls grid_wait() before it touches global
+// memory that a launch writes (the wait ends when everything before it has
+// completed and is visible), and grid_release() once its own sums are done, so
+// that the next kernel's launch, parameters and index arithmetic overlap its last
+// reduction and its stores. Released earlier, the waiting CTAs take the room of
+// running work: rank-10 train / rank-20 chain / 64 batched instances 11.34 / 29.28 /
+// 39.8 ms without, 10.33 / 28.55 / 39.4 with the release after the sums, 10.44 /
+// 29.18 / 41.1 right after the wait, 10.55 / 29.36 / 42.6 before it (contractions and
+// projections of the CUDA cores; the QR adds 0.1, the copies 0.5 ms to the chain's
+// gain). All CTAs of the earlier kernel are resident by then, so a waiting CTA
+// never keeps one from starting. The larger kernels are launched plainly: nothing
+// to win on the tensor cores' (within 0.3 %), and between the blocked QR's cooperative
+// panels it costs 5 % (rank-64 chain 99.3 -> 104.2 ms).
+// cluster: CTAs per cluster, 0 for a kernel without cluster instructions (a
+// kernel with remote stores needs the attribute for a cluster of one too: `mapa`
+// and `st.async` are illegal outside a cluster launch).
+#ifdef __CUDACC__
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+inline cudaError_t launch_dep(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int cluster,
+                              const A&... args) {
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)cluster;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster > 0 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+#endif
+
 // Device-side view of the job tables. Element type of bufs/mats is the
 // contraction type of the table (double2 or float2).
 struct DevTables {

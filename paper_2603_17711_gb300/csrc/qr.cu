@@ -192,7 +192,6 @@ __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int
   const bool six = n <= 6 * kGPW;
   const int slots = six ? 6 * kGPW : kSlots;
   const int cw = !six ? wid - 1 : wid < 4 ? wid - 1 : wid == 4 ? -1 : wid - 2;  // place among the column warps, -1: none
-  const uint64_t deadline = gtimer() + 2000000000ull;
 
   extern __shared__ double2 smem[];
   double2* A = smem;
@@ -219,6 +218,8 @@ __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
 
+  grid_wait();
+  const uint64_t deadline = gtimer() + 2000000000ull;
   // gather my rows: A[c][i] = U[.. row r0+i, column c ..] (panel: pn.A[c0+c][c0+r0+i])
   double fro = 0.0;
   for (int k = tid; k < n * rp; k += nt) {
@@ -567,6 +568,7 @@ __global__ void __launch_bounds__(kThreads) k_qr_cluster(double2* U, int d0, int
       dst[a * n + c] = buf[a];
     }
   }
+  grid_release();
   cluster.sync();  // M complete in every CTA; nobody reads another's rows any more
   // Q rows: Q[r][c] = delta_rc - sum_{a <= min(r,c)} v_a[r] M[a][c], column c scaled by phase_c
   // Entries (c, row) are laid along the lanes column after column, so that few
@@ -618,19 +620,9 @@ static bool launch_cluster(double2* U, int d0, int d1, int d2, int leg, double t
     cudaFuncSetAttribute(k_qr_cluster<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQrSmemCap);
     attr_done = true;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(C, 1, 1);
-  cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = qr_cluster_smem(m, n, C, pn.A ? 1 : pn.gtail ? 0 : pn.m_apart ? 2 : 1);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = C;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_qr_cluster<G>, U, d0, d1, d2, leg, tol, R, flag, U_lo, R_lo, pn) == cudaSuccess;
+  const size_t smem = qr_cluster_smem(m, n, C, pn.A ? 1 : pn.gtail ? 0 : pn.m_apart ? 2 : 1);
+  return launch_dep(k_qr_cluster<G>, dim3(C), dim3(kThreads), smem, s, C, U, d0, d1, d2, leg, tol, R, flag, U_lo, R_lo,
+                    pn) == cudaSuccess;
 }
 
 bool launch_qr_cluster(double2* U, int d0, int d1, int d2, int leg, double tol, double2* R, int* flag,
