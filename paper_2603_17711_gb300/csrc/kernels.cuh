@@ -402,8 +402,8 @@ void launch_write_pair(double2* Uf, float2* Uf_lo, const int* fd, int lf, double
 // Direct integration (vmf.cu), FP64. launch_vmf_edge: on edge p -> c with the
 // QR factor R (r x r, row-major) of the upper part and the class matrices at
 // slots_dev[0..n_classes) (isometric environments on entry): rho = R^H R,
-// rho_reg = rho + eps 1, E~ = rho_reg^-1 R^H E R in place, dmi = rho_reg^-1 rho - 1.
-// aug: 3 r^2, tmp: 2 r^2 per class. launch_vmf_finish: K (node derivative, r x
+// rho_reg = rho + eps 1, E~ = rho_reg^-1 R^H E R in place, dmi = rho_reg^-1 rho - 1
+// = -eps rho_reg^-1. aug: 3 r^2 (the inverse and, for wide bonds, the elimination), tmp: 2 r^2 per class. launch_vmf_finish: K (node derivative, r x
 // nc, row-major over the parent index) += dmi G_down, then K := (1 - P) K with
 // P the projector onto the rows of U (X: r^2 scratch).
 void launch_vmf_edge(double2* const* mats_dev, const int* slots_dev, int n_classes, const double2* R, int r,

@@ -15,19 +15,21 @@
 // then multiplies rho, not the identity, for those terms). P_c projects onto
 // the span of U_c's rows (parent index fixed): (1 - P) X = X - (X U^H) U.
 //
-//  k_vmf_rho    one CTA: rho = R^H R, the augmented [rho + eps 1 | 1 | rho]
-//  k_vmf_gj     one CTA: Gauss-Jordan elimination with partial pivoting of the
-//               augmented matrix -> [1 | rho_reg^-1 | D]; D - 1 stored
-//  k_vmf_class  one CTA per class: E~ = rho_reg^-1 (R^H (E R)), in place
-//  k_vmf_dmi    K += (D - 1) x_0 G_down
+//  k_vmf_inv    one CTA: rho = R^H R, rho_reg^-1 by Gauss-Jordan elimination with
+//               partial pivoting, D - 1 = -vmf_atol rho_reg^-1
+//  k_vmf_class  one cluster per class: E~ = rho_reg^-1 (R^H (E R)), in place
+//  k_vmf_addmul K += (D - 1) G_down; K -= X U
 //  k_vmf_px     X = K U^H (one CTA per entry, fixed-order sums)
-//  k_vmf_psub   K -= X U
 //  k_vmf_stage  out = y + sum_l c_l K_l over the flat state
 //  k_vmf_err    scaled squared error of the embedded pair, block partials;
 //  k_vmf_sum    the partials added in order
 #include <algorithm>
 
+#include <cooperative_groups.h>
+
 #include "kernels.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace ttn {
 
@@ -43,123 +45,146 @@ __device__ __forceinline__ double2 cmulc(double2 a, double2 b) {  // conj(a) b
 }
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 
-// aug: r x 3r row-major: [rho + eps 1 | 1 | rho]
-__global__ void k_vmf_rho(const double2* __restrict__ R, int r, double eps, double2* __restrict__ aug) {
-  const int w = 3 * r;
-  for (int e = threadIdx.x; e < r * r; e += blockDim.x) {
-    const int i = e / r, j = e % r;
-    double2 s = make_double2(0.0, 0.0);
-    for (int k = 0; k < r; ++k) s = cadd(s, cmulc(R[k * r + i], R[k * r + j]));  // (R^H R)[i][j]
-    aug[i * w + j] = make_double2(s.x + (i == j ? eps : 0.0), s.y);
-    aug[i * w + r + j] = make_double2(i == j ? 1.0 : 0.0, 0.0);
-    aug[i * w + 2 * r + j] = s;
-  }
+// Component comp (0 real, 1 imaginary) of s + a b and of s + conj(a) b.
+__device__ __forceinline__ double fma_part(double2 a, double2 b, int comp, double s) {
+  return fma(a.y, comp ? b.x : -b.y, fma(a.x, comp ? b.y : b.x, s));
+}
+__device__ __forceinline__ double fma_conj_part(double2 a, double2 b, int comp, double s) {
+  return fma(a.y, comp ? -b.x : b.y, fma(a.x, comp ? b.y : b.x, s));
 }
 
-// Gauss-Jordan on the r x 3r augmented matrix: pivot column j, the row of the
-// largest |entry| at or below j (lowest index on ties) swapped up, scaled, and
-// eliminated from every other row. Leaves [1 | rho_reg^-1 | D]; dmi = D - 1.
-__global__ void k_vmf_gj(double2* aug, int r, double2* __restrict__ dmi) {
-  __shared__ int s_piv;
-  __shared__ double2 s_inv;
-  const int w = 3 * r, tid = threadIdx.x;
+// inv = (rho + eps)^-1 with rho = R^H R, dmi = (rho + eps)^-1 rho - 1 = -eps inv, by
+// Gauss-Jordan on [rho + eps | 1], held in shared memory (in `aug` above
+// kGjSmemMaxR). Pivot: the largest |re| + |im| of the column among the rows not
+// yet used. Rows are neither swapped nor scaled until the end, so a pivot takes
+// two barriers: warp 0 finds it and divides the column's entries by it, then
+// all threads eliminate; of the left block only the columns still to come are
+// updated. A chain of latencies on one CTA (an FP64 instruction holds an SM
+// sub-partition for 64 cycles): r = 12 took 38 us with six barriers a pivot, the
+// matrix in global memory and rho as a third block.
+constexpr int kGjSmemMaxR = 64;
+size_t inv_smem(int r) { return sizeof(double2) * (size_t)(2 * r + (r <= kGjSmemMaxR ? 2 * r * r : 0)) + sizeof(int) * r; }
+__global__ void __launch_bounds__(kT) k_vmf_inv(const double2* __restrict__ R, int r, double eps, double2* aug,
+                                                double2* __restrict__ inv, double2* __restrict__ dmi) {
+  extern __shared__ double2 gj[];
+  const int tid = threadIdx.x, nt = blockDim.x, w = 2 * r;
+  double2* f = gj;       // multipliers of the current pivot
+  double2* sc = gj + r;  // 1 / pivot
+  double2* A = r <= kGjSmemMaxR ? gj + 2 * r : aug;
+  int* perm = (int*)(gj + 2 * r + (r <= kGjSmemMaxR ? 2 * r * r : 0));  // row of pivot j
+  grid_wait();
+  for (int e = tid; e < 2 * r * r; e += nt) {
+    const int comp = e & 1, i = (e >> 1) / r, j = (e >> 1) % r;
+    double s = 0.0;
+    for (int k = 0; k < r; ++k) s = fma_conj_part(R[k * r + i], R[k * r + j], comp, s);
+    reinterpret_cast<double*>(A + i * w + j)[comp] = i == j && comp == 0 ? s + eps : s;
+    reinterpret_cast<double*>(A + i * w + r + j)[comp] = i == j && comp == 0 ? 1.0 : 0.0;
+  }
+  __syncthreads();
   for (int j = 0; j < r; ++j) {
     if (tid < 32) {
-      double best = -1.0;
-      int bi = j;
-      for (int i = j + tid; i < r; i += 32) {
-        const double a = fabs(aug[i * w + j].x) + fabs(aug[i * w + j].y);
+      // nonnegative doubles compare as integers (a NaN above all numbers); + 1: a zero still beats no row
+      unsigned long long best = 0;
+      int bi = r;
+      for (int i = tid; i < r; i += 32) {
+        bool used = false;
+        for (int q = 0; q < j; ++q) used |= perm[q] == i;
+        const double2 v = A[i * w + j];
+        const unsigned long long a = used ? 0 : (unsigned long long)__double_as_longlong(fabs(v.x) + fabs(v.y)) + 1;
         if (a > best) {
           best = a;
           bi = i;
         }
       }
-      for (int o = 16; o > 0; o >>= 1) {
-        const double ob = __shfl_down_sync(0xffffffffu, best, o);
-        const int oi = __shfl_down_sync(0xffffffffu, bi, o);
-        if (ob > best || (ob == best && oi < bi)) {
-          best = ob;
-          bi = oi;
-        }
+      const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(best >> 32));
+      const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(best >> 32) == hi ? (unsigned)best : 0u);
+      const bool top = best == (((unsigned long long)hi << 32) | lo);
+      const int pv = (int)__reduce_min_sync(0xffffffffu, top ? (unsigned)bi : (unsigned)r);
+      const double2 p = A[pv * w + j];
+      const double n = fma(p.x, p.x, p.y * p.y), q = ((tid & 1) ? -p.y : p.x) / n;  // even lanes real, odd imaginary
+      const double2 pi = make_double2(__shfl_sync(0xffffffffu, q, 0), __shfl_sync(0xffffffffu, q, 1));
+      for (int i = tid; i < r; i += 32) f[i] = cmul(A[i * w + j], pi);
+      if (tid == 0) {
+        perm[j] = pv;
+        sc[j] = pi;
       }
-      if (tid == 0) s_piv = bi;
     }
     __syncthreads();
-    const int pv = s_piv;
-    if (pv != j)
-      for (int c = tid; c < w; c += blockDim.x) {
-        const double2 t = aug[j * w + c];
-        aug[j * w + c] = aug[pv * w + c];
-        aug[pv * w + c] = t;
-      }
-    __syncthreads();
-    if (tid == 0) {
-      const double2 p = aug[j * w + j];
-      const double n = p.x * p.x + p.y * p.y;
-      s_inv = make_double2(p.x / n, -p.y / n);
+    const int pv = perm[j], nc = w - j - 1;
+    for (int e = tid; e < r * nc; e += nt) {
+      const int i = e / nc, c = j + 1 + e % nc;
+      if (i == pv) continue;
+      const double2 p = A[pv * w + c], m = f[i];
+      double2 a = A[i * w + c];
+      a.x = fma(-m.x, p.x, fma(m.y, p.y, a.x));
+      a.y = fma(-m.x, p.y, fma(-m.y, p.x, a.y));
+      A[i * w + c] = a;
     }
-    __syncthreads();
-    for (int c = tid; c < w; c += blockDim.x) aug[j * w + c] = cmul(s_inv, aug[j * w + c]);
-    __syncthreads();
-    for (int e = tid; e < r * w; e += blockDim.x) {
-      const int i = e / w, c = e % w;
-      if (i == j || c == j) continue;
-      const double2 f = aug[i * w + j];
-      const double2 v = cmul(f, aug[j * w + c]);
-      aug[i * w + c] = make_double2(aug[i * w + c].x - v.x, aug[i * w + c].y - v.y);
-    }
-    __syncthreads();
-    for (int i = tid; i < r; i += blockDim.x)
-      if (i != j) aug[i * w + j] = make_double2(0.0, 0.0);
     __syncthreads();
   }
-  for (int e = tid; e < r * r; e += blockDim.x) {
+  grid_release();
+  for (int e = tid; e < r * r; e += nt) {
     const int i = e / r, c = e % r;
-    const double2 d = aug[i * w + 2 * r + c];
-    dmi[e] = make_double2(d.x - (i == c ? 1.0 : 0.0), d.y);
+    const double2 v = cmul(A[perm[i] * w + r + c], sc[i]);
+    inv[e] = v;
+    dmi[e] = make_double2(-eps * v.x, -eps * v.y);
   }
 }
 
-// E~ = rho_reg^-1 (R^H (E R)) for the class matrix of this CTA, in place; the
-// two intermediate products in `tmp` (2 r^2 per CTA).
-__global__ void k_vmf_class(double2* const* mats, const int* __restrict__ slots, const double2* __restrict__ R,
-                            const double2* __restrict__ aug, int r, double2* __restrict__ tmp) {
-  double2* E = mats[slots[blockIdx.x]];
-  double2* A = tmp + (size_t)blockIdx.x * 2 * r * r;  // E R
-  double2* B = A + r * r;                              // R^H E R
-  const int w = 3 * r;
-  for (int e = threadIdx.x; e < r * r; e += blockDim.x) {
-    const int i = e / r, j = e % r;
-    double2 s = make_double2(0.0, 0.0);
-    for (int k = 0; k < r; ++k) s = cadd(s, cmul(E[i * r + k], R[k * r + j]));
-    A[e] = s;
+// E~ = inv (R^H (E R)) for one class matrix per cluster, in place; a CTA makes
+// its own columns of all three products (one thread per component), the two
+// intermediate ones in `tmp` (2 r^2 per class), and E is overwritten once every
+// CTA has read it. FP64 issue of one SM bound a CTA per class: r = 12 12.7 us.
+__global__ void __launch_bounds__(128) k_vmf_class(double2* const* mats, const int* __restrict__ slots,
+                                                   const double2* __restrict__ R, const double2* __restrict__ inv, int r,
+                                                   double2* tmp) {
+  cg::cluster_group cluster = cg::this_cluster();
+  const int CC = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), cls = blockIdx.x / CC;
+  const int j0 = rank * r / CC, nj = (rank + 1) * r / CC - j0, n = 2 * r * nj;
+  double2* E = mats[slots[cls]];
+  double2* A = tmp + (size_t)cls * 2 * r * r;  // E R
+  double2* B = A + r * r;                      // R^H E R
+  grid_wait();
+  for (int e = threadIdx.x; e < n; e += blockDim.x) {
+    const int comp = e & 1, i = (e >> 1) / nj, j = j0 + (e >> 1) % nj;
+    double s = 0.0;
+    for (int k = 0; k < r; ++k) s = fma_part(E[i * r + k], R[k * r + j], comp, s);
+    reinterpret_cast<double*>(A + i * r + j)[comp] = s;
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < r * r; e += blockDim.x) {
-    const int i = e / r, j = e % r;
-    double2 s = make_double2(0.0, 0.0);
-    for (int k = 0; k < r; ++k) s = cadd(s, cmulc(R[k * r + i], A[k * r + j]));
-    B[e] = s;
+  for (int e = threadIdx.x; e < n; e += blockDim.x) {
+    const int comp = e & 1, i = (e >> 1) / nj, j = j0 + (e >> 1) % nj;
+    double s = 0.0;
+    for (int k = 0; k < r; ++k) s = fma_conj_part(R[k * r + i], A[k * r + j], comp, s);
+    reinterpret_cast<double*>(B + i * r + j)[comp] = s;
   }
-  __syncthreads();
-  for (int e = threadIdx.x; e < r * r; e += blockDim.x) {
-    const int i = e / r, j = e % r;
-    double2 s = make_double2(0.0, 0.0);
-    for (int k = 0; k < r; ++k) s = cadd(s, cmul(aug[i * w + r + k], B[k * r + j]));
-    E[e] = s;
+  grid_release();
+  cluster.sync();
+  for (int e = threadIdx.x; e < n; e += blockDim.x) {
+    const int comp = e & 1, i = (e >> 1) / nj, j = j0 + (e >> 1) % nj;
+    double s = 0.0;
+    for (int k = 0; k < r; ++k) s = fma_part(inv[i * r + k], B[k * r + j], comp, s);
+    reinterpret_cast<double*>(E + i * r + j)[comp] = s;
   }
 }
 
-// K (r x nc) += dmi (r x r) G (r x nc)
-__global__ void k_vmf_dmi(double2* __restrict__ K, const double2* __restrict__ G, const double2* __restrict__ dmi,
-                          int r, int64_t nc) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)r * nc;
+// K (r x nc) += sgn M (r x r) G (r x nc): dmi G_down added, X U taken off. One
+// thread per component and CTAs of two warps: at r = 12 (1728 elements) eight-warp
+// CTAs of one thread per element took 6.7 us, bound by the FP64 issue of the 7 SMs used.
+constexpr int kTs = 64;
+__global__ void __launch_bounds__(kTs) k_vmf_addmul(double2* __restrict__ K, const double2* __restrict__ G,
+                                                    const double2* __restrict__ M, double sgn, int r, int64_t nc) {
+  grid_wait();
+  grid_release();
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < 2 * (int64_t)r * nc;
        e += (int64_t)gridDim.x * blockDim.x) {
+    const int comp = (int)(e & 1);
     int64_t c;
-    const int a = (int)idivmod(e, nc, c);
-    double2 s = K[e];
-    for (int b = 0; b < r; ++b) s = cadd(s, cmul(dmi[a * r + b], G[(int64_t)b * nc + c]));
-    K[e] = s;
+    const int a = (int)idivmod(e >> 1, nc, c);
+    double s = 0.0;
+    for (int b = 0; b < r; ++b) s = fma_part(M[a * r + b], G[(int64_t)b * nc + c], comp, s);
+    double* k = reinterpret_cast<double*>(K) + e;
+    *k = fma(sgn, s, *k);
   }
 }
 
@@ -168,9 +193,11 @@ __global__ void k_vmf_px(const double2* __restrict__ K, const double2* __restric
                          double2* __restrict__ X) {
   __shared__ double2 red[kT / 32];
   const int a = blockIdx.x / r, b = blockIdx.x % r;
+  grid_wait();
   double2 s = make_double2(0.0, 0.0);
   for (int64_t c = threadIdx.x; c < nc; c += blockDim.x)
     s = cadd(s, cmulc(U[(int64_t)b * nc + c], K[(int64_t)a * nc + c]));
+  grid_release();
   for (int o = 16; o > 0; o >>= 1) {
     s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
     s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
@@ -184,20 +211,9 @@ __global__ void k_vmf_px(const double2* __restrict__ K, const double2* __restric
   }
 }
 
-// K[a][c] -= sum_b X[a][b] U[b][c]
-__global__ void k_vmf_psub(double2* __restrict__ K, const double2* __restrict__ U, const double2* __restrict__ X, int r,
-                           int64_t nc) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)r * nc;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    int64_t c;
-    const int a = (int)idivmod(e, nc, c);
-    double2 s = make_double2(0.0, 0.0);
-    for (int b = 0; b < r; ++b) s = cadd(s, cmul(X[a * r + b], U[(int64_t)b * nc + c]));
-    K[e] = make_double2(K[e].x - s.x, K[e].y - s.y);
-  }
-}
-
 __global__ void k_vmf_stage(double2* __restrict__ out, const double2* __restrict__ y, VmfComb cb, int64_t n) {
+  grid_wait();
+  grid_release();
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
     double2 s = y[e];
     for (int l = 0; l < cb.n; ++l) {
@@ -248,20 +264,29 @@ int grid_of(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n +
 
 void launch_vmf_edge(double2* const* mats_dev, const int* slots_dev, int n_classes, const double2* R, int r,
                      double eps, double2* aug, double2* dmi, double2* tmp, cudaStream_t s) {
-  k_vmf_rho<<<1, kT, 0, s>>>(R, r, eps, aug);
-  k_vmf_gj<<<1, kT, 0, s>>>(aug, r, dmi);
-  if (n_classes > 0) k_vmf_class<<<n_classes, kT, 0, s>>>(mats_dev, slots_dev, R, aug, r, tmp);
+  static bool attr = false;
+  if (!attr) {
+    cudaFuncSetAttribute(k_vmf_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)inv_smem(kGjSmemMaxR));
+    attr = true;
+  }
+  double2* inv = aug + 2 * (int64_t)r * r;
+  launch_dep(k_vmf_inv, dim3(1), dim3(kT), inv_smem(r), s, 0, R, r, eps, aug, inv, dmi);
+  const int cc = std::min(8, (r + 3) / 4);
+  if (n_classes > 0)
+    launch_dep(k_vmf_class, dim3((unsigned)(n_classes * cc)), dim3(128), 0, s, cc, mats_dev, slots_dev, R, inv, r, tmp);
 }
 
 void launch_vmf_finish(double2* K, const double2* Gdown, const double2* dmi, const double2* U, int r, int64_t nc,
                        double2* X, cudaStream_t s) {
-  k_vmf_dmi<<<grid_of((int64_t)r * nc), kT, 0, s>>>(K, Gdown, dmi, r, nc);
-  k_vmf_px<<<r * r, kT, 0, s>>>(K, U, r, nc, X);
-  k_vmf_psub<<<grid_of((int64_t)r * nc), kT, 0, s>>>(K, U, X, r, nc);
+  const int64_t n = 2 * (int64_t)r * nc;
+  const dim3 grid((unsigned)std::min<int64_t>((n + kTs - 1) / kTs, 8192));
+  launch_dep(k_vmf_addmul, grid, dim3(kTs), 0, s, 0, K, Gdown, dmi, 1.0, r, nc);
+  launch_dep(k_vmf_px, dim3(r * r), dim3(kT), 0, s, 0, K, U, r, nc, X);
+  launch_dep(k_vmf_addmul, grid, dim3(kTs), 0, s, 0, K, U, X, -1.0, r, nc);
 }
 
 void launch_vmf_stage(double2* out, const double2* y, const VmfComb& cb, int64_t n, cudaStream_t s) {
-  k_vmf_stage<<<grid_of(n), kT, 0, s>>>(out, y, cb, n);
+  launch_dep(k_vmf_stage, dim3(grid_of(n)), dim3(kT), 0, s, 0, out, y, cb, n);
 }
 
 void launch_vmf_err(const double2* y, const double2* y5, const VmfComb& cb, double rtol, double atol, int64_t n,
