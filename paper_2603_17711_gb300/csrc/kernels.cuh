@@ -186,7 +186,7 @@ int64_t tc_pool_floats(int d);
 void launch_tc_embed(void* const* mats32, const TcEmbedJob* jobs, int n, float* pool, cudaStream_t s);
 // FP64 lists on the tensor cores by an exact digit split (xs_apply.cu).
 // xs_applicable: the list qualifies (3 or 4 legs, contracted legs <= 64, all
-// outputs alike, work above kXsMinFlops). bufs / mats: host copies of the FP64
+// outputs alike, work above xs_min_flops). bufs / mats: host copies of the FP64
 // address tables (baked into the launch). planes: FP64 scratch of plane_elems
 // complex values (one-output lists: one plane per leg and term part, at most
 // max_split parts a leg). Returns
@@ -194,16 +194,26 @@ void launch_tc_embed(void* const* mats32, const TcEmbedJob* jobs, int n, float* 
 // The line: 19x11x11, 8 terms (2.1 MFLOP) 7.2 us on the CUDA cores, 10.4 here (the
 // second launch, the plane sum, is not won back); 16^3, 12 terms (6.3 MFLOP) 12.3 / 9.3;
 // 32x12x12, 12 terms (8.3 MFLOP) 15.8 / 12.0; 20^3, 12 terms (15 MFLOP) 22.9 / 12.9.
-// It lies above the crossing, at 8 MFLOP, and is the same for every max_split: runs
-// that differ only in the split of the CUDA-core launches then stay on one path,
-// and together through the rank events of a long trajectory.
-constexpr double kXsMinFlops = 8.0e6;
+// It lies above the crossing, at 8 MFLOP, and at 40 for nodes beside an open
+// or narrow leg (three legs, one of at most 16), whose gain is a few us a launch:
+// small trees are run at ranks far above the occupied ones, and there a
+// trajectory follows the rounding of the FMA chain (completion of dependent
+// columns): a spin-boson tree of rank 25, depth 11 parts by 5e-8 within 6 steps
+// between the two paths, both within 2e-16 of the exact sums; chains, Table 1
+// and two-site lists stay together to 1e-13. The line does not depend on max_split, so
+// runs that differ in it stay on one path.
+constexpr double kXsMinFlops = 8.0e6, kXsMinFlopsNarrow = 40.0e6;
+constexpr int kXsNarrow = 16;
+inline double xs_min_flops(int d0, int d1, int d2, int d3) {
+  const bool narrow = d0 <= kXsNarrow || d1 <= kXsNarrow || d2 <= kXsNarrow;
+  return d3 == 1 && narrow ? kXsMinFlopsNarrow : kXsMinFlops;
+}
 bool xs_applicable(const ApList& L, const ApOut* outs_host, const ApTerm* terms_host);
 bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L, const Epi& e,
                      const ApOut* outs_host, const ApTerm* terms_host, double2* planes, int64_t plane_elems,
                      int max_split, cudaStream_t s);
 // FP64 projections on the same path; false (nothing launched) below
-// kXsMinFlops or when the list does not qualify (all outputs alike, 8 <= bond
+// xs_min_flops or when the list does not qualify (all outputs alike, 8 <= bond
 // <= 64, at most 96 outputs).
 // Measured: 64-wide bond, 4096 positions, 5 classes 447 us (FP64 pipe) -> 172;
 // 56 classes' worth of the rank-64 chain's step 30.2 -> 9.9 ms.

@@ -647,7 +647,7 @@ bool xs_applicable(const ApList& L, const ApOut* outs, const ApTerm* terms) {
       if (!tm.pad) dense += 8.0 * P * dd[tm.leg];
     }
   }
-  return dense >= kXsMinFlops;
+  return dense >= xs_min_flops(f.d0, f.d1, f.d2, f.d3);
 }
 
 bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L, const Epi& e, const ApOut* outs,
@@ -761,8 +761,9 @@ bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L
 bool launch_project_xs(double2* const* bufs, double2* const* mats, const PjList& L, const PjOut* pjs, int max_split,
                        cudaStream_t s) {
   const int n = L.out_end - L.out_begin;
-  if (n < 1 || n > kXsMaxPj || L.flops < kXsMinFlops) return false;
+  if (n < 1 || n > kXsMaxPj) return false;
   const PjOut& f = pjs[L.out_begin];
+  if (L.flops < xs_min_flops(f.d0, f.d1, f.d2, 1)) return false;
   const int dd[3] = {f.d0, f.d1, f.d2}, d = dd[f.leg];
   const int64_t P = (int64_t)f.d0 * f.d1 * f.d2;
   if (d > kXsMaxD || d < 8 || P >= (int64_t)1 << 30) return false;
