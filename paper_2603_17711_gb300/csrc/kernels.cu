@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <cooperative_groups.h>
 #include <mutex>
+#include <type_traits>
 
 #include "kernels.cuh"
 
@@ -43,6 +44,10 @@ template <> struct Cx<double> {
   __device__ static T fma(T a, T b, T c) { return cfma(a, b, c); }
   __device__ static T fmaj(T a, T b, T c) { return cfma_conj(a, b, c); }
   __device__ static T add(T a, T b) { return cadd(a, b); }
+  // component comp (0 real, 1 imaginary) of fma(), the same operations in the same order
+  __device__ static double fma_part(T a, T b, int comp, double c) {
+    return ::fma(a.y, comp ? b.x : -b.y, ::fma(a.x, comp ? b.y : b.x, c));
+  }
   __device__ static double2 wide(T a) { return a; }
   __device__ static T narrow(double2 a) { return a; }
 };
@@ -88,6 +93,9 @@ template <> struct Cx<float> {
 // addition instead of a modulo per term, real and imaginary sums on two
 // sub-partitions, the stage update's state and accumulator loaded before the
 // sum, its step coefficient divided on the host. Same sums in the same order.
+// Small FP64 launches (CS) give an output two lanes, one component each: half a
+// tile per CTA, twice the CTAs, and half the FP64 instructions on a warp's
+// chain (8 a unit instead of 16, 64 cycles each), again the same sums.
 // Measured in the rank-10 spin-boson train: 8-CTA bond lists 5.0 -> 3.9 us,
 // 1-CTA lists 5.0 -> 3.6 us; rank-20 chain, 160-CTA lists 6.1 -> 4.6 us, 500-CTA
 // (FP64-issue bound) 20 -> 20 us.
@@ -149,14 +157,39 @@ __device__ __forceinline__ void geo_leg(const Geo& g, int leg, int& dl, int& il,
   }
 }
 
-// contribution of positions [x0, x0 + kApChunk) of one term (the whole term if
-// identity or sparse)
-template <typename R>
-__device__ __forceinline__ typename Cx<R>::T unit_dot(const ApTermV<typename Cx<R>::T>& term, int64_t idx, const Geo& g,
-                                                      int x0) {
+// What a lane sums: an output's complex value, or (CS) component comp of it.
+template <typename R, bool CS>
+struct LaneSum {
   using C = Cx<R>;
   using V = typename C::T;
-  if (!term.M) return term.X[idx];
+  using A = std::conditional_t<CS, R, V>;
+  __device__ static A zero() {
+    if constexpr (CS) return R(0);
+    else return C::zero();
+  }
+  __device__ static A add(A a, A b) {
+    if constexpr (CS) return a + b;
+    else return C::add(a, b);
+  }
+  __device__ static A fma(V a, V b, int comp, A c) {
+    if constexpr (CS) return C::fma_part(a, b, comp, c);
+    else return C::fma(a, b, c);
+  }
+  __device__ static A load(const V* p, int64_t i, int comp) {
+    if constexpr (CS) return reinterpret_cast<const R*>(p)[2 * i + comp];
+    else return p[i];
+  }
+};
+
+// contribution of positions [x0, x0 + kApChunk) of one term (the whole term if
+// identity or sparse)
+template <typename R, bool CS>
+__device__ __forceinline__ typename LaneSum<R, CS>::A unit_dot(const ApTermV<typename Cx<R>::T>& term, int64_t idx,
+                                                               const Geo& g, int x0, int comp) {
+  using C = Cx<R>;
+  using V = typename C::T;
+  using S = LaneSum<R, CS>;
+  if (!term.M) return S::load(term.X, idx, comp);
   int dl, il;
   int64_t stride;
   geo_leg(g, term.leg, dl, il, stride);
@@ -172,10 +205,10 @@ __device__ __forceinline__ typename Cx<R>::T unit_dot(const ApTermV<typename Cx<
       mv[k] = in ? row[x] : C::zero();
       sv[k] = in ? col[(int64_t)x * stride] : C::zero();
     }
-    V acc = C::zero();
+    typename S::A acc = S::zero();
 #pragma unroll
     for (int k = 0; k < 3; ++k)
-      if (k < nd) acc = C::fma(mv[k], sv[k], acc);
+      if (k < nd) acc = S::fma(mv[k], sv[k], comp, acc);
     return acc;
   }
 #pragma unroll
@@ -186,10 +219,10 @@ __device__ __forceinline__ typename Cx<R>::T unit_dot(const ApTermV<typename Cx<
       sv[k] = col[(int64_t)x * stride];
     }
   }
-  V acc = C::zero();
+  typename S::A acc = S::zero();
 #pragma unroll
   for (int k = 0; k < kApChunk; ++k)
-    if (x0 + k < dl) acc = C::fma(mv[k], sv[k], acc);
+    if (x0 + k < dl) acc = S::fma(mv[k], sv[k], comp, acc);
   return acc;
 }
 
@@ -197,30 +230,30 @@ __device__ __forceinline__ typename Cx<R>::T unit_dot(const ApTermV<typename Cx<
 // real parts, warp 1 the imaginary parts. An FP64 addition holds an SM
 // sub-partition for 64 cycles whatever the lane count, so the two components
 // on two sub-partitions take half the time of one warp adding complex values,
-// with the same sums; the epilogue follows the same split.
-template <typename R>
-__device__ __forceinline__ R comp_sum(const typename Cx<R>::T (*part)[32], int n) {
+// with the same sums; the epilogue follows the same split. Where the lanes hold
+// components already (CS), warp 0 does both.
+template <typename R, bool CS = false>
+__device__ __forceinline__ R comp_sum(const void* part, int n) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   R acc = R(0);
-  if (wid < 2) {
-    const R* p = reinterpret_cast<const R*>(part) + 2 * lane + wid;
+  if (wid < (CS ? 1 : 2)) {
+    const R* p = reinterpret_cast<const R*>(part) + (CS ? lane : 2 * lane + wid);
     acc = p[0];
-    for (int w = 1; w < n; ++w) acc += p[64 * w];
+    for (int w = 1; w < n; ++w) acc += p[(CS ? 32 : 64) * w];
   }
   return acc;
 }
 
 // Sum of one output tile over the units of CTA `rank` of the k sharing it;
 // the CTA's total (fixed order over warps) is returned in warps 0 (real part)
-// and 1 (imaginary part).
-template <typename R, int NW, typename TAB>
-__device__ __forceinline__ R tile_sum(const TAB& tab, const ApOutV<typename Cx<R>::T>& out, const Geo& g,
-                                                      int64_t idx, bool in, int rank, int K,
-                                                      typename Cx<R>::T (*part)[32]) {
-  using C = Cx<R>;
-  using V = typename C::T;
+// and 1 (imaginary part), or in warp 0 (CS).
+template <typename R, int NW, bool CS, typename TAB>
+__device__ __forceinline__ R tile_sum(const TAB& tab, const ApOutV<typename Cx<R>::T>& out, const Geo& g, int64_t idx,
+                                      int comp, bool in, int rank, int K, typename LaneSum<R, CS>::A (*part)[32]) {
+  using V = typename Cx<R>::T;
+  using S = LaneSum<R, CS>;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  V acc = C::zero();
+  typename S::A acc = S::zero();
   const int W = K * NW;
   int off = rank * NW + wid;  // this warp's first unit, relative to the current term's
   for (int t = out.tb; t < out.te; ++t) {
@@ -232,16 +265,15 @@ __device__ __forceinline__ R tile_sum(const TAB& tab, const ApOutV<typename Cx<R
     }
     int c = off;
     for (; c < nch; c += W)
-      if (in) acc = C::add(acc, unit_dot<R>(term, idx, g, c * kApChunk));
+      if (in) acc = S::add(acc, unit_dot<R, CS>(term, idx, g, c * kApChunk, comp));
     off = c - nch;
   }
   part[wid][lane] = acc;
   __syncthreads();
-  return comp_sum<R>(part, NW);
+  return comp_sum<R, CS>(part, NW);
 }
 
-// Epilogue of one component of one output element (warp `comp` of the CTA
-// owning the tile; at = 2 idx + comp); y0, a0: the state and the stage
+// Epilogue of one component of one output element (at = 2 idx + comp); y0, a0: the state and the stage
 // accumulator, loaded ahead of the sum.
 template <typename R>
 __device__ __forceinline__ void tile_store(R* dst, const Epi& ep, int64_t at, R acc, double y0, double a0) {
@@ -260,14 +292,15 @@ __device__ __forceinline__ void tile_store(R* dst, const Epi& ep, int64_t at, R 
   ((R*)ep.ys)[at] = (R)(y0 + ep.c * k);
 }
 
-template <typename R, int NW, typename TAB>
+template <typename R, int NW, bool CS, typename TAB>
 __global__ void __launch_bounds__(32 * NW, 32 / NW) k_apply(const __grid_constant__ TAB tab, ApList L, Epi ep) {
-  using C = Cx<R>;
-  using V = typename C::T;
-  __shared__ V part[NW][32];
-  __shared__ V slot[kMaxSplit][32];
+  using V = typename Cx<R>::T;
+  using A = typename LaneSum<R, CS>::A;
+  __shared__ A part[NW][32];
+  __shared__ A slot[kMaxSplit][32];
   const int K = L.k;
-  const int tile = blockIdx.x / K, rank = blockIdx.x % K;  // rank == block rank in the cluster
+  const int block = blockIdx.x / K, rank = blockIdx.x % K;  // rank == block rank in the cluster
+  const int tile = CS ? block >> 1 : block;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const ApOutV<V> out = tab.out(tab.find(L, tile));
   Geo g;
@@ -275,14 +308,17 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) k_apply(const __grid_constan
   g.s2 = g.d3;
   g.s1 = (int64_t)g.d2 * g.d3;
   g.s0 = g.s1 * g.d1;
-  const int64_t P = g.s0 * g.d0, idx = (int64_t)(tile - out.tile0) * kApTile + lane;
+  const int64_t P = g.s0 * g.d0, idx = (int64_t)(tile - out.tile0) * kApTile +
+                                    (CS ? (block & 1) * (kApTile / 2) + (lane >> 1) : lane);
   const bool in = idx < P;
+  const int comp = CS ? lane & 1 : wid & 1;  // of the lane's sum, or of the warp's share of the epilogue
+  const bool last = wid < (CS ? 1 : 2);      // warps that finish the tile
   g.i0 = g.i1 = g.i2 = g.i3 = 0;
-  const int64_t at = 2 * idx + (wid & 1);
+  const int64_t at = 2 * idx + comp;
   grid_wait();
   double y0 = 0.0, a0 = 0.0;
   if (in) {
-    if (ep.mode != EPI_STORE && wid < 2 && rank == 0) {
+    if (ep.mode != EPI_STORE && last && rank == 0) {
       y0 = ((const double*)ep.y)[at];
       if (ep.mode != EPI_RK1) a0 = ((const double*)ep.acc)[at];
     }
@@ -300,16 +336,18 @@ __global__ void __launch_bounds__(32 * NW, 32 / NW) k_apply(const __grid_constan
       g.i3 = (int)(idx % g.d3);
     }
   }
-  R acc = tile_sum<R, NW>(tab, out, g, idx, in, rank, K, part);
+  R acc = tile_sum<R, NW, CS>(tab, out, g, idx, comp, in, rank, K, part);
   grid_release();
   if (K > 1) {
     cg::cluster_group cluster = cg::this_cluster();
-    if (wid < 2) reinterpret_cast<R*>(cluster.map_shared_rank(&slot[0][0], 0))[rank * 64 + 2 * lane + wid] = acc;
+    if (last)
+      reinterpret_cast<R*>(cluster.map_shared_rank(&slot[0][0], 0))[CS ? rank * 32 + lane
+                                                                       : rank * 64 + 2 * lane + wid] = acc;
     cluster.sync();
     if (rank > 0) return;
-    acc = comp_sum<R>(slot, K);
+    acc = comp_sum<R, CS>(slot, K);
   }
-  if (wid > 1 || !in) return;
+  if (!last || !in) return;
   tile_store<R>(reinterpret_cast<R*>(out.dst), ep, at, acc, y0, a0);
 }
 
@@ -319,12 +357,23 @@ static void launch_split(Kern kern, int n_tiles, int k, int warps, cudaStream_t 
   launch_dep(kern, dim3((unsigned)(n_tiles * k)), dim3(32 * warps), 0, s, k > 1 ? k : 0, args...);
 }
 
+// CS: lists of at most half the SMs' number of CTAs, which still have an SM each
+// when doubled. Rank-10 train / rank-19 tree / Table 1 / FMO step: 10.27 / 17.83 / 14.39 /
+// 31.59 ms without, 9.97 / 17.62 / 14.23 / 31.41 up to 76 CTAs, 10.12 / 17.71 / 14.37 /
+// 31.41 up to 152, 10.11 / 18.38 / 14.46 / 31.52 up to 304 (the pipes are shared).
+constexpr int kCsMaxCtas = 76;
 template <typename R, typename TAB>
 static void launch_apply_w(const TAB& tab, const ApList& L, const Epi& e, cudaStream_t s) {
+  if constexpr (sizeof(R) == 8) {
+    if (L.w != 2 && L.w != 4 && L.n_tiles * L.k <= kCsMaxCtas) {
+      launch_split(k_apply<R, 8, true, TAB>, 2 * L.n_tiles, L.k, 8, s, tab, L, e);
+      return;
+    }
+  }
   switch (L.w) {
-    case 2: launch_split(k_apply<R, 2, TAB>, L.n_tiles, L.k, 2, s, tab, L, e); break;
-    case 4: launch_split(k_apply<R, 4, TAB>, L.n_tiles, L.k, 4, s, tab, L, e); break;
-    default: launch_split(k_apply<R, 8, TAB>, L.n_tiles, L.k, 8, s, tab, L, e); break;
+    case 2: launch_split(k_apply<R, 2, false, TAB>, L.n_tiles, L.k, 2, s, tab, L, e); break;
+    case 4: launch_split(k_apply<R, 4, false, TAB>, L.n_tiles, L.k, 4, s, tab, L, e); break;
+    default: launch_split(k_apply<R, 8, false, TAB>, L.n_tiles, L.k, 8, s, tab, L, e); break;
   }
 }
 
@@ -600,9 +649,10 @@ static void allow_wide(K kern) {
 }
 template <typename R, typename TAB>
 static void allow_wide_apply() {
-  allow_wide(k_apply<R, 8, TAB>);
-  allow_wide(k_apply<R, 4, TAB>);
-  allow_wide(k_apply<R, 2, TAB>);
+  allow_wide(k_apply<R, 8, false, TAB>);
+  allow_wide(k_apply<R, 4, false, TAB>);
+  allow_wide(k_apply<R, 2, false, TAB>);
+  if constexpr (sizeof(R) == 8) allow_wide(k_apply<R, 8, true, TAB>);
 }
 template <typename R>
 static void allow_wide_r() {
