@@ -286,7 +286,8 @@ ttn_status ttn_batch_step(ttn_t* hs, int32_t n, double dt, int32_t scheme, int32
  * stage update), 1 = environment update (mode products + projection),
  * 2 = Householder QR, 3 = everything else (absorb, copies, RDM, drive, checks).
  * ttn_stats: launches and algorithmic FLOPs issued since the last reset
- * (complex multiply-add = 8 FLOPs), counted on the host, always on. Kind 4
+ * (complex multiply-add = 8 FLOPs; an operator of at most three diagonals on a
+ * leg above 12 counts its entries), counted on the host, always on. Kind 4
  * (launches only) counts the job lists issued on the tensor-core ring path
  * (tensor_cores = 2), at issue time: a captured step graph counts once.
  * ttn_profile(h, 1) additionally brackets every launch with CUDA events on the
@@ -412,16 +413,16 @@ ttn_status ttn_tuning_set(ttn_t h, const int32_t* rows, int32_t n_rows, int32_t*
 
 /* Singular value decomposition a = U diag(sigma) V^H of a device matrix by
  * one-sided (Hestenes) Jacobi rotations in FP64: the factorisation the ps2
- * scheme uses to split a merged pair (Sec. 2.3, last paragraph), exposed for
- * callers and tests. a_dev: m x n complex, row-major (not modified); k =
+ * scheme uses to split a merged pair (Sec. 2.3, last paragraph; above 32 columns
+ * after a pivoted QR there), exposed for callers and tests. a_dev: m x n complex, row-major (not modified); k =
  * min(m, n). Outputs: u_dev m x k and vh_dev k x n (device, row-major), sigma_host
  * k values in descending order; singular vectors of sigma = 0 are returned as
  * zero. ws_dev: ttn_svd_workspace_size(m, n) bytes, 256-byte aligned. Matrices
  * whose smaller side has more than 16 columns run over several CTAs (the pairs
- * of each round of the circle ordering spread over the CTAs, one barrier per
- * round: a thread-block cluster's up to 32 columns, else a cooperative launch
- * over the whole GPU); every grid barrier wait is bounded by wait_s seconds
- * (0..60). *sweeps_out (nullable): sweeps that rotated.
+ * of each round of the circle ordering spread over the CTAs: up to 32 columns a
+ * thread-block cluster with one barrier per round, else a cooperative launch over
+ * the whole GPU with the columns handed over one by one and one barrier per sweep);
+ * every such wait is bounded by wait_s seconds (0..60). *sweeps_out (nullable): sweeps that rotated.
  * Synchronises `stream` (cudaStream_t as void*). Errors: TTN_EINVAL,
  * TTN_ENOMEM (workspace too small or misaligned), TTN_ETIMEOUT (a barrier
  * wait gave up; outputs undefined), TTN_ENUMERIC (no convergence within 60

@@ -220,7 +220,7 @@ __device__ __forceinline__ bool phase_sync(unsigned* lanes, unsigned target, uin
 // The two-site split of the rank-16 driven system (256 x 100 and 256 x 64), per
 // step of 14 splits: 148 ms with accumulated right vectors and one barrier a
 // round; 45 ms with R^H in place of the matrix, 41 with column hand-over and
-// the early last sweep, 40 with four warps a CTA.
+// the early last sweep, 40 with four warps a CTA, 37 with the pivoted QR's shorter sums.
 template <bool kCluster>
 __global__ void __launch_bounds__(kJThreads) k_jacobi_grid(double2* __restrict__ A, double2* __restrict__ V, int nr,
                                                           int nc_in, const int* nc_dev, double* __restrict__ sigma, int* __restrict__ info,
@@ -395,8 +395,8 @@ __global__ void __launch_bounds__(kJThreads) k_jacobi_grid(double2* __restrict__
 // grid barrier: every CTA publishes its largest remaining column and the norm,
 // then all pick the same pivot (ties: lower index), read that column from L2
 // and apply its reflector to their own columns. A step is a latency chain
-// (barrier, candidates, pivot column, scalars, dot, update) of about 5 us
-// whatever the size. *keff: the number of steps; it stops early when every
+// (barrier, candidates, pivot column, scalars, dot, update) of about 5.5 us
+// whatever the size (7.5 with the sums of three values over all warps). *keff: the number of steps; it stops early when every
 // remaining column is rounding noise of the matrix (jacobi_negligible).
 constexpr int kPivMaxCols = 8;  // columns per CTA
 constexpr int kPivSmem = 200 * 1024;
@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(kThreads) k_pivot_qr(const double2* __restrict
                                                        int* cand_i, double* fpart, int* keff, unsigned* sync, int* flag,
                                                        uint64_t wait_ns) {
   extern __shared__ double2 sm[];
-  __shared__ double s_nrm[kPivMaxCols], s_part[kWarps][3], s_sc[8];
+  __shared__ double s_nrm[kPivMaxCols], s_part1[kWarps], s_part2[kWarps][2], s_sc[8];
   __shared__ int s_done[kPivMaxCols], s_piv;
   __shared__ long long s_best;
   const int nb = iso_first ? n : m, ni = iso_first ? m : n;
@@ -419,31 +419,33 @@ __global__ void __launch_bounds__(kThreads) k_pivot_qr(const double2* __restrict
   const int my = wid / gs, gw = wid % gs;  // this warp's column and place in its group
   const bool on = my < ncl;
   double2* a = col + (size_t)my * nb;
-  auto group_sum = [&](double x, double y, double z, double& ox, double& oy, double& oz) {
-    // sums over the warps of a column, in order; block-uniform barriers
-    for (int o = 16; o > 0; o >>= 1) {
-      x += __shfl_xor_sync(0xffffffffu, x, o);
-      y += __shfl_xor_sync(0xffffffffu, y, o);
-      z += __shfl_xor_sync(0xffffffffu, z, o);
-    }
-    __syncthreads();
-    if (lane == 0) {
-      s_part[wid][0] = x;
-      s_part[wid][1] = y;
-      s_part[wid][2] = z;
-    }
-    __syncthreads();
-    const int w0 = (wid / gs) * gs;
-    ox = s_part[w0][0];
-    oy = s_part[w0][1];
-    oz = s_part[w0][2];
-    for (int w = w0 + 1; w < w0 + gs; ++w) {
-      ox += s_part[w][0];
-      oy += s_part[w][1];
-      oz += s_part[w][2];
-    }
+  // Sums over a column's lanes and warps (block-uniform barrier): of two values,
+  // left in every lane, lanes 0..15 carrying x and 16..31 y so that a step costs one
+  // FP64 addition; of one value, left in the column's first warp. Each has its own
+  // partials, so nothing has to be waited for before they are written. With three
+  // values in every lane and all warps adding the partials one by one, the two sums
+  // of a step took 9k cycles.
+  auto over_warps = [&](double t) {  // lane q of a half holds warp q's partial
+    for (int o = gs >> 1; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
   };
-  double nrm = 0.0, u1, u2;
+  auto group_sum2 = [&](double x, double y, double& ox, double& oy) {
+    const bool up = lane >= 16;
+    double t = (up ? y : x) + __shfl_xor_sync(0xffffffffu, up ? x : y, 16);
+    for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((lane & 15) == 0) s_part2[wid][lane >> 4] = t;
+    __syncthreads();
+    t = over_warps(s_part2[wid - gw + (lane & (gs - 1))][lane >> 4]);
+    ox = __shfl_sync(0xffffffffu, t, 0);
+    oy = __shfl_sync(0xffffffffu, t, 16);
+  };
+  auto group_sum1 = [&](double x) {
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if (lane == 0) s_part1[wid] = x;
+    __syncthreads();
+    return gw == 0 ? over_warps(s_part1[wid + (lane & (gs - 1))]) : 0.0;
+  };
+  double nrm = 0.0;
   {
     double f = 0.0;
     if (on) {
@@ -454,7 +456,7 @@ __global__ void __launch_bounds__(kThreads) k_pivot_qr(const double2* __restrict
         f = fma(t.x, t.x, fma(t.y, t.y, f));
       }
     }
-    group_sum(f, 0.0, 0.0, nrm, u1, u2);
+    nrm = group_sum1(f);
     if (on && gw == 0 && lane == 0) {
       s_nrm[my] = nrm;
       s_done[my] = 0;
@@ -490,7 +492,8 @@ __global__ void __launch_bounds__(kThreads) k_pivot_qr(const double2* __restrict
     if (!grid_sync(sync, nbar * (unsigned)G, wait_ns, flag)) return;
     if (c == 0) {
       double f = 0.0;
-      for (int q = 0; q < G; ++q) f += __ldcg(fpart + q);
+      for (int q = lane; q < G; q += 32) f += __ldcg(fpart + q);
+      f = wsum(f);
       tiny2 = jacobi_negligible(max(nb, ni), f);
       if (!isfinite(f)) {  // nothing to factor: report it, no columns (uniform over the grid)
         if (blockIdx.x == 0 && tid == 0) atomicOr(flag, 1);
@@ -556,8 +559,8 @@ __global__ void __launch_bounds__(kThreads) k_pivot_qr(const double2* __restrict
         wr = fma(x.x, y.x, fma(x.y, y.y, wr));
         wi = fma(x.x, y.y, fma(-x.y, y.x, wi));
       }
-    double sr, si, sn;
-    group_sum(wr, wi, 0.0, sr, si, sn);
+    double sr, si;
+    group_sum2(wr, wi, sr, si);
     const double beta = s_sc[2];
     sr *= beta;
     si *= beta;
@@ -571,7 +574,7 @@ __global__ void __launch_bounds__(kThreads) k_pivot_qr(const double2* __restrict
         a[r] = y;
         if (r > c) f = fma(y.x, y.x, fma(y.y, y.y, f));
       }
-    group_sum(f, 0.0, 0.0, nrm, u1, u2);
+    nrm = group_sum1(f);
     if (on && gw == 0 && lane == 0) {
       const int i = blockIdx.x + my * G;
       double2 t = make_double2(0.0, 0.0);  // a column finished earlier has no entry in this row of R
