@@ -396,8 +396,9 @@ __global__ void __launch_bounds__(kJThreads) k_jacobi_grid(double2* __restrict__
 // then all pick the same pivot (ties: lower index), read that column from L2
 // and apply its reflector to their own columns. A step is a latency chain
 // (barrier, candidates, pivot column, scalars, dot, update) of about 5.5 us
-// whatever the size (7.5 with the sums of three values over all warps). *keff: the number of steps; it stops early when every
-// remaining column is rounding noise of the matrix (jacobi_negligible).
+// whatever the size (7.5 with the sums of three values over all warps). *keff: the
+// number of steps; it stops early when every remaining column is rounding noise
+// of the matrix (jacobi_negligible).
 constexpr int kPivMaxCols = 8;  // columns per CTA
 constexpr int kPivSmem = 200 * 1024;
 __global__ void __launch_bounds__(kThreads) k_pivot_qr(const double2* __restrict__ theta, int m, int n, int iso_first,

@@ -106,3 +106,22 @@ def test_direct_integration_matches_the_oracle(pkg, rank, depth, K, tree):
     for u in range(g.n_nodes):
         assert np.max(np.abs(g.ttn_get_node(u) - o.tensors[u])) <= 1e-10, u
     g.close()
+
+
+@pytest.mark.parametrize("make", STEPS[1:5:3])
+def test_overlapped_launches_on_the_default_stream(pkg, make):
+    """Launch by launch on the legacy default stream, as a graph on a stream of its
+    own, and launch by launch there: the same bits (every kernel waits for the one before)."""
+    import torch
+    w = make()
+    out = []
+    for stream, prof in ((torch.cuda.default_stream(), 0), (None, 0), (None, 1)):
+        g = pkg.from_model(w.H, w.baths, w.depth, w.parent, w.leg_node, w.ranks, rho0=w.rho0, drives=w.drives,
+                           stream=stream)
+        g.ttn_profile(prof)
+        g.ttn_step(w.dt, pkg.TTN_PS1, 5)
+        out.append([g.ttn_rdm()] + [g.ttn_get_node(u) for u in range(g.n_nodes)])
+        g.close()
+    for other in out[1:]:
+        for a, b in zip(out[0], other):
+            assert np.array_equal(a, b)
