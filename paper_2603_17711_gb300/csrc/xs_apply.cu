@@ -693,7 +693,8 @@ bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L
     // (two are resident at a time)
     int ctas = 0, n_planes = 0, groups[4];
     for (int l = 0; l < 4; ++l) {
-      groups[l] = kXsWarps / ((dd[l] + 7) / 8);
+      // a leg without a dense term may be of any size, also above the kXsWarps row blocks of a CTA
+      groups[l] = nterm[l] ? kXsWarps / ((dd[l] + 7) / 8) : 0;
       gr.parts[l] = 1;
       if (nterm[l]) {
         ctas += tiles[l];
@@ -705,6 +706,7 @@ bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L
       int best = -1;
       double chain = 1.0;
       for (int l = 0; l < 4; ++l) {
+        if (!nterm[l]) continue;
         const int q = groups[l] * gr.parts[l];
         const double c = (double)((nterm[l] + q - 1) / q) * ((dd[l] + 7) / 8);
         if (nterm[l] > q && gr.parts[l] < max_split && c > chain) {

@@ -1,0 +1,52 @@
+"""Which FP64 job lists go to the tensor cores, and that the launcher's host part
+serves every list it is offered -- on the plans of real models, without a GPU."""
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import workloads as W
+from paper_2603_17711_gb300 import build, heom
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def harness(tmp_path_factory):
+    return compile_harness(tmp_path_factory.mktemp("harness"))
+
+
+def compile_harness(out_dir):
+    """The planner and the launcher with the harness, an integer division by zero made fatal on every host."""
+    exe = os.path.join(str(out_dir), "lists_harness")
+    src = [os.path.join(HERE, "lists_harness.cu")] + [os.path.join(build.CSRC, f) for f in ("plan.cpp", "xs_apply.cu")]
+    subprocess.run([build._nvcc(), *build.ARCH, "-O1", "-std=c++17", "-I", build.CSRC, "-Xcompiler",
+                    "-fsanitize=integer-divide-by-zero,-fno-sanitize-recover=integer-divide-by-zero", *src, "-lubsan", "-o", exe],
+                   check=True, capture_output=True)
+    return exe
+
+
+def lists(exe, w, max_split=16):
+    """Rows (applicable, launched, outputs, terms, d0, d1, d2, d3) of the model's lists."""
+    a = heom.heom_sop(w.H, w.baths, w.depth, w.drives)
+    nums = []
+    for x in (len(w.parent), w.parent, len(w.leg_node), w.leg_node, w.leg_dims, w.ranks, len(a["op_leg"]), a["op_leg"],
+              len(a["op_data"]), a["op_offset"], a["op_data"], len(a["term_offsets"]) - 1, a["term_offsets"],
+              len(a["term_ops"]), a["term_ops"], a["coef"], a["coef_drive"], max_split):
+        nums += [repr(float(v)) if isinstance(v, (float, np.floating)) else str(int(v)) for v in np.ravel(x)]
+    r = subprocess.run([exe, "lists"], input=" ".join(nums), capture_output=True, text=True,
+                       env={**os.environ, "CUDA_VISIBLE_DEVICES": ""})
+    assert r.returncode == 0, (r.returncode, r.stderr)
+    return np.array([[int(v) for v in line.split()] for line in r.stdout.splitlines()])
+
+
+@pytest.mark.parametrize("make", [
+    lambda: W.spin_boson_tt(rank=72, depth=8, n_pade=7, tree="btt"),  # nodes 72 x 64 x 64, terms on legs 1 and 2
+    lambda: W.exciton_chain(n_sites=3, rank=80, depth=9),
+    lambda: W.exciton_chain(n_sites=7, rank=64),
+])
+def test_a_leg_above_the_limit_that_carries_no_term(harness, make):
+    """Legs without a term do not limit the list, and their size divides nothing."""
+    r = lists(harness, make())
+    assert r[:, 0].any() and np.array_equal(r[:, 0], r[:, 1])
