@@ -186,11 +186,12 @@ int64_t tc_pool_floats(int d);
 void launch_tc_embed(void* const* mats32, const TcEmbedJob* jobs, int n, float* pool, cudaStream_t s);
 // FP64 lists on the tensor cores by an exact digit split (xs_apply.cu).
 // xs_applicable: the list qualifies (3 or 4 legs, contracted legs <= 64, all
-// outputs alike, work above xs_min_flops). bufs / mats: host copies of the FP64
+// outputs alike, at most 96 of them and 192 terms, work above xs_min_flops).
+// launch_apply_xs takes only lists that qualify. bufs / mats: host copies of the FP64
 // address tables (baked into the launch). planes: FP64 scratch of plane_elems
 // complex values (one-output lists: one plane per leg and term part, at most
 // max_split parts a leg). Returns
-// false (nothing launched) when the scratch or the launch's tables are too small.
+// false (nothing launched) when the scratch is too small.
 // The line: 19x11x11, 8 terms (2.1 MFLOP) 7.2 us on the CUDA cores, 10.4 here (the
 // second launch, the plane sum, is not won back); 16^3, 12 terms (6.3 MFLOP) 12.3 / 9.3;
 // 32x12x12, 12 terms (8.3 MFLOP) 15.8 / 12.0; 20^3, 12 terms (15 MFLOP) 22.9 / 12.9.

@@ -628,14 +628,17 @@ int sm_count() {
 }  // namespace
 
 // Lists that take this path: contracted legs of at most 64, all outputs alike,
-// fewer than 2^31 elements, and enough multiply-adds that the CUDA-core kernel
+// fewer than 2^30 elements an output, no more outputs and terms than a launch
+// has room for (everything else stays on the CUDA-core kernel and its tile
+// shapes, so ttn_autotune asks here too), and enough multiply-adds that the CUDA-core kernel
 // would be bound by FP64 issue instead of by its launch.
 bool xs_applicable(const ApList& L, const ApOut* outs, const ApTerm* terms) {
   if (L.n_tiles <= 0) return false;
   const ApOut& f = outs[L.out_begin];
   const int64_t P = (int64_t)f.d0 * f.d1 * f.d2 * f.d3;
   double dense = 0.0;  // sparse operators are cheap on the CUDA cores
-  if (P >= (int64_t)1 << 30 || L.out_end - L.out_begin > 65535) return false;
+  if (P >= (int64_t)1 << 30 || L.out_end - L.out_begin > kXsMaxOuts) return false;
+  if (outs[L.out_end - 1].term_end - f.term_begin > kXsMaxTerms) return false;
   for (int o = L.out_begin; o < L.out_end; ++o) {
     const ApOut& u = outs[o];
     if (u.d0 != f.d0 || u.d1 != f.d1 || u.d2 != f.d2 || u.d3 != f.d3) return false;
@@ -668,7 +671,6 @@ bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L
   for (int l = 0; l < 4; ++l) tiles[l] = (int)((P / dd[l] + kXsCols - 1) / kXsCols);
   XsWork gr{};
   XsSparse sp{};
-  if (n_outs > kXsMaxOuts || outs[L.out_end - 1].term_end - outs[L.out_begin].term_begin > kXsMaxTerms) return false;
   int nq = 0;
   for (int i = 0; i < 4; ++i) gr.dims[i] = sp.dims[i] = dd[i];
   for (int o = 0; o < n_outs; ++o) {

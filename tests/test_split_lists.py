@@ -50,3 +50,11 @@ def test_a_leg_above_the_limit_that_carries_no_term(harness, make):
     """Legs without a term do not limit the list, and their size divides nothing."""
     r = lists(harness, make())
     assert r[:, 0].any() and np.array_equal(r[:, 0], r[:, 1])
+
+
+def test_lists_too_long_for_a_launch_are_not_claimed(harness):
+    """More than 96 outputs: the list stays with the CUDA-core kernel from the
+    start, so the autotuner still finds its tile shape."""
+    r = lists(harness, W.exciton_chain(n_sites=60, rank=24, depth=4, n_pade=0))
+    assert r[:, 2].max() > 96 and r[:, 0].any()
+    assert np.array_equal(r[:, 0], r[:, 1])
