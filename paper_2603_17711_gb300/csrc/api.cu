@@ -235,6 +235,7 @@ struct Layout {
   std::vector<int64_t> tc_off_host;  // float offset of each matrix in tc_pool, -1 if none
   size_t svd_cand = 0, svd_small = 0, rsvd = 0, mlp = 0, xs = 0;
   int64_t xs_elems = 0;
+  bool xs_in_svd = false;
   // direct integration (vmf): committed state, per-node saves, 7 stage
   // derivatives (all as flat copies of the node region), edge scratch
   size_t vmf_y = 0, vmf_save = 0, vmf_k = 0, vmf_tmp = 0, vmf_r = 0, vmf_aug = 0, vmf_dmi = 0, vmf_x = 0,
@@ -300,10 +301,14 @@ Layout layout_of(const Plan& p, int prec) {
   L.rsvd = take(3 * p.theta_cap * sizeof(double2));
   L.mlp = take((24 + 13 + mlp_ws_floats(1) + 8) * sizeof(float) + 2 * sizeof(double));
   L.flag = take(sizeof(int) * 4);
-  // one plane per leg always fits; small nodes may cut their terms into more
-  L.xs_elems = std::max<int64_t>(4 * S, std::min<int64_t>(24 * p.P_cap_max, 1 << 20));
-  L.xs = take(L.xs_elems * sizeof(double2));
   if (prec == PREC_F64) {
+    // planes of the digit split (FP64 contractions only): one per leg always
+    // fits, small nodes may cut their terms into more. They take the two-site
+    // split's five matrices, which no contraction list overlaps, where those are
+    // large enough (every tree of two nodes or more at any but the smallest sizes)
+    L.xs_elems = std::max<int64_t>(4 * S, std::min<int64_t>(24 * p.P_cap_max, 1 << 20));
+    L.xs_in_svd = L.xs_elems <= 5 * p.theta_cap;
+    if (!L.xs_in_svd) L.xs = take(L.xs_elems * sizeof(double2));
     L.nodes_elems = acc;
     L.vmf_y = take(acc * sizeof(double2));
     L.vmf_save = take(acc * sizeof(double2));
@@ -1241,10 +1246,10 @@ ttn_status ttn_set_workspace(ttn_t h, void* dptr, size_t bytes) {
     h->rdm_off = L.rdm_off;
     h->rho_dev = (double2*)(base + L.rho);
     h->flag_dev = (int*)(base + L.flag);
-    h->xs_planes = (double2*)(base + L.xs);
-    h->xs_elems = L.xs_elems;
     h->node_off = L.node_off;
     if (h->prec == PREC_F64) {
+      h->xs_planes = L.xs_in_svd ? h->svd_A : (double2*)(base + L.xs);
+      h->xs_elems = L.xs_elems;
       h->vmf_n = L.nodes_elems;
       h->vmf_y = (double2*)(base + L.vmf_y);
       h->vmf_save = (double2*)(base + L.vmf_save);

@@ -58,3 +58,33 @@ def test_lists_too_long_for_a_launch_are_not_claimed(harness):
     r = lists(harness, W.exciton_chain(n_sites=60, rank=24, depth=4, n_pade=0))
     assert r[:, 2].max() > 96 and r[:, 0].any()
     assert np.array_equal(r[:, 0], r[:, 1])
+
+
+def workspace_bytes(w, precision):
+    import ctypes as C
+
+    from paper_2603_17711_gb300 import _lib
+    build.build()
+    lib = _lib.load()
+    par, ln = _lib.as_i32(w.parent), _lib.as_i32(w.leg_node)
+    tree = _lib.ttn_tree(len(par), _lib.ptr(par, C.c_int32), len(ln), _lib.ptr(ln, C.c_int32))
+    h, n = C.c_void_p(), C.c_size_t()
+    assert lib.ttn_create(C.byref(tree), _lib.ptr(_lib.as_i32(w.leg_dims), C.c_int32),
+                          _lib.ptr(_lib.as_i32(w.ranks), C.c_int32), precision, C.byref(h)) == 0
+    a = heom.heom_sop(w.H, w.baths, w.depth)
+    assert lib.sop_load(h, len(a["op_leg"]), _lib.ptr(a["op_leg"], C.c_int32), _lib.ptr(a["op_offset"], C.c_int64),
+                        _lib.ptr(a["op_data"], C.c_double), len(a["term_offsets"]) - 1,
+                        _lib.ptr(a["term_offsets"], C.c_int32), _lib.ptr(a["term_ops"], C.c_int32),
+                        _lib.ptr(a["coef"], C.c_double), _lib.ptr(a["coef_drive"], C.c_int32)) == 0
+    assert lib.ttn_workspace_size(h, C.byref(n)) == 0
+    lib.ttn_destroy(h)
+    return n.value
+
+
+@pytest.mark.parametrize("rank,precision,before", [
+    (20, 0, 902682880), (20, 1, 1223671808), (64, 0, 13959593728), (64, 1, 19299940096)])
+def test_workspace_without_room_for_planes(rank, precision, before):
+    """The mixed form has no digit split and the FP64 form keeps its planes in the
+    two-site split's matrices: `before`, the bytes without either, plus the split's
+    column counters and pivot candidates (below 32 KiB)."""
+    assert workspace_bytes(W.exciton_chain(rank=rank), precision) - before <= 32 << 10
