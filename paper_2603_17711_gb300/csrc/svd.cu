@@ -59,7 +59,8 @@ constexpr int kJWarps = kJThreads / 32;
 constexpr int kBarLanes = 8;
 constexpr int kVerOff = 128;  // first column counter in the sync words
 constexpr int kSvdMaxVer = kSvdSyncInts - kVerOff;
-static_assert(kBarLanes + kJacMaxSweeps <= kVerOff, "sweep counters fit before the column counters");
+constexpr int kSmallOff = kBarLanes + kJacMaxSweeps;  // first counter of small rotations
+static_assert(kSmallOff + kJacMaxSweeps <= kVerOff, "sweep counters fit before the column counters");
 
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
   return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -206,8 +207,8 @@ __device__ __forceinline__ bool phase_sync(unsigned* lanes, unsigned target, uin
   }
 }
 
-// sync: [0, 8) barrier lanes, [8, 8 + max_sweeps) rotations per sweep, then the columns' rounds; zeroed
-// before the launch. kCluster: the CTAs form one thread-block cluster. V may be
+// sync: [0, 8) barrier lanes, [8, 8 + max_sweeps) rotations per sweep that ask for another one, as many
+// counters of the small ones, then the columns' rounds; zeroed before the launch. kCluster: the CTAs form one thread-block cluster. V may be
 // null (no right vectors). nc_dev (nullable): the column count, at most nc,
 // found on the device; columns beyond it are zero.
 //
@@ -265,7 +266,7 @@ __global__ void __launch_bounds__(kJThreads) k_jacobi_grid(double2* __restrict__
   int sweep = 0;
   unsigned round = 0;  // rounds done, over all sweeps
   for (; sweep < max_sweeps; ++sweep) {
-    unsigned rot = 0;
+    unsigned rot = 0, small = 0;
     for (int rd = 0; rd < N - 1 && ok; ++rd) {
       for (int p = blockIdx.x; p < npairs; p += G) {
         int i, j;
@@ -340,6 +341,7 @@ __global__ void __launch_bounds__(kJThreads) k_jacobi_grid(double2* __restrict__
           }
         }
         rot += go == 2;
+        small += go == 1;
         if (p2p) {
           __syncthreads();  // the pair's columns are written
           if (tid < 2) st_release(ver + (tid == 0 ? i : j), round + 1);
@@ -349,6 +351,7 @@ __global__ void __launch_bounds__(kJThreads) k_jacobi_grid(double2* __restrict__
       if (!ok) break;
       // the sweep's count of rotations that ask for another sweep is published before its last barrier
       if (rd == N - 2 && tid == 0 && rot > 0) atomicAdd(sync + kBarLanes + sweep, rot);
+      if (rd == N - 2 && tid == 0 && small > 0) atomicAdd(sync + kSmallOff + sweep, small);
       if (p2p && rd < N - 2) continue;
       ++nbar;
       ok = phase_sync<kCluster>(sync, nbar * (unsigned)G, wait_ns, flag);
@@ -356,7 +359,10 @@ __global__ void __launch_bounds__(kJThreads) k_jacobi_grid(double2* __restrict__
     if (!ok) break;
     if (tid == 0) s_total = ld_acquire(sync + kBarLanes + sweep);
     __syncthreads();
-    if (s_total == 0) break;
+    if (s_total == 0) {
+      if (ld_acquire(sync + kSmallOff + sweep) > 0) ++sweep;  // the last sweep rotated too
+      break;
+    }
   }
   if (!ok) return;
   // sigma_j = |column j|, fixed-order sums; columns dealt round-robin to CTAs
