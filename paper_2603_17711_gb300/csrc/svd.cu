@@ -360,7 +360,8 @@ __global__ void __launch_bounds__(kJThreads) k_jacobi_grid(double2* __restrict__
     if (tid == 0) s_total = ld_acquire(sync + kBarLanes + sweep);
     __syncthreads();
     if (s_total == 0) {
-      if (ld_acquire(sync + kSmallOff + sweep) > 0) ++sweep;  // the last sweep rotated too
+      // the last sweep rotated too (max_sweeps itself says that the iteration did not end)
+      if (ld_acquire(sync + kSmallOff + sweep) > 0 && sweep + 1 < max_sweeps) ++sweep;
       break;
     }
   }
