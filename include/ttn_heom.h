@@ -287,10 +287,13 @@ ttn_status ttn_batch_step(ttn_t* hs, int32_t n, double dt, int32_t scheme, int32
  * 2 = Householder QR, 3 = everything else (absorb, copies, RDM, drive, checks).
  * ttn_stats: launches and algorithmic FLOPs issued since the last reset
  * (complex multiply-add = 8 FLOPs; an operator of at most three diagonals on a
- * leg above 12 counts its entries), counted on the host, always on. Kind 4
+ * leg above 12 counts its entries; a two-site split counts the rotations of a
+ * Jacobi SVD with right vectors over the sweeps run, also where it takes the
+ * pivoted route, which rotates none), counted on the host, always on: one job may
+ * be several launches, and FLOPs are of the mathematical operation, whichever unit does it. Kind 4
  * (launches only) counts the job lists issued on the tensor-core ring path
  * (tensor_cores = 2), at issue time: a captured step graph counts once.
- * ttn_profile(h, 1) additionally brackets every launch with CUDA events on the
+ * ttn_profile(h, 1) additionally brackets every job with CUDA events on the
  * handle's stream (the step is then issued launch by launch, not as a graph);
  * ttn_profile(h, 2) keeps the captured step graph and records the bracketing
  * events as event-record nodes inside it, so the times are those of the

@@ -389,13 +389,17 @@ struct Exec {
     return HostTables{h->h_bufs_lo.data(), h->h_mats_lo.data(), p.ap_outs.data(), p.ap_terms.data(), p.pj_outs.data()};
   }
 
-  // account one kernel launch of class `kind` and, when profiling, bracket it
-  // with CUDA events on the handle's stream
+  // account the kernel launches of one job of class `kind` and, when profiling,
+  // bracket them with CUDA events on the handle's stream
   template <typename F>
   void run(int kind, double flops, F&& launch) {
     if (err != cudaSuccess || fail_st != TTN_OK) return;  // a failed step launches nothing more
-    h->n_launch[kind] += 1;
     h->n_flops[kind] += flops;
+    struct Count {
+      int64_t& n;
+      const int64_t n0 = t_launched;
+      ~Count() { n += t_launched - n0; }
+    } count{h->n_launch[kind]};
     if (h->prof_mode == 0) {
       launch();
       return;
@@ -638,6 +642,7 @@ struct Exec {
                              " two-site matrix did not converge in " + std::to_string(kJacMaxSweeps) + " sweeps");
       return false;
     }
+    // nominal: Jacobi with right vectors over the sweeps run, also where the pivoted route rotates none
     const int nr = std::max(m, n);
     h->n_flops[2] += 8.0 * 4.0 * info[0] * 0.5 * nc * (nc - 1) * (double)(nr + nc);
     return true;

@@ -836,7 +836,7 @@ void launch_qr(double2* U, int d0, int d1, int d2, int leg, double tol, double2*
   if (launch_qr_cluster(U, d0, d1, d2, leg, tol, R, flag, U_lo, R_lo, work, work_elems, s)) return;
   if (launch_qr_blocked(U, d0, d1, d2, leg, tol, work, work_elems, qbuf, R, flag, U_lo, R_lo, s, grid_wait_ns))
     return;
-  k_qr<<<1, kQrThreads, 0, s>>>(U, d0, d1, d2, leg, tol, work, qbuf, R, flag, U_lo, R_lo);
+  k_qr<<<counted(1), kQrThreads, 0, s>>>(U, d0, d1, d2, leg, tol, work, qbuf, R, flag, U_lo, R_lo);
 }
 
 __global__ void k_copy(double2* dst, float2* dst_lo, const double2* src, int64_t n) {
@@ -948,7 +948,7 @@ __global__ void k_drive(double2* const* mats, float2* const* mats32, const Drive
 void launch_drive(double2* const* mats_dev, float2* const* mats32, const DriveMat* list, int n,
                   const DriveArgs& g, cudaStream_t s) {
   if (n <= 0) return;
-  k_drive<<<n, 128, 0, s>>>(mats_dev, mats32, list, n, g);
+  k_drive<<<counted(n), 128, 0, s>>>(mats_dev, mats32, list, n, g);
 }
 
 __global__ void k_check_finite(const double2* x, int64_t n, int* flag) {
@@ -959,7 +959,7 @@ __global__ void k_check_finite(const double2* x, int64_t n, int* flag) {
 }
 void launch_check_finite(const double2* x, int64_t n, int* flag, cudaStream_t s) {
   int blocks = (int)std::min<int64_t>((n + 255) / 256, 64);
-  k_check_finite<<<blocks, 256, 0, s>>>(x, n, flag);
+  k_check_finite<<<counted(blocks), 256, 0, s>>>(x, n, flag);
 }
 
 }  // namespace ttn

@@ -14,6 +14,13 @@ namespace ttn {
 // both modes; PREC_F32 runs the contractions in FP32 on FP32 shadow copies.
 enum Prec : int { PREC_F64 = 0, PREC_F32 = 1 };
 
+// Kernels launched by this thread: every grid of a launch passes through counted().
+inline thread_local int64_t t_launched = 0;
+inline dim3 counted(dim3 grid) {
+  ++t_launched;
+  return grid;
+}
+
 // Programmatic dependent launch. The kernels of a step form one chain of short
 // launches. launch_dep lets a launch start its CTAs while the previous kernel of
 // the stream still runs; such a kernel calls grid_wait() before it touches global
@@ -46,7 +53,7 @@ inline cudaError_t launch_dep(void (*kern)(P...), dim3 grid, dim3 block, size_t 
   at[1].val.clusterDim.y = 1;
   at[1].val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
+  cfg.gridDim = counted(grid);
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;

@@ -149,7 +149,7 @@ __global__ void k_adam(float* P, float* M, float* V, const float* G, int n, floa
 void launch_mlp_forward(const float* P, const float* x, int B, float* ws, float* logits, cudaStream_t s) {
   float* h1 = ws;
   float* h2 = h1 + (size_t)B * kH;
-  k_mlp_fwd<<<(B + kSamplesPerCta - 1) / kSamplesPerCta, 256, 0, s>>>(P, x, B, h1, h2, logits);
+  k_mlp_fwd<<<counted((B + kSamplesPerCta - 1) / kSamplesPerCta), 256, 0, s>>>(P, x, B, h1, h2, logits);
 }
 
 // ---------------------------------------------------------------------------
@@ -175,7 +175,7 @@ __global__ void k_gauss(double2* O, int64_t n, uint64_t seed) {
   }
 }
 void launch_gauss(double2* O, int64_t n, uint64_t seed, cudaStream_t s) {
-  k_gauss<<<(int)std::min<int64_t>((n + 255) / 256, 1024), 256, 0, s>>>(O, n, seed);
+  k_gauss<<<counted((int)std::min<int64_t>((n + 255) / 256, 1024)), 256, 0, s>>>(O, n, seed);
 }
 
 // C (M x N, row-major) = op(A) op(B); A is M x K (conjA: A given as K x M, use A^H),
@@ -197,7 +197,7 @@ __global__ void k_zgemm(const double2* A, const double2* Bm, double2* Cm, int M,
 }
 void launch_zgemm(const double2* A, const double2* B, double2* C, int M, int N, int K, bool conjA, cudaStream_t s) {
   const int64_t tot = (int64_t)M * N;
-  k_zgemm<<<(int)std::min<int64_t>((tot + 127) / 128, 4096), 128, 0, s>>>(A, B, C, M, N, K, conjA ? 1 : 0);
+  k_zgemm<<<counted((int)std::min<int64_t>((tot + 127) / 128, 4096)), 128, 0, s>>>(A, B, C, M, N, K, conjA ? 1 : 0);
 }
 
 // ||x||_2^2 in one block, fixed order
@@ -214,7 +214,7 @@ __global__ void k_norm2(const double2* x, int64_t n, double* out) {
     *out = t;
   }
 }
-void launch_norm2(const double2* x, int64_t n, double* out, cudaStream_t s) { k_norm2<<<1, 512, 0, s>>>(x, n, out); }
+void launch_norm2(const double2* x, int64_t n, double* out, cudaStream_t s) { k_norm2<<<counted(1), 512, 0, s>>>(x, n, out); }
 
 // Z / Cm of the randomised split. Theta ~ Q B, B (k x n) = Lb diag(sigma) Rb^H from
 // the Jacobi SVD of B (computed on B^H when n > k: Lb = V (k x k), Rb_j = A_j / sigma_j).
@@ -276,7 +276,7 @@ void launch_rsvd_vecs(const double2* Q, int m, int kk, const double2* A, const d
                       const int* perm, int r, int g, bool iso_first, double2* Z, double2* Zg, double2* Cm,
                       cudaStream_t s) {
   const int64_t tot = (int64_t)(m + n) * r;
-  k_rsvd_vecs<<<(int)std::min<int64_t>((tot + 127) / 128, 2048), 128, 0, s>>>(Q, m, kk, A, V, sigma, n, perm, r, g,
+  k_rsvd_vecs<<<counted((int)std::min<int64_t>((tot + 127) / 128, 2048)), 128, 0, s>>>(Q, m, kk, A, V, sigma, n, perm, r, g,
                                                                            iso_first ? 1 : 0, Z, Zg, Cm);
 }
 
@@ -319,16 +319,16 @@ ttn_status ttn_mlp_grad(const float* params, const float* x, const int32_t* labe
   float* d1 = d2 + (size_t)B * kH;
   float* lb = d1 + (size_t)B * kH;
   const int nb = (B + kSamplesPerCta - 1) / kSamplesPerCta;
-  k_mlp_fwd<<<nb, 256, 0, s>>>(params, x, B, h1, h2, z);
-  k_mlp_back<<<nb, 256, 0, s>>>(params, labels, B, h1, h2, z, dz, d2, d1, lb);
-  k_mlp_wgrad<<<(kNParams + 255) / 256, 256, 0, s>>>(x, B, h1, h2, dz, d2, d1, lb, grads, loss);
+  k_mlp_fwd<<<counted(nb), 256, 0, s>>>(params, x, B, h1, h2, z);
+  k_mlp_back<<<counted(nb), 256, 0, s>>>(params, labels, B, h1, h2, z, dz, d2, d1, lb);
+  k_mlp_wgrad<<<counted((kNParams + 255) / 256), 256, 0, s>>>(x, B, h1, h2, dz, d2, d1, lb, grads, loss);
   return cudaGetLastError() == cudaSuccess ? TTN_OK : TTN_ECUDA;
 }
 
 ttn_status ttn_mlp_adam(float* params, float* m, float* v, const float* grads, int32_t t, float lr, void* stream) {
   if (!params || !m || !v || !grads || t < 1 || !(lr > 0)) return TTN_EINVAL;
   const float c1 = 1.f - powf(0.9f, (float)t), c2 = 1.f - powf(0.999f, (float)t);
-  ttn::k_adam<<<(ttn::kNParams + 255) / 256, 256, 0, (cudaStream_t)stream>>>(params, m, v, grads, ttn::kNParams, lr,
+  ttn::k_adam<<<ttn::counted((ttn::kNParams + 255) / 256), 256, 0, (cudaStream_t)stream>>>(params, m, v, grads, ttn::kNParams, lr,
                                                                               c1, c2);
   return cudaGetLastError() == cudaSuccess ? TTN_OK : TTN_ECUDA;
 }

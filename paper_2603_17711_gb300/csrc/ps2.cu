@@ -65,7 +65,7 @@ void launch_merge(const double2* Uf, const int* fd, int lf, const double2* Us, c
                   double2* theta, float2* theta_lo, cudaStream_t s) {
   const int64_t n = (int64_t)fd[0] * fd[1] * fd[2] / fd[lf] * ((int64_t)sd[0] * sd[1] * sd[2] / sd[ls]);
   const int blocks = (int)std::min<int64_t>((n + 255) / 256, 2048);
-  k_merge<<<blocks, 256, 0, s>>>(Uf, fd[0], fd[1], fd[2], lf, Us, sd[0], sd[1], sd[2], ls, theta, theta_lo);
+  k_merge<<<counted(blocks), 256, 0, s>>>(Uf, fd[0], fd[1], fd[2], lf, Us, sd[0], sd[1], sd[2], ls, theta, theta_lo);
 }
 
 constexpr int kJacThreads = 512;
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kJacThreads) k_jacobi(const double2* theta, in
 
 void launch_jacobi_svd(const double2* theta, int m, int n, double2* A, double2* V, double* sigma, int* info,
                        cudaStream_t s) {
-  k_jacobi<<<1, kJacThreads, 0, s>>>(theta, m, n, A, V, sigma, info, jacobi_tol(m, n), kJacMaxSweeps);
+  k_jacobi<<<counted(1), kJacThreads, 0, s>>>(theta, m, n, A, V, sigma, info, jacobi_tol(m, n), kJacMaxSweeps);
 }
 
 // Z (rows_iso x r, row-major) and the centre factor Cm (row-major: first side
@@ -263,7 +263,7 @@ void launch_svd_vecs(const double2* A, const double2* V, const double* sigma, in
                      int g, bool iso_first, double2* Z, double2* Zg, double2* Cm, cudaStream_t s) {
   const int64_t tot = (int64_t)(m + n) * r;
   const int blocks = (int)std::min<int64_t>((tot + 255) / 256, 1024);
-  k_svd_vecs<<<blocks, 256, 0, s>>>(A, V, sigma, m, n, perm, r, g, iso_first ? 1 : 0, Z, Zg, Cm);
+  k_svd_vecs<<<counted(blocks), 256, 0, s>>>(A, V, sigma, m, n, perm, r, g, iso_first ? 1 : 0, Z, Zg, Cm);
 }
 
 // Z[:, a] := Zg[:, a] for a < g (restore the determined columns after the QR completion).
@@ -275,7 +275,7 @@ __global__ void k_restore_cols(double2* Z, const double2* Zg, int rows, int r, i
 
 void launch_restore_cols(double2* Z, const double2* Zg, int rows, int r, int g, cudaStream_t s) {
   const int64_t tot = (int64_t)rows * r;
-  k_restore_cols<<<(int)std::min<int64_t>((tot + 255) / 256, 1024), 256, 0, s>>>(Z, Zg, rows, r, g);
+  k_restore_cols<<<counted((int)std::min<int64_t>((tot + 255) / 256, 1024)), 256, 0, s>>>(Z, Zg, rows, r, g);
 }
 
 // New node tensors of the pair (canonical leg order, bond of new rank r at
@@ -318,7 +318,7 @@ __global__ void k_write_pair(double2* Uf, float2* Uf_lo, int f0, int f1, int f2,
 void launch_write_pair(double2* Uf, float2* Uf_lo, const int* fd, int lf, double2* Us, float2* Us_lo, const int* sd,
                        int ls, const double2* Z, const double2* Cm, int r, bool iso_first, cudaStream_t s) {
   const int64_t tot = (int64_t)fd[0] * fd[1] * fd[2] + (int64_t)sd[0] * sd[1] * sd[2];
-  k_write_pair<<<(int)std::min<int64_t>((tot + 255) / 256, 2048), 256, 0, s>>>(
+  k_write_pair<<<counted((int)std::min<int64_t>((tot + 255) / 256, 2048)), 256, 0, s>>>(
       Uf, Uf_lo, fd[0], fd[1], fd[2], lf, Us, Us_lo, sd[0], sd[1], sd[2], ls, Z, Cm, r, iso_first ? 1 : 0);
 }
 

@@ -590,7 +590,7 @@ bool launch_qr_blocked(double2* U, int d0, int d1, int d2, int leg, double tol, 
     const int G = (int)std::min<int64_t>(std::min(sms, kBlkCap), (rows + 7) / 8);
     if (coop && occ >= 1 && G >= 1 && (rows + G - 1) / G <= kPgRows) {
       cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(G, 1, 1);
+      cfg.gridDim = counted(dim3(G, 1, 1));
       cfg.blockDim = dim3(256, 1, 1);
       cfg.stream = s;
       cudaLaunchAttribute at[1];
@@ -605,8 +605,8 @@ bool launch_qr_blocked(double2* U, int d0, int d1, int d2, int leg, double tol, 
     return launch_qr_panel(pn, s);
   };
   const int g1 = (int)std::min<int64_t>(kGatherMax, (m * n + 255) / 256);
-  k_qb_gather<<<g1, 256, 0, s>>>(U, d0, d1, d2, leg, A, m, n, part);
-  k_qb_norm<<<1, 32, 0, s>>>(part, g1, tol, sc, flag, bar);
+  k_qb_gather<<<counted(g1), 256, 0, s>>>(U, d0, d1, d2, leg, A, m, n, part);
+  k_qb_norm<<<counted(1), 32, 0, s>>>(part, g1, tol, sc, flag, bar);
   // factorisation: panel, then its reflectors on the trailing columns
   for (int c0 = 0; c0 < n; c0 += kNB) {
     const int nb = std::min(kNB, n - c0);
@@ -616,23 +616,23 @@ bool launch_qr_blocked(double2* U, int d0, int d1, int d2, int leg, double tol, 
     if (k0 >= n) break;
     const int rbs = rows_per_block(m - c0, sms);
     const int nblk = (int)((m - c0 + rbs - 1) / rbs);
-    k_qb_ypart<<<nblk, 256, 0, s>>>(A, A, m, c0, nb, k0, n, rbs, Y, sc);
-    k_qb_zsum<<<n - k0, 256, 0, s>>>(Y, nblk, nb, k0, n, pn.T, 1, Z, sc);
-    k_qb_update<<<nblk, 256, 0, s>>>(A, A, m, c0, nb, k0, n, rbs, Z, sc);
+    k_qb_ypart<<<counted(nblk), 256, 0, s>>>(A, A, m, c0, nb, k0, n, rbs, Y, sc);
+    k_qb_zsum<<<counted(n - k0), 256, 0, s>>>(Y, nblk, nb, k0, n, pn.T, 1, Z, sc);
+    k_qb_update<<<counted(nblk), 256, 0, s>>>(A, A, m, c0, nb, k0, n, rbs, Z, sc);
   }
   // Q = H_0 .. H_{n-1} [I_n; 0], panels applied last to first
   const int gi = (int)std::min<int64_t>(2048, (m * n + 255) / 256);
-  k_qb_identity<<<gi, 256, 0, s>>>(X, m, n, sc);
+  k_qb_identity<<<counted(gi), 256, 0, s>>>(X, m, n, sc);
   for (int c0 = (n - 1) / kNB * kNB; c0 >= 0; c0 -= kNB) {
     const int nb = std::min(kNB, n - c0);
     const double2* Tp = T + (int64_t)(c0 / kNB) * kNB * kNB;
     const int rbs = rows_per_block(m - c0, sms);
     const int nblk = (int)((m - c0 + rbs - 1) / rbs);
-    k_qb_ypart<<<nblk, 256, 0, s>>>(A, X, m, c0, nb, c0, n, rbs, Y, sc);
-    k_qb_zsum<<<n - c0, 256, 0, s>>>(Y, nblk, nb, c0, n, Tp, 0, Z, sc);
-    k_qb_update<<<nblk, 256, 0, s>>>(A, X, m, c0, nb, c0, n, rbs, Z, sc);
+    k_qb_ypart<<<counted(nblk), 256, 0, s>>>(A, X, m, c0, nb, c0, n, rbs, Y, sc);
+    k_qb_zsum<<<counted(n - c0), 256, 0, s>>>(Y, nblk, nb, c0, n, Tp, 0, Z, sc);
+    k_qb_update<<<counted(nblk), 256, 0, s>>>(A, X, m, c0, nb, c0, n, rbs, Z, sc);
   }
-  k_qb_finish<<<gi, 256, 0, s>>>(A, X, m, n, alpha, phase, skip, U, d0, d1, d2, leg, R, U_lo, R_lo, sc);
+  k_qb_finish<<<counted(gi), 256, 0, s>>>(A, X, m, n, alpha, phase, skip, U, d0, d1, d2, leg, R, U_lo, R_lo, sc);
   return true;
 }
 

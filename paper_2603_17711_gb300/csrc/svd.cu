@@ -640,7 +640,7 @@ bool launch_jacobi_svd_grid(const double2* theta, int m, int n, double2* A, doub
     return cudaGetLastError() == cudaSuccess;
   }
   const int64_t tot = (int64_t)nr * nc + (int64_t)nc * nc;
-  k_svd_load<<<(int)std::min<int64_t>((tot + 255) / 256, 4096), 256, 0, s>>>(theta, m, n, A, V);
+  k_svd_load<<<counted((int)std::min<int64_t>((tot + 255) / 256, 4096)), 256, 0, s>>>(theta, m, n, A, V);
   if (cudaMemsetAsync(sync, 0, kSvdSyncInts * sizeof(unsigned), s) != cudaSuccess) return false;
   const int tr = n > m ? 1 : 0;
   const double tol = jacobi_tol(m, n);
@@ -651,7 +651,7 @@ bool launch_jacobi_svd_grid(const double2* theta, int m, int n, double2* A, doub
   cfg.attrs = at;
   cfg.numAttrs = 1;
   if (cluster) {  // one pair per CTA, the CTAs one cluster
-    cfg.gridDim = dim3(npairs, 1, 1);
+    cfg.gridDim = counted(dim3(npairs, 1, 1));
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = npairs;
     at[0].val.clusterDim.y = 1;
@@ -660,7 +660,7 @@ bool launch_jacobi_svd_grid(const double2* theta, int m, int n, double2* A, doub
                               wait_ns) == cudaSuccess;
   }
   const int G = std::max(1, std::min(npairs, gi.sms * std::min(gi.occ, 2)));
-  cfg.gridDim = dim3(G, 1, 1);
+  cfg.gridDim = counted(dim3(G, 1, 1));
   at[0].id = cudaLaunchAttributeCooperative;
   at[0].val.cooperative = 1;
   return cudaLaunchKernelEx(&cfg, k_jacobi_grid<false>, A, V, nr, nc, (const int*)nullptr, sigma, info, sync, flag, tol, kJacMaxSweeps, tr,
@@ -688,7 +688,7 @@ bool launch_pivot_svd(const double2* theta, int m, int n, bool iso_first, double
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  cfg.gridDim = dim3(G, 1, 1);
+  cfg.gridDim = counted(dim3(G, 1, 1));
   cfg.dynamicSmemBytes = pivot_smem(nb, ni, G);
   double* fpart = cand + 2 * kPivMaxGrid;
   int* cand_i = (int*)(fpart + kPivMaxGrid);
@@ -698,7 +698,7 @@ bool launch_pivot_svd(const double2* theta, int m, int n, bool iso_first, double
   if (cudaMemsetAsync(sync, 0, kSvdSyncInts * sizeof(unsigned), s) != cudaSuccess) return false;
   cfg.dynamicSmemBytes = 0;
   cfg.blockDim = dim3(kJThreads, 1, 1);
-  cfg.gridDim = dim3(std::max(1, std::min((k + 1) / 2, gi.sms * std::min(gi.occ, 2))), 1, 1);
+  cfg.gridDim = counted(dim3(std::max(1, std::min((k + 1) / 2, gi.sms * std::min(gi.occ, 2))), 1, 1));
   return cudaLaunchKernelEx(&cfg, k_jacobi_grid<false>, X, (double2*)nullptr, ni, k, (const int*)(info + 2), sigma,
                             info, sync, flag, jacobi_tol(m, n), kJacMaxSweeps, iso_first ? 0 : 1,
                             wait_ns) == cudaSuccess;
@@ -748,9 +748,9 @@ __global__ void __launch_bounds__(256) k_pivot_centre(const double2* __restrict_
 void launch_pivot_vecs(const double2* theta, int m, int n, bool iso_first, const double2* X, const double* sigma,
                        const int* perm, int r, int g, double2* Z, double2* Zg, double2* Cm, cudaStream_t s) {
   const int ni = iso_first ? m : n, no = iso_first ? n : m;
-  k_pivot_iso<<<(int)std::min<int64_t>(((int64_t)ni * r + 255) / 256, 1024), 256, 0, s>>>(X, sigma, perm, ni, r, g,
+  k_pivot_iso<<<counted((int)std::min<int64_t>(((int64_t)ni * r + 255) / 256, 1024)), 256, 0, s>>>(X, sigma, perm, ni, r, g,
                                                                                           iso_first ? 1 : 0, Z, Zg);
-  k_pivot_centre<<<(int)std::min<int64_t>(((int64_t)no * r + 7) / 8, 4096), 256, 0, s>>>(theta, m, n, Z, r,
+  k_pivot_centre<<<counted((int)std::min<int64_t>(((int64_t)no * r + 7) / 8, 4096)), 256, 0, s>>>(theta, m, n, Z, r,
                                                                                          iso_first ? 1 : 0, Cm);
 }
 
@@ -865,7 +865,7 @@ extern "C" ttn_status ttn_svd(const void* a_dev, int32_t m, int32_t n, void* u_d
   for (int i = 0; i < nc; ++i) sigma_host[i] = sig[pm[i]];
   if (cudaMemcpyAsync(perm, pm.data(), nc * sizeof(int), cudaMemcpyHostToDevice, s) != cudaSuccess) return TTN_ECUDA;
   const int64_t tot = (int64_t)(m + n) * nc;
-  k_svd_write<<<(int)std::min<int64_t>((tot + 255) / 256, 4096), 256, 0, s>>>(A, V, sigma, perm, m, n,
+  k_svd_write<<<counted((int)std::min<int64_t>((tot + 255) / 256, 4096)), 256, 0, s>>>(A, V, sigma, perm, m, n,
                                                                              (double2*)u_dev, (double2*)vh_dev);
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return TTN_ECUDA;
   return TTN_OK;

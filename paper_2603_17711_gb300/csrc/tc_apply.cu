@@ -998,7 +998,7 @@ bool launch_apply_tc(const DevTables& T, const ApList& L, const Epi& e, const Ap
     cudaFuncSetAttribute(k_tc_apply_ring, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingSmem);
     ring_attr = true;
   }
-  if (ring && J.start[J.n] > 0) k_tc_split<<<J.start[J.n], kTcThreads, 0, s>>>(T, J, bsplit);
+  if (ring && J.start[J.n] > 0) k_tc_split<<<counted(J.start[J.n]), kTcThreads, 0, s>>>(T, J, bsplit);
   if (used_ring) *used_ring = ring;
   const bool rk = e.mode != EPI_STORE;
   const bool one = L.out_end - L.out_begin == 1;
@@ -1075,12 +1075,12 @@ bool launch_apply_tc(const DevTables& T, const ApList& L, const Epi& e, const Ap
     }
     if (lg.lt[3] > 0) {
       if (ring)
-        k_tc_apply_ring<<<lg.lt[3], kTcThreads, kRingSmem, s>>>(T, L, -1, lg, acc, P, flag, pool, pool_off, bsplit,
+        k_tc_apply_ring<<<counted(lg.lt[3]), kTcThreads, kRingSmem, s>>>(T, L, -1, lg, acc, P, flag, pool, pool_off, bsplit,
                                                                 B);
       else
-        k_tc_apply<<<lg.lt[3], kTcThreads, kTcSmem, s>>>(T, L, -1, lg, acc, P, flag, pool, pool_off);
+        k_tc_apply<<<counted(lg.lt[3]), kTcThreads, kTcSmem, s>>>(T, L, -1, lg, acc, P, flag, pool, pool_off);
     }
-    k_tc_epilogue<<<L.n_tiles, 32, 0, s>>>(T, L, e, acc, q, P);
+    k_tc_epilogue<<<counted(L.n_tiles), 32, 0, s>>>(T, L, e, acc, q, P);
     return true;
   }
   const TcLegs none{};
@@ -1088,12 +1088,12 @@ bool launch_apply_tc(const DevTables& T, const ApList& L, const Epi& e, const Ap
     if (has[l]) {
       float2* part = rk ? acc : nullptr;  // RK lists: the single output's sum goes to acc
       if (ring)
-        k_tc_apply_ring<<<tiles[l], kTcThreads, kRingSmem, s>>>(T, L, l, none, part, 0, flag, pool, pool_off, bsplit,
+        k_tc_apply_ring<<<counted(tiles[l]), kTcThreads, kRingSmem, s>>>(T, L, l, none, part, 0, flag, pool, pool_off, bsplit,
                                                                 B);
       else
-        k_tc_apply<<<tiles[l], kTcThreads, kTcSmem, s>>>(T, L, l, none, part, 0, flag, pool, pool_off);
+        k_tc_apply<<<counted(tiles[l]), kTcThreads, kTcSmem, s>>>(T, L, l, none, part, 0, flag, pool, pool_off);
     }
-  if (rk || ident) k_tc_epilogue<<<L.n_tiles, 32, 0, s>>>(T, L, e, acc, 0, 0);
+  if (rk || ident) k_tc_epilogue<<<counted(L.n_tiles), 32, 0, s>>>(T, L, e, acc, 0, 0);
   return true;
 }
 
@@ -1104,7 +1104,7 @@ void launch_tc_embed(void* const* mats32, const TcEmbedJob* jobs, int n, float* 
     TcEmbedBatch b{};
     b.n = std::min(kTcEmbedBatch, n - i0);
     for (int i = 0; i < b.n; ++i) b.job[i] = jobs[i0 + i];
-    k_tc_embed<<<dim3(b.n, (kTcM + kTcK - 1) / kTcK), kTcThreads, 0, s>>>(mats32, b, pool);
+    k_tc_embed<<<counted(dim3(b.n, (kTcM + kTcK - 1) / kTcK)), kTcThreads, 0, s>>>(mats32, b, pool);
   }
 }
 

@@ -291,8 +291,8 @@ void launch_vmf_stage(double2* out, const double2* y, const VmfComb& cb, int64_t
 
 void launch_vmf_err(const double2* y, const double2* y5, const VmfComb& cb, double rtol, double atol, int64_t n,
                     double* part, double* out, cudaStream_t s) {
-  k_vmf_err<<<kErrBlocks, kT, 0, s>>>(y, y5, cb, rtol, atol, n, part);
-  k_vmf_sum<<<1, 32, 0, s>>>(part, kErrBlocks, out);
+  k_vmf_err<<<counted(kErrBlocks), kT, 0, s>>>(y, y5, cb, rtol, atol, n, part);
+  k_vmf_sum<<<counted(1), 32, 0, s>>>(part, kErrBlocks, out);
 }
 
 }  // namespace ttn

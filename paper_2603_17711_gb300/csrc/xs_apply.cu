@@ -872,8 +872,8 @@ bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L
     }
     gr.leg = -1;
     gr.planes = planes;
-    k_xs_apply<<<dim3(gr.lt[4], 1), kXsThreads, 0, s>>>(gr);
-    k_xs_epilogue<<<(int)((P + 127) / 128), 128, 0, s>>>(planes, q, P, with_coef(e), gr.dst[0], sp);
+    k_xs_apply<<<counted(dim3(gr.lt[4], 1)), kXsThreads, 0, s>>>(gr);
+    k_xs_epilogue<<<counted((int)((P + 127) / 128)), 128, 0, s>>>(planes, q, P, with_coef(e), gr.dst[0], sp);
     return true;
   }
   if (e.mode != EPI_STORE) return false;
@@ -894,13 +894,13 @@ bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L
   }
   if (!multi_leg) {
     gr.leg = -2;
-    k_xs_apply<<<dim3(gmax, n_outs), kXsThreads, 0, s>>>(gr);
+    k_xs_apply<<<counted(dim3(gmax, n_outs)), kXsThreads, 0, s>>>(gr);
     return true;
   }
   for (int l = 0; l < 4; ++l)
     if (nterm[l]) {
       gr.leg = l;
-      k_xs_apply<<<dim3(gx[l], n_outs), kXsThreads, 0, s>>>(gr);
+      k_xs_apply<<<counted(dim3(gx[l], n_outs)), kXsThreads, 0, s>>>(gr);
     }
   return true;
 }
@@ -930,7 +930,7 @@ bool launch_project_xs(double2* const* bufs, double2* const* mats, const PjList&
   w.KS = 1;
   while (w.KS < std::min(8, max_split) && w.KS * G < nch && (int64_t)tiles * n * w.KS < 2 * sm_count()) ++w.KS;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(tiles * w.KS), (unsigned)n, 1);
+  cfg.gridDim = counted(dim3((unsigned)(tiles * w.KS), (unsigned)n, 1));
   cfg.blockDim = dim3(kXsThreads, 1, 1);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
