@@ -192,7 +192,9 @@ ttn_status ttn_set_drive(ttn_t h, int32_t id, ttn_drive_fn g, void* user, double
  * scratch (sized for the rank caps). Valid after sop_load. */
 ttn_status ttn_workspace_size(ttn_t h, size_t* bytes);
 /* Bind a device buffer of at least ttn_workspace_size bytes, 256-byte aligned,
- * on the current CUDA device. Uploads operators, builds the initial product
+ * on the current CUDA device. (FP64: the last bytes may be planes of the
+ * tensor-core contractions; a buffer that ends before them is accepted, and the
+ * lists that need them then run on the CUDA cores.) Uploads operators, builds the initial product
  * state rho0 = |0><0| (x) |0..0> and its environments. */
 ttn_status ttn_set_workspace(ttn_t h, void* device_ptr, size_t bytes);
 /* cudaStream_t passed as void*. */

@@ -71,7 +71,6 @@ struct ttn_ctx {
   double* svd_sigma = nullptr;
   int* svd_perm = nullptr;
   int* svd_info = nullptr;
-  double* svd_cand = nullptr;  // pivot candidates of the two-site QR
   unsigned* svd_sync = nullptr;  // barrier counters of the grid Jacobi SVD
   // direct integration (vmf), FP64 form only
   double2 *vmf_y = nullptr, *vmf_save = nullptr, *vmf_tmp = nullptr, *vmf_r = nullptr, *vmf_aug = nullptr,
@@ -232,12 +231,13 @@ ttn_status cuda_fail(ttn_t h, cudaError_t e, const char* what) {
 // Workspace layout
 // ---------------------------------------------------------------------------
 struct Layout {
-  size_t nodes, pool, scratch, qr, rdm, rho, bufs_tab, mats_tab, terms, outs, pjs, drives, flag, total;
+  size_t nodes, pool, scratch, qr, rdm, rho, bufs_tab, mats_tab, terms, outs, pjs, drives, flag;
+  size_t required, total;  // without and with the planes of the digit split
   size_t nodes32 = 0, pool32 = 0, scratch32 = 0, bufs_tab_lo = 0, mats_tab_lo = 0, tc_acc = 0, tc_bsplit = 0;
   int64_t tc_bsplit_floats = 0;  // FP32 mode only
   size_t tc_pool = 0, tc_off = 0;
   std::vector<int64_t> tc_off_host;  // float offset of each matrix in tc_pool, -1 if none
-  size_t svd_cand = 0, svd_small = 0, rsvd = 0, mlp = 0, xs = 0;
+  size_t svd_small = 0, rsvd = 0, mlp = 0, xs = 0;
   int64_t xs_elems = 0;
   bool xs_in_svd = false;
   // direct integration (vmf): committed state, per-node saves, 7 stage
@@ -293,7 +293,9 @@ Layout layout_of(const Plan& p, int prec) {
   }
   L.rdm_elems = ra;
   L.rdm = take(ra * sizeof(double2));
-  L.rho = take(((size_t)p.leg_dims[0] * p.leg_dims[0] + 1) * sizeof(double2));  // rho, then the error flag
+  const size_t n_rho = (size_t)p.leg_dims[0] * p.leg_dims[0];
+  L.rho = take((n_rho + 1) * sizeof(double2) + 4 * sizeof(int));  // rho, its copy of the error flag, the flag
+  L.flag = L.rho + (n_rho + 1) * sizeof(double2);
   L.bufs_tab = take(p.buf.n_bufs * sizeof(double2*));
   L.mats_tab = take(p.mats.size() * sizeof(double2*));
   L.terms = take(p.ap_terms.size() * sizeof(ApTerm));
@@ -301,18 +303,9 @@ Layout layout_of(const Plan& p, int prec) {
   L.pjs = take(p.pj_outs.size() * sizeof(PjOut));
   L.drives = take(p.locals.size() * sizeof(DriveMat));
   L.svd_small = take(p.theta_cap * sizeof(double) + (p.theta_cap + 4 + kSvdSyncInts) * sizeof(int));
-  L.svd_cand = take(kPivScratch * sizeof(double));
   L.rsvd = take(3 * p.theta_cap * sizeof(double2));
   L.mlp = take((24 + 13 + mlp_ws_floats(1) + 8) * sizeof(float) + 2 * sizeof(double));
-  L.flag = take(sizeof(int) * 4);
   if (prec == PREC_F64) {
-    // planes of the digit split (FP64 contractions only): one per leg always
-    // fits, small nodes may cut their terms into more. They take the two-site
-    // split's five matrices, which no contraction list overlaps, where those are
-    // large enough (every tree of two nodes or more at any but the smallest sizes)
-    L.xs_elems = std::max<int64_t>(4 * S, std::min<int64_t>(24 * p.P_cap_max, 1 << 20));
-    L.xs_in_svd = L.xs_elems <= 5 * p.theta_cap;
-    if (!L.xs_in_svd) L.xs = take(L.xs_elems * sizeof(double2));
     L.nodes_elems = acc;
     L.vmf_y = take(acc * sizeof(double2));
     L.vmf_save = take(acc * sizeof(double2));
@@ -371,6 +364,18 @@ Layout layout_of(const Plan& p, int prec) {
             std::max(L.tc_bsplit_floats, tc_split_floats(al, p.ap_outs.data(), p.ap_terms.data(), L.tc_off_host.data()));
     L.tc_bsplit = take(std::max<int64_t>(L.tc_bsplit_floats, 1) * sizeof(float));
     L.mats_tab_lo = take(p.mats.size() * sizeof(void*));
+  }
+  L.required = off;
+  if (prec == PREC_F64) {
+    // planes of the digit split (FP64 contractions only): one per leg always
+    // fits, small nodes may cut their terms into more. They take the two-site
+    // split's five matrices, which no contraction list overlaps, where those are
+    // large enough, else the workspace's end; one that ends before them is taken
+    // too, as it was without the split, and its one-output lists stay on the
+    // CUDA cores
+    L.xs_elems = std::max<int64_t>(4 * S, std::min<int64_t>(24 * p.P_cap_max, 1 << 20));
+    L.xs_in_svd = L.xs_elems <= 5 * p.theta_cap;
+    if (!L.xs_in_svd) L.xs = take(L.xs_elems * sizeof(double2));
   }
   L.total = off;
   return L;
@@ -606,7 +611,8 @@ struct Exec {
     }
   }
   uint64_t wait_ns() const { return (uint64_t)(h->params.wait_s * 1e9); }
-  // launch the Jacobi SVD (one CTA or the whole GPU) and read back sigma; false
+  // launch the Jacobi SVD (one CTA or the whole GPU; its column counters and pivot candidates
+  // lie in the isometry's buffers, which are written after it) and read back sigma; false
   // (with fail_st set) when it did not converge or a grid wait gave up
   // pivoted (nullable in): ask for the pivoted-QR route of a two-site matrix with
   // the isometry on the first / second side; out: whether it was taken
@@ -615,8 +621,8 @@ struct Exec {
     const int nc = std::min(m, n);
     run(2, 0.0, [&] {
       if (pivoted) {
-        *pivoted = launch_pivot_svd(theta, m, n, iso_first, h->svd_A, h->svd_V, h->svd_sigma, h->svd_cand, h->svd_info,
-                                    h->svd_sync, h->flag_dev, wait_ns(), s);
+        *pivoted = launch_pivot_svd(theta, m, n, iso_first, h->svd_A, h->svd_V, h->svd_sigma, (double*)h->svd_Zg, h->svd_info,
+                                    h->svd_sync, (unsigned*)h->svd_Z, h->flag_dev, wait_ns(), s);
         if (*pivoted) return;
         if (const cudaError_t e = cudaGetLastError(); e != cudaSuccess) {
           note(e);
@@ -624,7 +630,7 @@ struct Exec {
         }
       }
       if (!launch_jacobi_svd_grid(theta, m, n, h->svd_A, h->svd_V, h->svd_sigma, h->svd_info, h->svd_sync,
-                                  h->flag_dev, wait_ns(), s))
+                                  (unsigned*)h->svd_Z, h->flag_dev, wait_ns(), s))
         {
           const cudaError_t e = cudaGetLastError();
           note(e != cudaSuccess ? e : cudaErrorLaunchFailure);
@@ -979,6 +985,17 @@ bool ensure_capture(ttn_t h, double dt) {
   h->graph_prof = h->prof_mode;
   return true;
 }
+// The same with its executable form. A batch replays the captures of its members
+// as children of one graph and needs none of theirs: they were 50 of the 160 ms
+// that the first batched step of 64 instances took.
+bool ensure_graph(ttn_t h, double dt) {
+  if (!ensure_capture(h, dt)) return false;
+  if (h->graph || cudaGraphInstantiate(&h->graph, h->graph_src, 0) == cudaSuccess) return true;
+  cudaGetLastError();
+  h->drop_graph();
+  h->graph_disabled = true;
+  return false;
+}
 
 template <typename F>
 ttn_status guarded(ttn_t h, F&& f) {
@@ -990,17 +1007,6 @@ ttn_status guarded(ttn_t h, F&& f) {
   } catch (const std::exception& e) {
     return h->fail(TTN_EINVAL, e.what());
   }
-}
-// The same with its executable form. A batch replays the captures of its members
-// as children of one graph and needs none of theirs: they were 50 of the 160 ms
-// that the first batched step of 64 instances took.
-bool ensure_graph(ttn_t h, double dt) {
-  if (!ensure_capture(h, dt)) return false;
-  if (h->graph || cudaGraphInstantiate(&h->graph, h->graph_src, 0) == cudaSuccess) return true;
-  cudaGetLastError();
-  h->drop_graph();
-  h->graph_disabled = true;
-  return false;
 }
 
 ttn_status status_of(const std::string& e) {
@@ -1206,7 +1212,7 @@ ttn_status ttn_set_workspace(ttn_t h, void* dptr, size_t bytes) {
     allow_wide_splits();
     Plan& p = h->plan;
     Layout L = layout_of(p, h->prec);
-    if (bytes < L.total) return h->fail(TTN_ENOMEM, "workspace smaller than ttn_workspace_size");
+    if (bytes < L.required) return h->fail(TTN_ENOMEM, "workspace smaller than ttn_workspace_size");
     char* base = (char*)dptr;
     h->ws = base;
     h->ws_bytes = bytes;
@@ -1241,7 +1247,6 @@ ttn_status ttn_set_workspace(ttn_t h, void* dptr, size_t bytes) {
     h->svd_perm = (int*)(h->svd_sigma + p.theta_cap);
     h->svd_info = h->svd_perm + p.theta_cap;
     h->svd_sync = (unsigned*)(h->svd_info + 4);
-    h->svd_cand = (double*)(base + L.svd_cand);
     h->rs_omega = (double2*)(base + L.rsvd);
     h->rs_Y = h->rs_omega + p.theta_cap;
     h->rs_B = h->rs_Y + p.theta_cap;
@@ -1270,7 +1275,7 @@ ttn_status ttn_set_workspace(ttn_t h, void* dptr, size_t bytes) {
     h->node_off = L.node_off;
     if (h->prec == PREC_F64) {
       h->xs_planes = L.xs_in_svd ? h->svd_A : (double2*)(base + L.xs);
-      h->xs_elems = L.xs_elems;
+      h->xs_elems = L.xs_in_svd || bytes >= L.total ? L.xs_elems : 0;
       h->vmf_n = L.nodes_elems;
       h->vmf_y = (double2*)(base + L.vmf_y);
       h->vmf_save = (double2*)(base + L.vmf_save);
@@ -2139,7 +2144,7 @@ ttn_status ttn_autotune(ttn_t h, int32_t reps) {
       if (!f64[i] && h->prec == PREC_F32 && h->params.tensor_cores &&
           tc_applicable(L, p.ap_outs.data(), p.ap_terms.data()))
         continue;
-      if (h->prec == PREC_F64 && xs_applicable(L, p.ap_outs.data(), p.ap_terms.data())) continue;
+      if (h->prec == PREC_F64 && h->xs_elems > 0 && xs_applicable(L, p.ap_outs.data(), p.ap_terms.data())) continue;
       const bool epi = p.ap_outs[L.out_begin].dst < 0;
       const TuneKey key = ap_key(p, L, prec);
       auto seen = done.find(key);

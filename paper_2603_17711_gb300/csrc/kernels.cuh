@@ -380,13 +380,13 @@ __device__ __forceinline__ double warp_sum4(double v0, double v1, double v2, dou
 // one thread-block cluster for up to 2 * kJacClusterMax columns, else a grid
 // barrier of one cooperative launch. Used when the smaller side has more than
 // kJacOneCtaMaxCols columns (else the one-CTA kernel). sync: kSvdSyncInts device
-// ints (cleared by the launch); a grid wait longer than wait_ns sets bit 4 (16)
+// ints, ver: min(m, n) more (both cleared by the launch); a grid wait longer than wait_ns sets bit 4 (16)
 // of *flag. Same outputs as launch_jacobi_svd.
 constexpr int kJacOneCtaMaxCols = 16;
 constexpr int kJacClusterMax = 16;
-constexpr int kSvdSyncInts = 128 + 2048;  // barrier and sweep counters, column round counters
+constexpr int kSvdSyncInts = 128;  // barrier and sweep counters
 bool launch_jacobi_svd_grid(const double2* theta, int m, int n, double2* A, double2* V, double* sigma, int* info,
-                            unsigned* sync, int* flag, uint64_t wait_ns, cudaStream_t s);
+                            unsigned* sync, unsigned* ver, int* flag, uint64_t wait_ns, cudaStream_t s);
 // The split of a two-site matrix theta (m x n, row-major) with more columns on
 // its smaller side than a cluster's Jacobi takes: pivoted QR, then Jacobi on R^H
 // (svd.cu). X (ni x k, column-major; ni rows of the isometry side, k = min(m, n))
@@ -397,7 +397,7 @@ bool launch_jacobi_svd_grid(const double2* theta, int m, int n, double2* A, doub
 constexpr int kPivMaxGrid = 256;
 constexpr int kPivScratch = 2 * kPivMaxGrid + kPivMaxGrid + kPivMaxGrid;  // norms, partial sums, indices
 bool launch_pivot_svd(const double2* theta, int m, int n, bool iso_first, double2* X, double2* Bg, double* sigma,
-                      double* cand, int* info, unsigned* sync, int* flag, uint64_t wait_ns, cudaStream_t s);
+                      double* cand, int* info, unsigned* sync, unsigned* ver, int* flag, uint64_t wait_ns, cudaStream_t s);
 // Isometry Z (ni x r, row-major; columns beyond g zero), its copy Zg, and the
 // centre factor Cm = theta contracted with conj(Z), in the layouts of launch_svd_vecs.
 void launch_pivot_vecs(const double2* theta, int m, int n, bool iso_first, const double2* X, const double* sigma,

@@ -5,21 +5,22 @@
 // The working matrix holds the columns of Theta (or of Theta^H when Theta is
 // wider than tall), column-major; V starts as the identity. A sweep visits every
 // column pair once, in the rounds of the circle method: the pairs of one round
-// are disjoint, so they are dealt to the CTAs and the round ends with one
-// barrier -- the hardware barrier of a thread-block cluster when the pairs fit
-// one cluster (at most 16 CTAs), else a grid barrier of one cooperative launch.
-// A pair is handled by one CTA: its threads split the rows, the three Gram
-// entries a = |x|^2, b = |y|^2, c = x^H y are summed in a fixed order (threads
-// -> warps -> warp order), thread 0 computes the complex rotation
-// (jacobi_rotation: skipped when |c| <= tol sqrt(a b) or a column is rounding
+// are disjoint, so they are dealt to the CTAs. Between rounds stands the hardware
+// barrier of a thread-block cluster when the pairs fit one cluster (at most 16
+// CTAs); in the grid form (one cooperative launch) a CTA waits for its two columns
+// only, handed over by a counter each, and a grid barrier ends the sweep.
+// A pair is handled by one CTA of four warps: its threads split the rows, the three
+// Gram entries a = |x|^2, b = |y|^2, c = x^H y are summed in a fixed order (threads
+// -> warps -> a butterfly over the warps), warp 0 computes the complex rotation
+// (rotate_warp: skipped when |c| <= tol sqrt(a b) or a column is rounding
 // noise) and the threads apply it to the pair's rows of the working matrix and
 // of V. GB300 retires about one FP64 warp instruction per 19 cycles per SM, and
 // a square root or quotient is a dozen of them: computing the rotation in one
-// thread instead of all eight warps keeps the FP64 pipe for the rows.
-// A sweep without any rotation ends the iteration: every CTA reads the sweep's
-// rotation count after the sweep's last barrier. Which CTA handles a pair, and
-// which barrier ends a round, does not change the arithmetic, so the result
-// does not depend on the launch shape.
+// warp instead of all keeps the FP64 pipe for the rows.
+// A sweep without a rotation, or of small rotations only (kBigCos, kBigSin), ends
+// the iteration: every CTA reads the sweep's counts after the sweep's last barrier.
+// Which CTA handles a pair, and what ends a round, does not change the arithmetic,
+// so the result does not depend on the launch shape.
 //
 // The convergence threshold tol = 2 sqrt(max(rows, 64)) * DBL_EPSILON sits above
 // the rounding noise of the Gram entries summed over the rows, so a converged
@@ -29,7 +30,7 @@
 // Every grid wait is bounded (wait_ns from the moment the CTA starts waiting);
 // a CTA whose wait gives up sets bit 4 (value 16) of *flag and returns. Nothing
 // is in flight when it does (plain loads and stores only), so any CTA may leave
-// at any time; the others give up at their next barrier. The cluster barrier is
+// at any time; the others give up at their next wait. The cluster barrier is
 // the hardware's: all CTAs of a cluster are resident together and every CTA
 // passes the same number of barriers.
 #include <algorithm>
@@ -57,10 +58,9 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kJThreads = 128;
 constexpr int kJWarps = kJThreads / 32;
 constexpr int kBarLanes = 8;
-constexpr int kVerOff = 128;  // first column counter in the sync words
-constexpr int kSvdMaxVer = kSvdSyncInts - kVerOff;
+constexpr int kSvdMaxVer = 2048;  // more columns than this keep one barrier a round
 constexpr int kSmallOff = kBarLanes + kJacMaxSweeps;  // first counter of small rotations
-static_assert(kSmallOff + kJacMaxSweeps <= kVerOff, "sweep counters fit before the column counters");
+static_assert(kSmallOff + kJacMaxSweeps <= kSvdSyncInts, "the counters of all sweeps fit");
 
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
   return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -207,9 +207,10 @@ __device__ __forceinline__ bool phase_sync(unsigned* lanes, unsigned target, uin
   }
 }
 
-// sync: [0, 8) barrier lanes, [8, 8 + max_sweeps) rotations per sweep that ask for another one, as many
-// counters of the small ones, then the columns' rounds; zeroed before the launch. kCluster: the CTAs form one thread-block cluster. V may be
-// null (no right vectors). nc_dev (nullable): the column count, at most nc,
+// sync: [0, 8) barrier lanes, [8, 8 + max_sweeps) rotations per sweep that ask for
+// another one, then as many counters of the small ones; ver: the columns' rounds (grid
+// form); both zeroed before the launch. kCluster: the CTAs form one thread-block
+// cluster. V may be null (no right vectors). nc_dev (nullable): the column count, at most nc,
 // found on the device; columns beyond it are zero.
 //
 // Between the rounds of the grid form a CTA waits for its two columns only:
@@ -217,7 +218,7 @@ __device__ __forceinline__ bool phase_sync(unsigned* lanes, unsigned target, uin
 // the CTA that finished it and polled with acquire by the one that takes it
 // next. A round's hand-over is then one flag to one reader instead of a
 // barrier over all CTAs; one grid barrier a sweep remains, for its rotation count.
-// (sync + kVerOff: up to kSvdMaxVer columns; wider matrices keep the barrier.)
+// (Up to kSvdMaxVer columns; wider matrices keep the barrier.)
 // The two-site split of the rank-16 driven system (256 x 100 and 256 x 64), per
 // step of 14 splits: 148 ms with accumulated right vectors and one barrier a
 // round; 45 ms with R^H in place of the matrix, 41 with column hand-over and
@@ -225,7 +226,7 @@ __device__ __forceinline__ bool phase_sync(unsigned* lanes, unsigned target, uin
 template <bool kCluster>
 __global__ void __launch_bounds__(kJThreads) k_jacobi_grid(double2* __restrict__ A, double2* __restrict__ V, int nr,
                                                           int nc_in, const int* nc_dev, double* __restrict__ sigma, int* __restrict__ info,
-                                                          unsigned* sync, int* flag, double tol, int max_sweeps,
+                                                          unsigned* sync, unsigned* ver, int* flag, double tol, int max_sweeps,
                                                           int tr, uint64_t wait_ns) {
   static_assert(kJWarps * 4 <= 32 && (kJWarps & (kJWarps - 1)) == 0, "warp 0 adds four sums of each warp, one per lane");
   __shared__ double s_red[kJWarps][4];
@@ -260,7 +261,6 @@ __global__ void __launch_bounds__(kJThreads) k_jacobi_grid(double2* __restrict__
   double fro2 = 0.0;
   for (int jc = 0; jc < nc; ++jc) fro2 += sigma[jc];
   const double tiny2 = jacobi_negligible(nr, fro2);
-  unsigned* ver = sync + kVerOff;
   const bool p2p = !kCluster && nc <= kSvdMaxVer;
   __shared__ int s_alive;
   int sweep = 0;
@@ -630,7 +630,7 @@ double jacobi_tol(int m, int n) {
 }
 
 bool launch_jacobi_svd_grid(const double2* theta, int m, int n, double2* A, double2* V, double* sigma, int* info,
-                            unsigned* sync, int* flag, uint64_t wait_ns, cudaStream_t s) {
+                            unsigned* sync, unsigned* ver, int* flag, uint64_t wait_ns, cudaStream_t s) {
   const int nc = std::min(m, n), nr = std::max(m, n);
   const GridInfo gi = grid_info();
   const int npairs = (nc + 1) / 2;
@@ -641,7 +641,9 @@ bool launch_jacobi_svd_grid(const double2* theta, int m, int n, double2* A, doub
   }
   const int64_t tot = (int64_t)nr * nc + (int64_t)nc * nc;
   k_svd_load<<<counted((int)std::min<int64_t>((tot + 255) / 256, 4096)), 256, 0, s>>>(theta, m, n, A, V);
-  if (cudaMemsetAsync(sync, 0, kSvdSyncInts * sizeof(unsigned), s) != cudaSuccess) return false;
+  if (cudaMemsetAsync(sync, 0, kSvdSyncInts * sizeof(unsigned), s) != cudaSuccess ||
+      cudaMemsetAsync(ver, 0, nc * sizeof(unsigned), s) != cudaSuccess)
+    return false;
   const int tr = n > m ? 1 : 0;
   const double tol = jacobi_tol(m, n);
   cudaLaunchConfig_t cfg = {};
@@ -656,19 +658,21 @@ bool launch_jacobi_svd_grid(const double2* theta, int m, int n, double2* A, doub
     at[0].val.clusterDim.x = npairs;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
-    return cudaLaunchKernelEx(&cfg, k_jacobi_grid<true>, A, V, nr, nc, (const int*)nullptr, sigma, info, sync, flag, tol, kJacMaxSweeps, tr,
+    return cudaLaunchKernelEx(&cfg, k_jacobi_grid<true>, A, V, nr, nc, (const int*)nullptr, sigma, info, sync, ver, flag, tol,
+                              kJacMaxSweeps, tr,
                               wait_ns) == cudaSuccess;
   }
   const int G = std::max(1, std::min(npairs, gi.sms * std::min(gi.occ, 2)));
   cfg.gridDim = counted(dim3(G, 1, 1));
   at[0].id = cudaLaunchAttributeCooperative;
   at[0].val.cooperative = 1;
-  return cudaLaunchKernelEx(&cfg, k_jacobi_grid<false>, A, V, nr, nc, (const int*)nullptr, sigma, info, sync, flag, tol, kJacMaxSweeps, tr,
+  return cudaLaunchKernelEx(&cfg, k_jacobi_grid<false>, A, V, nr, nc, (const int*)nullptr, sigma, info, sync, ver, flag, tol,
+                              kJacMaxSweeps, tr,
                             wait_ns) == cudaSuccess;
 }
 
 bool launch_pivot_svd(const double2* theta, int m, int n, bool iso_first, double2* X, double2* Bg, double* sigma,
-                      double* cand, int* info, unsigned* sync, int* flag, uint64_t wait_ns, cudaStream_t s) {
+                      double* cand, int* info, unsigned* sync, unsigned* ver, int* flag, uint64_t wait_ns, cudaStream_t s) {
   const int nb = iso_first ? n : m, ni = iso_first ? m : n, k = std::min(m, n);
   const GridInfo gi = grid_info();
   // the pivoted QR pays its ~5 us a column where the sweeps it saves are those
@@ -695,12 +699,14 @@ bool launch_pivot_svd(const double2* theta, int m, int n, bool iso_first, double
   if (cudaLaunchKernelEx(&cfg, k_pivot_qr, theta, m, n, iso_first ? 1 : 0, Bg, X, cand, cand_i, fpart, info + 2, sync,
                          flag, wait_ns) != cudaSuccess)
     return false;
-  if (cudaMemsetAsync(sync, 0, kSvdSyncInts * sizeof(unsigned), s) != cudaSuccess) return false;
+  if (cudaMemsetAsync(sync, 0, kSvdSyncInts * sizeof(unsigned), s) != cudaSuccess ||
+      cudaMemsetAsync(ver, 0, k * sizeof(unsigned), s) != cudaSuccess)
+    return false;
   cfg.dynamicSmemBytes = 0;
   cfg.blockDim = dim3(kJThreads, 1, 1);
   cfg.gridDim = counted(dim3(std::max(1, std::min((k + 1) / 2, gi.sms * std::min(gi.occ, 2))), 1, 1));
   return cudaLaunchKernelEx(&cfg, k_jacobi_grid<false>, X, (double2*)nullptr, ni, k, (const int*)(info + 2), sigma,
-                            info, sync, flag, jacobi_tol(m, n), kJacMaxSweeps, iso_first ? 0 : 1,
+                            info, sync, ver, flag, jacobi_tol(m, n), kJacMaxSweeps, iso_first ? 0 : 1,
                             wait_ns) == cudaSuccess;
 }
 
@@ -847,7 +853,8 @@ extern "C" ttn_status ttn_svd(const void* a_dev, int32_t m, int32_t n, void* u_d
   const int nc = std::min(m, n);
   if (cudaMemsetAsync(flag, 0, sizeof(int), s) != cudaSuccess) return TTN_ECUDA;
   const double wns = std::min(wait_s, 60.0) * 1e9;
-  if (!launch_jacobi_svd_grid((const double2*)a_dev, m, n, A, V, sigma, info, sync, flag, (uint64_t)wns, s))
+  // the columns' counters lie in U, which is written last
+  if (!launch_jacobi_svd_grid((const double2*)a_dev, m, n, A, V, sigma, info, sync, (unsigned*)u_dev, flag, (uint64_t)wns, s))
     return TTN_ECUDA;
   std::vector<double> sig(nc);
   int hinfo[2] = {0, 0}, hflag = 0;

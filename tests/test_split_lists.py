@@ -88,3 +88,9 @@ def test_workspace_without_room_for_planes(rank, precision, before):
     two-site split's matrices: `before`, the bytes without either, plus the split's
     column counters and pivot candidates (below 32 KiB)."""
     assert workspace_bytes(W.exciton_chain(rank=rank), precision) - before <= 32 << 10
+
+
+def test_the_two_site_split_has_no_room_of_its_own_either():
+    """Its column counters and pivot candidates lie in buffers that are written after them."""
+    for rank, precision, before in [(20, 0, 902682880), (20, 1, 1223671808), (64, 0, 13959593728), (64, 1, 19299940096)]:
+        assert workspace_bytes(W.exciton_chain(rank=rank), precision) <= before
