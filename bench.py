@@ -710,7 +710,7 @@ def bench_ours(args, rank, world, local_rank):
 
     if rank != 0:
         return
-    names = {0: "node/bond application (k_apply)", 1: "environment update", 2: "Householder QR", 3: "other"}
+    names = {0: "node/bond application (k_apply, k_xs_apply)", 1: "environment update", 2: "Householder QR", 3: "other"}
     dom = max(range(4), key=lambda k: prof[k][2])
     n_l, fl, t_ms = prof[dom]
     # the class's share of the summed device time of the replayed step graph
@@ -744,6 +744,8 @@ def bench_ours(args, rank, world, local_rank):
                      "kernel_time": "share of the device time of the replayed step graph (CUDA events recorded "
                                     "as graph nodes, ttn_profile 2) x ms_per_step of the timed run",
                      "kernel_ms_per_step": t_dom / args.steps,
+                     "peak_note": "FP64 results per second against the FP64 pipe; lists of 8 MFLOP and more run on the "
+                                  "tensor cores (exact digit split), so this is no bound where those dominate",
                      "frac_of_nominal_fp64": achieved / FP64_PEAK_TFLOPS,
                      "launches_per_step": n_l / args.steps},
         "node_contraction": {"tflops_kernel": (k1_flops / args.steps) / (share[0] * (ms_max / args.steps) * 1e-3) / 1e12
