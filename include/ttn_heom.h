@@ -102,6 +102,8 @@ typedef struct {
  *                    (no counterpart in the paper: GB300 work distribution).
  *                    Use 1 for instances advanced concurrently by
  *                    ttn_batch_step, which fill the GPU by themselves.
+ *                    FP64 lists then go to the tensor cores from 8 instead
+ *                    of 100 MFLOP.
  *  tensor_cores (1)  mixed form only: run the mode products of large nodes
  *                    (contracted legs <= 64, >= 16384 elements) on the
  *                    tcgen05 tensor cores in 3xTF32 (hi/lo split, FP32

@@ -453,7 +453,7 @@ struct Exec {
   }
   // an FP64 list: large ones on the tensor cores (exact digit split), the others on the CUDA cores
   void apply64(const ApList& L, const Epi& e) {
-    if (xs_applicable(L, p.ap_outs.data(), p.ap_terms.data()) &&
+    if (xs_applicable(L, p.ap_outs.data(), p.ap_terms.data(), h->params.max_split) &&
         launch_apply_xs(h->h_bufs.data(), h->h_mats.data(), L, e, p.ap_outs.data(), p.ap_terms.data(), h->xs_planes,
                         h->xs_elems, h->params.max_split, s))
       return;
@@ -2144,7 +2144,9 @@ ttn_status ttn_autotune(ttn_t h, int32_t reps) {
       if (!f64[i] && h->prec == PREC_F32 && h->params.tensor_cores &&
           tc_applicable(L, p.ap_outs.data(), p.ap_terms.data()))
         continue;
-      if (h->prec == PREC_F64 && h->xs_elems > 0 && xs_applicable(L, p.ap_outs.data(), p.ap_terms.data())) continue;
+      if (h->prec == PREC_F64 && h->xs_elems > 0 &&
+          xs_applicable(L, p.ap_outs.data(), p.ap_terms.data(), h->params.max_split))
+        continue;
       const bool epi = p.ap_outs[L.out_begin].dst < 0;
       const TuneKey key = ap_key(p, L, prec);
       auto seen = done.find(key);

@@ -199,24 +199,18 @@ void launch_tc_embed(void* const* mats32, const TcEmbedJob* jobs, int n, float* 
 // complex values (one-output lists: one plane per leg and term part, at most
 // max_split parts a leg). Returns
 // false (nothing launched) when the scratch is too small.
-// The line: 19x11x11, 8 terms (2.1 MFLOP) 7.2 us on the CUDA cores, 10.4 here (the
-// second launch, the plane sum, is not won back); 16^3, 12 terms (6.3 MFLOP) 12.3 / 9.3;
-// 32x12x12, 12 terms (8.3 MFLOP) 15.8 / 12.0; 20^3, 12 terms (15 MFLOP) 22.9 / 12.9.
-// It lies above the crossing, at 8 MFLOP, and at 40 for nodes beside an open
-// or narrow leg (three legs, one of at most 16), whose gain is a few us a launch:
-// small trees are run at ranks far above the occupied ones, and there a
-// trajectory follows the rounding of the FMA chain (completion of dependent
-// columns): a spin-boson tree of rank 25, depth 11 parts by 5e-8 within 6 steps
-// between the two paths, both within 2e-16 of the exact sums; chains, Table 1
-// and two-site lists stay together to 1e-13. The line does not depend on max_split, so
-// runs that differ in it stay on one path.
-constexpr double kXsMinFlops = 8.0e6, kXsMinFlopsNarrow = 40.0e6;
-constexpr int kXsNarrow = 16;
-inline double xs_min_flops(int d0, int d1, int d2, int d3) {
-  const bool narrow = d0 <= kXsNarrow || d1 <= kXsNarrow || d2 <= kXsNarrow;
-  return d3 == 1 && narrow ? kXsMinFlopsNarrow : kXsMinFlops;
-}
-bool xs_applicable(const ApList& L, const ApOut* outs_host, const ApTerm* terms_host);
+// The line lies where the split still pays with the weak outputs of a run from the
+// product state (xs_apply.cu). ms a step, CUDA cores / split: chains of rank 20 (20^3, 12
+// terms, 15 MFLOP) 12.3 / 15.5, 28 24.2 / 28.9, 32 (100 MFLOP) 34.4 / 36.5, 36 49.5 / 50,
+// 40 69 / 62, 64 288 / 156; trees 32 x 32 x 24 (60 MFLOP) 18.3 / 17.0, 40 x 40 x 24 28.4 /
+// 23.3. From a generic state it pays from 8 MFLOP (rank 20 28.7 / 28.1, 64 300 / 101).
+// Handles that share the GPU (max_split = 1: a tile on one CTA) start at 8 MFLOP: together
+// they are bound by FP64 issue, and 256 instances of rank 8 to 32 make 1444 / 1888
+// steps/s. The two paths agree as two orders of the sums do, so a handle may be on
+// either.
+constexpr double kXsMinFlops = 100.0e6, kXsMinFlopsShared = 8.0e6;
+inline double xs_min_flops(int max_split) { return max_split <= 1 ? kXsMinFlopsShared : kXsMinFlops; }
+bool xs_applicable(const ApList& L, const ApOut* outs_host, const ApTerm* terms_host, int max_split);
 bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L, const Epi& e,
                      const ApOut* outs_host, const ApTerm* terms_host, double2* planes, int64_t plane_elems,
                      int max_split, cudaStream_t s);

@@ -10,9 +10,10 @@
 // enter one f32 accumulator (2d <= 128, digit pairs i + j = g <= 7), so every
 // accumulator is an exact integer below 2^24: the only errors are the two
 // truncations at 2^-62 and the dropped digit pairs i + j > 7, together below
-// 2^-60 of (row maximum x fiber maximum), where a chain of FP64 FMAs loses
-// 2^-53 per addition. 36 digit products replace 64-cycle FMAs by MMAs at
-// 2048 * 592 / (36 * 8.2) = 4.1k multiply-adds per clock against 259 FMAs.
+// 2^-56.8 of (row scale x position scale) for each real product (2^-60 as a root
+// mean square), where a chain of FP64 FMAs loses 2^-53 of the sum per addition. 36
+// digit products replace 64-cycle FMAs by MMAs at 2048 * 592 / (36 * 8.2) = 4.1k
+// multiply-adds per clock against 259 FMAs.
 //
 // One term Y += M x_l X (complex, d = d_l <= 64) is a real GEMM: output index
 // i gives rows i (real part) and i + 8 (imaginary part) of an MMA tile, leg
@@ -20,15 +21,42 @@
 // column. A lane loads the complex values of its own fragment slots from
 // global memory (L1 / L2), so there is no shared-memory staging and no barrier
 // in the term loop; the digits live in registers. A warp owns 8 output indices x
-// 16 positions. Before the split, X[x] of the tile is scaled to equal size over x and
-// the scale moved to operator column x. The operator's fixed point of row i is
-// then set by the largest contribution |M[i][x]| |X[x]| that the row receives, and what is
-// lost stays below 2^-60 of that, as a chain of FMAs loses 2^-53 of it: the small
-// components of a graded state (weights down to 1e-9 and below beside 1) keep
-// their relative accuracy, also where the operator couples them to themselves
-// by 1 and to the large ones by 1e-9. (With the columns of M scaled to equal size
-// instead, a rank-20 chain's bond directions of weight 1e-9 differed by 2e-9
-// from the FMA chain after 30 steps.)
+// 16 positions.
+//
+// Scales. X[x] of the tile is scaled to equal size over x and the scale moved to
+// operator column x. The operator's fixed point of row i is then set by the
+// largest |M[i][x]| S[x], S[x] = max_n |X[x][n]| over the tile's 16 positions, the
+// tensor's of position n by its largest scaled element |X[x][n]| / S[x]. Where the
+// grading is a row factor times a position factor these are the size of the output's own
+// largest product. (With the columns of M scaled to equal size instead, a
+// rank-20 chain's bond directions of weight 1e-9 differed by 2e-9 from the FMA chain
+// after 30 steps.)
+//
+// Weak outputs. Otherwise row and position may reach their scales at different x,
+// and an output that is small against both would keep few digits of its own: 1e-6
+// for a row that sees only x = 0 at a position where X[0] is 1e-12 of S[0]. A run from
+// the product state is full of them (padded directions), and they decide its weakly
+// occupied directions: without what follows the nodes of chains of rank 20 to 32 were
+// 6e-7 to 5e-6 from the FMA chain's after 20 to 60 steps and as far from those of
+// another max_split (the chain's, in another order of sums: 1e-13 to 2e-11), rho up to
+// 1e-12 (1e-17). So the products' magnitudes are summed too (powers of two, two MMAs
+// per 8 x), and an output below kXsWeak of the scales is made from the operands by
+// FMAs: nodes within 4e-14 to 1e-11 again. (Only where the row's scale also exceeds the position's
+// largest output by 2^12, 2^16, 2^20: cheaper, but up to 2e-4 away.)
+// What the split keeps is within 2 d 2^-44.8 sum |a b| of the exact sum whatever
+// the operands. Largest and root mean square error over sum |a b| in units of 2^-53
+// over the 64^3 outputs of a product, chain / split: flat operands 1.5, 0.22 / 0.38,
+// 0.07; graded as the perf cases' states 6.6, 1.0 / 2.1, 0.29; tensor 10^(-0.6 |x - n|)
+// 8.0, 1.0 / 9.3, 0.36; operator 1 + 1e-9 G on a graded tensor 7.1, 1.2 / 38, 0.42; rows
+// that see what is small 1.8, 0.40 / 2.2, 0.31 (4e10, 4e8 without). One output's
+// parts are not told apart: a part that is small beside the other is as accurate as
+// the other.
+// Cost: from a generic state, where 3e-4 of the outputs are below 2^-8 and none below
+// 2^-12, the check alone (rank-64 chain 100.0 -> 101.4 ms; at 2^-8 102.3); in a run from the
+// product state a third of the work at rank 64 (94 -> 156 ms, FMA chain 288), more
+// than the split gives at rank 20; hence the line (xs_min_flops). Sharing the weak outputs
+// of a CTA among its warps at the end, or leaving out the MMAs of warps that have no
+// others, is no cheaper.
 //
 // A non-finite operand makes its whole row or column of outputs NaN.
 //
@@ -61,6 +89,9 @@ constexpr int kXsNT = 2;              // n tiles (8 positions) per warp
 constexpr int kXsCols = 8 * kXsNT;    // positions per warp
 constexpr int kXsTermSplit = 2;       // more terms than this on a leg: the warp groups split the terms
 constexpr int kXsMaxD = 64;           // 2 d <= 128: exactness of the f32 accumulators
+// An output whose products sum to less than this of row scale x position scale is
+// made by FP64 multiply-adds (weak outputs, above).
+constexpr float kXsWeak = 1.0f / 4096;
 constexpr unsigned kFull = 0xffffffffu;
 
 __device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
@@ -70,8 +101,23 @@ __device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], u
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// The same with 8 rows (the other 8 zero) and 8 K positions, for the magnitudes.
+__device__ __forceinline__ void mma_f16_k8(float (&c)[4], uint32_t a, uint32_t b) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a), "r"(0), "r"(b));
+}
+
 __device__ __forceinline__ int exp_field(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
 __device__ __forceinline__ int exp_c(double2 v) { return max(exp_field(v.x), exp_field(v.y)); }
+__device__ __forceinline__ uint32_t pack2(int lo, int hi) { return (uint32_t)lo | ((uint32_t)hi << 16); }
+__device__ __forceinline__ uint32_t both(int v) { return (uint32_t)(v & 0xffff) * 0x10001u; }
+__device__ __forceinline__ uint32_t nonzero2(uint32_t e) { return __vminu2(e, 0x00010001u) * 0xffffu; }  // mask of 16-bit halves
+// two exponents e <= 0 as f16x2 magnitudes 2^(e + 15), e at least -29; 0 where the mask is
+__device__ __forceinline__ uint32_t magnitudes(uint32_t e, uint32_t mask) {
+  return (__vmaxs2(__vadd2(e, both(30)), 0x00010001u) & mask) << 10;
+}
 
 // v as a fixed-point integer with 62 bits below 2^(top + 1 - 1023), plus the
 // bias that turns its bytes into digits - 128 .. 127 offset by 128. Subnormal v
@@ -148,6 +194,8 @@ struct XsGroup {
                     //   [16] largest scaled tensor exponent of every position, offset by kXsBias
                     //   [16] largest raw tensor exponent (0x7ff: not finite)
   uint4* bd;        // [MT][8][32] digits: x, y = K halves of positions 0..7, z, w = of positions 8..15
+  uint2* be;        // [MT][32] magnitudes of the same values: x of positions 0..7, y of 8..15, f16x2 of the K halves
+  uint8_t* weak;    // [128] this warp's list of weak outputs
 };
 struct XsSrc {
   const double2* a;  // operator row of this lane, or null
@@ -158,6 +206,69 @@ __device__ __forceinline__ void gsync(const XsGroup& G) {
     __syncwarp();
   else
     asm volatile("bar.sync %0, %1;" ::"r"(G.bar), "r"(32 * G.MT) : "memory");
+}
+
+// The outputs of the masks `weak` (bit 2 t + j of a lane: row lane >> 2, position
+// 8 t + 2 (lane & 3) + j) by FP64 multiply-adds, into add. The warp lists them and takes
+// up to 32 at a time, 32 / (their number) lanes each, so a few cost the latency of a
+// short chain (four at a time, without a list: 4 % of a rank-20 chain's step more).
+// Not inlined: its registers would be the product's spills (300 bytes against 208;
+// rank-64 chain 102.8 ms against 101.4).
+template <bool PROJ, typename KA, typename KB>
+__device__ __noinline__ void weak_sums(uint8_t* list, const double2* sa, const double2* sb0, const double2* sb1, int K,
+                                       KA ka, KB kb, uint32_t weak, double* add) {
+  const int lane = threadIdx.x & 31, cnt = __popc(weak);
+  int end = cnt;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(kFull, end, o);
+    if (lane >= o) end += v;
+  }
+  const int total = __shfl_sync(kFull, end, 31), off = end - cnt;
+  __syncwarp();  // the previous product's list is done with
+#pragma unroll 1
+  for (uint32_t w = weak, q = off; w != 0; w &= w - 1, ++q) list[q] = (uint8_t)(lane << 2 | (__ffs(w) - 1));
+  __syncwarp();
+#pragma unroll 1
+  for (int base = 0; base < total;) {
+    const int rem = total - base, lg = max(0, __clz(rem - 1) - 27), nb = 32 >> lg;
+    const int slot = lane >> lg, L = 1 << lg;
+    const bool on = slot < rem;
+    const int code = on ? list[base + slot] : 0;
+    const int from = code >> 2, t = code >> 1 & 1, pos = (2 * (from & 3) + (code & 1)) * 4;
+    const double2* a = (const double2*)__shfl_sync(kFull, (unsigned long long)sa, from);
+    const double2* b0 = (const double2*)__shfl_sync(kFull, (unsigned long long)sb0, pos);
+    const double2* b1 = (const double2*)__shfl_sync(kFull, (unsigned long long)sb1, pos);
+    const double2* b = t == 0 ? b0 : b1;
+    double x = 0.0, y = 0.0;
+#pragma unroll 2
+    for (int k = lane & (L - 1); on && k < K; k += L) {
+      const double2 u = a[ka(k)];
+      double2 v = b[kb(k)];
+      if (PROJ) v.y = -v.y;
+      x = fma(u.x, v.x, fma(-u.y, v.y, x));
+      y = fma(u.x, v.y, fma(u.y, v.x, y));
+    }
+#pragma unroll 1
+    for (int o = L >> 1; o > 0; o >>= 1) {
+      x += __shfl_xor_sync(kFull, x, o);
+      y += __shfl_xor_sync(kFull, y, o);
+    }
+    int q = off - base;
+#pragma unroll
+    for (int e = 0; e < 2 * kXsNT; ++e) {  // back to the owners
+      const int at = (q & (nb - 1)) << lg;
+      const double gx = __shfl_sync(kFull, x, at), gy = __shfl_sync(kFull, y, at);
+      if (weak >> e & 1u) {
+        if (q >= 0 && q < nb) {
+          add[2 * e] += gx;
+          add[2 * e + 1] += gy;
+        }
+        ++q;
+      }
+    }
+    base += nb;
+  }
 }
 
 // acc += block product. PROJ: conj(B) instead of B.
@@ -196,7 +307,7 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, int turn, const XsSrc
   for (int t = 0; t < kXsNT; ++t) {
     eb[t][0] = exp_c(braw[t][0]);
     eb[t][1] = exp_c(braw[t][1]);
-    xr = __vmaxu2(xr, (uint32_t)eb[t][0] | ((uint32_t)eb[t][1] << 16));
+    xr = __vmaxu2(xr, pack2(eb[t][0], eb[t][1]));
   }
   xr = __vmaxu2(xr, __shfl_xor_sync(kFull, xr, 4));
   xr = __vmaxu2(xr, __shfl_xor_sync(kFull, xr, 8));
@@ -223,33 +334,55 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, int turn, const XsSrc
   gsync(G);  // also: every warp is done with the previous product's scales and digits
   for (int e = 64 + G.m * 32 + lane; e < 96; e += 32 * G.MT) G.sc[96 * ((turn & 1) ^ 1) + e] = 0;
   // 2: row scale of the scaled operator; tensor digits of this warp's K positions
-  int row = -kXsBias, rraw = 0;
+  uint32_t rowp = 0, rawp = 0;
 #pragma unroll
   for (int ks = 0; ks < 8; ++ks)
     if (ks < KS) {
-      const int e0 = ep[ks] & 0xffff, e1 = ep[ks] >> 16;
-      const int x0 = scx[ks * 8 + kq], x1 = scx[ks * 8 + 4 + kq];
-      if (e0 && x0) row = max(row, e0 + x0);
-      if (e1 && x1) row = max(row, e1 + x1);
-      rraw = max(rraw, max(e0, e1));
+      const uint32_t x = pack2(scx[ks * 8 + kq], scx[ks * 8 + 4 + kq]);
+      rawp = __vmaxu2(rawp, ep[ks]);
+      ep[ks] = (ep[ks] + x) & nonzero2(ep[ks]) & nonzero2(x);  // exponents of the scaled operator
+      rowp = __vmaxu2(rowp, ep[ks]);
     }
+  int row = max((int)(rowp & 0xffff), (int)(rowp >> 16)), rraw = max((int)(rawp & 0xffff), (int)(rawp >> 16));
+  if (row == 0) row = -kXsBias;
   row = max(row, __shfl_xor_sync(kFull, row, 1));
   row = max(row, __shfl_xor_sync(kFull, row, 2));
   rraw = max(rraw, __shfl_xor_sync(kFull, rraw, 1));
   rraw = max(rraw, __shfl_xor_sync(kFull, rraw, 2));
   {
-    uint32_t d[kXsNT][2][8];
+    uint32_t d[kXsNT][2][8], q[kXsNT];
 #pragma unroll
     for (int t = 0; t < kXsNT; ++t) {
       const int top = scol[8 * t + (lane >> 2)] - kXsBias;
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf) digits8(braw[t][hf], top + xk[hf], d[t][hf]);
+      const uint32_t e = pack2(eb[t][0], eb[t][1]);
+      q[t] = magnitudes(__vsub2(__vsub2(e, xr), both(top)), nonzero2(e));
     }
+    G.be[G.m * 32 + lane] = make_uint2(q[0], q[1]);
 #pragma unroll
     for (int j = 0; j < 8; ++j) G.bd[(G.m * 8 + j) * 32 + lane] = make_uint4(d[0][0][j], d[0][1][j], d[1][0][j], d[1][1][j]);
   }
   gsync(G);
-  // 3: operator digits and MMAs
+  // 3: this lane's weak outputs (bit 2 t + j: row lane >> 2, position 8 t + 2 kq + j)
+  uint32_t weak = 0;
+  {
+    float s[kXsNT][4] = {};
+#pragma unroll
+    for (int ks = 0; ks < 8; ++ks)
+      if (ks < KS) {
+        const uint32_t a = magnitudes(__vsub2(ep[ks], both(row)), nonzero2(ep[ks]));
+        const uint2 b = G.be[ks * 32 + lane];
+        mma_f16_k8(s[0], a, b.x);
+        mma_f16_k8(s[1], a, b.y);
+      }
+#pragma unroll
+    for (int t = 0; t < kXsNT; ++t)
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+        if (s[t][j] > 0.f && s[t][j] < kXsWeak * 0x1p30f) weak |= 1u << (2 * t + j);
+  }
+  // 4: operator digits and MMAs
   float c[kXsNT][8][4];
 #pragma unroll
   for (int t = 0; t < kXsNT; ++t)
@@ -297,6 +430,8 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, int turn, const XsSrc
       const int ex = row + ec - kXsBias;  // no scale: the sums are zero, and 2^0 keeps join() off its slow path
       const bool none = row < 0 || ec == 0;
       const bool bad = rraw == 0x7ff || scraw[n] == 0x7ff;
+      if (bad) weak &= ~(1u << (2 * t + j));
+      if (weak >> (2 * t + j) & 1u) continue;
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
         float cc[8];
@@ -308,6 +443,14 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, int turn, const XsSrc
                                 : join(cc, none ? 0 : ex - 2 * 1084 + 56, acc[t][2 * j + p]);
       }
     }
+  if (__any_sync(kFull, weak != 0)) {
+    double add[4 * kXsNT] = {};
+    weak_sums<PROJ>(G.weak, S.a, S.b[0], S.b[1], K, ka, kb, weak, add);
+#pragma unroll
+    for (int t = 0; t < kXsNT; ++t)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[t][q] += add[4 * t + q];
+  }
 }
 
 // Leg geometry: element = outer * (d * inner) + x * inner + in, position n = outer * inner + in.
@@ -351,6 +494,8 @@ struct XsWork {
 // (one 16-position tile per group, no sum).
 __global__ void __launch_bounds__(kXsThreads, 2) k_xs_apply(const __grid_constant__ XsWork w) {
   __shared__ __align__(16) uint4 sm_bd[kXsWarps * 8 * 32];  // digits; the groups' sums at the end
+  __shared__ uint2 sm_be[kXsWarps * 32];
+  __shared__ uint8_t sm_weak[kXsWarps][128];
   __shared__ int sm_sc[kXsWarps][2 * 96];
   double2(*red)[kXsCols * 8] = reinterpret_cast<double2(*)[kXsCols * 8]>(sm_bd);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -387,7 +532,7 @@ __global__ void __launch_bounds__(kXsThreads, 2) k_xs_apply(const __grid_constan
 #pragma unroll
     for (int r = 0; r < 4; ++r) acc[t][r] = 0.0;
   const int i = mt * 8 + (lane >> 2);
-  const XsGroup gp{mt, MT, 1 + grp, sm_sc[grp], sm_bd + (size_t)grp * MT * 8 * 32};
+  const XsGroup gp{mt, MT, 1 + grp, sm_sc[grp], sm_bd + (size_t)grp * MT * 8 * 32, sm_be + (size_t)grp * MT * 32, sm_weak[wid]};
   for (int e = threadIdx.x; e < kXsWarps * 2 * 96; e += kXsThreads) sm_sc[0][e] = 0;
   __syncthreads();
   if (on) {
@@ -536,6 +681,8 @@ struct XsPj {
 };
 __global__ void __launch_bounds__(kXsThreads, 2) k_xs_project(const __grid_constant__ XsPj w) {
   __shared__ __align__(16) uint4 sm_bd[kXsWarps * 8 * 32];
+  __shared__ uint2 sm_be[kXsWarps * 32];
+  __shared__ uint8_t sm_weak[kXsWarps][128];
   __shared__ int sm_sc[kXsWarps][2 * 96];
   __shared__ double2 tot[kXsWarps * kXsCols * 8];  // this CTA's 8 MT x 16 tile
   double2(*red)[kXsCols * 8] = reinterpret_cast<double2(*)[kXsCols * 8]>(sm_bd);
@@ -545,7 +692,7 @@ __global__ void __launch_bounds__(kXsThreads, 2) k_xs_project(const __grid_const
   const int MT = (g.d + 7) >> 3, G = kXsWarps / MT;
   const int mt = wid % MT, grp = wid / MT;
   const int rank = blockIdx.x % w.KS, tile = blockIdx.x / w.KS, o = blockIdx.y;
-  const XsGroup gp{mt, MT, 1 + grp, sm_sc[grp], sm_bd + (size_t)grp * MT * 8 * 32};
+  const XsGroup gp{mt, MT, 1 + grp, sm_sc[grp], sm_bd + (size_t)grp * MT * 8 * 32, sm_be + (size_t)grp * MT * 32, sm_weak[wid]};
   for (int e = threadIdx.x; e < kXsWarps * 2 * 96; e += kXsThreads) sm_sc[0][e] = 0;
   __syncthreads();
   double acc[kXsNT][4];
@@ -632,7 +779,7 @@ int sm_count() {
 // has room for (everything else stays on the CUDA-core kernel and its tile
 // shapes, so ttn_autotune asks here too), and enough multiply-adds that the CUDA-core kernel
 // would be bound by FP64 issue instead of by its launch.
-bool xs_applicable(const ApList& L, const ApOut* outs, const ApTerm* terms) {
+bool xs_applicable(const ApList& L, const ApOut* outs, const ApTerm* terms, int max_split) {
   if (L.n_tiles <= 0) return false;
   const ApOut& f = outs[L.out_begin];
   const int64_t P = (int64_t)f.d0 * f.d1 * f.d2 * f.d3;
@@ -650,7 +797,7 @@ bool xs_applicable(const ApList& L, const ApOut* outs, const ApTerm* terms) {
       if (!tm.pad) dense += 8.0 * P * dd[tm.leg];
     }
   }
-  return dense >= xs_min_flops(f.d0, f.d1, f.d2, f.d3);
+  return dense >= xs_min_flops(max_split);
 }
 
 bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L, const Epi& e, const ApOut* outs,
@@ -767,7 +914,7 @@ bool launch_project_xs(double2* const* bufs, double2* const* mats, const PjList&
   const int n = L.out_end - L.out_begin;
   if (n < 1 || n > kXsMaxPj) return false;
   const PjOut& f = pjs[L.out_begin];
-  if (L.flops < xs_min_flops(f.d0, f.d1, f.d2, 1)) return false;
+  if (L.flops < xs_min_flops(max_split)) return false;
   const int dd[3] = {f.d0, f.d1, f.d2}, d = dd[f.leg];
   const int64_t P = (int64_t)f.d0 * f.d1 * f.d2;
   if (d > kXsMaxD || d < 8 || P >= (int64_t)1 << 30) return false;

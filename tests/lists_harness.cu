@@ -65,7 +65,7 @@ int lists() {
   const int64_t planes = std::max<int64_t>(4 * std::max(p.P_cap_max, p.theta_cap), std::min<int64_t>(24 * p.P_cap_max, 1 << 20));
   for (const ApList& L : p.ap_lists) {
     const ApOut& f = p.ap_outs[L.out_begin];
-    const bool ok = xs_applicable(L, p.ap_outs.data(), p.ap_terms.data());
+    const bool ok = xs_applicable(L, p.ap_outs.data(), p.ap_terms.data(), 1);  // the lower line claims the most lists
     const Epi store{EPI_STORE, nullptr, nullptr, nullptr, nullptr, 0.0};
     const bool done = ok && launch_apply_xs(bufs.data(), mats.data(), L, store, p.ap_outs.data(), p.ap_terms.data(),
                                             nullptr, planes, max_split, nullptr);
