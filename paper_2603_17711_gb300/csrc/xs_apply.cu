@@ -58,7 +58,8 @@
 // of a CTA among its warps at the end, or leaving out the MMAs of warps that have no
 // others, is no cheaper.
 //
-// A non-finite operand makes its whole row or column of outputs NaN.
+// A non-finite operand makes its whole row or column of outputs NaN; it sets no
+// scale, so the outputs beside them are what they are without it.
 //
 // Measured (graph replay, CUDA-core kernel / this one): 64^3 node, 14 terms
 // 1799 / 244 us (7.7 TFLOP/s of FP64 results against the 1.1 of the FP64 pipe;
@@ -111,6 +112,8 @@ __device__ __forceinline__ void mma_f16_k8(float (&c)[4], uint32_t a, uint32_t b
 
 __device__ __forceinline__ int exp_field(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
 __device__ __forceinline__ int exp_c(double2 v) { return max(exp_field(v.x), exp_field(v.y)); }
+// an exponent that sets a scale: not of a zero, and not of a non-finite value
+__device__ __forceinline__ bool scales(int e) { return (unsigned)(e - 1) < 0x7feu; }
 __device__ __forceinline__ uint32_t pack2(int lo, int hi) { return (uint32_t)lo | ((uint32_t)hi << 16); }
 __device__ __forceinline__ uint32_t both(int v) { return (uint32_t)(v & 0xffff) * 0x10001u; }
 __device__ __forceinline__ uint32_t nonzero2(uint32_t e) { return __vminu2(e, 0x00010001u) * 0xffffu; }  // mask of 16-bit halves
@@ -307,7 +310,7 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, int turn, const XsSrc
   for (int t = 0; t < kXsNT; ++t) {
     eb[t][0] = exp_c(braw[t][0]);
     eb[t][1] = exp_c(braw[t][1]);
-    xr = __vmaxu2(xr, pack2(eb[t][0], eb[t][1]));
+    xr = __vmaxu2(xr, pack2(scales(eb[t][0]) ? eb[t][0] : 0, scales(eb[t][1]) ? eb[t][1] : 0));
   }
   xr = __vmaxu2(xr, __shfl_xor_sync(kFull, xr, 4));
   xr = __vmaxu2(xr, __shfl_xor_sync(kFull, xr, 8));
@@ -319,7 +322,7 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, int turn, const XsSrc
     int c = 0, r = 0;
 #pragma unroll
     for (int hf = 0; hf < 2; ++hf) {
-      if (eb[t][hf]) c = max(c, eb[t][hf] - xk[hf] + kXsBias);
+      if (scales(eb[t][hf])) c = max(c, eb[t][hf] - xk[hf] + kXsBias);
       r = max(r, eb[t][hf]);
     }
     c = max(c, __shfl_xor_sync(kFull, c, 1));
@@ -340,7 +343,8 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, int turn, const XsSrc
     if (ks < KS) {
       const uint32_t x = pack2(scx[ks * 8 + kq], scx[ks * 8 + 4 + kq]);
       rawp = __vmaxu2(rawp, ep[ks]);
-      ep[ks] = (ep[ks] + x) & nonzero2(ep[ks]) & nonzero2(x);  // exponents of the scaled operator
+      const uint32_t fin = pack2(scales(ep[ks] & 0xffff) ? 0xffff : 0, scales(ep[ks] >> 16) ? 0xffff : 0);
+      ep[ks] = (ep[ks] + x) & fin & nonzero2(x);  // exponents of the scaled operator
       rowp = __vmaxu2(rowp, ep[ks]);
     }
   int row = max((int)(rowp & 0xffff), (int)(rowp >> 16)), rraw = max((int)(rawp & 0xffff), (int)(rawp >> 16));
@@ -356,7 +360,7 @@ __device__ __forceinline__ void xs_block(const XsGroup& G, int turn, const XsSrc
       const int top = scol[8 * t + (lane >> 2)] - kXsBias;
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf) digits8(braw[t][hf], top + xk[hf], d[t][hf]);
-      const uint32_t e = pack2(eb[t][0], eb[t][1]);
+      const uint32_t e = pack2(scales(eb[t][0]) ? eb[t][0] : 0, scales(eb[t][1]) ? eb[t][1] : 0);
       q[t] = magnitudes(__vsub2(__vsub2(e, xr), both(top)), nonzero2(e));
     }
     G.be[G.m * 32 + lane] = make_uint2(q[0], q[1]);

@@ -135,6 +135,27 @@ def test_powers_of_two_and_zeros(harness):
     assert not y[:, 5].any() and y[:, 4].all()
 
 
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf, complex(0.0, np.inf)])
+def test_what_is_not_finite_spreads(harness, bad):
+    """A non-finite operand makes the outputs that it enters non-finite, and leaves the others as they are."""
+    dims, rng = (41, 29, 30), np.random.default_rng(6)
+    M, X = cnormal(rng, (41, 41)), cnormal(rng, dims)
+    M[9, 2] = X[7, 3, 11] = 0.0
+    good = call(harness, 0, dims, [0], [M, X], dims)
+    X[7, 3, 11] = bad
+    y = call(harness, 0, dims, [0], [M, X], dims)
+    hit = np.zeros(dims, bool)
+    hit[:, 3, 11] = True
+    assert np.array_equal(~np.isfinite(y), hit)
+    assert np.array_equal(y[~hit], good[~hit])
+    X[7, 3, 11] = 0.0
+    M[9, 2] = bad
+    y = call(harness, 0, dims, [0], [M, X], dims)
+    hit = np.broadcast_to((np.arange(41) == 9)[:, None, None], dims)
+    assert np.array_equal(~np.isfinite(y), hit)
+    assert np.array_equal(y[~hit], good[~hit])
+
+
 @pytest.mark.parametrize("args,steps", [(dict(n_sites=3, rank=28, depth=8), 10), (dict(n_sites=4, rank=32, depth=8), 20)])
 def test_a_run_keeps_its_weak_directions(args, steps):
     """From the product state on the tensor cores (max_split 1: lists from 8 MFLOP) and
