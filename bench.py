@@ -45,7 +45,7 @@ METRIC = "HEOM-TTN steps/s & node-contraction TFLOP/s vs plain FP64 at RDM err <
 FP64_PEAK_TFLOPS = 1.25  # nominal GB300 FP64 (152 SMs x 2 FP64 FMA/clk/SM x ~2.07 GHz)
 WORKLOAD = "7-site Frenkel exciton chain, 21 features (1 Drude + 2 Pade per site), depth 8, BTT, rank 20, ps1, dt 0.05 fs"
 L2_FLUSH_BYTES = 256 << 20  # > 129 MB L2
-APPLY_DRAM_BYTES = 283730   # ncu: mean DRAM bytes (read + write) per contraction launch of one timed step
+APPLY_DRAM_BYTES = 232246   # ncu: mean DRAM bytes (read + write) per contraction launch of one timed step
 
 
 def workload():
@@ -736,16 +736,16 @@ def bench_ours(args, rank, world, local_rank):
         "roofline": {"bound": "alu", "kernel": names[dom], "achieved": achieved,
                      "peak": fp64_peak, "unit": "TFLOP/s", "frac": achieved / fp64_peak,
                      "traffic": APPLY_DRAM_BYTES if names[dom].startswith("node/bond") else None,
-                     "traffic_source": "mean dram__bytes_read+write per launch over the 940 k_apply, k_xs_apply and "
-                                       "k_xs_epilogue launches of one timed step, ncu (1 pass; caches flushed before each launch) "
+                     "traffic_source": "mean dram__bytes_read+write per launch over the 854 k_apply launches of one "
+                                       "timed step, ncu (1 pass; caches flushed before each launch) "
                                        "(profiles/apply_traffic_exciton7_r20_fp64.md)",
                      "peak_source": "FP64 torch.matmul 4096^3 measured in this run (peaks.fp64_tflops); "
                                     "nominal FP64 is %.2f" % FP64_PEAK_TFLOPS,
                      "kernel_time": "share of the device time of the replayed step graph (CUDA events recorded "
                                     "as graph nodes, ttn_profile 2) x ms_per_step of the timed run",
                      "kernel_ms_per_step": t_dom / args.steps,
-                     "peak_note": "FP64 results per second against the FP64 pipe; lists of 8 MFLOP and more run on the "
-                                  "tensor cores (exact digit split), so this is no bound where those dominate",
+                     "peak_note": "FP64 results per second against the FP64 pipe; lists of 100 MFLOP and more run on the "
+                                  "tensor cores (exact digit split; none at this size), where this is no bound",
                      "frac_of_nominal_fp64": achieved / FP64_PEAK_TFLOPS,
                      "launches_per_step": n_l / args.steps},
         "node_contraction": {"tflops_kernel": (k1_flops / args.steps) / (share[0] * (ms_max / args.steps) * 1e-3) / 1e12

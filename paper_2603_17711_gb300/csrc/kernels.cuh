@@ -205,7 +205,7 @@ void launch_tc_embed(void* const* mats32, const TcEmbedJob* jobs, int n, float* 
 // 40 69 / 62, 64 288 / 156; trees 32 x 32 x 24 (60 MFLOP) 18.3 / 17.0, 40 x 40 x 24 28.4 /
 // 23.3. From a generic state it pays from 8 MFLOP (rank 20 28.7 / 28.1, 64 300 / 101).
 // Handles that share the GPU (max_split = 1: a tile on one CTA) start at 8 MFLOP: together
-// they are bound by FP64 issue, and 256 instances of rank 8 to 32 make 1444 / 1888
+// they are bound by FP64 issue, and 256 instances of rank 8 to 32 make 1444 / 1952
 // steps/s. The two paths agree as two orders of the sums do, so a handle may be on
 // either.
 constexpr double kXsMinFlops = 100.0e6, kXsMinFlopsShared = 8.0e6;
@@ -217,8 +217,9 @@ bool launch_apply_xs(double2* const* bufs, double2* const* mats, const ApList& L
 // FP64 projections on the same path; false (nothing launched) below
 // xs_min_flops or when the list does not qualify (all outputs alike, 8 <= bond
 // <= 64, at most 96 outputs).
-// Measured: 64-wide bond, 4096 positions, 5 classes 447 us (FP64 pipe) -> 172;
-// 56 classes' worth of the rank-64 chain's step 30.2 -> 9.9 ms.
+// Measured without the check for weak outputs: 64-wide bond, 4096 positions, 5
+// classes 447 us (FP64 pipe) -> 172; 56 classes' worth of the rank-64 chain's step
+// 30.2 -> 9.9 ms.
 bool launch_project_xs(double2* const* bufs, double2* const* mats, const PjList& L, const PjOut* pjs_host,
                        int max_split, cudaStream_t s);
 void launch_project(int prec, const DevTables& T, const HostTables& H, const PjList& L, cudaStream_t s);
@@ -370,12 +371,12 @@ __device__ __forceinline__ double warp_sum4(double v0, double v1, double v2, dou
   return k;
 }
 // The same SVD spread over several CTAs (svd.cu): pairs of a circle-method
-// round dealt to the CTAs, one barrier per round -- the hardware barrier of
-// one thread-block cluster for up to 2 * kJacClusterMax columns, else a grid
-// barrier of one cooperative launch. Used when the smaller side has more than
-// kJacOneCtaMaxCols columns (else the one-CTA kernel). sync: kSvdSyncInts device
-// ints, ver: min(m, n) more (both cleared by the launch); a grid wait longer than wait_ns sets bit 4 (16)
-// of *flag. Same outputs as launch_jacobi_svd.
+// round dealt to the CTAs; up to 2 * kJacClusterMax columns one thread-block
+// cluster with a hardware barrier per round, else one cooperative launch whose CTAs
+// hand the columns over one by one and meet once a sweep. Used when the smaller side has
+// more than kJacOneCtaMaxCols columns (else the one-CTA kernel). sync: kSvdSyncInts
+// device ints, ver: min(m, n) more (both cleared by the launch); a grid wait longer
+// than wait_ns sets bit 4 (16) of *flag. Same outputs as launch_jacobi_svd.
 constexpr int kJacOneCtaMaxCols = 16;
 constexpr int kJacClusterMax = 16;
 constexpr int kSvdSyncInts = 128;  // barrier and sweep counters

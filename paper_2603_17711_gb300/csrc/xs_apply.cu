@@ -61,7 +61,8 @@
 // A non-finite operand makes its whole row or column of outputs NaN; it sets no
 // scale, so the outputs beside them are what they are without it.
 //
-// Measured (graph replay, CUDA-core kernel / this one): 64^3 node, 14 terms
+// Measured without the check for weak outputs (graph replay, CUDA-core kernel /
+// this one): 64^3 node, 14 terms
 // 1799 / 244 us (7.7 TFLOP/s of FP64 results against the 1.1 of the FP64 pipe;
 // the tensor pipe is half busy, the rest is operand latency and digit
 // arithmetic); 20^3, 12 terms 22.9 / 12.9 us; 20x25x25, 12 terms 38.4 / 16.8 us.
